@@ -9,6 +9,7 @@
 #include "hla_common.cuh"
 #include "hla_simt.cuh"
 #include "hla_tc.cuh"
+#include "hla_simt_tiled.cuh"
 #include "hla_tc_phi.cuh"
 #include "hla_tc_fused.cuh"
 #include "hla_tc_fused_k.cuh"
@@ -171,8 +172,33 @@ hla_status simt_phi_backward(hla_ctx* c, const void* Q, const void* K, void* dQ,
     return HLA_OK;
 }
 
+// The arguments of the tiled kernels that both directions share.
+simt::TiledArgs tiled_args(const hla_ctx* c, const void* Q, const void* K, const void* V, char* ws) {
+    simt::TiledArgs a{};
+    const bool mlp = c->cfg.phi == HLA_PHI_MLP;
+    a.D = c->D;
+    a.BH = c->BH;
+    a.Q = Q; a.K = K; a.V = V;
+    a.qf_out = mlp ? reinterpret_cast<float*>(ws + c->L.qf) : nullptr;
+    a.kf_out = mlp ? reinterpret_cast<float*>(ws + c->L.kf) : nullptr;
+    a.qf = mlp ? a.qf_out : static_cast<const float*>(Q);
+    a.kf = mlp ? a.kf_out : static_cast<const float*>(K);
+    a.part = reinterpret_cast<float*>(ws + c->off_part);
+    a.state = reinterpret_cast<float*>(ws + c->L.state);
+    a.dstate = reinterpret_cast<float*>(ws + c->L.dstate);
+    a.eta = reinterpret_cast<float*>(ws + c->L.eta);
+    a.phi_q = mlp ? &c->phi_q : nullptr;
+    a.phi_k = mlp ? c->phi_k : nullptr;
+    return a;
+}
+
 template <typename T>
 hla_status forward_simt(hla_ctx* c, const void* Q, const void* K, const void* V, void* O, char* ws, cudaStream_t st) {
+    if (simt::tiled(c->D)) {
+        simt::TiledArgs a = tiled_args(c, Q, K, V, ws);
+        a.Oout = O;
+        return simt::run_tiled<T>(a, true, c->rec) ? HLA_OK : HLA_ERR_CUDA;
+    }
     const float *qf, *kf;
     if (c->cfg.phi == HLA_PHI_MLP) {
         hla_status s = simt_phi_forward<T>(c, Q, K, ws, st);
@@ -190,6 +216,14 @@ template <typename T>
 hla_status backward_simt(hla_ctx* c, const void* Q, const void* K, const void* V, const void* O, const void* dO, void* dQ,
                          void* dK, void* dV, char* ws, cudaStream_t st) {
     const bool mlp = c->cfg.phi == HLA_PHI_MLP;
+    if (simt::tiled(c->D)) {
+        simt::TiledArgs a = tiled_args(c, Q, K, V, ws);
+        a.O = O; a.dO = dO;
+        a.dQ = dQ; a.dK = dK; a.dV = dV;
+        a.dqf = mlp ? reinterpret_cast<float*>(ws + c->L.dqf) : static_cast<float*>(dQ);
+        a.dkf = mlp ? reinterpret_cast<float*>(ws + c->L.dkf) : static_cast<float*>(dK);
+        return simt::run_tiled<T>(a, false, c->rec) ? HLA_OK : HLA_ERR_CUDA;
+    }
     const float* qf = mlp ? reinterpret_cast<const float*>(ws + c->L.qf) : static_cast<const float*>(Q);
     const float* kf = mlp ? reinterpret_cast<const float*>(ws + c->L.kf) : static_cast<const float*>(K);
     float* dqf = mlp ? reinterpret_cast<float*>(ws + c->L.dqf) : static_cast<float*>(dQ);
@@ -285,7 +319,7 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
                 if (score > best + 1e-9) { best = score; S = cand; }
             }
         } else {
-            S = (2 * x->sm_count + x->BH - 1) / x->BH;
+            S = simt::tiled(D) ? simt::tiled_splits(x->BH, c.N, P, x->sm_count) : (2 * x->sm_count + x->BH - 1) / x->BH;
         }
     }
     if (S > tiles) S = tiles;

@@ -1,0 +1,675 @@
+// fp32 kernels for the paper's two geometries, (F, d_phi) = (3, 6) and (2, 12), at any head width d <= 128, d % 4 == 0: register-tiled
+// products on the FMA units (fp32 inputs, and bf16 inputs of widths the tensor-core kernels do not take).  The kernels of hla_simt.cuh
+// serve the other geometries.
+//
+// What bounds them is the FMA pipe, so each product is a tile of 8 tokens (or state rows) x 4 columns per thread that reads 16 bytes
+// at a time from shared memory: 12 loads for 128 FMAs.  The kernels of hla_simt.cuh form 16-token tiles with one scalar load and one
+// predicate per four FMAs and decode every index of T with divisions.
+//
+// The symmetry of the query tensor folds every contraction but one from P = 216 (144) products to M = 56 (78) monomials (the same
+// argument as in hla_tc.cuh): the readout sees the state summed over index permutations, its gradient is the same for all
+// permutations of an index, and so is G = X S^T of the key side.  Only the state itself is formed in full, because it is the layout
+// the workspace promises (P rows); the folded rows are summed when a block stages the state.
+//
+// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2547 -> 431 us (two
+// state builds 1236 -> 170, two feature gradients 557 -> 51, two readouts 277 -> 39, feature networks backward 387 -> 101, forward 104 ->
+// 72); forward with B*H = 2, N = 256, d = 16: 95 -> 37 us.
+#pragma once
+#include "hla_simt.cuh"
+#include "hla_tc.cuh"
+
+namespace hla {
+namespace simt {
+
+constexpr int kTm = 64;           // tokens per tile of the per-token kernels; a thread holds the tokens tg + 8 i, i < 8
+constexpr int kSbTok = 32;        // tokens per step of the state build
+constexpr int kSbRows = 64;       // state rows per block of the state build
+
+template <int F> struct Geo {
+    using M = tc::MT<F>;
+    static constexpr int kDphi = M::kDphi, kN = M::kN, kKf = M::kKf;
+    static constexpr int kNp = (kN + 3) / 4 * 4;             // rows of a folded operand, padded for 16-byte steps
+    static constexpr int kP = F == 3 ? 216 : 144;
+};
+
+// The state row whose index digits are those of monomial m in ascending order.
+template <int F> __host__ __device__ constexpr int first_row(int m) {
+    int idx = 0;
+    for (int a = 0; a < Geo<F>::kDphi; ++a)
+        for (int b = a; b < Geo<F>::kDphi; ++b) {
+            if (F == 2) {
+                if (idx++ == m) return a * 12 + b;
+            } else {
+                for (int c = b; c < 6; ++c)
+                    if (idx++ == m) return 36 * a + 6 * b + c;
+            }
+        }
+    return 0;
+}
+template <int F> struct RowTable {
+    short v[Geo<F>::kN];
+    constexpr RowTable() : v() {
+        for (int m = 0; m < Geo<F>::kN; ++m) v[m] = (short)first_row<F>(m);
+    }
+};
+template <int F> __device__ constexpr RowTable<F> kRowTable{};
+
+// ---- tiles -------------------------------------------------------------------------------------
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(p));
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(tc::pack_bf16(v.x, v.y), tc::pack_bf16(v.z, v.w));
+}
+
+// rows [row0, row0 + n) of a matrix [.][d] into a tile with row stride ld; rows from `limit` on are zero.  All threads.
+template <typename T> __device__ __forceinline__ void stage_rows(float* tile, int ld, const T* __restrict__ src, size_t row0, int n, size_t limit, int d) {
+    const int q = d >> 2;
+    for (int i = threadIdx.x; i < n * q; i += blockDim.x) {
+        const int r = i / q, c = 4 * (i - r * q);
+        const float4 v = row0 + r < limit ? load4(src + (row0 + r) * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(tile + r * ld + c) = v;
+    }
+}
+
+// acc[i][j] += sum_k A[8 i][k] B[k][j], j < 4;  K a multiple of 4
+__device__ __forceinline__ void tile_nn(float (&acc)[8][4], const float* A, int lda, const float* B, int ldb, int K) {
+#pragma unroll 1
+    for (int k = 0; k < K; k += 4) {
+        float4 b[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) b[e] = ld4(B + (k + e) * ldb);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 a = ld4(A + 8 * i * lda + k);
+            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[i][0] = fmaf(av[e], b[e].x, acc[i][0]);
+                acc[i][1] = fmaf(av[e], b[e].y, acc[i][1]);
+                acc[i][2] = fmaf(av[e], b[e].z, acc[i][2]);
+                acc[i][3] = fmaf(av[e], b[e].w, acc[i][3]);
+            }
+        }
+    }
+}
+// acc[i][j] += sum_k A[8 i][k] B[CG j][k], j < JN  (rows of B past its end are the caller's padding)
+template <int CG, int JN> __device__ __forceinline__ void tile_nt(float (&acc)[8][JN], const float* A, int lda, const float* B, int ldb, int K) {
+#pragma unroll 1
+    for (int k = 0; k < K; k += 4) {
+        float4 b[JN];
+#pragma unroll
+        for (int j = 0; j < JN; ++j) b[j] = ld4(B + CG * j * ldb + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 a = ld4(A + 8 * i * lda + k);
+#pragma unroll
+            for (int j = 0; j < JN; ++j) acc[i][j] = fmaf(a.x, b[j].x, fmaf(a.y, b[j].y, fmaf(a.z, b[j].z, fmaf(a.w, b[j].w, acc[i][j]))));
+        }
+    }
+}
+
+// The value-side tile: X = V, xz = 1 (forward), or X = r dO, xz = -r (dO . O), r = 1 / (eta + eps) (backward; a warp per row).
+template <typename T, bool BWD>
+__device__ __forceinline__ void stage_values(float* Xs, int ld, float* xz, const T* __restrict__ X, const T* __restrict__ O, const float* __restrict__ eta,
+                                             const Dims& D, int bh, int tok0, int n, int limit) {
+    if (!BWD) {
+        stage_rows(Xs, ld, X + (size_t)bh * D.N * D.d, (size_t)tok0, n, (size_t)limit, D.d);
+        for (int t = threadIdx.x; t < n; t += blockDim.x) xz[t] = tok0 + t < limit ? 1.f : 0.f;
+        return;
+    }
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5, c = 4 * lane;
+#pragma unroll 4
+    for (int t = threadIdx.x >> 5; t < n; t += nwarp) {
+        const int tok = tok0 + t;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        float s = 0.f, r = 0.f;
+        if (tok < limit) {
+            const size_t row = (size_t)bh * D.N + tok;
+            r = 1.f / (__ldg(eta + row) + D.eps);
+            if (c < D.d) {
+                x = load4(X + row * D.d + c);
+                const float4 o = load4(O + row * D.d + c);
+                s = fmaf(x.x, o.x, fmaf(x.y, o.y, fmaf(x.z, o.z, x.w * o.w)));
+            }
+        }
+        s = warp_sum(s);
+        if (c < D.d) *reinterpret_cast<float4*>(Xs + t * ld + c) = make_float4(r * x.x, r * x.y, r * x.z, r * x.w);
+        if (lane == 0) xz[t] = -r * s;
+    }
+}
+
+// ---- state build -------------------------------------------------------------------------------
+// Forward: rows = the P products T_k[p], X = V.  Backward: rows = the M monomials of q (the gradient is the same for every permutation
+// of a row's indices), X = r dO.  Block = (split, 64 rows, head), thread = 8 rows x 4 columns; the T tile of a step is formed by threads
+// that own one row each, so that a row's digits are decoded once per block.
+template <typename T, int F, int CG, bool BWD>
+__global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X, const T* __restrict__ O,
+                                                                   const float* __restrict__ eta, float* __restrict__ part) {
+    using G = Geo<F>;
+    constexpr int NT = CG * 8, DP = G::kDphi, LD = 4 * CG + 4, LT = kSbRows + 4, KF = BWD ? DP : G::kKf, ROWS = BWD ? G::kN : G::kP;
+    __shared__ __align__(16) float Ts[kSbTok * LT];
+    __shared__ __align__(16) float Xs[kSbTok * LD];
+    __shared__ float fs[kSbTok * KF];
+    __shared__ float xz[kSbTok];
+    const int s = blockIdx.x, row0 = blockIdx.y * kSbRows, bh = blockIdx.z;
+    const int cg = threadIdx.x % CG, rg = threadIdx.x / CG;      // columns 4 cg .., rows 8 rg ..
+    const int per = ((D.N + D.S - 1) / D.S + kSbTok - 1) / kSbTok * kSbTok;
+    const int t0 = s * per, t1 = min(D.N, t0 + per);
+    // the row this thread forms: feature indices of its factors
+    const int row = row0 + (threadIdx.x & 63);
+    int dig[F];
+    {
+        int rem = BWD ? kRowTable<F>.v[row < ROWS ? row : 0] : row;
+#pragma unroll
+        for (int f = F - 1; f >= 0; --f) {
+            dig[f] = rem % DP + (BWD ? 0 : f * DP);
+            rem /= DP;
+        }
+        if (row >= ROWS)
+            for (int f = 0; f < F; ++f) dig[f] = 0;
+    }
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();
+    float acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    float zacc = 0.f;
+    if (4 * cg >= D.d) {      // columns past the head width: never staged, kept finite
+        for (int t = rg; t < kSbTok; t += 8) *reinterpret_cast<float4*>(Xs + t * LD + 4 * cg) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int tok0 = t0; tok0 < t1; tok0 += kSbTok) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < kSbTok * KF; i += NT) {
+            const int f = i / (kSbTok * DP), j = i - f * (kSbTok * DP), t = j / DP, k = j - t * DP;      // (BWD: f = 0)
+            const size_t at = BWD ? ((size_t)bh * D.N + tok0 + t) * DP + k : (((size_t)bh * F + f) * D.N + tok0 + t) * DP + k;
+            fs[t * KF + f * DP + k] = tok0 + t < t1 ? __ldg(feat + at) : 0.f;
+        }
+        stage_values<T, BWD>(Xs, LD, xz, X, O, eta, D, bh, tok0, kSbTok, t1);
+        __syncthreads();
+        for (int t = threadIdx.x >> 6; t < kSbTok; t += NT / 64) {
+            const float* f = fs + t * KF;
+            float v = f[dig[0]] * f[dig[1]];
+            if (F == 3) v *= f[dig[F - 1]];
+            Ts[t * LT + (threadIdx.x & 63)] = row < ROWS ? v : 0.f;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int t = 0; t < kSbTok; ++t) {
+            const float4 a0 = ld4(Ts + t * LT + 8 * rg), a1 = ld4(Ts + t * LT + 8 * rg + 4), x = ld4(Xs + t * LD + 4 * cg);
+            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                acc[i][0] = fmaf(av[i], x.x, acc[i][0]);
+                acc[i][1] = fmaf(av[i], x.y, acc[i][1]);
+                acc[i][2] = fmaf(av[i], x.z, acc[i][2]);
+                acc[i][3] = fmaf(av[i], x.w, acc[i][3]);
+            }
+        }
+        if (threadIdx.x < kSbRows) {
+#pragma unroll 4
+            for (int t = 0; t < kSbTok; ++t) zacc = fmaf(Ts[t * LT + threadIdx.x], xz[t], zacc);
+        }
+    }
+    float* out = part + ((size_t)bh * D.S + s) * ROWS * D.ld;
+    if (4 * cg < D.d) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (row0 + 8 * rg + i < ROWS) store4(out + (size_t)(row0 + 8 * rg + i) * D.ld + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+    }
+    if (threadIdx.x < kSbRows && row < ROWS) store4(out + (size_t)row * D.ld + D.d, make_float4(zacc, 0.f, 0.f, 0.f));
+}
+
+// Sum of the split partials in a fixed order (bit-reproducible) -> state [BH][P][ld].  FOLDED: the partials hold the M monomial rows;
+// every row of the state takes the sum of its monomial.
+template <int F, bool FOLDED>
+__global__ void __launch_bounds__(256) tiled_reduce_kernel(float* __restrict__ out, const float* __restrict__ part, int BH, int S, int ld) {
+    using G = Geo<F>;
+    constexpr int ROWS = FOLDED ? G::kN : G::kP;
+    const int q = ld >> 2, total = BH * ROWS * q;
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
+        const int c = i % q, row = (i / q) % ROWS, bh = i / (q * ROWS);
+        const float4* src = reinterpret_cast<const float4*>(part) + ((size_t)bh * S * ROWS + row) * q + c;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int s = 0; s < S; ++s) {
+            const float4 v = __ldg(src + (size_t)s * ROWS * q);
+            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+        }
+        float4* o = reinterpret_cast<float4*>(out) + (size_t)bh * G::kP * q + c;
+        if (!FOLDED) {
+            o[(size_t)row * q] = a;
+        } else {
+            const int p = kRowTable<F>.v[row];
+            if (F == 2) {
+                o[(size_t)p * q] = a;
+                o[(size_t)((p % 12) * 12 + p / 12) * q] = a;
+            } else {
+                const int d0 = p / 36, d1 = (p / 6) % 6, d2 = p % 6;
+                const int perm[6] = {36 * d0 + 6 * d1 + d2, 36 * d0 + 6 * d2 + d1, 36 * d1 + 6 * d0 + d2, 36 * d1 + 6 * d2 + d0, 36 * d2 + 6 * d0 + d1, 36 * d2 + 6 * d1 + d0};
+#pragma unroll
+                for (int e = 0; e < 6; ++e) o[(size_t)perm[e] * q] = a;
+            }
+        }
+    }
+}
+
+// Folded rows of a head's state into a tile [kNp][ldt] (columns 0 .. d: d values, then z; the padding rows are zero).
+//   SUM = true: sum over the distinct permutations of the row's indices (what the readout of q (x) .. (x) q sees);
+//   SUM = false: the row itself (a gradient state, the same for all permutations).
+template <int F, bool SUM> __device__ __forceinline__ void stage_state(float* tile, int ldt, const float* __restrict__ st, int ld) {
+    using G = Geo<F>;
+    const int q = ld >> 2;
+    for (int i = threadIdx.x; i < G::kNp * q; i += blockDim.x) {
+        const int m = i / q, c = 4 * (i - m * q);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (m < G::kN) {
+            const int p = kRowTable<F>.v[m];
+            auto add = [&](int r, bool on) {
+                if (on) {
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(st + (size_t)r * ld + c));
+                    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+                }
+            };
+            add(p, true);
+            if (SUM && F == 2) add((p % 12) * 12 + p / 12, p / 12 != p % 12);
+            if (SUM && F == 3) {
+                const int d0 = p / 36, d1 = (p / 6) % 6, d2 = p % 6;      // d0 <= d1 <= d2
+                const bool n01 = d0 != d1, n12 = d1 != d2;
+                add(36 * d0 + 6 * d2 + d1, n12);
+                add(36 * d1 + 6 * d0 + d2, n01);
+                add(36 * d1 + 6 * d2 + d0, n01 && n12);
+                add(36 * d2 + 6 * d0 + d1, n01 && n12);
+                add(36 * d2 + 6 * d1 + d0, n01 || n12);
+            }
+        }
+        *reinterpret_cast<float4*>(tile + m * ldt + c) = a;
+    }
+}
+
+// Features of one token into registers (key side: F sets).
+template <int F, bool QSIDE> __device__ __forceinline__ void load_token(float* f, const float* __restrict__ feat, const Dims& D, int bh, int tok) {
+    using G = Geo<F>;
+    if (QSIDE) {
+        tc::load_feat<G::kDphi>(f, feat + ((size_t)bh * D.N + tok) * G::kDphi);
+    } else {
+#pragma unroll
+        for (int m = 0; m < F; ++m) tc::load_feat<G::kDphi>(f + m * G::kDphi, feat + (((size_t)bh * F + m) * D.N + tok) * G::kDphi);
+    }
+}
+
+// ---- readout -----------------------------------------------------------------------------------
+// QSIDE: Y = (mono Csym) / (eta + eps), eta = mono . zsym saved.  Key side: dV = Tsym_k dC.  Tile of 64 tokens, thread = 8 tokens x 4
+// columns; the 64 operand rows are formed by 64 threads, one token each, from registers.
+template <typename T, int F, int CG, bool QSIDE>
+__global__ void __launch_bounds__(CG * 8) tiled_readout_kernel(Dims D, const float* __restrict__ feat, const float* __restrict__ state, T* __restrict__ Y,
+                                                               float* __restrict__ eta_out) {
+    using G = Geo<F>;
+    constexpr int LD = 4 * CG + 4, LA = G::kNp + 4;
+    extern __shared__ __align__(16) float dyn[];
+    float* Ss = dyn;                          // [kNp][LD]
+    float* As = Ss + G::kNp * LD;             // [64][LA]
+    float* inv = As + kTm * LA;               // [64]
+    const int bh = blockIdx.y, tok0 = blockIdx.x * kTm;
+    const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();
+    stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
+    if (threadIdx.x < kTm) {
+        const int tok = tok0 + threadIdx.x;
+        constexpr int KF = QSIDE ? G::kDphi : G::kKf;
+        float f[KF], v[G::kN];
+        load_token<F, QSIDE>(f, feat, D, bh, tok < D.N ? tok : D.N - 1);
+        if constexpr (QSIDE) tc::query_monomials_t<F>(f, v);
+        else tc::key_folded_t<F>(f, v);
+        float* a = As + threadIdx.x * LA;
+#pragma unroll
+        for (int m = 0; m < G::kNp; ++m) a[m] = m < G::kN ? v[m < G::kN ? m : 0] : 0.f;
+    }
+    __syncthreads();
+    if (QSIDE) {
+        for (int t = threadIdx.x; t < kTm; t += CG * 8) {
+            float e0 = 0.f, e1 = 0.f;
+#pragma unroll 4
+            for (int m = 0; m < G::kN; m += 2) {
+                e0 = fmaf(As[t * LA + m], Ss[m * LD + D.d], e0);
+                e1 = fmaf(As[t * LA + m + 1], Ss[(m + 1) * LD + D.d], e1);
+            }
+            inv[t] = 1.f / (e0 + e1 + D.eps);
+            if (tok0 + t < D.N) eta_out[(size_t)bh * D.N + tok0 + t] = e0 + e1;
+        }
+    }
+    float acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    if (4 * cg < D.d) tile_nn(acc, As + tg * LA, LA, Ss + 4 * cg, LD, G::kNp);
+    if (QSIDE) __syncthreads();
+    if (4 * cg >= D.d) return;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int tok = tok0 + tg + 8 * i;
+        const float r = QSIDE ? inv[tg + 8 * i] : 1.f;
+        if (tok < D.N) store4(Y + ((size_t)bh * D.N + tok) * D.d + 4 * cg, make_float4(acc[i][0] * r, acc[i][1] * r, acc[i][2] * r, acc[i][3] * r));
+    }
+}
+
+// ---- feature gradients -------------------------------------------------------------------------
+// G[t][m] = sum_g X[t][g] S[m][g] + xz[t] S[m][d], then the product rule through the folded outer product, one token per thread.
+// QSIDE: X = r dO, xz = -r (dO . O), S = (C|z) summed over permutations.  Key side: X = V, xz = 1, S = (dC|dz).
+template <typename T, int F, int CG, bool QSIDE>
+__global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X, const T* __restrict__ O,
+                                                                    const float* __restrict__ eta, const float* __restrict__ state, float* __restrict__ dfeat) {
+    using G = Geo<F>;
+    constexpr int LD = 4 * CG + 4, JN = (G::kN + CG - 1) / CG, LG = G::kN + 1;
+    extern __shared__ __align__(16) float dyn[];
+    float* Xs = dyn;                          // [64][LD]
+    float* Ss = Xs + kTm * LD;                // [CG * JN][LD] (kNp rows are staged; the columns of the rest are not used)
+    float* xz = Ss + CG * JN * LD;            // [64]
+    float* Gs = xz + kTm;                     // [64][LG], an odd stride
+    const int bh = blockIdx.y, tok0 = blockIdx.x * kTm;
+    const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();
+    stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
+    stage_values<T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, kTm, D.N);
+    __syncthreads();
+    float acc[8][JN];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < JN; ++j) acc[i][j] = 0.f;
+    tile_nt<CG, JN>(acc, Xs + tg * LD, LD, Ss + cg * LD, LD, D.d);
+#pragma unroll
+    for (int j = 0; j < JN; ++j) {
+        const int m = cg + CG * j;
+        if (m < G::kN) {
+            const float z = Ss[m * LD + D.d];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) Gs[(tg + 8 * i) * LG + m] = fmaf(xz[tg + 8 * i], z, acc[i][j]);
+        }
+    }
+    __syncthreads();
+    const int tok = tok0 + threadIdx.x;
+    if (threadIdx.x < kTm && tok < D.N) {
+        float g[G::kN];
+#pragma unroll
+        for (int m = 0; m < G::kN; ++m) g[m] = Gs[threadIdx.x * LG + m];
+        if constexpr (QSIDE) {
+            float q[G::kDphi], dq[G::kDphi];
+            load_token<F, true>(q, feat, D, bh, tok);
+            tc::query_monomials_grad_t<F>(q, g, dq);
+            tc::store_feat<G::kDphi>(dfeat + ((size_t)bh * D.N + tok) * G::kDphi, dq);
+        } else {
+            float k[G::kKf], dk[G::kKf];
+            load_token<F, false>(k, feat, D, bh, tok);
+            tc::key_folded_grad_t<F>(k, g, dk);
+#pragma unroll
+            for (int m = 0; m < F; ++m) tc::store_feat<G::kDphi>(dfeat + (((size_t)bh * F + m) * D.N + tok) * G::kDphi, dk + m * G::kDphi);
+        }
+    }
+}
+
+// ---- feature networks --------------------------------------------------------------------------
+// feat = ReLU(W2^T GELU(W1^T x + b1) + b2) of 64 rows and one map (blockIdx.y).  rows = B*H*N; key side: out [bh][maps][N][d_phi].
+template <typename T, int DP, int CG, bool KSIDE>
+__global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __restrict__ X, PhiWeights<T> W, float* __restrict__ out, size_t rows, int N, int d) {
+    constexpr int NT = CG * 8, LD = 4 * CG + 4;
+    extern __shared__ __align__(16) float dyn[];
+    float* Xs = dyn;                  // [64][LD]; the hidden layer later
+    float* Ws = Xs + kTm * LD;        // [d][LD]
+    float* W2s = Ws + 4 * CG * LD;    // [DP][LD], transposed
+    const size_t row0 = (size_t)blockIdx.x * kTm;
+    const int m = blockIdx.y, cg = threadIdx.x % CG, tg = threadIdx.x / CG;
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();
+    stage_rows(Xs, LD, X, row0, kTm, rows, d);
+    stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
+    for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
+    __syncthreads();
+    float acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    const bool live = 4 * cg < d;
+    if (live) {
+        tile_nn(acc, Xs + tg * LD, LD, Ws + 4 * cg, LD, d);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float b = ldf(W.b1[m] + 4 * cg + j);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i][j] = gelu_erf(acc[i][j] + b);
+        }
+    }
+    __syncthreads();      // the input tile has been read
+    if (live) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) store4(Xs + (tg + 8 * i) * LD + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kTm * DP; i += NT) {
+        const int t = i / DP, o = i - t * DP;
+        float p0 = 0.f, p1 = 0.f;
+        for (int j = 0; j < d; j += 4) {
+            const float4 g = ld4(Xs + t * LD + j), w = ld4(W2s + o * LD + j);
+            p0 = fmaf(g.x, w.x, fmaf(g.y, w.y, p0));
+            p1 = fmaf(g.z, w.z, fmaf(g.w, w.w, p1));
+        }
+        const size_t row = row0 + t;
+        if (row < rows) {
+            const float v = fmaxf(p0 + p1 + ldf(W.b2[m] + o), 0.f);
+            if (KSIDE) {
+                const size_t bh = row / N, n = row - bh * N;
+                out[((bh * W.nmaps + m) * N + n) * DP + o] = v;
+            } else {
+                out[row * DP + o] = v;
+            }
+        }
+    }
+}
+
+// dX[row][:] = sum over maps of W1 (GELU'(h) (.) (W2 (dfeat (.) [feat > 0]))), h recomputed, the ReLU mask from the kept features.
+template <typename T, int DP, int CG, bool KSIDE>
+__global__ void __launch_bounds__(CG * 8) tiled_phi_backward_kernel(const T* __restrict__ X, PhiWeights<T> W, const float* __restrict__ feat,
+                                                                    const float* __restrict__ dfeat, T* __restrict__ dX, size_t rows, int N, int d) {
+    constexpr int NT = CG * 8, LD = 4 * CG + 4, LP = DP + 2;
+    extern __shared__ __align__(16) float dyn[];
+    float* Xs = dyn;                          // [64][LD]
+    float* Ws = Xs + kTm * LD;                // [4 CG][LD]
+    float* Hs = Ws + 4 * CG * LD;             // [64][LD] dh
+    float* W2s = Hs + kTm * LD;               // [DP][LD], transposed
+    float* dps = W2s + DP * LD;               // [64][LP]
+    const size_t row0 = (size_t)blockIdx.x * kTm;
+    const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
+    const bool live = 4 * cg < d;
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();
+    stage_rows(Xs, LD, X, row0, kTm, rows, d);
+    for (int i = threadIdx.x; i < (4 * CG - d) * (d >> 2); i += NT)      // rows of W1 past the head width: read by tile_nt, kept finite
+        *reinterpret_cast<float4*>(Ws + (d + i / (d >> 2)) * LD + 4 * (i % (d >> 2))) = make_float4(0.f, 0.f, 0.f, 0.f);
+    float dx[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dx[i][j] = 0.f;
+    for (int m = 0; m < W.nmaps; ++m) {
+        if (m > 0) __syncthreads();      // the previous map's tiles have been read
+        stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
+        for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
+        for (int i = threadIdx.x; i < kTm * DP; i += NT) {
+            const int t = i / DP, o = i - t * DP;
+            const size_t row = row0 + t;
+            float g = 0.f;
+            if (row < rows) {
+                size_t at = row * DP + o;
+                if (KSIDE) {
+                    const size_t bh = row / N, n = row - bh * N;
+                    at = ((bh * W.nmaps + m) * N + n) * DP + o;
+                }
+                g = __ldg(feat + at) > 0.f ? __ldg(dfeat + at) : 0.f;
+            }
+            dps[t * LP + o] = g;
+        }
+        __syncthreads();
+        if (live) {
+            float h[8][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float b = ldf(W.b1[m] + 4 * cg + j);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) h[i][j] = b;
+            }
+            tile_nn(h, Xs + tg * LD, LD, Ws + 4 * cg, LD, d);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float dg[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int o = 0; o < DP; ++o) {
+                    const float p = dps[(tg + 8 * i) * LP + o];
+                    const float4 w = ld4(W2s + o * LD + 4 * cg);
+                    dg[0] = fmaf(p, w.x, dg[0]);
+                    dg[1] = fmaf(p, w.y, dg[1]);
+                    dg[2] = fmaf(p, w.z, dg[2]);
+                    dg[3] = fmaf(p, w.w, dg[3]);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) dg[j] *= gelu_erf_grad(h[i][j]);
+                store4(Hs + (tg + 8 * i) * LD + 4 * cg, make_float4(dg[0], dg[1], dg[2], dg[3]));
+            }
+        }
+        __syncthreads();
+        tile_nt<CG, 4>(dx, Hs + tg * LD, LD, Ws + cg * LD, LD, d);      // column cg + CG j of dX
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j)      // through shared memory: whole rows leave with 16-byte stores
+#pragma unroll
+        for (int i = 0; i < 8; ++i) Hs[(tg + 8 * i) * LD + cg + CG * j] = dx[i][j];
+    __syncthreads();
+    if (live) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const size_t row = row0 + tg + 8 * i;
+            if (row < rows) store4(dX + row * d + 4 * cg, ld4(Hs + (tg + 8 * i) * LD + 4 * cg));
+        }
+    }
+}
+
+// ---- host --------------------------------------------------------------------------------------
+inline bool tiled(const Dims& D) { return (D.F == 3 && D.dphi == 6) || (D.F == 2 && D.dphi == 12); }
+// Token splits of a state build: three blocks per SM over all row blocks and heads (each block then walks several 32-token steps at
+// every size but the smallest, and the partials, S x P x ld floats per head, stay a few MB).
+inline int tiled_splits(int BH, int N, int P, int sm_count) {
+    const int blocks = BH * ((P + kSbRows - 1) / kSbRows), S = (3 * sm_count + blocks - 1) / blocks, most = (N + kSbTok - 1) / kSbTok;
+    return S < most ? S : most;
+}
+template <int F, int CG> struct TiledSmem {
+    using G = Geo<F>;
+    static constexpr int LD = 4 * CG + 4;
+    static constexpr size_t readout = sizeof(float) * (G::kNp * LD + kTm * (G::kNp + 4) + kTm);
+    static constexpr size_t grad = sizeof(float) * (kTm * LD + (G::kN + CG - 1) / CG * CG * LD + kTm + kTm * (G::kN + 1));
+    static_assert((G::kN + CG - 1) / CG * CG >= G::kNp, "staged rows");
+    static constexpr size_t phi_fwd = sizeof(float) * (kTm * LD + 4 * CG * LD + G::kDphi * LD);
+    static constexpr size_t phi_bwd = sizeof(float) * (2 * kTm * LD + 4 * CG * LD + G::kDphi * LD + kTm * (G::kDphi + 2));
+};
+
+struct TiledArgs {
+    Dims D;
+    int BH;
+    const void *Q, *K, *V, *O, *dO;
+    void *Oout, *dQ, *dK, *dV;
+    const float *qf, *kf;      // features: given, or in the workspace
+    float *qf_out, *kf_out, *dqf, *dkf, *part, *state, *dstate, *eta;
+    const hla_mlp *phi_q, *phi_k;      // null: features are given
+};
+
+// Launch sequences.  Every kernel is launched with programmatic stream serialization and waits for its predecessor at its top.
+template <typename T, int F, int CG> struct Tiled {
+    using G = Geo<F>;
+    using S = TiledSmem<F, CG>;
+    static constexpr int NT = CG * 8;
+
+    template <typename... KArgs, typename... Args>
+    static bool launch(LaunchRec& rec, const char* name, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, Args... args) {
+        if (smem > 48 * 1024 && !tc::set_smem(kernel, (int)smem)) return false;
+        rec.begin(name);
+        tc::launch_pdl(kernel, grid, dim3(threads), smem, rec.st, KArgs(args)...);
+        return rec.end();
+    }
+    static PhiWeights<T> weights(const hla_mlp* m, int n) {
+        PhiWeights<T> w{};
+        w.nmaps = n;
+        for (int i = 0; i < n; ++i) {
+            w.W1[i] = static_cast<const T*>(m[i].W1);
+            w.b1[i] = static_cast<const T*>(m[i].b1);
+            w.W2[i] = static_cast<const T*>(m[i].W2);
+            w.b2[i] = static_cast<const T*>(m[i].b2);
+        }
+        return w;
+    }
+    static dim3 reduce_grid(const TiledArgs& a, int rows) {
+        const long long n = (long long)a.BH * rows * (a.D.ld / 4), b = (n + 255) / 256;
+        return dim3((unsigned)(b < 8192 ? b : 8192));
+    }
+    static const T* in(const void* p) { return static_cast<const T*>(p); }
+    static T* out(void* p) { return static_cast<T*>(p); }
+
+    static bool forward(const TiledArgs& a, LaunchRec& rec) {
+        const Dims& D = a.D;
+        const size_t rows = (size_t)a.BH * D.N;
+        const unsigned rb = (unsigned)((rows + kTm - 1) / kTm), tb = (unsigned)((D.N + kTm - 1) / kTm);
+        if (a.phi_q) {
+            if (!launch(rec, "simt_phi_forward", tiled_phi_forward_kernel<T, G::kDphi, CG, false>, dim3(rb, 1), NT, S::phi_fwd, in(a.Q), weights(a.phi_q, 1), a.qf_out, rows,
+                        D.N, D.d))
+                return false;
+            if (!launch(rec, "simt_phi_forward", tiled_phi_forward_kernel<T, G::kDphi, CG, true>, dim3(rb, F), NT, S::phi_fwd, in(a.K), weights(a.phi_k, F), a.kf_out, rows,
+                        D.N, D.d))
+                return false;
+        }
+        return launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, false>, dim3(D.S, (G::kP + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.kf, in(a.V),
+                      in(nullptr), a.eta, a.part) &&
+               launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, false>, reduce_grid(a, G::kP), 256, 0, a.state, a.part, a.BH, D.S, D.ld) &&
+               launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, true>, dim3(tb, a.BH), NT, S::readout, D, a.qf, a.state, out(a.Oout), a.eta);
+    }
+    static bool backward(const TiledArgs& a, LaunchRec& rec) {
+        const Dims& D = a.D;
+        const size_t rows = (size_t)a.BH * D.N;
+        const unsigned rb = (unsigned)((rows + kTm - 1) / kTm), tb = (unsigned)((D.N + kTm - 1) / kTm);
+        // pass over the queries: dC, dz, then dq;  pass over the keys: dV, dk^f
+        if (!(launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(D.S, (G::kN + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.qf, in(a.dO), in(a.O),
+                     a.eta, a.part) &&
+              launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, D.S, D.ld) &&
+              launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state, a.dqf) &&
+              launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, false>, dim3(tb, a.BH), NT, S::readout, D, a.kf, a.dstate, out(a.dV), a.eta) &&
+              launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, false>, dim3(tb, a.BH), NT, S::grad, D, a.kf, in(a.V), in(nullptr), a.eta, a.dstate, a.dkf)))
+            return false;
+        if (!a.phi_q) return true;
+        return launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, false>, dim3(rb), NT, S::phi_bwd, in(a.Q), weights(a.phi_q, 1), a.qf, a.dqf,
+                      out(a.dQ), rows, D.N, D.d) &&
+               launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, true>, dim3(rb), NT, S::phi_bwd, in(a.K), weights(a.phi_k, F), a.kf, a.dkf, out(a.dK),
+                      rows, D.N, D.d);
+    }
+};
+
+// The column groups of a block: the smallest of 8, 16, 32 (x 4 columns) that covers the head width.
+template <typename T, int F> inline bool run_tiled_f(const TiledArgs& a, bool fwd, LaunchRec& rec) {
+    if (a.D.d <= 32) return fwd ? Tiled<T, F, 8>::forward(a, rec) : Tiled<T, F, 8>::backward(a, rec);
+    if (a.D.d <= 64) return fwd ? Tiled<T, F, 16>::forward(a, rec) : Tiled<T, F, 16>::backward(a, rec);
+    return fwd ? Tiled<T, F, 32>::forward(a, rec) : Tiled<T, F, 32>::backward(a, rec);
+}
+template <typename T> inline bool run_tiled(const TiledArgs& a, bool fwd, LaunchRec& rec) {
+    return a.D.F == 3 ? run_tiled_f<T, 3>(a, fwd, rec) : run_tiled_f<T, 2>(a, fwd, rec);
+}
+
+}  // namespace simt
+}  // namespace hla
