@@ -344,14 +344,15 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
     L.tensor_core = x->tc ? 1 : 0;
     // partial states: S per head from the split kernels, or the pieces of the fused key-side kernel (folded rows)
     x->k_pieces = 0;
-    size_t part_bytes = (size_t)x->BH * S * P * D.ld * 4;
+    const int part_rows = x->tc && !c.causal ? tc::n_mono(c.F) : P;
+    size_t part_bytes = (size_t)x->BH * S * part_rows * D.ld * 4;
     if (x->tc && mlp) {
         x->k_pieces = tc::fused_key_max_pieces(x->BH, tiles, tc::fused_key_grid(x->BH, c.N, x->sm_count));
         const size_t need = (size_t)x->BH * x->k_pieces * tc::n_mono(c.F) * D.ld * 4;
         if (need > part_bytes) part_bytes = need;
     }
     x->off_part = cv.take(part_bytes);
-    x->off_wpart = (x->tc && mlp) ? cv.take(tc::wgrad_part_bytes(c.d, (long long)x->BH * c.N, x->sm_count)) : kNone;
+    x->off_wpart = (x->tc && mlp) ? cv.take(tc::wgrad_part_bytes(c.d, c.F, (long long)x->BH * c.N, x->sm_count)) : kNone;
     if (x->tc) cv.off = tc::plan(x->tcp, D, x->BH, cv.off);
     x->off_delta = c.causal ? cv.take(tok * 4) : kNone;      // dO . o per token (causal backward)
     x->carry = false;

@@ -6,11 +6,13 @@
 //
 // Both weight gradients contract over the tokens, so neither operand can stay in TMEM (a TMEM operand has one token per
 // lane): the 16 arithmetic warps write the G and dh tiles to shared memory, where X^T, G^T (A operands) and dh, dp (B
-// operands) are all read token-major ("MN-major").  Persistent CTAs take one map at a time over all their tiles, keep
+// operands) are all read token-major ("MN-major").  Every CTA serves ONE map: the maps of a side share the grid, a contiguous run of
+// CTAs each, so that a side leaves one partial per CTA.  (With every CTA walking all maps of its side one after the other the partials
+// of three key maps were 33 MB at d = 128: 159 -> 139 us for the four launches of a call at 12 heads x 12600 tokens.)  It keeps
 //   dW1     [d x d]   accumulator lane = input index, column = hidden unit
 //   dW2ext  [d x 64]  accumulator lane = hidden unit, columns 0..5 = G^T dp_hi, 6..11 = G^T dp_lo
-// in TMEM for the whole map and leave one partial per (CTA, map) in the workspace; a second kernel adds the partials in
-// CTA order, so the result is bit-reproducible.
+// in TMEM and leaves one partial in the workspace; a second kernel adds a map's partials in CTA order, so the result is
+// bit-reproducible.
 //
 // warp 0: TMA loads, warp 1: dg, dW1 and dW2 MMAs, warp 2: h MMAs, warps 3..18: arithmetic (thread = token row x quarter
 // of the hidden units), warps 19..22: column sums of the dh tile (db1), warps 23..26: dp tiles and db2 (thread = token row;
@@ -25,34 +27,43 @@ constexpr int kWgThreads = 27 * 32;
 constexpr int kWgEpiWarp0 = 3, kWgSumWarp0 = 19, kWgDpWarp0 = 23;
 constexpr int kWgColDg = 128, kWgColW1 = 256, kWgColW2 = 384;      // TMEM columns (h at 0)
 
-template <int DV, int NMAPS, int DP> struct WgCfg {
+template <int DV, int DP> struct WgCfg {
     static constexpr int kXBytes = 2 * kBlk;                     // two 64-column blocks per stage (the second stays zero for d = 64)
     static constexpr int kW1Bytes = DV * DV * 2;
     static constexpr int kDgSteps = DP == 6 ? 1 : 2;             // K = 16 steps of the dg product: [dp_hi | dp_lo] is 2 DP columns wide
     static constexpr int kW2tBlock = kDgSteps * 2048;
-    static constexpr int kW2tBytes = (DV / 64) * kW2tBlock;      // per map: [16 kDgSteps K rows][DV] bf16 (W2^T twice, halved; row 12 of the last step: b1)
+    static constexpr int kW2tBytes = (DV / 64) * kW2tBlock;      // [16 kDgSteps K rows][DV] bf16 (W2^T twice, halved; row 12 of the last step: b1)
     static constexpr int kOffX = 0;                              // 2 stages
-    static constexpr int kOffW1 = 2 * kXBytes;                   // the current map's W1
+    static constexpr int kOffW1 = 2 * kXBytes;                   // the map's W1
     static constexpr int kOffDp = kOffW1 + kW1Bytes;             // 3 dp blocks [128 tok][64]: K columns 0..5 dp_hi, 6..11 dp_lo; column 44 of block 0 is 1
     static constexpr int kOffW2t = kOffDp + 3 * kBlk;
-    static constexpr int kOffG = ((kOffW2t + NMAPS * kW2tBytes + 1023) / 1024) * 1024;   // G tile, two 64-column blocks
+    static constexpr int kOffG = ((kOffW2t + kW2tBytes + 1023) / 1024) * 1024;   // G tile, two 64-column blocks
     static constexpr int kOffDh = kOffG + 2 * kBlk;              // dh tile
     static constexpr int kOffBars = kOffDh + 2 * kBlk;
     static constexpr int kSmemUsed = 1024 + kOffBars + 256;
     static_assert(kSmemUsed <= 227 * 1024, "shared memory");
     static constexpr int kSmem = kSmemUsed > 120 * 1024 ? kSmemUsed : 120 * 1024;   // one CTA per SM (512 TMEM columns)
     static constexpr int kB1Row = 12;
-    // one partial per (CTA, map), in floats: dW1 [DV][DV], dW2ext [DV][kW2Cols], db1 [DV], db2 [4 token quarters][16]
+    // one partial per CTA, in floats: dW1 [DV][DV], dW2ext [DV][kW2Cols], db1 [DV], db2 [4 token quarters][16]
     static constexpr int kW2Cols = 16 * kDgSteps;
     static constexpr int kPartW2 = DV * DV, kPartB1 = kPartW2 + DV * kW2Cols, kPartB2 = kPartB1 + DV, kPartFloats = kPartB2 + 64;
 };
 
-// X [rows][DV] bf16.  KSIDE: feat / dfeat are [bh][NMAPS][N][6], else [rows][6].  wpart: [gridDim.x][NMAPS][kPartFloats].
-template <int DV, int NMAPS, bool KSIDE, int DP>
-__global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ PhiMaps maps,
-                                                                     PhiBwdPtrs P, const float* __restrict__ feat, const float* __restrict__ dfeat,
-                                                                     float* __restrict__ wpart, long long rows, int N, int* status) {
-    using Cfg = WgCfg<DV, NMAPS, DP>;
+// The maps of one side: map i is served by the CTAs first[i] .. first[i + 1] - 1.
+struct WgMaps {
+    CUtensorMap x, w1[3];
+    const __nv_bfloat16* b1[3];
+    const __nv_bfloat16* W2[3];
+    int first[4];
+    int n;
+};
+
+// X [rows][DV] bf16.  feat / dfeat: key side (N > 0) [bh][n][N][DP], query side (N = 0) [rows][DP].  wpart: [gridDim.x][kPartFloats].
+template <int DV, int DP>
+__global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __grid_constant__ WgMaps maps, const float* __restrict__ feat,
+                                                                     const float* __restrict__ dfeat, float* __restrict__ wpart, long long rows, int N,
+                                                                     int* status) {
+    using Cfg = WgCfg<DV, DP>;
     constexpr int HC = DV / 4;
     extern __shared__ uint8_t smem_raw[];
     grid_launch_dependents();
@@ -60,8 +71,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
     uint64_t* x_full = bars;           // [2] TMA
     uint64_t* x_empty = bars + 2;      // [2] MMA commit (dW1 of the unit has read the tile)
-    uint64_t* w_full = bars + 4;       // TMA: W1 of the current map
-    uint64_t* w_empty = bars + 5;      // MMA commit after the map's last product
+    uint64_t* w_full = bars + 4;       // TMA: W1 of the map
     uint64_t* h_full = bars + 6;       // MMA commit
     uint64_t* h_empty = bars + 7;      // 512 arrivals
     uint64_t* dp_full = bars + 8;      // [3] 128 arrivals
@@ -70,23 +80,26 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     uint64_t* dg_empty = bars + 12;    // 512 arrivals
     uint64_t* gd_full = bars + 13;     // 512 arrivals: G and dh tiles written
     uint64_t* gd_empty = bars + 14;    // MMA commit + the column-sum warps
-    uint64_t* acc_full = bars + 15;    // MMA commit, once per map
-    uint64_t* acc_empty = bars + 16;   // 512 arrivals, once per map
+    uint64_t* acc_full = bars + 15;    // MMA commit after the last product
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int map = 0;
+    while (map + 1 < maps.n && (int)blockIdx.x >= maps.first[map + 1]) ++map;
+    const int slot = blockIdx.x - maps.first[map], nslots = maps.first[map + 1] - maps.first[map];
     const long long tiles = (rows + kTileTokens - 1) / kTileTokens;
-    const long long t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
-    const int ntiles = (int)(t1 - t0);
-    const int nunits = ntiles * NMAPS;      // unit u = map (u / ntiles), tile (u % ntiles)
-    float* out_cta = wpart + (size_t)blockIdx.x * NMAPS * Cfg::kPartFloats;
+    const long long t0 = tiles * slot / nslots, t1 = tiles * (slot + 1) / nslots;
+    const int ntiles = (int)(t1 - t0);      // >= 1: a map has at most as many CTAs as there are tiles
+    const __nv_bfloat16 *W2g = maps.W2[map], *b1g = maps.b1[map];
+    const CUtensorMap* mapX = &maps.x;
+    float* out_cta = wpart + (size_t)blockIdx.x * Cfg::kPartFloats;
 
     constexpr int kRows = 16 * Cfg::kDgSteps, kB1Abs = kRows - 16 + Cfg::kB1Row;
-    for (int i = tid; i < NMAPS * kRows * DV; i += kWgThreads) {
-        const int m = i / (kRows * DV), k = (i / DV) % kRows, j = i % DV;
-        uint8_t* base = smem + Cfg::kOffW2t + m * Cfg::kW2tBytes + (j >> 6) * Cfg::kW2tBlock;
+    for (int i = tid; i < kRows * DV; i += kWgThreads) {
+        const int k = i / DV, j = i % DV;
+        uint8_t* base = smem + Cfg::kOffW2t + (j >> 6) * Cfg::kW2tBlock;
         *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(k, (j & 63) >> 3) + (j & 7) * 2) =
-            k < 2 * DP ? half_bf16(P.W2[m][j * DP + (k % DP)]) : (k == kB1Abs ? P.b1[m][j] : __float2bfloat16_rn(0.f));
+            k < 2 * DP ? half_bf16(W2g[j * DP + (k % DP)]) : (k == kB1Abs ? b1g[j] : __float2bfloat16_rn(0.f));
     }
     for (int i = tid; i < 3 * kBlk / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffDp)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < 2 * Cfg::kXBytes / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffX)[i] = make_uint4(0, 0, 0, 0);
@@ -101,7 +114,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
             mbar_init(&x_empty[i], 1);
         }
         mbar_init(w_full, 1);
-        mbar_init(w_empty, 1);
         mbar_init(h_full, 1);
         mbar_init(h_empty, 512);
         for (int i = 0; i < 3; ++i) {
@@ -113,9 +125,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
         mbar_init(gd_full, 512);
         mbar_init(gd_empty, 1 + DV / 32);
         mbar_init(acc_full, 1);
-        mbar_init(acc_empty, 512);
         fence_mbar_init();
-        prefetch_tmap(&mapX);
+        prefetch_tmap(mapX);
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
@@ -129,31 +140,27 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0 && ntiles > 0) {
-            for (int unit = 0; unit < nunits; ++unit) {
-                const int m = unit / ntiles, it = unit - m * ntiles, st = unit & 1;
-                if (it == 0) {      // the previous map's products have finished with the W1 image
-                    if (!mbar_wait(w_empty, (m & 1) ^ 1)) { report_timeout(status, 1001); break; }
-                    mbar_arrive_expect_tx(w_full, Cfg::kW1Bytes);
-                    for (int b = 0; b < DV / 64; ++b) tma_load_2d(smem + Cfg::kOffW1 + b * (DV * 128), &maps.w1[m], w_full, b * 64, 0);
-                }
+        if (elect_one()) {
+            mbar_arrive_expect_tx(w_full, Cfg::kW1Bytes);
+            for (int b = 0; b < DV / 64; ++b) tma_load_2d(smem + Cfg::kOffW1 + b * (DV * 128), &maps.w1[map], w_full, b * 64, 0);
+            for (int unit = 0; unit < ntiles; ++unit) {
+                const int st = unit & 1;
                 if (!mbar_wait(&x_empty[st], ((unit >> 1) & 1) ^ 1)) { report_timeout(status, 1002); break; }
                 mbar_arrive_expect_tx(&x_full[st], DV * kTileTokens * 2);
                 for (int b = 0; b < DV / 64; ++b)
-                    tma_load_2d(smem + Cfg::kOffX + st * Cfg::kXBytes + b * kBlk, &mapX, &x_full[st], b * 64, (int)((t0 + it) * kTileTokens));
+                    tma_load_2d(smem + Cfg::kOffX + st * Cfg::kXBytes + b * kBlk, mapX, &x_full[st], b * 64, (int)((t0 + unit) * kTileTokens));
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && ntiles > 0) {      // h = X * W1[m] + 1 * b1[m]
+        if (elect_one()) {      // h = X * W1 + 1 * b1
             const uint32_t idesc1 = idesc_bf16(128, DV, false, true);    // X K-major, W1 [in][hidden] MN-major
             const uint64_t xd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffX), 16, 1024);
             const uint64_t wd = smem_desc_sw128(smem_u32(smem + Cfg::kOffW1), DV * 128, 1024);
             const uint64_t od = smem_desc_sw128(smem_u32(smem + Cfg::kOffDp) + 64, 16, 1024);
             const uint64_t bd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffW2t) + (Cfg::kDgSteps - 1) * 2048, Cfg::kW2tBlock, 1024);      // the K step with the b1 row
-            bool good = true;
-            for (int unit = 0; unit < nunits && good; ++unit) {
-                const int m = unit / ntiles, it = unit - m * ntiles, st = unit & 1;
-                if (it == 0 && !mbar_wait(w_full, m & 1)) { good = false; break; }
+            bool good = mbar_wait(w_full, 0);
+            for (int unit = 0; unit < ntiles && good; ++unit) {
+                const int st = unit & 1;
                 if (!(mbar_wait(&x_full[st], (unit >> 1) & 1) && mbar_wait(h_empty, (unit & 1) ^ 1))) { good = false; break; }
                 // the unit's dg product must be complete too, so that h_full tells the arithmetic warps both
                 if (!mbar_wait(dg_full, unit & 1)) { good = false; break; }
@@ -162,13 +169,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
 #pragma unroll
                 for (int ks = 0; ks < DV / 16; ++ks)
                     umma_bf16(tmem, desc_advance(xd, (ks >> 2) * kBlk + (ks & 3) * 32), desc_advance(wd, ks * 2048), idesc1, ks > 0 ? 1u : 0u);
-                umma_bf16(tmem, od, desc_advance(bd0, m * Cfg::kW2tBytes), idesc1, 1u);      // + 1 * b1
+                umma_bf16(tmem, od, bd0, idesc1, 1u);      // + 1 * b1
                 umma_commit(h_full);
             }
             if (!good) report_timeout(status, 1003);
         }
     } else if (warp == 1) {
-        if (lane == 0 && ntiles > 0) {
+        if (elect_one()) {
             const uint32_t idesc_dg = idesc_bf16(128, DV, false, true);   // dg = dp (K-major) * W2^T (MN-major)
             const uint32_t idesc_w1 = idesc_bf16(128, DV, true, true);    // dW1 = X^T (MN-major, M = input index) * dh (MN-major, N = hidden)
             const uint32_t idesc_w2 = idesc_bf16(128, 64, true, true);    // dW2ext = G^T (MN-major, M = hidden) * dp block (MN-major, N = 64)
@@ -177,49 +184,42 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
             const uint64_t vd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffW2t), Cfg::kW2tBlock, 1024);
             bool good = true;
             auto issue_dg = [&](int unit) -> bool {      // the arithmetic warps of unit - 1 must have taken their dg into registers
-                const int m = unit / ntiles;
                 if (unit > 0 && !mbar_wait(dg_empty, (unit - 1) & 1)) return false;
                 if (!mbar_wait(&dp_full[unit % 3], (unit / 3) & 1)) return false;
                 tc_fence_after();
 #pragma unroll
                 for (int ks = 0; ks < Cfg::kDgSteps; ++ks)
-                    umma_bf16(tmem + kWgColDg, smem_desc_sw128(dpa + (unit % 3) * kBlk + ks * 32, 16, 1024), desc_advance(vd0, m * Cfg::kW2tBytes + ks * 2048), idesc_dg,
+                    umma_bf16(tmem + kWgColDg, smem_desc_sw128(dpa + (unit % 3) * kBlk + ks * 32, 16, 1024), desc_advance(vd0, ks * 2048), idesc_dg,
                               ks > 0 ? 1u : 0u);
                 umma_commit(dg_full);
                 return true;
             };
-            if (nunits > 0) good = issue_dg(0);
-            for (int unit = 0; unit < nunits && good; ++unit) {
-                const int m = unit / ntiles, it = unit - m * ntiles, st = unit & 1;
-                if (unit + 1 < nunits && !issue_dg(unit + 1)) { good = false; break; }
-                // the accumulators of the previous map must have been drained before this map's first product overwrites them
-                if (it == 0 && m > 0 && !mbar_wait(acc_empty, (m - 1) & 1)) { good = false; break; }
+            good = issue_dg(0);
+            for (int unit = 0; unit < ntiles && good; ++unit) {
+                const int st = unit & 1;
+                if (unit + 1 < ntiles && !issue_dg(unit + 1)) { good = false; break; }
                 if (!mbar_wait(gd_full, unit & 1)) { good = false; break; }
                 tc_fence_after();
                 const uint32_t xs = xa + st * Cfg::kXBytes, dps = dpa + (unit % 3) * kBlk;
 #pragma unroll
                 for (int ks = 0; ks < kTileTokens / 16; ++ks)
                     umma_bf16(tmem + kWgColW1, smem_desc_sw128(xs + ks * 2048, kBlk, 1024), smem_desc_sw128(da + ks * 2048, kBlk, 1024), idesc_w1,
-                              (it > 0 || ks > 0) ? 1u : 0u);
+                              (unit > 0 || ks > 0) ? 1u : 0u);
 #pragma unroll
                 for (int ks = 0; ks < kTileTokens / 16; ++ks)
                     umma_bf16(tmem + kWgColW2, smem_desc_sw128(ga + ks * 2048, kBlk, 1024), smem_desc_sw128(dps + ks * 2048, kBlk, 1024), idesc_w2,
-                              (it > 0 || ks > 0) ? 1u : 0u);
+                              (unit > 0 || ks > 0) ? 1u : 0u);
                 umma_commit(gd_empty);
                 umma_commit(&dp_free[unit % 3]);
                 umma_commit(&x_empty[st]);
-                if (it == ntiles - 1) {
-                    umma_commit(acc_full);
-                    umma_commit(w_empty);
-                }
+                if (unit == ntiles - 1) umma_commit(acc_full);
             }
             if (!good) report_timeout(status, 1004);
         }
     } else if (warp >= kWgSumWarp0 && warp < kWgDpWarp0) {
         // db1: column sums of the dh tile as the dW1 product sees it (bf16 values, fp32 sums).  Warp w owns the 32 hidden
         // units 32 w ..: one 16-byte load per lane and step, lane l adds the eight columns of chunk 4 w + (l & 3) over the
-        // rows l >> 2, l >> 2 + 8, ... and keeps its partial sums for the whole map; the lanes' sums meet after the map's last
-        // tile, in a fixed order.  (Two warps with one 4-byte load per row took as long as a whole unit: a lone warp issues
+        // rows l >> 2, l >> 2 + 8, ... and keeps its partial sums; the lanes' sums meet after the last tile, in a fixed order.  (Two warps with one 4-byte load per row took as long as a whole unit: a lone warp issues
         // an instruction every five cycles or so.)
         const int sw = warp - kWgSumWarp0;
         if (sw < DV / 32) {
@@ -228,8 +228,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
             float sm[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) sm[e] = 0.f;
-            for (int unit = 0; unit < nunits; ++unit) {
-                const int m = unit / ntiles, it = unit - m * ntiles;
+            for (int unit = 0; unit < ntiles; ++unit) {
                 if (ok && !mbar_wait(gd_full, unit & 1)) { ok = false; report_timeout(status, 1005); }
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -245,15 +244,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(gd_empty);
-                if (it == ntiles - 1) {
-                    float* o = out_cta + (size_t)m * Cfg::kPartFloats + Cfg::kPartB1 + (sw >> 1) * 64 + 8 * chunk;
+                if (unit == ntiles - 1) {
+                    float* o = out_cta + Cfg::kPartB1 + (sw >> 1) * 64 + 8 * chunk;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
                         float v = sm[e];
 #pragma unroll
                         for (int x = 4; x < 32; x <<= 1) v += __shfl_xor_sync(0xffffffffu, v, x);
                         if (lane < 4) o[e] = v;
-                        sm[e] = 0.f;
                     }
                 }
             }
@@ -266,15 +264,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
         float b2s[DP];
 #pragma unroll
         for (int i = 0; i < DP; ++i) b2s[i] = 0.f;
-        for (int unit = 0; unit < nunits; ++unit) {
-            const int m = unit / ntiles, it = unit - m * ntiles;
-            long long grow = (t0 + it) * kTileTokens + row;
+        for (int unit = 0; unit < ntiles; ++unit) {
+            long long grow = (t0 + unit) * kTileTokens + row;
             const bool live = grow < rows;
             grow = live ? grow : rows - 1;
             size_t off;
-            if (KSIDE) {
+            if (N > 0) {
                 const uint32_t bh = (uint32_t)grow / (uint32_t)N, n = (uint32_t)grow - bh * (uint32_t)N;   // rows < 2^31 (checked on the host)
-                off = (((size_t)bh * NMAPS + m) * N + n) * DP;
+                off = (((size_t)bh * maps.n + map) * N + n) * DP;
             } else {
                 off = (size_t)grow * DP;
             }
@@ -302,13 +299,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
             }
             fence_proxy_async();
             mbar_arrive(&dp_full[unit % 3]);
-            if (it == ntiles - 1) {      // the map is complete: its db2 partial of this token quarter
-                float* o = out_cta + (size_t)m * Cfg::kPartFloats + Cfg::kPartB2 + quarter * 16;
+            if (unit == ntiles - 1) {      // the db2 partial of this token quarter
+                float* o = out_cta + Cfg::kPartB2 + quarter * 16;
 #pragma unroll
                 for (int i = 0; i < DP; ++i) {
                     const float a = warp_sum(b2s[i]);
                     if (lane == 0) o[i] = a;
-                    b2s[i] = 0.f;
                 }
                 if (lane < 16 - DP) o[DP + lane] = 0.f;
             }
@@ -317,8 +313,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
         const int quarter = warp & 3, part = (warp - kWgEpiWarp0) >> 2;
         const int row = quarter * 32 + lane;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-        for (int unit = 0; unit < nunits && ok; ++unit) {
-            const int m = unit / ntiles, it = unit - m * ntiles;
+        for (int unit = 0; unit < ntiles && ok; ++unit) {
             // h_full(unit) also says that dg(unit) is complete (the thread that issues the h products waits for it first)
             if (!mbar_wait(h_full, unit & 1)) { ok = false; report_timeout(status, 1007); }
             ok = __all_sync(0xffffffffu, ok);
@@ -358,13 +353,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
             }
             fence_proxy_async();
             mbar_arrive(gd_full);
-            if (it == ntiles - 1) {
-                // the map is complete: drain dW1 (lane = input index) and dW2ext (lane = hidden unit)
-                if (!mbar_wait(acc_full, m & 1)) { ok = false; report_timeout(status, 1009); }
+            if (unit == ntiles - 1) {
+                // drain dW1 (lane = input index) and dW2ext (lane = hidden unit)
+                if (!mbar_wait(acc_full, 0)) { ok = false; report_timeout(status, 1009); }
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                float* o = out_cta + (size_t)m * Cfg::kPartFloats;
+                float* o = out_cta;
                 if (row < DV) {
 #pragma unroll
                     for (int c = 0; c < HC / 16; ++c) {
@@ -389,8 +384,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
                         }
                     }
                 }
-                tc_fence_before();
-                mbar_arrive(acc_empty);
             }
         }
     }
@@ -399,29 +392,29 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// Adds the partials of `nctas` CTAs in CTA order and writes one map's gradients (fp32, the shapes of the weights).
-// grid = (blocks, maps); partial layout as WgCfg::kPart*.  A CTA that had no tiles left its partial untouched: it is skipped.
 struct WgradOut {
-    float* dW1[4];
-    float* db1[4];
-    float* dW2[4];
-    float* db2[4];
+    float* dW1[3];
+    float* db1[3];
+    float* dW2[3];
+    float* db2[3];
+    int first[4];      // map i: the partials first[i] .. first[i + 1] - 1
 };
-// Sum of the per-CTA partials in a fixed order (bit-reproducible): a block owns 32 consecutive outputs, warp w adds the
-// partials of the CTAs w, w + 8, ... (coalesced 128-byte reads, a dozen and a half independent loads per thread), and
-// the eight warp sums are added in warp order.
+// Adds a map's partials in a fixed order (bit-reproducible) and writes its gradients (fp32, the shapes of the weights); grid = (blocks,
+// maps).  A block owns 32 consecutive outputs, warp w adds the partials w, w + 8, ... of the map (coalesced 128-byte reads, independent
+// loads), and the eight warp sums are added in warp order.
 template <int DV, int DP>
-__global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __restrict__ wpart, WgradOut out, int nmaps_in_part, int map0, int nctas) {
-    using C1 = WgCfg<DV, 1, DP>;
+__global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __restrict__ wpart, WgradOut out) {
+    using C1 = WgCfg<DV, DP>;
     constexpr int PF = C1::kPartFloats, oW2 = C1::kPartW2, oB1 = C1::kPartB1, oB2 = C1::kPartB2, W2C = C1::kW2Cols;
     __shared__ float red[8][32];
     grid_launch_dependents();
     grid_dependency_wait();
-    const int m = blockIdx.y;                        // map of this launch
+    const int m = blockIdx.y;
+    const int nctas = out.first[m + 1] - out.first[m];
     const int total = DV * DV + DV * DP + DV + DP;   // outputs of one map
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float* src = wpart + (size_t)m * PF;
-    const size_t stride = (size_t)nmaps_in_part * PF;
+    const float* src = wpart + (size_t)out.first[m] * PF;
+    constexpr size_t stride = PF;
     for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
         const int i = base + lane;
         // an output is the sum over the CTAs of `nterm` partial entries `step` floats apart, starting at `off`
@@ -439,7 +432,7 @@ __global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __res
         }
         float a = 0.f;
         if (nterm == 1) {
-#pragma unroll 4
+#pragma unroll 8
             for (int c = warp; c < nctas; c += 8) a += src[c * stride + off];
         } else {
             for (int c = warp; c < nctas; c += 8)
@@ -452,23 +445,31 @@ __global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __res
 #pragma unroll
             for (int w = 1; w < 8; ++w) t += red[w][lane];
             t *= scale;
-            if (i < DV * DV) out.dW1[map0 + m][i] = t;
-            else if (i < DV * DV + DV * DP) out.dW2[map0 + m][i - DV * DV] = t;
-            else if (i < DV * DV + DV * DP + DV) out.db1[map0 + m][i - DV * DV - DV * DP] = t;
-            else out.db2[map0 + m][i - DV * DV - DV * DP - DV] = t;
+            if (i < DV * DV) out.dW1[m][i] = t;
+            else if (i < DV * DV + DV * DP) out.dW2[m][i - DV * DV] = t;
+            else if (i < DV * DV + DV * DP + DV) out.db1[m][i - DV * DV - DV * DP] = t;
+            else out.db2[m][i - DV * DV - DV * DP - DV] = t;
         }
         __syncthreads();
     }
 }
 
-inline size_t wgrad_part_bytes(int d, long long rows, int sm_count) {
+// CTAs of the query map, and of each of n key maps: an even share of the SMs, and no more partials in all than three per tile (or four
+// for a single tile), which bounds the workspace of short inputs.
+inline int wgrad_query_ctas(long long tiles, int sm_count) { return (int)(tiles < sm_count ? tiles : sm_count); }
+inline int wgrad_key_ctas(long long tiles, int sm_count, int n) {
+    const int q = wgrad_query_ctas(tiles, sm_count), most = 2 * q < sm_count ? 2 * q : sm_count;
+    return most / n > 1 ? most / n : 1;
+}
+inline size_t wgrad_part_bytes(int d, int n, long long rows, int sm_count) {
     const long long tiles = (rows + kTileTokens - 1) / kTileTokens;
-    const int grid = (int)(tiles < sm_count ? tiles : sm_count);
-    const size_t pf = d == 128 ? WgCfg<128, 1, 12>::kPartFloats : WgCfg<64, 1, 12>::kPartFloats;      // the larger of the two geometries
-    return (size_t)grid * 3 * pf * 4;      // the key side's maps share one launch; the query side reuses the region
+    const size_t pf = d == 128 ? WgCfg<128, 12>::kPartFloats : WgCfg<64, 12>::kPartFloats;      // the larger of the two geometries
+    return (size_t)(wgrad_query_ctas(tiles, sm_count) + n * wgrad_key_ctas(tiles, sm_count, n)) * pf * 4;
 }
 
 // dphi_q / dphi_k: fp32 device outputs with the shapes of the weights (dphi_k points to one entry per key map); either may be null.
+// Both passes come first, then both reductions: the partials of the sides have regions of their own, so the key pass is set up while the
+// query pass drains.
 template <int DV, int F>
 inline hla_status launch_phi_wgrad(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K,
                                    const hla_mlp_grad* dphi_q, const hla_mlp_grad* dphi_k, char* ws, const hla_ws_layout& L, size_t off_wpart,
@@ -476,54 +477,44 @@ inline hla_status launch_phi_wgrad(const Dims& D, int BH, const hla_mlp* phi_q, 
     constexpr int NM = MT<F>::kMaps, DP = MT<F>::kDphi;
     const long long rows = (long long)BH * D.N;
     const long long tiles = (rows + kTileTokens - 1) / kTileTokens;
-    const int grid = (int)(tiles < sm_count ? tiles : sm_count);
     int* status = reinterpret_cast<int*>(ws + L.status);
-    float* wpart = reinterpret_cast<float*>(ws + off_wpart);
-    cudaStream_t st = rec.st;
-    if (dphi_q) {
-        CUtensorMap mapQ;
-        PhiMaps mq;
-        PhiBwdPtrs pq{};
-        if (!make_map_2d(&mapQ, Q, (size_t)rows, DV, kTileTokens) || !make_map_2d(&mq.w1[0], phi_q->W1, DV, DV, DV)) return HLA_ERR_CUDA;
-        mq.w1[1] = mq.w1[0];
-        mq.w1[2] = mq.w1[0];
-        pq.b1[0] = static_cast<const __nv_bfloat16*>(phi_q->b1);
-        pq.W2[0] = static_cast<const __nv_bfloat16*>(phi_q->W2);
-        if (!set_smem(tc_phi_wgrad_kernel<DV, 1, false, DP>, WgCfg<DV, 1, DP>::kSmem)) return HLA_ERR_CUDA;
-        rec.begin("tc_phi_wgrad_q");
-        launch_serial(tc_phi_wgrad_kernel<DV, 1, false, DP>, grid, dim3(kWgThreads), WgCfg<DV, 1, DP>::kSmem, st, mapQ, mq, pq,
-                      reinterpret_cast<const float*>(ws + L.qf), reinterpret_cast<const float*>(ws + L.dqf), wpart, rows, D.N, status);
-        if (!rec.end()) return HLA_ERR_CUDA;
-        WgradOut o{};
-        o.dW1[0] = static_cast<float*>(dphi_q->dW1); o.db1[0] = static_cast<float*>(dphi_q->db1);
-        o.dW2[0] = static_cast<float*>(dphi_q->dW2); o.db2[0] = static_cast<float*>(dphi_q->db2);
-        rec.begin("tc_wgrad_reduce");
-        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((DV * DV + DV * DP + DV + DP + 31) / 32, 1), dim3(256), 0, st, (const float*)wpart, o, 1, 0, grid);
+    if (!set_smem(tc_phi_wgrad_kernel<DV, DP>, WgCfg<DV, DP>::kSmem)) return HLA_ERR_CUDA;
+    WgradOut out[2] = {};
+    float* wpart[2];
+    int nmaps[2] = {dphi_q ? 1 : 0, dphi_k ? NM : 0};
+    bool first = true;
+    for (int key = 0; key < 2; ++key) {
+        const int n = nmaps[key];
+        wpart[key] = reinterpret_cast<float*>(ws + off_wpart) + (key ? (size_t)wgrad_query_ctas(tiles, sm_count) * WgCfg<DV, DP>::kPartFloats : 0);
+        if (n == 0) continue;
+        const hla_mlp* w = key ? phi_k : phi_q;
+        const hla_mlp_grad* g = key ? dphi_k : dphi_q;
+        WgMaps maps{};
+        WgradOut& o = out[key];
+        if (!make_map_2d(&maps.x, key ? K : Q, (size_t)rows, DV, kTileTokens)) return HLA_ERR_CUDA;
+        for (int i = 0; i < n; ++i) {
+            if (!make_map_2d(&maps.w1[i], w[i].W1, DV, DV, DV)) return HLA_ERR_CUDA;
+            maps.b1[i] = static_cast<const __nv_bfloat16*>(w[i].b1);
+            maps.W2[i] = static_cast<const __nv_bfloat16*>(w[i].W2);
+            o.dW1[i] = static_cast<float*>(g[i].dW1); o.db1[i] = static_cast<float*>(g[i].db1);
+            o.dW2[i] = static_cast<float*>(g[i].dW2); o.db2[i] = static_cast<float*>(g[i].db2);
+            maps.first[i + 1] = o.first[i + 1] = maps.first[i] + (key ? wgrad_key_ctas(tiles, sm_count, n) : wgrad_query_ctas(tiles, sm_count));
+        }
+        maps.n = n;
+        const float* feat = reinterpret_cast<const float*>(ws + (key ? L.kf : L.qf));
+        const float* dfeat = reinterpret_cast<const float*>(ws + (key ? L.dkf : L.dqf));
+        const int per_head = key ? D.N : 0;
+        rec.begin(key ? "tc_phi_wgrad_k" : "tc_phi_wgrad_q");
+        // the first pass stages caller-provided weights before its dependency wait: no overlap with what precedes it
+        if (first) launch_serial(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status);
+        else launch_pdl(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status);
+        first = false;
         if (!rec.end()) return HLA_ERR_CUDA;
     }
-    if (dphi_k) {
-        CUtensorMap mapK;
-        PhiMaps mk;
-        PhiBwdPtrs pk{};
-        if (!make_map_2d(&mapK, K, (size_t)rows, DV, kTileTokens)) return HLA_ERR_CUDA;
-        WgradOut o{};
-        for (int f = 0; f < NM; ++f) {
-            if (!make_map_2d(&mk.w1[f], phi_k[f].W1, DV, DV, DV)) return HLA_ERR_CUDA;
-            pk.b1[f] = static_cast<const __nv_bfloat16*>(phi_k[f].b1);
-            pk.W2[f] = static_cast<const __nv_bfloat16*>(phi_k[f].W2);
-            o.dW1[f] = static_cast<float*>(dphi_k[f].dW1); o.db1[f] = static_cast<float*>(dphi_k[f].db1);
-            o.dW2[f] = static_cast<float*>(dphi_k[f].dW2); o.db2[f] = static_cast<float*>(dphi_k[f].db2);
-        }
-        for (int f = NM; f < 3; ++f) mk.w1[f] = mk.w1[0];
-        if (!set_smem(tc_phi_wgrad_kernel<DV, NM, true, DP>, WgCfg<DV, NM, DP>::kSmem)) return HLA_ERR_CUDA;
-        rec.begin("tc_phi_wgrad_k");
-        // it stages caller-provided weights before its dependency wait, and the reduction before it still reads the
-        // partial region: no overlap with what precedes it
-        launch_serial(tc_phi_wgrad_kernel<DV, NM, true, DP>, grid, dim3(kWgThreads), WgCfg<DV, NM, DP>::kSmem, st, mapK, mk, pk,
-                      reinterpret_cast<const float*>(ws + L.kf), reinterpret_cast<const float*>(ws + L.dkf), wpart, rows, D.N, status);
-        if (!rec.end()) return HLA_ERR_CUDA;
+    for (int key = 0; key < 2; ++key) {
+        if (nmaps[key] == 0) continue;
         rec.begin("tc_wgrad_reduce");
-        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((DV * DV + DV * DP + DV + DP + 31) / 32, NM), dim3(256), 0, st, (const float*)wpart, o, NM, 0, grid);
+        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((DV * DV + DV * DP + DV + DP + 31) / 32, nmaps[key]), dim3(256), 0, rec.st, (const float*)wpart[key], out[key]);
         if (!rec.end()) return HLA_ERR_CUDA;
     }
     return HLA_OK;
