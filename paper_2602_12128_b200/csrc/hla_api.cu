@@ -189,6 +189,7 @@ simt::TiledArgs tiled_args(const hla_ctx* c, const void* Q, const void* K, const
     a.eta = reinterpret_cast<float*>(ws + c->L.eta);
     a.phi_q = mlp ? &c->phi_q : nullptr;
     a.phi_k = mlp ? c->phi_k : nullptr;
+    a.clear = reinterpret_cast<int*>(ws + c->L.status);
     return a;
 }
 
@@ -420,7 +421,8 @@ hla_status forward_impl(hla_ctx* ctx, const void* Q, const void* K, const void* 
     char* ws = static_cast<char*>(workspace);
     ctx->rec.start_call(st);
     (void)cudaGetLastError();
-    if (phase != 2 && cudaMemsetAsync(ws + ctx->L.status, 0, 64, st) != cudaSuccess) return HLA_ERR_CUDA;
+    // the first kernel of a forward clears the status words (a memset node cost 2 us per call); the kernels of hla_simt.cuh do not
+    if (!ctx->tc && !simt::tiled(ctx->D) && cudaMemsetAsync(ws + ctx->L.status, 0, 64, st) != cudaSuccess) return HLA_ERR_CUDA;
     follow_device(ctx);
     tc::HostCacheScope scope(&ctx->hc);
     if (ctx->tc) {
@@ -431,8 +433,10 @@ hla_status forward_impl(hla_ctx* ctx, const void* Q, const void* K, const void* 
             if (phase != 2) {
                 s = tc::phik_state(ctx->D, ctx->BH, ctx->phi_k, K, V, ws, ctx->L, ctx->off_part, ctx->k_pieces, ctx->sm_count, ctx->rec);
                 if (s != HLA_OK) return s;
-                s = tc::reduce_pieces(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, ctx->off_part, ctx->k_pieces,
-                                      tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count), ctx->rec, ctx->cfg.causal != 0);
+                // (the causal sweep reads the pieces themselves)
+                if (!ctx->cfg.causal)
+                    s = tc::reduce_pieces(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count),
+                                          ctx->rec);
                 if (s != HLA_OK || phase == 1) return s;
             } else {
                 s = tc::emit_from_state(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, false, ctx->rec);
@@ -590,8 +594,6 @@ hla_status value_mod_call(hla_ctx* ctx, const void* T, const void* V, const void
     tc::HostCacheScope scope(&ctx->hc);
     const long long rows = (long long)ctx->BH * ctx->D.N;
     int* status = reinterpret_cast<int*>(ws + ctx->L.status);
-    // like hla_forward, the forward starts a new record of device-side time-outs
-    if (!backward && cudaMemsetAsync(ws + ctx->L.status, 0, 64, st) != cudaSuccess) return HLA_ERR_CUDA;
     if (ctx->D.d == 128)
         return tc::launch_vmod<128>(ctx->vmp, rows, ctx->phi_v, T, V, dOut, Out, dT, dV, accumulate, backward, ws, status, ctx->sm_count, ctx->rec);
     return tc::launch_vmod<64>(ctx->vmp, rows, ctx->phi_v, T, V, dOut, Out, dT, dV, accumulate, backward, ws, status, ctx->sm_count, ctx->rec);

@@ -149,7 +149,7 @@ __device__ __forceinline__ void stage_values(float* Xs, int ld, float* xz, const
 // that own one row each, so that a row's digits are decoded once per block.
 template <typename T, int F, int CG, bool BWD>
 __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X, const T* __restrict__ O,
-                                                                   const float* __restrict__ eta, float* __restrict__ part) {
+                                                                   const float* __restrict__ eta, float* __restrict__ part, int* __restrict__ clear) {
     using G = Geo<F>;
     constexpr int NT = CG * 8, DP = G::kDphi, LD = 4 * CG + 4, LT = kSbRows + 4, KF = BWD ? DP : G::kKf, ROWS = BWD ? G::kN : G::kP;
     __shared__ __align__(16) float Ts[kSbTok * LT];
@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
     }
     tc::grid_launch_dependents();
     tc::grid_dependency_wait();
+    if (clear && s == 0 && blockIdx.y == 0 && bh == 0 && threadIdx.x < 16) clear[threadIdx.x] = 0;
     float acc[8][4];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -591,6 +592,7 @@ struct TiledArgs {
     const float *qf, *kf;      // features: given, or in the workspace
     float *qf_out, *kf_out, *dqf, *dkf, *part, *state, *dstate, *eta;
     const hla_mlp *phi_q, *phi_k;      // null: features are given
+    int* clear;                // status words, cleared by a kernel of the forward (none of these kernels waits, so none reports)
 };
 
 // Launch sequences.  Every kernel is launched with programmatic stream serialization and waits for its predecessor at its top.
@@ -637,7 +639,7 @@ template <typename T, int F, int CG> struct Tiled {
                 return false;
         }
         return launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, false>, dim3(D.S, (G::kP + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.kf, in(a.V),
-                      in(nullptr), a.eta, a.part) &&
+                      in(nullptr), a.eta, a.part, a.clear) &&
                launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, false>, reduce_grid(a, G::kP), 256, 0, a.state, a.part, a.BH, D.S, D.ld) &&
                launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, true>, dim3(tb, a.BH), NT, S::readout, D, a.qf, a.state, out(a.Oout), a.eta);
     }
@@ -647,7 +649,7 @@ template <typename T, int F, int CG> struct Tiled {
         const unsigned rb = (unsigned)((rows + kTm - 1) / kTm), tb = (unsigned)((D.N + kTm - 1) / kTm);
         // pass over the queries: dC, dz, then dq;  pass over the keys: dV, dk^f
         if (!(launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(D.S, (G::kN + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.qf, in(a.dO), in(a.O),
-                     a.eta, a.part) &&
+                     a.eta, a.part, nullptr) &&
               launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, D.S, D.ld) &&
               launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state, a.dqf) &&
               launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, false>, dim3(tb, a.BH), NT, S::readout, D, a.kf, a.dstate, out(a.dV), a.eta) &&

@@ -405,7 +405,7 @@ template <int DV, int F, bool GRAD = false>
 __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __grid_constant__ CUtensorMap mapV, const float* __restrict__ kf,
                                                                        float* __restrict__ part, int N, int S, int ld, int* status,
                                                                        const float* __restrict__ eta = nullptr, const float* __restrict__ delta = nullptr,
-                                                                       float eps = 0.f) {
+                                                                       float eps = 0.f, int clear = 0) {
     using M = MT<F>;
     using Cfg = SbCfg<F>;
     constexpr int kStages = Cfg::kStages, kStageBytes = Cfg::kStageBytes;
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     float* out = part + ((size_t)bh * S + s) * M::kN * ld;
 
     grid_launch_dependents();
-    if (ntiles == 0) {   // an empty split contributes zeros
+    if (ntiles == 0) {   // an empty split contributes zeros (never split 0)
         grid_dependency_wait();
         for (int i = tid; i < M::kN * ld; i += kSbThreads) out[i] = 0.f;
         return;
@@ -459,6 +459,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     grid_dependency_wait();
+    if (clear && s == 0 && bh == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
     bool ok = true;
 
     if (warp == 0) {
@@ -1424,7 +1425,7 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
     if (!set_smem(tc_state_build_kernel<DV, F>, SbCfg<F>::kSmem) || !set_smem(tc_readout_kernel<DV, F>, RoCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
     cudaStream_t st = rec.st;
     rec.begin("tc_state_build");
-    launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (const float*)nullptr, 0.f);
+    launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (const float*)nullptr, 0.f, 1);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_reduce_emit");
     launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, state, b3, bq, D.S, D.ld, 0, 0);
@@ -1439,25 +1440,20 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
 }
 
 // Reduction of the pieces the fused key-side kernel (G CTAs over heads x T tiles, at most `smax` pieces per head) left.
-// scratch_state: the fp32 sum goes to the gradient-state region instead of the state region (the causal forward keeps
-// the state region for the state it carries from call to call).
 template <int F>
-inline hla_status reduce_pieces_f(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec,
-                                  bool scratch_state) {
+inline hla_status reduce_pieces_f(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec) {
     __nv_bfloat16* b3 = reinterpret_cast<__nv_bfloat16*>(ws + P.b3);
     __nv_bfloat16* bq = reinterpret_cast<__nv_bfloat16*>(ws + P.bq);
     float* part = reinterpret_cast<float*>(ws + off_part);
-    float* state = reinterpret_cast<float*>(ws + (scratch_state ? L.dstate : L.state));
+    float* state = reinterpret_cast<float*>(ws + L.state);
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_reduce_emit");
     if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T);
     else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
-inline hla_status reduce_pieces(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec,
-                                bool scratch_state = false) {
-    return D.F == 3 ? reduce_pieces_f<3>(P, D, BH, ws, L, off_part, smax, G, rec, scratch_state)
-                    : reduce_pieces_f<2>(P, D, BH, ws, L, off_part, smax, G, rec, scratch_state);
+inline hla_status reduce_pieces(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec) {
+    return D.F == 3 ? reduce_pieces_f<3>(P, D, BH, ws, L, off_part, smax, G, rec) : reduce_pieces_f<2>(P, D, BH, ws, L, off_part, smax, G, rec);
 }
 
 // The two bf16 operand images of a state that already sits, summed, in the workspace (the state region, or with

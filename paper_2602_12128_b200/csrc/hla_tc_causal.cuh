@@ -587,7 +587,7 @@ inline hla_status launch_causal_state_build(const Dims& D, int BH, const float* 
     if (!set_smem(tc_state_build_kernel<DV, 3>, SbCfg<3>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_state_build");
     launch_pdl(tc_state_build_kernel<DV, 3>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapV, kf, reinterpret_cast<float*>(ws + off_part), D.N, D.S,
-               D.ld, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, (const float*)nullptr, 0.f);
+               D.ld, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, (const float*)nullptr, 0.f, 1);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
@@ -651,7 +651,7 @@ inline hla_status launch_causal_backward_values(const Dims& D, int BH, const flo
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_dstate_build");
     launch_pdl(tc_state_build_kernel<DV, 3, true>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapdO, qf, part, D.N, D.S, D.ld, status,
-               (const float*)eta, (const float*)delta, D.eps);
+               (const float*)eta, (const float*)delta, D.eps, 0);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_scan_pieces");
     launch_pdl(tc_scan_pieces_kernel<3, true>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, dstate, D.S, D.ld, 0, T, 0);

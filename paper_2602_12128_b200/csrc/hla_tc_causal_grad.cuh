@@ -494,7 +494,7 @@ inline hla_status launch_causal_backward_features(const Dims& D, int BH, const f
         if (!set_smem(tc_state_build_kernel<DV, 3>, SbCfg<3>::kSmem) || !set_smem(tc_causal_grad_kernel<DV, 0>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
         rec.begin("tc_state_build");
         launch_pdl(tc_state_build_kernel<DV, 3>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapV, kf, part, D.N, D.S, D.ld, status,
-                   (const float*)nullptr, (const float*)nullptr, 0.f);
+                   (const float*)nullptr, (const float*)nullptr, 0.f, 0);
         if (!rec.end()) return HLA_ERR_CUDA;
         rec.begin("tc_scan_pieces");
         launch_pdl(tc_scan_pieces_kernel<3>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, state, D.S, D.ld, 0, T, 0);

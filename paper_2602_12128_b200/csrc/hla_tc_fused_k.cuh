@@ -165,20 +165,9 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
     auto head_of = [&](int it) { return (w0 + it) / T; };
     auto piece_ends = [&](int it) { return it == nwork - 1 || head_of(it + 1) != head_of(it); };
 
-    // second-layer weights as a K-major MMA operand [16 rows (outputs, 6 used)][DV] per map, halved (the GELU warps
-    // form 2 GELU); row kFkB1Row of the same tile holds b1: read as an MN-major operand [16 K rows][DV] it is the B
-    // operand of the bias step of the first layer
     for (int i = tid; i < NM * Cfg::kW2Bytes / 16; i += kFkThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffW2)[i] = make_uint4(0, 0, 0, 0);
     if (DV == 64)
         for (int i = tid; i < kBlk / 16; i += kFkThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffV + kBlk)[i] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    for (int i = tid; i < NM * DV * (DP + 1); i += kFkThreads) {
-        const int m = i / (DV * (DP + 1)), j = (i / (DP + 1)) % DV, o = i % (DP + 1);
-        uint8_t* base = smem + Cfg::kOffW2 + m * Cfg::kW2Bytes + (j >> 6) * 2048;
-        const int r = o < DP ? o : kFkB1Row;
-        *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(r, (j & 63) >> 3) + (j & 7) * 2) = o < DP ? half_bf16(P.W2[m][j * DP + o]) : P.b1[m][j];
-    }
-    for (int i = tid; i < NM * 16; i += kFkThreads) b2s[i] = (i & 15) < DP ? __bfloat162float(P.b2[i >> 4][i & 15]) : 0.f;
     fence_proxy_async();
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -221,10 +210,25 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
         tmem_st8(tmem + Col::kOnes + ((uint32_t)((warp & 3) * 32) << 16), c[0], c[1], c[2], c[3], c[4], c[5], c[6], c[7]);
         tmem_st_wait();
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
     grid_dependency_wait();
+    if (blockIdx.x == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
+    if (warp > 0) {
+        // second-layer weights as a K-major MMA operand [16 rows (outputs, 6 used)][DV] per map, halved (the GELU warps
+        // form 2 GELU); row kFkB1Row of the same tile holds b1: read as an MN-major operand [16 K rows][DV] it is the B
+        // operand of the bias step of the first layer.  (After the dependency wait: a kernel of the caller may have just written
+        // the weights.  Warp 0 has started the loads of the tiles meanwhile.)
+        for (int i = tid - 32; i < NM * DV * (DP + 1); i += kFkThreads - 32) {
+            const int m = i / (DV * (DP + 1)), j = (i / (DP + 1)) % DV, o = i % (DP + 1);
+            uint8_t* base = smem + Cfg::kOffW2 + m * Cfg::kW2Bytes + (j >> 6) * 2048;
+            const int r = o < DP ? o : kFkB1Row;
+            *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(r, (j & 63) >> 3) + (j & 7) * 2) = o < DP ? half_bf16(P.W2[m][j * DP + o]) : P.b1[m][j];
+        }
+        for (int i = tid - 32; i < NM * 16; i += kFkThreads - 32) b2s[i] = (i & 15) < DP ? __bfloat162float(P.b2[i >> 4][i & 15]) : 0.f;
+        fence_proxy_async();
+        tc_fence_before();
+        named_barrier(1, kFkThreads - 32);
+        tc_fence_after();
+    }
     bool ok = true;
 
     if (warp == 0) {
@@ -524,8 +528,7 @@ inline hla_status launch_phik_state(const Dims& D, int BH, const hla_mlp* phi_k,
     if (!set_smem(tc_phik_state_kernel<DV, F>, FkCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
     const int grid = fused_key_grid(BH, D.N, sm_count);
     rec.begin("tc_phik_state");
-    // first kernel of hla_forward, and it stages the weights before its dependency wait: no overlap with what precedes it
-    launch_serial(tc_phik_state_kernel<DV, F>, grid, dim3(kFkThreads), FkCfg<DV, F>::kSmem, rec.st, mapK, mk, mapV, pk, reinterpret_cast<float*>(ws + L.kf),
+    launch_pdl(tc_phik_state_kernel<DV, F>, grid, dim3(kFkThreads), FkCfg<DV, F>::kSmem, rec.st, mapK, mk, mapV, pk, reinterpret_cast<float*>(ws + L.kf),
                   reinterpret_cast<float*>(ws + off_part), D.N, BH, D.ld, smax, reinterpret_cast<int*>(ws + L.status));
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
