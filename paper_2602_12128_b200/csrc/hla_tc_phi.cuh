@@ -34,21 +34,23 @@ __device__ __forceinline__ float2 gelu2_twice(float2 x) {
     return __ffma2_rn(x, make_float2(tanh_approx(u.x), tanh_approx(u.y)), x);
 }
 __device__ __forceinline__ __nv_bfloat16 half_bf16(__nv_bfloat16 w) { return __float2bfloat16_rn(0.5f * __bfloat162float(w)); }
-// GELU'(x) = Phi(x) + x pdf(x) through one tanh.approx per element:
-//   th = tanh(x (a + b x^2)),   2 GELU'(x) ~ (1 + th) (1 + V (1 - th)) = 1 + V + th (1 - V th),   V = x (C0 + C1 x^2) / 2
-// (the derivative of a tanh-form GELU whose inner derivative is a free polynomial); a, b, C0, C1 are fitted against the
-// exact derivative (fit_gelu_tanh.py: |error| < 1.5e-4 before the 2^-11 relative error of tanh.approx, < 1.3e-3 with
-// it).  The kernel evaluates it with -V (negated constants) so that every step is one packed multiply or fma, and the
-// factor 1/2 sits in the staged W2^T of the dg product (exact in bf16): 9 packed + 2 special-function instructions
-// per pair of elements; the polynomial Phi plus exp form needed sixteen.
-__device__ __forceinline__ float2 gelu_grad2_twice(float2 x) {
+// dg GELU'(x) of a pair of elements, with dg already halved (the 1/2 sits in the staged W2^T, exact in bf16), through one tanh.approx
+// per element:
+//   th = tanh(x (a + b x^2)),   2 GELU'(x) ~ (1 + th) (1 + C0 x (1 - th)) = 1 + th + C0 x (1 - th^2)
+// (the derivative of a tanh-form GELU with a linear inner derivative); a, b, C0 are fitted against the exact derivative
+// (fit_gelu_tanh.py: |error| < 1.33e-4 before the 2^-11 relative error of tanh.approx).  Seven packed instructions per pair; the form
+// with a cubic inner derivative (1.23e-4) needed nine, and a packed fp32 instruction holds the FMA pipe for two cycles: sixteen
+// warps with 32 elements per thread took 1445 cycles, with this form 1265 (the special-function pipe alone needs 1024).  Phi backward of
+// the training shape (B = 2, H = 24, N = 32760, d = 128): key side 424 -> 398 us, query side 189 -> 184 us (at the power cap, where fewer
+// instructions count and more overlap does not: h single- and dg double-buffered, with a fifth fewer cycles, took 404 and 190 us).
+constexpr float kGradA = 0.70650562f, kGradB = 0.03061539f, kGradC0 = 0.88953152f;
+__device__ __forceinline__ float2 times_gelu_grad2(float2 dg, float2 x) {
     const float2 t = __fmul2_rn(x, x);
-    const float2 u = __fmul2_rn(x, __ffma2_rn(t, splat2(0.02936904f), splat2(0.69631102f)));
+    const float2 u = __fmul2_rn(x, __ffma2_rn(t, splat2(kGradB), splat2(kGradA)));
+    const float2 v = __fmul2_rn(x, splat2(-kGradC0));
     const float2 th = make_float2(tanh_approx(u.x), tanh_approx(u.y));
-    const float2 vn = __fmul2_rn(x, __ffma2_rn(t, splat2(0.010848315f), splat2(-0.89902785f)));   // -V
-    const float2 a1 = __ffma2_rn(vn, th, splat2(1.f));          // 1 - V th
-    const float2 b1 = __ffma2_rn(th, a1, splat2(1.f));          // 1 + th (1 - V th)
-    return __ffma2_rn(vn, splat2(-1.f), b1);                    // + V
+    const float2 q = __ffma2_rn(v, __ffma2_rn(th, th, splat2(-1.f)), th);
+    return __ffma2_rn(dg, q, dg);
 }
 
 // 2 GELU(x) and 2 GELU'(x) of the same elements through ONE tanh.approx each (the weight gradients need both): the tanh
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
                 for (int e = 0; e < 8; ++e) {
                     const float2 h = make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
                     const float2 dg = make_float2(__uint_as_float(dgr[16 * c + 2 * e]), __uint_as_float(dgr[16 * c + 2 * e + 1]));
-                    const float2 dh = __fmul2_rn(dg, gelu_grad2_twice(h));      // dg holds dg / 2 (halved W2^T)
+                    const float2 dh = times_gelu_grad2(dg, h);
                     w[e] = pack_bf16(dh.x, dh.y);
                 }
                 // dh as the A operand of the dX product, packed into the h columns this thread has already read

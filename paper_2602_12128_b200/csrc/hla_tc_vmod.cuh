@@ -777,7 +777,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
                     const int j = part * HC + 16 * c + 2 * e;
                     const float2 h = __fmul2_rn(make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), splat2(rstd));
                     const float2 dg = make_float2(__uint_as_float(dgr[16 * c + 2 * e]), __uint_as_float(dgr[16 * c + 2 * e + 1]));
-                    const float2 dh = __fmul2_rn(dg, gelu_grad2_twice(h));      // twice dh: the output warps halve
+                    const float2 dh = times_gelu_grad2(dg, h);      // twice dh: the output warps halve
                     w[e] = pack_bf16(dh.x, dh.y);
                     const float2 dr = make_float2(bf_lo(w[e]), bf_hi(w[e]));      // dh as the dxhat product sees it
                     const float2 cj = *reinterpret_cast<const float2*>(cb + j), bj = *reinterpret_cast<const float2*>(cb + DV + j);
