@@ -35,6 +35,7 @@ struct hla_ctx {
     hla_vmlp phi_v[2];
     tc::VmodPlan vmp;   // scratch of the value modulation inside the workspace
     size_t off_delta;   // dO . o per token (scratch of the causal backward)
+    size_t off_gpart;   // gradient states of the pieces (scratch of the causal backward; off_part keeps the forward's prefix states)
     bool carry;         // causal forward starts from the state the previous call left in the workspace
     size_t off_wpart;   // per-CTA partials of the weight gradients (scratch; tensor-core path with the phi maps)
     tc::Plan tcp;       // tensor-core operand buffers inside the workspace
@@ -334,19 +335,19 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
     L.status = cv.take(64);
     L.qf = mlp ? cv.take(tok * c.d_phi * 4) : kNone;
     L.kf = mlp ? cv.take(tok * c.F * c.d_phi * 4) : kNone;
-    L.state = cv.take((size_t)x->BH * P * D.ld * 4);
+    const int state_rows = x->tc ? tc::n_mono(c.F) : P;
+    L.state = cv.take((size_t)x->BH * state_rows * D.ld * 4);
     L.eta = cv.take(tok * 4);
-    L.dstate = cv.take((size_t)x->BH * P * D.ld * 4);
+    L.dstate = cv.take((size_t)x->BH * state_rows * D.ld * 4);
     L.dqf = mlp ? cv.take(tok * c.d_phi * 4) : kNone;
     L.dkf = mlp ? cv.take(tok * c.F * c.d_phi * 4) : kNone;
     L.state_ld = D.ld;
-    L.state_rows = x->tc ? tc::n_mono(c.F) : P;
+    L.state_rows = state_rows;
     L.n_splits = S;
     L.tensor_core = x->tc ? 1 : 0;
     // partial states: S per head from the split kernels, or the pieces of the fused key-side kernel (folded rows)
     x->k_pieces = 0;
-    const int part_rows = x->tc && !c.causal ? tc::n_mono(c.F) : P;
-    size_t part_bytes = (size_t)x->BH * S * part_rows * D.ld * 4;
+    size_t part_bytes = (size_t)x->BH * S * state_rows * D.ld * 4;
     if (x->tc && mlp) {
         x->k_pieces = tc::fused_key_max_pieces(x->BH, tiles, tc::fused_key_grid(x->BH, c.N, x->sm_count));
         const size_t need = (size_t)x->BH * x->k_pieces * tc::n_mono(c.F) * D.ld * 4;
@@ -356,6 +357,7 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
     x->off_wpart = (x->tc && mlp) ? cv.take(tc::wgrad_part_bytes(c.d, c.F, (long long)x->BH * c.N, x->sm_count)) : kNone;
     if (x->tc) cv.off = tc::plan(x->tcp, D, x->BH, cv.off);
     x->off_delta = c.causal ? cv.take(tok * 4) : kNone;      // dO . o per token (causal backward)
+    x->off_gpart = c.causal ? cv.take((size_t)x->BH * S * state_rows * D.ld * 4) : kNone;
     x->carry = false;
     x->vmod = c.value_mod != 0;
     x->phi_v_set = false;
@@ -503,7 +505,9 @@ hla_status backward_impl(hla_ctx* ctx, const void* Q, const void* K, const void*
         float* dkf = mlp ? reinterpret_cast<float*>(ws + ctx->L.dkf) : static_cast<float*>(dK);
         if (ctx->cfg.causal) {
             if (ctx->carry) return HLA_ERR_UNSUPPORTED;      // a chunk that started from a carried state has no backward here
-            s = tc::causal_backward(ctx->D, ctx->BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, ctx->L, ctx->off_part, ctx->off_delta, ctx->rec);
+            const tc::CausalPieces fwd = mlp ? tc::CausalPieces{ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count)}
+                                             : tc::CausalPieces{ctx->off_part, ctx->D.S, 0};
+            s = tc::causal_backward(ctx->D, ctx->BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, ctx->L, fwd, ctx->off_gpart, ctx->off_delta, ctx->rec);
         } else {
             s = tc::core_backward(ctx->tcp, ctx->D, ctx->BH, qf, kf, V, dO, dqf, dkf, dV, ws, ctx->L, ctx->off_part, ctx->sm_count, ctx->rec, phase);
         }

@@ -122,6 +122,24 @@ __device__ __forceinline__ void shifted_key_row(uint32_t blk, uint32_t row, floa
     (shifted_key_chunk<C + 1>(blk, row, s12, k3, std::make_integer_sequence<int, 8>{}), ...);
 }
 
+// Chunks c0 .. c0 + kStateBatch - 1 (8 floats each) of one row of a piece's initial state; zeros past its ld floats.  All loads of a batch
+// are in flight together: one chunk at a time, a piece began with 17 dependent round trips to L2, 8 us.
+constexpr int kStateBatch = 4;
+__device__ __forceinline__ void load_state_chunks(float (&v)[kStateBatch][8], const float* __restrict__ src, int c0, int ld, bool mine) {
+#pragma unroll
+    for (int k = 0; k < kStateBatch; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int at = 8 * (c0 + k) + 4 * h;
+            const float4 a = mine && at < ld ? *reinterpret_cast<const float4*>(src + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[k][4 * h] = a.x; v[k][4 * h + 1] = a.y; v[k][4 * h + 2] = a.z; v[k][4 * h + 3] = a.w;
+        }
+}
+__device__ __forceinline__ void tmem_st_state(uint32_t taddr, const float (&v)[8]) {
+    tmem_st8(taddr, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]), __float_as_uint(v[4]), __float_as_uint(v[5]),
+             __float_as_uint(v[6]), __float_as_uint(v[7]));
+}
+
 // In-place exclusive scan of the piece states of every head, in piece order (bit-reproducible); the sum of all pieces,
 // i.e. the state after the last token, goes to `state`.  REVERSE: the scan runs from the last piece to the first (every
 // piece gets the sum of the pieces after it).  carry != 0: the scan starts from what `state` holds (the state an earlier
@@ -428,25 +446,22 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
         for (int it = 0; it < nwork; ++it) {
             const int work = work_of(it), bh = work / T;
             if (starts(it)) {
-                // a piece begins: its initial state goes to tensor memory (fp32) and to the image (bf16)
+                // a piece begins: its initial state goes to tensor memory (fp32) and to the image (bf16), which was last read by the
+                // readout of the tile before the previous one
+                if (it >= 2 && ok && !mbar_wait_c(&rd_done[it & 1], ((it - 2) >> 1) & 1)) { ok = false; report_timeout(status, 914); }
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
                 const float* src = init + ((size_t)causal_slot(bh, T, BH, S, G) * kMono + (mine ? m : 0)) * ld;
 #pragma unroll 1
-                for (int c = 0; c < kChunks; ++c) {
-                    float v[8];
+                for (int c0 = 0; c0 < kChunks; c0 += kStateBatch) {
+                    float v[kStateBatch][8];
+                    load_state_chunks(v, src, c0, ld, mine);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = 0.f;
-                    if (mine && 8 * c < ld) {
-                        const float4 a = *reinterpret_cast<const float4*>(src + 8 * c);
-                        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-                        if (8 * c + 4 < ld) {
-                            const float4 b = *reinterpret_cast<const float4*>(src + 8 * c + 4);
-                            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-                        }
+                    for (int k = 0; k < kStateBatch; ++k) {
+                        const int c = c0 + k;
+                        if (8 * c < Cfg::kNState) tmem_st_state(sa + 8 * c, v[k]);
+                        if (c < kChunks) store_chunk(it, c, v[k]);
                     }
-                    if (8 * c < Cfg::kNState)
-                        tmem_st8(sa + 8 * c, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]), __float_as_uint(v[4]),
-                                 __float_as_uint(v[5]), __float_as_uint(v[6]), __float_as_uint(v[7]));
-                    store_chunk(it, c, v);
                 }
                 tmem_st_wait();
                 tc_fence_before();
@@ -639,11 +654,11 @@ inline hla_status launch_causal_delta(const Dims& D, int BH, const void* O, cons
 // and the sweep that gives dV (delta must have been computed).
 template <int DV>
 inline hla_status launch_causal_backward_values(const Dims& D, int BH, const float* qf, const float* kf, const void* dO, void* dV, char* ws,
-                                                const hla_ws_layout& L, size_t off_part, size_t off_delta, LaunchRec& rec) {
+                                                const hla_ws_layout& L, size_t off_gpart, size_t off_delta, LaunchRec& rec) {
     CUtensorMap mapdO, mapdV;
     if (!make_map_bhnd(&mapdO, dO, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapdV, dV, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
     int* status = reinterpret_cast<int*>(ws + L.status);
-    float* part = reinterpret_cast<float*>(ws + off_part);
+    float* part = reinterpret_cast<float*>(ws + off_gpart);
     float* dstate = reinterpret_cast<float*>(ws + L.dstate);
     float* eta = reinterpret_cast<float*>(ws + L.eta);
     float* delta = reinterpret_cast<float*>(ws + off_delta);

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                                                                        const float* __restrict__ qf, const float* __restrict__ kf,
                                                                        const float* __restrict__ eta, const float* __restrict__ delta,
                                                                        const float* __restrict__ init, float* __restrict__ out, int N, int BH, int S, int ld,
-                                                                       float eps, int* status) {
+                                                                       int G, float eps, int* status) {
     using Cfg = CgCfg<DV>;
     constexpr int kStageBytes = Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
@@ -83,10 +83,21 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int T = (N + kTileTokens - 1) / kTileTokens;
-    const CaWork cw = causal_work(T, BH, S, 0);
+    const CaWork cw = causal_work(T, BH, S, G);      // (G > 0, several heads per CTA, for DIR 0 only)
     const int w0 = cw.w0, nwork = cw.w1 - cw.w0;
-    const int bh = blockIdx.y;
-    auto tile_of = [&](int it) { return (DIR == 0 ? w0 + it : w0 + nwork - 1 - it) - bh * T; };
+    auto work_of = [&](int it) { return DIR == 0 ? w0 + it : w0 + nwork - 1 - it; };
+    // (head, tile) of an item, stepped along instead of divided for each one (two divisions per thread and tile cost dq a tenth)
+    struct Pos { int bh, tile; };
+    auto pos_of = [&](int it) { const int w = work_of(it), h = w / T; return Pos{h, w - h * T}; };
+    auto step = [&](Pos& p, int n) {
+        if (DIR == 0) {
+            p.tile += n;
+            while (p.tile >= T) { p.tile -= T; ++p.bh; }
+        } else {
+            p.tile -= n;
+        }
+    };
+    auto starts = [&](int it) { return it == 0 || (DIR == 0 && (w0 + it) % T == 0); };      // a piece begins with this item
     grid_launch_dependents();
 
     if (tid == 0) {
@@ -129,8 +140,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
         const int qt = warp & 3, row = qt * 32 + lane, grp = (warp - kCgEpiWarp0) >> 2;
         const uint32_t aa = tmem + Cfg::kColAcc + ((uint32_t)(qt * 32) << 16);
         float fn[DIR == 0 ? 6 : 18], en = 0.f, dn = 0.f;
-        auto prefetch = [&](int it) {
-            const int tok = min(tile_of(it) * kTileTokens + row, N - 1);
+        auto prefetch = [&](const Pos& p) {
+            const int tok = min(p.tile * kTileTokens + row, N - 1), bh = p.bh;
             if (DIR == 0) {
                 load_feat<6>(fn, qf + ((size_t)bh * N + tok) * 6);
                 en = __ldg(eta + (size_t)bh * N + tok);
@@ -140,14 +151,18 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                 for (int f = 0; f < 3; ++f) load_feat<6>(fn + 6 * f, kf + (((size_t)bh * 3 + f) * N + tok) * 6);
             }
         };
-        if (nwork > grp) prefetch(grp);
+        Pos pn = pos_of(grp < nwork ? grp : 0);
+        if (nwork > grp) prefetch(pn);
         for (int it = grp; it < nwork; it += 2) {
-            const int tok = tile_of(it) * kTileTokens + row;
+            const int tok = pn.tile * kTileTokens + row, bh = pn.bh;
             float f[DIR == 0 ? 6 : 18];
 #pragma unroll
             for (int i = 0; i < (DIR == 0 ? 6 : 18); ++i) f[i] = fn[i];
             const float r = 1.f / (en + eps), dl = dn;
-            if (it + 2 < nwork) prefetch(it + 2);
+            if (it + 2 < nwork) {
+                step(pn, 2);
+                prefetch(pn);
+            }
             if (ok && !mbar_wait(&acc_full[grp], (it >> 1) & 1)) { ok = false; report_timeout(status, 934); }
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -188,8 +203,9 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
         reg_dec<kCgIssueRegs>();
         if (warp == 0) {
             if (lane == 0) {
-                for (int it = 0; it < nwork; ++it) {
-                    const int st = it & 1, u = it >> 1, tile = tile_of(it);
+                Pos p = pos_of(0);
+                for (int it = 0; it < nwork; ++it, step(p, 1)) {
+                    const int st = it & 1, u = it >> 1, tile = p.tile, bh = p.bh;
                     if (!mbar_wait(&stage_free[st], (u & 1) ^ 1)) { report_timeout(status, 921); break; }
                     mbar_arrive_expect_tx(&stage_ready[st], 2 * DV * kTileTokens * 2);
                     for (int b = 0; b < Cfg::kVB; ++b) {
@@ -261,7 +277,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                     const int st = it & 1, u = it >> 1;
                     const uint32_t ya = smem_u32(smem + st * kStageBytes), wa = ya + Cfg::kOffW;
                     if (it > 0 && !mbar_wait(state_read, (it - 1) & 1)) { report_timeout(status, 926); break; }
-                    if (it == 0 && !mbar_wait(&b3_ready[0], 0)) { report_timeout(status, 927); break; }
+                    if (starts(it) && !mbar_wait(&b3_ready[it & 1], (it >> 1) & 1)) { report_timeout(status, 927); break; }
                     if (!mbar_wait(&stage_ready[st], u & 1)) { report_timeout(status, 928); break; }
                     tc_fence_after();
                     {      // state += W^T [Y | W]
@@ -281,15 +297,16 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
             const int row = tid - kCgRowWarp0 * 32;
             if (DIR == 0) {
                 float kn[18];
-                auto prefetch = [&](int it) {
-                    const int tok = min(tile_of(it) * kTileTokens + row, N - 1);
+                auto prefetch = [&](const Pos& p) {
+                    const int tok = min(p.tile * kTileTokens + row, N - 1), bh = p.bh;
 #pragma unroll
                     for (int f = 0; f < 3; ++f) load_feat<6>(kn + 6 * f, kf + (((size_t)bh * 3 + f) * N + tok) * 6);
                 };
-                if (nwork > 0) prefetch(0);
+                Pos pn = pos_of(0);
+                if (nwork > 0) prefetch(pn);
                 for (int it = 0; it < nwork; ++it) {
                     const int st = it & 1, u = it >> 1;
-                    const bool valid = tile_of(it) * kTileTokens + row < N;
+                    const bool valid = pn.tile * kTileTokens + row < N;
                     float k[18];
 #pragma unroll
                     for (int i = 0; i < 18; ++i) k[i] = valid ? kn[i] : 0.f;
@@ -305,20 +322,24 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                     shifted_key_row(smem_u32(smem + st * kStageBytes) + Cfg::kOffW, row, valid ? 1.f : 0.f, s12, k3, std::make_integer_sequence<int, 7>{});
                     fence_proxy_async();
                     mbar_arrive(&stage_ready[st]);
-                    if (it + 1 < nwork) prefetch(it + 1);
+                    if (it + 1 < nwork) {
+                        step(pn, 1);
+                        prefetch(pn);
+                    }
                 }
             } else {
                 float qn[6], en = 0.f, dn = 0.f;
-                auto prefetch = [&](int it) {
-                    const int tok = min(tile_of(it) * kTileTokens + row, N - 1);
+                auto prefetch = [&](const Pos& p) {
+                    const int tok = min(p.tile * kTileTokens + row, N - 1), bh = p.bh;
                     load_feat<6>(qn, qf + ((size_t)bh * N + tok) * 6);
                     en = __ldg(eta + (size_t)bh * N + tok);
                     dn = __ldg(delta + (size_t)bh * N + tok);
                 };
-                if (nwork > 0) prefetch(0);
+                Pos pn = pos_of(0);
+                if (nwork > 0) prefetch(pn);
                 for (int it = 0; it < nwork; ++it) {
                     const int st = it & 1, u = it >> 1;
-                    const bool valid = tile_of(it) * kTileTokens + row < N;
+                    const bool valid = pn.tile * kTileTokens + row < N;
                     float q[6], qs[6];
                     const float r = valid ? 1.f / (en + eps) : 0.f, dl = valid ? dn : 0.f;
 #pragma unroll
@@ -332,7 +353,10 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                     dvec[st * 128 + row] = dl;
                     fence_proxy_async();
                     mbar_arrive(&stage_ready[st]);
-                    if (it + 1 < nwork) prefetch(it + 1);
+                    if (it + 1 < nwork) {
+                        step(pn, 1);
+                        prefetch(pn);
+                    }
                 }
             }
         } else if (warp < kCgConvWarp0) {
@@ -342,14 +366,18 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
             const int qt = warp & 3, half = (warp - kCgMaskWarp0) >> 2;
             const uint32_t pa0 = tmem + Cfg::kColS + 64 * half + ((uint32_t)(qt * 32) << 16);
             float dn = 0.f;
-            auto prefetch = [&](int it) {
-                const int tok = min(tile_of(it) * kTileTokens + qt * 32 + lane, N - 1);
-                dn = __ldg(delta + (size_t)bh * N + tok);
+            auto prefetch = [&](const Pos& p) {
+                const int tok = min(p.tile * kTileTokens + qt * 32 + lane, N - 1);
+                dn = __ldg(delta + (size_t)p.bh * N + tok);
             };
-            if (DIR == 0 && nwork > 0) prefetch(0);
+            Pos pn = pos_of(0);
+            if (DIR == 0 && nwork > 0) prefetch(pn);
             for (int it = 0; it < nwork; ++it) {
                 const float dl = dn;
-                if (DIR == 0 && it + 1 < nwork) prefetch(it + 1);
+                if (DIR == 0 && it + 1 < nwork) {
+                    step(pn, 1);
+                    prefetch(pn);
+                }
                 if (ok && !mbar_wait(&p_full[it & 1], (it >> 1) & 1)) { ok = false; report_timeout(status, 931); }
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -399,40 +427,37 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
             const uint32_t sa = tmem + Cfg::kColState + ((uint32_t)(qt * 32) << 16);
             const uint32_t b3base = smem_u32(smem + Cfg::kOffB3);
             for (int it = 0; it < nwork; ++it) {
-                if (it == 0) {
-                    const float* src = init + ((size_t)(bh * S + blockIdx.x) * kMono + (mine ? m : 0)) * ld;
+                if (starts(it)) {
+                    // the image and the vector written now were last read for the tile before the previous one
+                    if (it >= 2 && ok && !mbar_wait(&acc_free[it & 1], ((it - 2) >> 1) & 1)) { ok = false; report_timeout(status, 937); }
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const float* src = init + ((size_t)causal_slot(pos_of(it).bh, T, BH, S, G) * kMono + (mine ? m : 0)) * ld;
+                    const uint32_t b3img = b3base + (it & 1) * Cfg::kB3Bytes;
 #pragma unroll 1
-                    for (int c = 0; c < (DV + 8) / 8; ++c) {
-                        float v[8];
+                    for (int c0 = 0; c0 < (DV + 8) / 8; c0 += kStateBatch) {
+                        float v[kStateBatch][8];
+                        load_state_chunks(v, src, c0, ld, mine);
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) v[e] = 0.f;
-                        if (mine && 8 * c < ld) {
-                            const float4 a = *reinterpret_cast<const float4*>(src + 8 * c);
-                            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-                            if (8 * c + 4 < ld) {
-                                const float4 b = *reinterpret_cast<const float4*>(src + 8 * c + 4);
-                                v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-                            }
-                        }
-                        tmem_st8(sa + 8 * c, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]), __float_as_uint(v[4]),
-                                 __float_as_uint(v[5]), __float_as_uint(v[6]), __float_as_uint(v[7]));
-                        if (mine) {
-                            if (8 * c < DV)
-                                st_shared_v4(b3base + (c >> 3) * Cfg::kB3Block + sw128_off(R, c & 7), pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                                             pack_bf16(v[6], v[7]));
-                            else
-                                zvec[R] = v[0];
+                        for (int k = 0; k < kStateBatch; ++k) {
+                            const int c = c0 + k;
+                            if (c < (DV + 8) / 8) tmem_st_state(sa + 8 * c, v[k]);
+                            if (mine && c < DV / 8)
+                                st_shared_v4(b3img + (c >> 3) * Cfg::kB3Block + sw128_off(R, c & 7), pack_bf16(v[k][0], v[k][1]), pack_bf16(v[k][2], v[k][3]),
+                                             pack_bf16(v[k][4], v[k][5]), pack_bf16(v[k][6], v[k][7]));
+                            if (mine && c == DV / 8) zvec[(it & 1) * 64 + R] = v[k][0];
                         }
                     }
                     tmem_st_wait();
                     tc_fence_before();
                     fence_proxy_async();
-                    mbar_arrive(&b3_ready[0]);
+                    mbar_arrive(&b3_ready[it & 1]);
                 }
                 if (ok && !mbar_wait(state_full, it & 1)) { ok = false; report_timeout(status, 932); }
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                if (it + 1 < nwork) {
+                if (it + 1 < nwork && !starts(it + 1)) {
                     // the image and the vector written now were last read for the previous tile: its epilogue must have read the
                     // vector, which also means that every product of that tile has completed
                     if (it > 0 && ok && !mbar_wait(&acc_free[(it - 1) & 1], ((it - 1) >> 1) & 1)) { ok = false; report_timeout(status, 933); }
@@ -477,59 +502,54 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// Feature gradients of the causal operator: the state of every piece and its prefix scan (as in the forward), the forward
-// sweep for dq; then, on the gradient states the value-gradient pass left in `part` (suffix sums), the backward sweep for dk.
+// The pieces the forward swept, and the prefix states of which it left in the workspace: S slots per head, G as in CaWork.
+struct CausalPieces {
+    size_t off;
+    int S, G;
+};
+
+// Feature gradients of the causal operator: the forward sweep for dq on the prefix states that the forward left in the workspace (they were
+// rebuilt here at first: a pass over the keys and V and a scan, 59 us of a training step with 24 heads x 32760 tokens); then, on the
+// gradient states the value-gradient pass left (suffix sums), the backward sweep for dk.
 template <int DV>
 inline hla_status launch_causal_backward_features(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* dO, float* dqf, float* dkf,
-                                                  char* ws, const hla_ws_layout& L, size_t off_part, size_t off_delta, bool second, LaunchRec& rec) {
+                                                  char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta, bool second,
+                                                  LaunchRec& rec) {
     CUtensorMap mapV, mapdO;
     if (!make_map_bhnd(&mapV, V, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapdO, dO, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
     int* status = reinterpret_cast<int*>(ws + L.status);
-    float* part = reinterpret_cast<float*>(ws + off_part);
-    float* state = reinterpret_cast<float*>(ws + L.state);
     const float* eta = reinterpret_cast<const float*>(ws + L.eta);
     const float* delta = reinterpret_cast<const float*>(ws + off_delta);
-    const int T = (D.N + kTileTokens - 1) / kTileTokens;
     if (!second) {
-        if (!set_smem(tc_state_build_kernel<DV, 3>, SbCfg<3>::kSmem) || !set_smem(tc_causal_grad_kernel<DV, 0>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
-        rec.begin("tc_state_build");
-        launch_pdl(tc_state_build_kernel<DV, 3>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapV, kf, part, D.N, D.S, D.ld, status,
-                   (const float*)nullptr, (const float*)nullptr, 0.f, 0);
-        if (!rec.end()) return HLA_ERR_CUDA;
-        rec.begin("tc_scan_pieces");
-        launch_pdl(tc_scan_pieces_kernel<3>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, state, D.S, D.ld, 0, T, 0);
-        if (!rec.end()) return HLA_ERR_CUDA;
+        if (!set_smem(tc_causal_grad_kernel<DV, 0>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
         rec.begin("tc_causal_dq");
-        launch_pdl(tc_causal_grad_kernel<DV, 0>, dim3(D.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapdO, mapV, qf, kf, eta, delta, (const float*)part, dqf,
-                   D.N, BH, D.S, D.ld, D.eps, status);
+        launch_pdl(tc_causal_grad_kernel<DV, 0>, fwd.G > 0 ? dim3(fwd.G) : dim3(fwd.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapdO, mapV, qf, kf, eta, delta,
+                   reinterpret_cast<const float*>(ws + fwd.off), dqf, D.N, BH, fwd.S, D.ld, fwd.G, D.eps, status);
         return rec.end() ? HLA_OK : HLA_ERR_CUDA;
     }
     if (!set_smem(tc_causal_grad_kernel<DV, 1>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dk");
-    launch_pdl(tc_causal_grad_kernel<DV, 1>, dim3(D.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapV, mapdO, qf, kf, eta, delta, (const float*)part, dkf, D.N,
-               BH, D.S, D.ld, D.eps, status);
+    launch_pdl(tc_causal_grad_kernel<DV, 1>, dim3(D.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapV, mapdO, qf, kf, eta, delta,
+               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, D.ld, 0, D.eps, status);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
-// dO . o, then dq on the forward states, then the gradient states, dV and dk on them.
-inline hla_status causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf, float* dkf,
-                                  void* dV, char* ws, const hla_ws_layout& L, size_t off_part, size_t off_delta, LaunchRec& rec) {
-    if (D.F != 3) return HLA_ERR_UNSUPPORTED;
-    hla_status s;
-    // the value-gradient pass computes delta first; the forward sweep for dq needs it, so the order is: delta (inside the
-    // first call below), dq, then the gradient states with dV, then dk
-    if (D.d == 128) {
-        s = launch_causal_delta<128>(D, BH, O, dO, ws, off_delta, rec);
-        if (s == HLA_OK) s = launch_causal_backward_features<128>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, off_part, off_delta, false, rec);
-        if (s == HLA_OK) s = launch_causal_backward_values<128>(D, BH, qf, kf, dO, dV, ws, L, off_part, off_delta, rec);
-        if (s == HLA_OK) s = launch_causal_backward_features<128>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, off_part, off_delta, true, rec);
-    } else {
-        s = launch_causal_delta<64>(D, BH, O, dO, ws, off_delta, rec);
-        if (s == HLA_OK) s = launch_causal_backward_features<64>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, off_part, off_delta, false, rec);
-        if (s == HLA_OK) s = launch_causal_backward_values<64>(D, BH, qf, kf, dO, dV, ws, L, off_part, off_delta, rec);
-        if (s == HLA_OK) s = launch_causal_backward_features<64>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, off_part, off_delta, true, rec);
-    }
+// dO . o, then dq on the forward states, then the gradient states (in a region of their own, so that the forward's stay), dV and dk on them.
+template <int DV>
+inline hla_status launch_causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf,
+                                         float* dkf, void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta,
+                                         LaunchRec& rec) {
+    hla_status s = launch_causal_delta<DV>(D, BH, O, dO, ws, off_delta, rec);
+    if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, false, rec);
+    if (s == HLA_OK) s = launch_causal_backward_values<DV>(D, BH, qf, kf, dO, dV, ws, L, off_gpart, off_delta, rec);
+    if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, true, rec);
     return s;
+}
+inline hla_status causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf, float* dkf,
+                                  void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta, LaunchRec& rec) {
+    if (D.F != 3) return HLA_ERR_UNSUPPORTED;
+    if (D.d == 128) return launch_causal_backward<128>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec);
+    return launch_causal_backward<64>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec);
 }
 
 }  // namespace tc
