@@ -48,7 +48,10 @@ template <int DV, int F> struct FqCfg {
 
 // Q [BH][N][DV] bf16 (3-D map, rows past N read as zero), O the same (stores are clipped at N).  READOUT = false: the feature
 // map only (the causal operator reads its states tile by tile in a sweep of its own and needs just the query features):
-// the readout product, its epilogue and the monomial tile are left out, O and eta are not written.
+// the readout product, its epilogue and the monomial tile are left out, O and eta are not written.  It then needs nothing of the kernel
+// before it (the key side of the same call, which lets it start only once everything before the call is complete): it waits for that
+// kernel at its end instead of its start, so that the two run side by side where they do not fill the SMs (12 heads x 500 tokens: a
+// quarter of a call).
 template <int DV, int F, bool READOUT = true>
 __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapW1,
                                                                         const __grid_constant__ CUtensorMap mapB3, const __grid_constant__ CUtensorMap mapO,
@@ -137,7 +140,8 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;     // D1[b] at columns 128*b, D2[b] at 256 + 32*b, readout accumulator at 320
-    grid_dependency_wait();
+    if (READOUT) grid_dependency_wait();
+    else grid_start_beside();
     bool ok = true;
 
     if (warp == 0) {
@@ -341,6 +345,7 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
+    if (!READOUT) grid_dependency_wait();      // what follows this kernel may rely on the key side too
 }
 
 template <int DV, int F, bool READOUT>

@@ -133,7 +133,6 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
     constexpr int NM = M::kMaps, DP = M::kDphi;
     constexpr int HC = DV / 4;          // hidden units per GELU thread
     extern __shared__ uint8_t smem_raw[];
-    grid_launch_dependents();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float* b2s = reinterpret_cast<float*>(smem + Cfg::kOffB2);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
@@ -212,6 +211,9 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
     }
     grid_dependency_wait();
     if (blockIdx.x == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
+    // Only now may the next kernel start: the kernels of a call that stage weights before their own wait (or, the causal query map, do
+    // not wait at all until their end) rely on everything before the call being complete.
+    grid_launch_dependents();
     if (warp > 0) {
         // second-layer weights as a K-major MMA operand [16 rows (outputs, 6 used)][DV] per map, halved (the GELU warps
         // form 2 GELU); row kFkB1Row of the same tile holds b1: read as an MN-major operand [16 K rows][DV] it is the B

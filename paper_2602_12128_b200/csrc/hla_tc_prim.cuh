@@ -36,6 +36,10 @@ template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setma
 // staging) and then wait here until the previous kernel has completed and its writes are visible.  No global memory
 // that another kernel of the library writes or reads is touched before this wait.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The start of a kernel that needs nothing of its predecessor, only of the kernels before that one: the predecessor lets it be scheduled
+// after its own dependency wait (so those kernels are complete), and it calls grid_dependency_wait at its end, so that what follows may
+// rely on both.  The fence orders its reads after that; nothing is waited for.
+__device__ __forceinline__ void grid_start_beside() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // Lets the next kernel's blocks be scheduled as soon as every block of this one has started.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
