@@ -199,7 +199,7 @@ hla_status forward_simt(hla_ctx* c, const void* Q, const void* K, const void* V,
     if (simt::tiled(c->D)) {
         simt::TiledArgs a = tiled_args(c, Q, K, V, ws);
         a.Oout = O;
-        return simt::run_tiled<T>(a, true, c->rec) ? HLA_OK : HLA_ERR_CUDA;
+        return simt::run_tiled<T>(a, true, c->sm_count, c->rec) ? HLA_OK : HLA_ERR_CUDA;
     }
     const float *qf, *kf;
     if (c->cfg.phi == HLA_PHI_MLP) {
@@ -224,7 +224,7 @@ hla_status backward_simt(hla_ctx* c, const void* Q, const void* K, const void* V
         a.dQ = dQ; a.dK = dK; a.dV = dV;
         a.dqf = mlp ? reinterpret_cast<float*>(ws + c->L.dqf) : static_cast<float*>(dQ);
         a.dkf = mlp ? reinterpret_cast<float*>(ws + c->L.dkf) : static_cast<float*>(dK);
-        return simt::run_tiled<T>(a, false, c->rec) ? HLA_OK : HLA_ERR_CUDA;
+        return simt::run_tiled<T>(a, false, c->sm_count, c->rec) ? HLA_OK : HLA_ERR_CUDA;
     }
     const float* qf = mlp ? reinterpret_cast<const float*>(ws + c->L.qf) : static_cast<const float*>(Q);
     const float* kf = mlp ? reinterpret_cast<const float*>(ws + c->L.kf) : static_cast<const float*>(K);

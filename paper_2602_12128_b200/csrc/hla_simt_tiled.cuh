@@ -11,9 +11,10 @@
 // permutations of an index, and so is G = X S^T of the key side.  Only the state itself is formed in full, because it is the layout
 // the workspace promises (P rows); the folded rows are summed when a block stages the state.
 //
-// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2547 -> 431 us (two
-// state builds 1236 -> 170, two feature gradients 557 -> 51, two readouts 277 -> 39, feature networks backward 387 -> 101, forward 104 ->
-// 72); forward with B*H = 2, N = 256, d = 16: 95 -> 37 us.
+// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2547 -> 332 us (two
+// state builds 1236 -> 98, two feature gradients 557 -> 56, two readouts 277 -> 37, feature networks backward 387 -> 105, forward 104 ->
+// 72); forward with B*H = 2, N = 256, d = 16: 95 -> 25 us.  Of these, independent neighbours side by side, more splits of the gradient
+// state and the small tiles: 431 -> 332 and 37 -> 25 us.
 #pragma once
 #include "hla_simt.cuh"
 #include "hla_tc.cuh"
@@ -21,7 +22,8 @@
 namespace hla {
 namespace simt {
 
-constexpr int kTm = 64;           // tokens per tile of the per-token kernels; a thread holds the tokens tg + 8 i, i < 8
+// The per-token kernels work on tiles of TM = 8 R tokens, a thread holds the tokens tg + 8 i, i < R: R = 8 where that gives every SM a
+// block, else R = 2 (512 rows: 32 blocks instead of 8, and a quarter of the serial work in each).
 constexpr int kSbTok = 32;        // tokens per step of the state build
 constexpr int kSbRows = 64;       // state rows per block of the state build
 
@@ -54,6 +56,18 @@ template <int F> struct RowTable {
 };
 template <int F> __device__ constexpr RowTable<F> kRowTable{};
 
+// ---- order ------------------------------------------------------------------------------------
+// A kernel that needs the one before it waits for it first and then lets the next start.  `beside`: it needs only what is complete when
+// that one has begun (see grid_start_beside), runs next to it and waits at its end.
+__device__ __forceinline__ void begin_kernel(bool beside) {
+    if (beside) tc::grid_start_beside();
+    else tc::grid_dependency_wait();
+    tc::grid_launch_dependents();
+}
+__device__ __forceinline__ void end_kernel(bool beside) {
+    if (beside) tc::grid_dependency_wait();
+}
+
 // ---- tiles -------------------------------------------------------------------------------------
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -77,14 +91,14 @@ template <typename T> __device__ __forceinline__ void stage_rows(float* tile, in
 }
 
 // acc[i][j] += sum_k A[8 i][k] B[k][j], j < 4;  K a multiple of 4
-__device__ __forceinline__ void tile_nn(float (&acc)[8][4], const float* A, int lda, const float* B, int ldb, int K) {
+template <int R> __device__ __forceinline__ void tile_nn(float (&acc)[R][4], const float* A, int lda, const float* B, int ldb, int K) {
 #pragma unroll 1
     for (int k = 0; k < K; k += 4) {
         float4 b[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) b[e] = ld4(B + (k + e) * ldb);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < R; ++i) {
             const float4 a = ld4(A + 8 * i * lda + k);
             const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
@@ -98,14 +112,14 @@ __device__ __forceinline__ void tile_nn(float (&acc)[8][4], const float* A, int 
     }
 }
 // acc[i][j] += sum_k A[8 i][k] B[CG j][k], j < JN  (rows of B past its end are the caller's padding)
-template <int CG, int JN> __device__ __forceinline__ void tile_nt(float (&acc)[8][JN], const float* A, int lda, const float* B, int ldb, int K) {
+template <int CG, int JN, int R> __device__ __forceinline__ void tile_nt(float (&acc)[R][JN], const float* A, int lda, const float* B, int ldb, int K) {
 #pragma unroll 1
     for (int k = 0; k < K; k += 4) {
         float4 b[JN];
 #pragma unroll
         for (int j = 0; j < JN; ++j) b[j] = ld4(B + CG * j * ldb + k);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < R; ++i) {
             const float4 a = ld4(A + 8 * i * lda + k);
 #pragma unroll
             for (int j = 0; j < JN; ++j) acc[i][j] = fmaf(a.x, b[j].x, fmaf(a.y, b[j].y, fmaf(a.z, b[j].z, fmaf(a.w, b[j].w, acc[i][j]))));
@@ -149,7 +163,7 @@ __device__ __forceinline__ void stage_values(float* Xs, int ld, float* xz, const
 // that own one row each, so that a row's digits are decoded once per block.
 template <typename T, int F, int CG, bool BWD>
 __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X, const T* __restrict__ O,
-                                                                   const float* __restrict__ eta, float* __restrict__ part, int* __restrict__ clear) {
+                                                                   const float* __restrict__ eta, float* __restrict__ part, int S, bool beside, int* __restrict__ clear) {
     using G = Geo<F>;
     constexpr int NT = CG * 8, DP = G::kDphi, LD = 4 * CG + 4, LT = kSbRows + 4, KF = BWD ? DP : G::kKf, ROWS = BWD ? G::kN : G::kP;
     __shared__ __align__(16) float Ts[kSbTok * LT];
@@ -158,7 +172,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
     __shared__ float xz[kSbTok];
     const int s = blockIdx.x, row0 = blockIdx.y * kSbRows, bh = blockIdx.z;
     const int cg = threadIdx.x % CG, rg = threadIdx.x / CG;      // columns 4 cg .., rows 8 rg ..
-    const int per = ((D.N + D.S - 1) / D.S + kSbTok - 1) / kSbTok * kSbTok;
+    const int per = ((D.N + S - 1) / S + kSbTok - 1) / kSbTok * kSbTok;
     const int t0 = s * per, t1 = min(D.N, t0 + per);
     // the row this thread forms: feature indices of its factors
     const int row = row0 + (threadIdx.x & 63);
@@ -173,8 +187,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
         if (row >= ROWS)
             for (int f = 0; f < F; ++f) dig[f] = 0;
     }
-    tc::grid_launch_dependents();
-    tc::grid_dependency_wait();
+    begin_kernel(beside);
     if (clear && s == 0 && blockIdx.y == 0 && bh == 0 && threadIdx.x < 16) clear[threadIdx.x] = 0;
     float acc[8][4];
 #pragma unroll
@@ -218,13 +231,14 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
             for (int t = 0; t < kSbTok; ++t) zacc = fmaf(Ts[t * LT + threadIdx.x], xz[t], zacc);
         }
     }
-    float* out = part + ((size_t)bh * D.S + s) * ROWS * D.ld;
+    float* out = part + ((size_t)bh * S + s) * ROWS * D.ld;
     if (4 * cg < D.d) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             if (row0 + 8 * rg + i < ROWS) store4(out + (size_t)(row0 + 8 * rg + i) * D.ld + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
     }
     if (threadIdx.x < kSbRows && row < ROWS) store4(out + (size_t)row * D.ld + D.d, make_float4(zacc, 0.f, 0.f, 0.f));
+    end_kernel(beside);
 }
 
 // Sum of the split partials in a fixed order (bit-reproducible) -> state [BH][P][ld].  FOLDED: the partials hold the M monomial rows;
@@ -234,8 +248,7 @@ __global__ void __launch_bounds__(256) tiled_reduce_kernel(float* __restrict__ o
     using G = Geo<F>;
     constexpr int ROWS = FOLDED ? G::kN : G::kP;
     const int q = ld >> 2, total = BH * ROWS * q;
-    tc::grid_launch_dependents();
-    tc::grid_dependency_wait();
+    begin_kernel(false);
     for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
         const int c = i % q, row = (i / q) % ROWS, bh = i / (q * ROWS);
         const float4* src = reinterpret_cast<const float4*>(part) + ((size_t)bh * S * ROWS + row) * q + c;
@@ -310,21 +323,20 @@ template <int F, bool QSIDE> __device__ __forceinline__ void load_token(float* f
 // ---- readout -----------------------------------------------------------------------------------
 // QSIDE: Y = (mono Csym) / (eta + eps), eta = mono . zsym saved.  Key side: dV = Tsym_k dC.  Tile of 64 tokens, thread = 8 tokens x 4
 // columns; the 64 operand rows are formed by 64 threads, one token each, from registers.
-template <typename T, int F, int CG, bool QSIDE>
+template <typename T, int F, int CG, int R, bool QSIDE>
 __global__ void __launch_bounds__(CG * 8) tiled_readout_kernel(Dims D, const float* __restrict__ feat, const float* __restrict__ state, T* __restrict__ Y,
-                                                               float* __restrict__ eta_out) {
+                                                               float* __restrict__ eta_out, bool beside) {
     using G = Geo<F>;
-    constexpr int LD = 4 * CG + 4, LA = G::kNp + 4;
+    constexpr int TM = 8 * R, LD = 4 * CG + 4, LA = G::kNp + 4;
     extern __shared__ __align__(16) float dyn[];
     float* Ss = dyn;                          // [kNp][LD]
-    float* As = Ss + G::kNp * LD;             // [64][LA]
-    float* inv = As + kTm * LA;               // [64]
-    const int bh = blockIdx.y, tok0 = blockIdx.x * kTm;
+    float* As = Ss + G::kNp * LD;             // [TM][LA]
+    float* inv = As + TM * LA;               // [TM]
+    const int bh = blockIdx.y, tok0 = blockIdx.x * TM;
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
-    tc::grid_launch_dependents();
-    tc::grid_dependency_wait();
+    begin_kernel(beside);
     stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
-    if (threadIdx.x < kTm) {
+    if (threadIdx.x < TM) {
         const int tok = tok0 + threadIdx.x;
         constexpr int KF = QSIDE ? G::kDphi : G::kKf;
         float f[KF], v[G::kN];
@@ -337,7 +349,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_readout_kernel(Dims D, const flo
     }
     __syncthreads();
     if (QSIDE) {
-        for (int t = threadIdx.x; t < kTm; t += CG * 8) {
+        for (int t = threadIdx.x; t < TM; t += CG * 8) {
             float e0 = 0.f, e1 = 0.f;
 #pragma unroll 4
             for (int m = 0; m < G::kN; m += 2) {
@@ -348,60 +360,59 @@ __global__ void __launch_bounds__(CG * 8) tiled_readout_kernel(Dims D, const flo
             if (tok0 + t < D.N) eta_out[(size_t)bh * D.N + tok0 + t] = e0 + e1;
         }
     }
-    float acc[8][4];
+    float acc[R][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     if (4 * cg < D.d) tile_nn(acc, As + tg * LA, LA, Ss + 4 * cg, LD, G::kNp);
     if (QSIDE) __syncthreads();
-    if (4 * cg >= D.d) return;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < R; ++i) {
         const int tok = tok0 + tg + 8 * i;
         const float r = QSIDE ? inv[tg + 8 * i] : 1.f;
-        if (tok < D.N) store4(Y + ((size_t)bh * D.N + tok) * D.d + 4 * cg, make_float4(acc[i][0] * r, acc[i][1] * r, acc[i][2] * r, acc[i][3] * r));
+        if (tok < D.N && 4 * cg < D.d) store4(Y + ((size_t)bh * D.N + tok) * D.d + 4 * cg, make_float4(acc[i][0] * r, acc[i][1] * r, acc[i][2] * r, acc[i][3] * r));
     }
+    end_kernel(beside);
 }
 
 // ---- feature gradients -------------------------------------------------------------------------
 // G[t][m] = sum_g X[t][g] S[m][g] + xz[t] S[m][d], then the product rule through the folded outer product, one token per thread.
 // QSIDE: X = r dO, xz = -r (dO . O), S = (C|z) summed over permutations.  Key side: X = V, xz = 1, S = (dC|dz).
-template <typename T, int F, int CG, bool QSIDE>
+template <typename T, int F, int CG, int R, bool QSIDE>
 __global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X, const T* __restrict__ O,
-                                                                    const float* __restrict__ eta, const float* __restrict__ state, float* __restrict__ dfeat) {
+                                                                    const float* __restrict__ eta, const float* __restrict__ state, float* __restrict__ dfeat, bool beside) {
     using G = Geo<F>;
-    constexpr int LD = 4 * CG + 4, JN = (G::kN + CG - 1) / CG, LG = G::kN + 1;
+    constexpr int TM = 8 * R, LD = 4 * CG + 4, JN = (G::kN + CG - 1) / CG, LG = G::kN + 1;
     extern __shared__ __align__(16) float dyn[];
-    float* Xs = dyn;                          // [64][LD]
-    float* Ss = Xs + kTm * LD;                // [CG * JN][LD] (kNp rows are staged; the columns of the rest are not used)
-    float* xz = Ss + CG * JN * LD;            // [64]
-    float* Gs = xz + kTm;                     // [64][LG], an odd stride
-    const int bh = blockIdx.y, tok0 = blockIdx.x * kTm;
+    float* Xs = dyn;                          // [TM][LD]
+    float* Ss = Xs + TM * LD;                // [CG * JN][LD] (kNp rows are staged; the columns of the rest are not used)
+    float* xz = Ss + CG * JN * LD;            // [TM]
+    float* Gs = xz + TM;                     // [TM][LG], an odd stride
+    const int bh = blockIdx.y, tok0 = blockIdx.x * TM;
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
-    tc::grid_launch_dependents();
-    tc::grid_dependency_wait();
+    begin_kernel(beside);
     stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
-    stage_values<T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, kTm, D.N);
+    stage_values<T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, TM, D.N);
     __syncthreads();
-    float acc[8][JN];
+    float acc[R][JN];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < JN; ++j) acc[i][j] = 0.f;
-    tile_nt<CG, JN>(acc, Xs + tg * LD, LD, Ss + cg * LD, LD, D.d);
+    tile_nt<CG, JN, R>(acc, Xs + tg * LD, LD, Ss + cg * LD, LD, D.d);
 #pragma unroll
     for (int j = 0; j < JN; ++j) {
         const int m = cg + CG * j;
         if (m < G::kN) {
             const float z = Ss[m * LD + D.d];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) Gs[(tg + 8 * i) * LG + m] = fmaf(xz[tg + 8 * i], z, acc[i][j]);
+            for (int i = 0; i < R; ++i) Gs[(tg + 8 * i) * LG + m] = fmaf(xz[tg + 8 * i], z, acc[i][j]);
         }
     }
     __syncthreads();
     const int tok = tok0 + threadIdx.x;
-    if (threadIdx.x < kTm && tok < D.N) {
+    if (threadIdx.x < TM && tok < D.N) {
         float g[G::kN];
 #pragma unroll
         for (int m = 0; m < G::kN; ++m) g[m] = Gs[threadIdx.x * LG + m];
@@ -418,28 +429,28 @@ __global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, cons
             for (int m = 0; m < F; ++m) tc::store_feat<G::kDphi>(dfeat + (((size_t)bh * F + m) * D.N + tok) * G::kDphi, dk + m * G::kDphi);
         }
     }
+    end_kernel(beside);
 }
 
 // ---- feature networks --------------------------------------------------------------------------
 // feat = ReLU(W2^T GELU(W1^T x + b1) + b2) of 64 rows and one map (blockIdx.y).  rows = B*H*N; key side: out [bh][maps][N][d_phi].
-template <typename T, int DP, int CG, bool KSIDE>
-__global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __restrict__ X, PhiWeights<T> W, float* __restrict__ out, size_t rows, int N, int d) {
-    constexpr int NT = CG * 8, LD = 4 * CG + 4;
+template <typename T, int DP, int CG, int R, bool KSIDE>
+__global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __restrict__ X, PhiWeights<T> W, float* __restrict__ out, size_t rows, int N, int d, bool beside) {
+    constexpr int TM = 8 * R, NT = CG * 8, LD = 4 * CG + 4;
     extern __shared__ __align__(16) float dyn[];
-    float* Xs = dyn;                  // [64][LD]; the hidden layer later
-    float* Ws = Xs + kTm * LD;        // [d][LD]
+    float* Xs = dyn;                  // [TM][LD]; the hidden layer later
+    float* Ws = Xs + TM * LD;        // [d][LD]
     float* W2s = Ws + 4 * CG * LD;    // [DP][LD], transposed
-    const size_t row0 = (size_t)blockIdx.x * kTm;
+    const size_t row0 = (size_t)blockIdx.x * TM;
     const int m = blockIdx.y, cg = threadIdx.x % CG, tg = threadIdx.x / CG;
-    tc::grid_launch_dependents();
-    tc::grid_dependency_wait();
-    stage_rows(Xs, LD, X, row0, kTm, rows, d);
+    begin_kernel(beside);
+    stage_rows(Xs, LD, X, row0, TM, rows, d);
     stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
     for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
     __syncthreads();
-    float acc[8][4];
+    float acc[R][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     const bool live = 4 * cg < d;
@@ -449,16 +460,16 @@ __global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __re
         for (int j = 0; j < 4; ++j) {
             const float b = ldf(W.b1[m] + 4 * cg + j);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i][j] = gelu_erf(acc[i][j] + b);
+            for (int i = 0; i < R; ++i) acc[i][j] = gelu_erf(acc[i][j] + b);
         }
     }
     __syncthreads();      // the input tile has been read
     if (live) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) store4(Xs + (tg + 8 * i) * LD + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+        for (int i = 0; i < R; ++i) store4(Xs + (tg + 8 * i) * LD + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kTm * DP; i += NT) {
+    for (int i = threadIdx.x; i < TM * DP; i += NT) {
         const int t = i / DP, o = i - t * DP;
         float p0 = 0.f, p1 = 0.f;
         for (int j = 0; j < d; j += 4) {
@@ -477,37 +488,38 @@ __global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __re
             }
         }
     }
+    end_kernel(beside);
 }
 
 // dX[row][:] = sum over maps of W1 (GELU'(h) (.) (W2 (dfeat (.) [feat > 0]))), h recomputed, the ReLU mask from the kept features.
-template <typename T, int DP, int CG, bool KSIDE>
-__global__ void __launch_bounds__(CG * 8) tiled_phi_backward_kernel(const T* __restrict__ X, PhiWeights<T> W, const float* __restrict__ feat,
-                                                                    const float* __restrict__ dfeat, T* __restrict__ dX, size_t rows, int N, int d) {
-    constexpr int NT = CG * 8, LD = 4 * CG + 4, LP = DP + 2;
+// (At least 16 warps per SM where shared memory allows it: at most 128 registers a thread.)
+template <typename T, int DP, int CG, int R, bool KSIDE>
+__global__ void __launch_bounds__(CG * 8, CG == 32 ? 1 : 64 / CG) tiled_phi_backward_kernel(const T* __restrict__ X, PhiWeights<T> W, const float* __restrict__ feat,
+                                                                    const float* __restrict__ dfeat, T* __restrict__ dX, size_t rows, int N, int d, bool beside) {
+    constexpr int TM = 8 * R, NT = CG * 8, LD = 4 * CG + 4, LP = DP + 2;
     extern __shared__ __align__(16) float dyn[];
-    float* Xs = dyn;                          // [64][LD]
-    float* Ws = Xs + kTm * LD;                // [4 CG][LD]
-    float* Hs = Ws + 4 * CG * LD;             // [64][LD] dh
-    float* W2s = Hs + kTm * LD;               // [DP][LD], transposed
-    float* dps = W2s + DP * LD;               // [64][LP]
-    const size_t row0 = (size_t)blockIdx.x * kTm;
+    float* Xs = dyn;                          // [TM][LD]
+    float* Ws = Xs + TM * LD;                // [4 CG][LD]
+    float* Hs = Ws + 4 * CG * LD;             // [TM][LD] dh
+    float* W2s = Hs + TM * LD;               // [DP][LD], transposed
+    float* dps = W2s + DP * LD;               // [TM][LP]
+    const size_t row0 = (size_t)blockIdx.x * TM;
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
     const bool live = 4 * cg < d;
-    tc::grid_launch_dependents();
-    tc::grid_dependency_wait();
-    stage_rows(Xs, LD, X, row0, kTm, rows, d);
+    begin_kernel(beside);
+    stage_rows(Xs, LD, X, row0, TM, rows, d);
     for (int i = threadIdx.x; i < (4 * CG - d) * (d >> 2); i += NT)      // rows of W1 past the head width: read by tile_nt, kept finite
         *reinterpret_cast<float4*>(Ws + (d + i / (d >> 2)) * LD + 4 * (i % (d >> 2))) = make_float4(0.f, 0.f, 0.f, 0.f);
-    float dx[8][4];
+    float dx[R][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) dx[i][j] = 0.f;
     for (int m = 0; m < W.nmaps; ++m) {
         if (m > 0) __syncthreads();      // the previous map's tiles have been read
         stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
         for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
-        for (int i = threadIdx.x; i < kTm * DP; i += NT) {
+        for (int i = threadIdx.x; i < TM * DP; i += NT) {
             const int t = i / DP, o = i - t * DP;
             const size_t row = row0 + t;
             float g = 0.f;
@@ -523,65 +535,76 @@ __global__ void __launch_bounds__(CG * 8) tiled_phi_backward_kernel(const T* __r
         }
         __syncthreads();
         if (live) {
-            float h[8][4];
+            float h[R][4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float b = ldf(W.b1[m] + 4 * cg + j);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) h[i][j] = b;
+                for (int i = 0; i < R; ++i) h[i][j] = b;
             }
             tile_nn(h, Xs + tg * LD, LD, Ws + 4 * cg, LD, d);
+            float dg[R][4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                float dg[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int o = 0; o < DP; ++o) {
+                for (int j = 0; j < 4; ++j) dg[i][j] = 0.f;
+#pragma unroll
+            for (int o = 0; o < DP; ++o) {
+                const float4 w = ld4(W2s + o * LD + 4 * cg);
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
                     const float p = dps[(tg + 8 * i) * LP + o];
-                    const float4 w = ld4(W2s + o * LD + 4 * cg);
-                    dg[0] = fmaf(p, w.x, dg[0]);
-                    dg[1] = fmaf(p, w.y, dg[1]);
-                    dg[2] = fmaf(p, w.z, dg[2]);
-                    dg[3] = fmaf(p, w.w, dg[3]);
+                    dg[i][0] = fmaf(p, w.x, dg[i][0]);
+                    dg[i][1] = fmaf(p, w.y, dg[i][1]);
+                    dg[i][2] = fmaf(p, w.z, dg[i][2]);
+                    dg[i][3] = fmaf(p, w.w, dg[i][3]);
                 }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) dg[j] *= gelu_erf_grad(h[i][j]);
-                store4(Hs + (tg + 8 * i) * LD + 4 * cg, make_float4(dg[0], dg[1], dg[2], dg[3]));
             }
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+                store4(Hs + (tg + 8 * i) * LD + 4 * cg, make_float4(dg[i][0] * gelu_erf_grad(h[i][0]), dg[i][1] * gelu_erf_grad(h[i][1]),
+                                                                    dg[i][2] * gelu_erf_grad(h[i][2]), dg[i][3] * gelu_erf_grad(h[i][3])));
         }
         __syncthreads();
-        tile_nt<CG, 4>(dx, Hs + tg * LD, LD, Ws + cg * LD, LD, d);      // column cg + CG j of dX
+        tile_nt<CG, 4, R>(dx, Hs + tg * LD, LD, Ws + cg * LD, LD, d);      // column cg + CG j of dX
     }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < 4; ++j)      // through shared memory: whole rows leave with 16-byte stores
 #pragma unroll
-        for (int i = 0; i < 8; ++i) Hs[(tg + 8 * i) * LD + cg + CG * j] = dx[i][j];
+        for (int i = 0; i < R; ++i) Hs[(tg + 8 * i) * LD + cg + CG * j] = dx[i][j];
     __syncthreads();
     if (live) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < R; ++i) {
             const size_t row = row0 + tg + 8 * i;
             if (row < rows) store4(dX + row * d + 4 * cg, ld4(Hs + (tg + 8 * i) * LD + 4 * cg));
         }
     }
+    end_kernel(beside);
 }
 
 // ---- host --------------------------------------------------------------------------------------
 inline bool tiled(const Dims& D) { return (D.F == 3 && D.dphi == 6) || (D.F == 2 && D.dphi == 12); }
-// Token splits of a state build: three blocks per SM over all row blocks and heads (each block then walks several 32-token steps at
-// every size but the smallest, and the partials, S x P x ld floats per head, stay a few MB).
+// Token splits of a state build: six blocks per SM over all row blocks and heads (a step is loads, two barriers and 1024 FMAs per thread,
+// so it takes that many blocks side by side to cover them; three per SM: 85 us a build against 49 at B*H = 12, N = 3000, d = 64).
 inline int tiled_splits(int BH, int N, int P, int sm_count) {
-    const int blocks = BH * ((P + kSbRows - 1) / kSbRows), S = (3 * sm_count + blocks - 1) / blocks, most = (N + kSbTok - 1) / kSbTok;
+    const int blocks = BH * ((P + kSbRows - 1) / kSbRows), S = (6 * sm_count + blocks - 1) / blocks, most = (N + kSbTok - 1) / kSbTok;
     return S < most ? S : most;
 }
-template <int F, int CG> struct TiledSmem {
+// The gradient state has M instead of P rows: as many more splits for the same bytes of partials.
+template <int F> inline int tiled_gradient_splits(const Dims& D) {
+    const int S = (int)((long long)D.S * Geo<F>::kP / Geo<F>::kN), most = (D.N + kSbTok - 1) / kSbTok;
+    return S < most ? S : (most > D.S ? most : D.S);
+}
+template <int F, int CG, int R> struct TiledSmem {
     using G = Geo<F>;
-    static constexpr int LD = 4 * CG + 4;
-    static constexpr size_t readout = sizeof(float) * (G::kNp * LD + kTm * (G::kNp + 4) + kTm);
-    static constexpr size_t grad = sizeof(float) * (kTm * LD + (G::kN + CG - 1) / CG * CG * LD + kTm + kTm * (G::kN + 1));
+    static constexpr int LD = 4 * CG + 4, TM = 8 * R;
+    static constexpr size_t readout = sizeof(float) * (G::kNp * LD + TM * (G::kNp + 4) + TM);
+    static constexpr size_t grad = sizeof(float) * (TM * LD + (G::kN + CG - 1) / CG * CG * LD + TM + TM * (G::kN + 1));
     static_assert((G::kN + CG - 1) / CG * CG >= G::kNp, "staged rows");
-    static constexpr size_t phi_fwd = sizeof(float) * (kTm * LD + 4 * CG * LD + G::kDphi * LD);
-    static constexpr size_t phi_bwd = sizeof(float) * (2 * kTm * LD + 4 * CG * LD + G::kDphi * LD + kTm * (G::kDphi + 2));
+    static constexpr size_t phi_fwd = sizeof(float) * (TM * LD + 4 * CG * LD + G::kDphi * LD);
+    static constexpr size_t phi_bwd = sizeof(float) * (2 * TM * LD + 4 * CG * LD + G::kDphi * LD + TM * (G::kDphi + 2));
 };
 
 struct TiledArgs {
@@ -596,10 +619,10 @@ struct TiledArgs {
 };
 
 // Launch sequences.  Every kernel is launched with programmatic stream serialization and waits for its predecessor at its top.
-template <typename T, int F, int CG> struct Tiled {
+template <typename T, int F, int CG, int R> struct Tiled {
     using G = Geo<F>;
-    using S = TiledSmem<F, CG>;
-    static constexpr int NT = CG * 8;
+    using S = TiledSmem<F, CG, R>;
+    static constexpr int NT = CG * 8, TM = 8 * R;
 
     template <typename... KArgs, typename... Args>
     static bool launch(LaunchRec& rec, const char* name, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, Args... args) {
@@ -629,48 +652,55 @@ template <typename T, int F, int CG> struct Tiled {
     static bool forward(const TiledArgs& a, LaunchRec& rec) {
         const Dims& D = a.D;
         const size_t rows = (size_t)a.BH * D.N;
-        const unsigned rb = (unsigned)((rows + kTm - 1) / kTm), tb = (unsigned)((D.N + kTm - 1) / kTm);
+        const unsigned rb = (unsigned)((rows + TM - 1) / TM), tb = (unsigned)((D.N + TM - 1) / TM);
+        // the key maps run beside the query map
         if (a.phi_q) {
-            if (!launch(rec, "simt_phi_forward", tiled_phi_forward_kernel<T, G::kDphi, CG, false>, dim3(rb, 1), NT, S::phi_fwd, in(a.Q), weights(a.phi_q, 1), a.qf_out, rows,
-                        D.N, D.d))
+            if (!launch(rec, "simt_phi_forward", tiled_phi_forward_kernel<T, G::kDphi, CG, R, false>, dim3(rb, 1), NT, S::phi_fwd, in(a.Q), weights(a.phi_q, 1), a.qf_out,
+                        rows, D.N, D.d, false))
                 return false;
-            if (!launch(rec, "simt_phi_forward", tiled_phi_forward_kernel<T, G::kDphi, CG, true>, dim3(rb, F), NT, S::phi_fwd, in(a.K), weights(a.phi_k, F), a.kf_out, rows,
-                        D.N, D.d))
+            if (!launch(rec, "simt_phi_forward", tiled_phi_forward_kernel<T, G::kDphi, CG, R, true>, dim3(rb, F), NT, S::phi_fwd, in(a.K), weights(a.phi_k, F), a.kf_out,
+                        rows, D.N, D.d, true))
                 return false;
         }
         return launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, false>, dim3(D.S, (G::kP + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.kf, in(a.V),
-                      in(nullptr), a.eta, a.part, a.clear) &&
+                      in(nullptr), a.eta, a.part, D.S, false, a.clear) &&
                launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, false>, reduce_grid(a, G::kP), 256, 0, a.state, a.part, a.BH, D.S, D.ld) &&
-               launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, true>, dim3(tb, a.BH), NT, S::readout, D, a.qf, a.state, out(a.Oout), a.eta);
+               launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, R, true>, dim3(tb, a.BH), NT, S::readout, D, a.qf, a.state, out(a.Oout), a.eta, false);
     }
     static bool backward(const TiledArgs& a, LaunchRec& rec) {
         const Dims& D = a.D;
         const size_t rows = (size_t)a.BH * D.N;
-        const unsigned rb = (unsigned)((rows + kTm - 1) / kTm), tb = (unsigned)((D.N + kTm - 1) / kTm);
-        // pass over the queries: dC, dz, then dq;  pass over the keys: dV, dk^f
-        if (!(launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(D.S, (G::kN + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.qf, in(a.dO), in(a.O),
-                     a.eta, a.part, nullptr) &&
-              launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, D.S, D.ld) &&
-              launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state, a.dqf) &&
-              launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, false>, dim3(tb, a.BH), NT, S::readout, D, a.kf, a.dstate, out(a.dV), a.eta) &&
-              launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, false>, dim3(tb, a.BH), NT, S::grad, D, a.kf, in(a.V), in(nullptr), a.eta, a.dstate, a.dkf)))
+        const unsigned rb = (unsigned)((rows + TM - 1) / TM), tb = (unsigned)((D.N + TM - 1) / TM);
+        const int Sg = tiled_gradient_splits<F>(D);
+        // dq, and beside it the partials of dC, dz;  their sum;  dk^f, and beside it dV;  the feature networks of Q (dq is long complete) beside
+        // that, then those of K
+        if (!(launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state, a.dqf,
+                     false) &&
+              launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(Sg, (G::kN + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.qf, in(a.dO), in(a.O),
+                     a.eta, a.part, Sg, true, nullptr) &&
+              launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, Sg, D.ld) &&
+              launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::grad, D, a.kf, in(a.V), in(nullptr), a.eta, a.dstate,
+                     a.dkf, false) &&
+              launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::readout, D, a.kf, a.dstate, out(a.dV), a.eta, true)))
             return false;
         if (!a.phi_q) return true;
-        return launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, false>, dim3(rb), NT, S::phi_bwd, in(a.Q), weights(a.phi_q, 1), a.qf, a.dqf,
-                      out(a.dQ), rows, D.N, D.d) &&
-               launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, true>, dim3(rb), NT, S::phi_bwd, in(a.K), weights(a.phi_k, F), a.kf, a.dkf, out(a.dK),
-                      rows, D.N, D.d);
+        return launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, R, false>, dim3(rb), NT, S::phi_bwd, in(a.Q), weights(a.phi_q, 1), a.qf, a.dqf,
+                      out(a.dQ), rows, D.N, D.d, true) &&
+               launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, R, true>, dim3(rb), NT, S::phi_bwd, in(a.K), weights(a.phi_k, F), a.kf, a.dkf,
+                      out(a.dK), rows, D.N, D.d, false);
     }
 };
 
 // The column groups of a block: the smallest of 8, 16, 32 (x 4 columns) that covers the head width.
-template <typename T, int F> inline bool run_tiled_f(const TiledArgs& a, bool fwd, LaunchRec& rec) {
-    if (a.D.d <= 32) return fwd ? Tiled<T, F, 8>::forward(a, rec) : Tiled<T, F, 8>::backward(a, rec);
-    if (a.D.d <= 64) return fwd ? Tiled<T, F, 16>::forward(a, rec) : Tiled<T, F, 16>::backward(a, rec);
-    return fwd ? Tiled<T, F, 32>::forward(a, rec) : Tiled<T, F, 32>::backward(a, rec);
+template <typename T, int F, int R> inline bool run_tiled_r(const TiledArgs& a, bool fwd, LaunchRec& rec) {
+    if (a.D.d <= 32) return fwd ? Tiled<T, F, 8, R>::forward(a, rec) : Tiled<T, F, 8, R>::backward(a, rec);
+    if (a.D.d <= 64) return fwd ? Tiled<T, F, 16, R>::forward(a, rec) : Tiled<T, F, 16, R>::backward(a, rec);
+    return fwd ? Tiled<T, F, 32, R>::forward(a, rec) : Tiled<T, F, 32, R>::backward(a, rec);
 }
-template <typename T> inline bool run_tiled(const TiledArgs& a, bool fwd, LaunchRec& rec) {
-    return a.D.F == 3 ? run_tiled_f<T, 3>(a, fwd, rec) : run_tiled_f<T, 2>(a, fwd, rec);
+template <typename T> inline bool run_tiled(const TiledArgs& a, bool fwd, int sm_count, LaunchRec& rec) {
+    const bool few = (long long)a.BH * ((a.D.N + 63) / 64) < sm_count;
+    if (a.D.F == 3) return few ? run_tiled_r<T, 3, 2>(a, fwd, rec) : run_tiled_r<T, 3, 8>(a, fwd, rec);
+    return few ? run_tiled_r<T, 2, 2>(a, fwd, rec) : run_tiled_r<T, 2, 8>(a, fwd, rec);
 }
 
 }  // namespace simt
