@@ -15,10 +15,12 @@ EPS = 1e-6
 f64 = lambda a: np.asarray(a, np.float64)
 
 
+# (the last three: enough heads for the tiles of 64 tokens, the others run on tiles of 16)
 @pytest.mark.parametrize("F,dphi", [(3, 6), (2, 12)])
-@pytest.mark.parametrize("d,N,splits", [(4, 1, 0), (28, 63, 0), (32, 64, 5), (36, 65, 0), (64, 31, 0), (64, 129, 3), (68, 33, 0), (128, 200, 0)])
-def test_core_forward_backward(F, dphi, d, N, splits):
-    s = synth.HlaShape("t", 1, 3, N, d, "f32", "inv_sqrt_d", F=F, d_phi=dphi)
+@pytest.mark.parametrize("H,d,N,splits", [(3, 4, 1, 0), (3, 28, 63, 0), (3, 32, 64, 5), (3, 36, 65, 0), (3, 64, 31, 0), (3, 64, 129, 3), (3, 68, 33, 0), (3, 128, 200, 0),
+                                          (150, 32, 63, 0), (75, 64, 65, 0), (50, 128, 130, 2)])
+def test_core_forward_backward(F, dphi, H, d, N, splits):
+    s = synth.HlaShape("t", 1, H, N, d, "f32", "inv_sqrt_d", F=F, d_phi=dphi)
     _, _, V = synth.make_qkv(s)
     V = V * np.float32(np.sqrt(d))
     qf, kf = synth.make_features(s)
@@ -39,11 +41,12 @@ def test_core_forward_backward(F, dphi, d, N, splits):
     assert np.abs(dk - rk).max() < TOL["f32"] * max(np.abs(rk).max(), term)
 
 
-@pytest.mark.parametrize("F,dphi,d,N,dtype", [(3, 6, 16, 70, "f32"), (2, 12, 20, 64, "f32"), (3, 6, 64, 65, "f32"), (2, 12, 128, 33, "f32"), (3, 6, 100, 130, "f32"),
-                                              (3, 6, 32, 65, "bf16"), (2, 12, 72, 40, "bf16")])
-def test_with_phi_stage_by_stage(F, dphi, d, N, dtype):
+@pytest.mark.parametrize("F,dphi,H,d,N,dtype", [(3, 6, 2, 16, 70, "f32"), (2, 12, 2, 20, 64, "f32"), (3, 6, 2, 64, 65, "f32"), (2, 12, 2, 128, 33, "f32"),
+                                                (3, 6, 2, 100, 130, "f32"), (3, 6, 2, 32, 65, "bf16"), (2, 12, 2, 72, 40, "bf16"), (3, 6, 75, 20, 63, "f32"),
+                                                (2, 12, 38, 64, 129, "f32"), (3, 6, 38, 128, 129, "f32"), (3, 6, 75, 32, 63, "bf16")])
+def test_with_phi_stage_by_stage(F, dphi, H, d, N, dtype):
     """Feature networks forward and backward, each stage on the features and feature gradients the library kept."""
-    s = synth.HlaShape("t", 2, 2, N, d, dtype, "rms_qk", F=F, d_phi=dphi)
+    s = synth.HlaShape("t", 2, H, N, d, dtype, "rms_qk", F=F, d_phi=dphi)
     Q, K, V = synth.make_qkv(s)
     dO = synth.make_dO(s)
     pq, pk = synth.make_phi_weights(d, dphi, F, dtype)
