@@ -503,16 +503,23 @@ hla_status backward_impl(hla_ctx* ctx, const void* Q, const void* K, const void*
         const float* kf = mlp ? reinterpret_cast<const float*>(ws + ctx->L.kf) : static_cast<const float*>(K);
         float* dqf = mlp ? reinterpret_cast<float*>(ws + ctx->L.dqf) : static_cast<float*>(dQ);
         float* dkf = mlp ? reinterpret_cast<float*>(ws + ctx->L.dkf) : static_cast<float*>(dK);
+        // the feature network of the queries needs only the query side's result: its backward is launched in the middle of the core's
+        const bool inside = mlp && phase == 0;
+        auto query_map = [&]() { return tc::phi_backward<false>(ctx->D, ctx->BH, &ctx->phi_q, Q, dQ, ws, ctx->L, ctx->sm_count, ctx->rec); };
         if (ctx->cfg.causal) {
             if (ctx->carry) return HLA_ERR_UNSUPPORTED;      // a chunk that started from a carried state has no backward here
             const tc::CausalPieces fwd = mlp ? tc::CausalPieces{ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count)}
                                              : tc::CausalPieces{ctx->off_part, ctx->D.S, 0};
-            s = tc::causal_backward(ctx->D, ctx->BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, ctx->L, fwd, ctx->off_gpart, ctx->off_delta, ctx->rec);
+            s = tc::causal_backward(ctx->D, ctx->BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, ctx->L, fwd, ctx->off_gpart, ctx->off_delta, ctx->rec, inside, query_map);
         } else {
-            s = tc::core_backward(ctx->tcp, ctx->D, ctx->BH, qf, kf, V, dO, dqf, dkf, dV, ws, ctx->L, ctx->off_part, ctx->sm_count, ctx->rec, phase);
+            s = tc::core_backward(ctx->tcp, ctx->D, ctx->BH, qf, kf, V, dO, dqf, dkf, dV, ws, ctx->L, ctx->off_part, ctx->sm_count, ctx->rec, phase, inside, query_map);
         }
         if (s != HLA_OK || !mlp || phase == 1) return s;
-        return tc::phi_backward(ctx->D, ctx->BH, &ctx->phi_q, ctx->phi_k, Q, K, dQ, dK, ws, ctx->L, ctx->sm_count, ctx->rec);
+        if (!inside) {
+            s = query_map();
+            if (s != HLA_OK) return s;
+        }
+        return tc::phi_backward<true>(ctx->D, ctx->BH, ctx->phi_k, K, dK, ws, ctx->L, ctx->sm_count, ctx->rec);
     }
     if (ctx->cfg.dtype == HLA_F32) return backward_simt<float>(ctx, Q, K, V, O, dO, dQ, dK, dV, ws, st);
     return backward_simt<__nv_bfloat16>(ctx, Q, K, V, O, dO, dQ, dK, dV, ws, st);

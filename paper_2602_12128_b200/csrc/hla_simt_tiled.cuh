@@ -56,18 +56,6 @@ template <int F> struct RowTable {
 };
 template <int F> __device__ constexpr RowTable<F> kRowTable{};
 
-// ---- order ------------------------------------------------------------------------------------
-// A kernel that needs the one before it waits for it first and then lets the next start.  `beside`: it needs only what is complete when
-// that one has begun (see grid_start_beside), runs next to it and waits at its end.
-__device__ __forceinline__ void begin_kernel(bool beside) {
-    if (beside) tc::grid_start_beside();
-    else tc::grid_dependency_wait();
-    tc::grid_launch_dependents();
-}
-__device__ __forceinline__ void end_kernel(bool beside) {
-    if (beside) tc::grid_dependency_wait();
-}
-
 // ---- tiles -------------------------------------------------------------------------------------
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -187,7 +175,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
         if (row >= ROWS)
             for (int f = 0; f < F; ++f) dig[f] = 0;
     }
-    begin_kernel(beside);
+    tc::grid_begin(beside);
     if (clear && s == 0 && blockIdx.y == 0 && bh == 0 && threadIdx.x < 16) clear[threadIdx.x] = 0;
     float acc[8][4];
 #pragma unroll
@@ -238,7 +226,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
             if (row0 + 8 * rg + i < ROWS) store4(out + (size_t)(row0 + 8 * rg + i) * D.ld + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
     }
     if (threadIdx.x < kSbRows && row < ROWS) store4(out + (size_t)row * D.ld + D.d, make_float4(zacc, 0.f, 0.f, 0.f));
-    end_kernel(beside);
+    tc::grid_end(beside);
 }
 
 // Sum of the split partials in a fixed order (bit-reproducible) -> state [BH][P][ld].  FOLDED: the partials hold the M monomial rows;
@@ -248,7 +236,7 @@ __global__ void __launch_bounds__(256) tiled_reduce_kernel(float* __restrict__ o
     using G = Geo<F>;
     constexpr int ROWS = FOLDED ? G::kN : G::kP;
     const int q = ld >> 2, total = BH * ROWS * q;
-    begin_kernel(false);
+    tc::grid_begin(false);
     for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
         const int c = i % q, row = (i / q) % ROWS, bh = i / (q * ROWS);
         const float4* src = reinterpret_cast<const float4*>(part) + ((size_t)bh * S * ROWS + row) * q + c;
@@ -334,7 +322,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_readout_kernel(Dims D, const flo
     float* inv = As + TM * LA;               // [TM]
     const int bh = blockIdx.y, tok0 = blockIdx.x * TM;
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
-    begin_kernel(beside);
+    tc::grid_begin(beside);
     stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
     if (threadIdx.x < TM) {
         const int tok = tok0 + threadIdx.x;
@@ -373,7 +361,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_readout_kernel(Dims D, const flo
         const float r = QSIDE ? inv[tg + 8 * i] : 1.f;
         if (tok < D.N && 4 * cg < D.d) store4(Y + ((size_t)bh * D.N + tok) * D.d + 4 * cg, make_float4(acc[i][0] * r, acc[i][1] * r, acc[i][2] * r, acc[i][3] * r));
     }
-    end_kernel(beside);
+    tc::grid_end(beside);
 }
 
 // ---- feature gradients -------------------------------------------------------------------------
@@ -391,7 +379,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, cons
     float* Gs = xz + TM;                     // [TM][LG], an odd stride
     const int bh = blockIdx.y, tok0 = blockIdx.x * TM;
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
-    begin_kernel(beside);
+    tc::grid_begin(beside);
     stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
     stage_values<T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, TM, D.N);
     __syncthreads();
@@ -429,7 +417,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, cons
             for (int m = 0; m < F; ++m) tc::store_feat<G::kDphi>(dfeat + (((size_t)bh * F + m) * D.N + tok) * G::kDphi, dk + m * G::kDphi);
         }
     }
-    end_kernel(beside);
+    tc::grid_end(beside);
 }
 
 // ---- feature networks --------------------------------------------------------------------------
@@ -443,7 +431,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __re
     float* W2s = Ws + 4 * CG * LD;    // [DP][LD], transposed
     const size_t row0 = (size_t)blockIdx.x * TM;
     const int m = blockIdx.y, cg = threadIdx.x % CG, tg = threadIdx.x / CG;
-    begin_kernel(beside);
+    tc::grid_begin(beside);
     stage_rows(Xs, LD, X, row0, TM, rows, d);
     stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
     for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
@@ -488,7 +476,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __re
             }
         }
     }
-    end_kernel(beside);
+    tc::grid_end(beside);
 }
 
 // dX[row][:] = sum over maps of W1 (GELU'(h) (.) (W2 (dfeat (.) [feat > 0]))), h recomputed, the ReLU mask from the kept features.
@@ -506,7 +494,7 @@ __global__ void __launch_bounds__(CG * 8, CG == 32 ? 1 : 64 / CG) tiled_phi_back
     const size_t row0 = (size_t)blockIdx.x * TM;
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
     const bool live = 4 * cg < d;
-    begin_kernel(beside);
+    tc::grid_begin(beside);
     stage_rows(Xs, LD, X, row0, TM, rows, d);
     for (int i = threadIdx.x; i < (4 * CG - d) * (d >> 2); i += NT)      // rows of W1 past the head width: read by tile_nt, kept finite
         *reinterpret_cast<float4*>(Ws + (d + i / (d >> 2)) * LD + 4 * (i % (d >> 2))) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -581,7 +569,7 @@ __global__ void __launch_bounds__(CG * 8, CG == 32 ? 1 : 64 / CG) tiled_phi_back
             if (row < rows) store4(dX + row * d + 4 * cg, ld4(Hs + (tg + 8 * i) * LD + 4 * cg));
         }
     }
-    end_kernel(beside);
+    tc::grid_end(beside);
 }
 
 // ---- host --------------------------------------------------------------------------------------

@@ -405,7 +405,7 @@ template <int DV, int F, bool GRAD = false>
 __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __grid_constant__ CUtensorMap mapV, const float* __restrict__ kf,
                                                                        float* __restrict__ part, int N, int S, int ld, int* status,
                                                                        const float* __restrict__ eta = nullptr, const float* __restrict__ delta = nullptr,
-                                                                       float eps = 0.f, int clear = 0) {
+                                                                       float eps = 0.f, int clear = 0, bool beside = false) {
     using M = MT<F>;
     using Cfg = SbCfg<F>;
     constexpr int kStages = Cfg::kStages, kStageBytes = Cfg::kStageBytes;
@@ -427,10 +427,10 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     const int ntiles = max(0, min(tiles, tile0 + tiles_per) - tile0);
     float* out = part + ((size_t)bh * S + s) * M::kN * ld;
 
-    grid_launch_dependents();
     if (ntiles == 0) {   // an empty split contributes zeros (never split 0)
-        grid_dependency_wait();
+        grid_begin(beside);
         for (int i = tid; i < M::kN * ld; i += kSbThreads) out[i] = 0.f;
+        grid_end(beside);
         return;
     }
     if (DV == 64) {      // rows 64..127 of the MMA's M dimension read a second V block: keep it zero
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    grid_begin(beside);
     if (clear && s == 0 && bh == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
     bool ok = true;
 
@@ -576,6 +576,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, Cfg::kTmemCols);
+    grid_end(beside);
 }
 
 // =======================================================================================
@@ -590,12 +591,11 @@ __host__ __device__ inline int owner_of_work(long long w, long long total, int G
 
 template <int DV, int F>
 __global__ void __launch_bounds__(256) tc_reduce_emit_kernel(const float* __restrict__ part, float* __restrict__ state,
-                                                             __nv_bfloat16* __restrict__ b3, __nv_bfloat16* __restrict__ bq, int S, int ld, int G, int T) {
+                                                             __nv_bfloat16* __restrict__ b3, __nv_bfloat16* __restrict__ bq, int S, int ld, int G, int T, bool beside) {
     constexpr int kN = MT<F>::kN, kPad = MT<F>::kPad;
     __shared__ float sm[8][kMaxD + 8];
     const int m0 = 8 * blockIdx.x, bh = blockIdx.y, tid = threadIdx.x;      // gridDim.x = kPad / 8
-    grid_launch_dependents();
-    grid_dependency_wait();
+    grid_begin(beside);
     const size_t n_per = (size_t)kN * ld;
     int count = S;
     if (G > 0) {
@@ -625,6 +625,7 @@ __global__ void __launch_bounds__(256) tc_reduce_emit_kernel(const float* __rest
         const int mm = i / DV, g = i - mm * DV;
         oq[(size_t)(m0 + mm) * DV + g] = __float2bfloat16_rn(sm[mm][g]);
     }
+    grid_end(beside);
 }
 
 // =======================================================================================
@@ -1425,10 +1426,10 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
     if (!set_smem(tc_state_build_kernel<DV, F>, SbCfg<F>::kSmem) || !set_smem(tc_readout_kernel<DV, F>, RoCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
     cudaStream_t st = rec.st;
     rec.begin("tc_state_build");
-    launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (const float*)nullptr, 0.f, 1);
+    launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (const float*)nullptr, 0.f, 1, false);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_reduce_emit");
-    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, state, b3, bq, D.S, D.ld, 0, 0);
+    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, state, b3, bq, D.S, D.ld, 0, 0, false);
     if (!rec.end()) return HLA_ERR_CUDA;
     if (!readout) return HLA_OK;
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
@@ -1448,8 +1449,8 @@ inline hla_status reduce_pieces_f(const Plan& P, const Dims& D, int BH, char* ws
     float* state = reinterpret_cast<float*>(ws + L.state);
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_reduce_emit");
-    if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T);
-    else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T);
+    if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T, false);
+    else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 inline hla_status reduce_pieces(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec) {
@@ -1465,7 +1466,7 @@ inline hla_status launch_emit_from_state(const Plan& P, const Dims& D, int BH, c
     __nv_bfloat16* b3 = reinterpret_cast<__nv_bfloat16*>(ws + (gradient ? P.bd3 : P.b3));
     __nv_bfloat16* bq = reinterpret_cast<__nv_bfloat16*>(ws + (gradient ? P.bdq : P.bq));
     rec.begin("tc_reduce_emit");
-    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, (const float*)st, st, b3, bq, 1, D.ld, 0, 0);
+    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, (const float*)st, st, b3, bq, 1, D.ld, 0, 0, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 inline hla_status emit_from_state(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, bool gradient, LaunchRec& rec) {
@@ -1505,10 +1506,11 @@ inline hla_status core_forward(const Plan& P, const Dims& D, int BH, const float
     return launch_core_forward<64, 2>(P, D, BH, qf, kf, V, O, ws, L, off_part, sm_count, rec, readout);
 }
 
-template <int DV, int F>
+// `between` (run_between: there is such a step) is launched after the query pass; the reduction then runs beside it.
+template <int DV, int F, typename Between>
 inline hla_status launch_core_backward(const Plan& P, const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* dO,
                                        float* dqf, float* dkf, void* dV, char* ws, const hla_ws_layout& L, size_t off_part, int sm_count,
-                                       LaunchRec& rec, int phase) {
+                                       LaunchRec& rec, int phase, bool run_between, Between&& between) {
     // phase 0: the whole backward; 1: query pass and reduction only (leaves the gradient state in the workspace);
     // 2: key pass only, on the gradient state in the workspace (its operand images are formed first)
     constexpr int kPad = MT<F>::kPad;
@@ -1532,8 +1534,12 @@ inline hla_status launch_core_backward(const Plan& P, const Dims& D, int BH, con
         launch_pdl(tc_bwd_query_kernel<DV, F>, dim3(D.S, BH), dim3(kBqThreads), BqCfg<F>::kSmem, st, mapdO, mapBq, qf, eta, state, dqf, part, D.N, D.S, D.ld, D.eps,
                    status);
         if (!rec.end()) return HLA_ERR_CUDA;
+        if (run_between) {
+            const hla_status e = between();
+            if (e != HLA_OK) return e;
+        }
         rec.begin("tc_reduce_emit");
-        launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, dstate, bd3, bdq, D.S, D.ld, 0, 0);
+        launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, dstate, bd3, bdq, D.S, D.ld, 0, 0, run_between);
         if (!rec.end()) return HLA_ERR_CUDA;
         if (phase == 1) return HLA_OK;
     } else {
@@ -1549,15 +1555,16 @@ inline hla_status launch_core_backward(const Plan& P, const Dims& D, int BH, con
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
+template <typename Between>
 inline hla_status core_backward(const Plan& P, const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* dO,
                                 float* dqf, float* dkf, void* dV, char* ws, const hla_ws_layout& L, size_t off_part, int sm_count, LaunchRec& rec,
-                                int phase = 0) {
+                                int phase, bool run_between, Between&& between) {
     if (D.F == 3) {
-        if (D.d == 128) return launch_core_backward<128, 3>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase);
-        return launch_core_backward<64, 3>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase);
+        if (D.d == 128) return launch_core_backward<128, 3>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase, run_between, between);
+        return launch_core_backward<64, 3>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase, run_between, between);
     }
-    if (D.d == 128) return launch_core_backward<128, 2>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase);
-    return launch_core_backward<64, 2>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase);
+    if (D.d == 128) return launch_core_backward<128, 2>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase, run_between, between);
+    return launch_core_backward<64, 2>(P, D, BH, qf, kf, V, dO, dqf, dkf, dV, ws, L, off_part, sm_count, rec, phase, run_between, between);
 }
 
 }  // namespace tc

@@ -145,11 +145,11 @@ __device__ __forceinline__ void tmem_st_state(uint32_t taddr, const float (&v)[8
 // piece gets the sum of the pieces after it).  carry != 0: the scan starts from what `state` holds (the state an earlier
 // call left there: Eq. "seq.updates" continued across calls) instead of zero.
 template <int F, bool REVERSE = false>
-__global__ void __launch_bounds__(256) tc_scan_pieces_kernel(float* __restrict__ part, float* __restrict__ state, int S, int ld, int G, int T, int carry) {
+__global__ void __launch_bounds__(256) tc_scan_pieces_kernel(float* __restrict__ part, float* __restrict__ state, int S, int ld, int G, int T, int carry,
+                                                             bool beside) {
     constexpr int kN = MT<F>::kN;
     const int bh = blockIdx.y;
-    grid_launch_dependents();
-    grid_dependency_wait();
+    grid_begin(beside);
     const size_t n_per = (size_t)kN * ld;
     int count = S;
     if (G > 0) {
@@ -157,9 +157,10 @@ __global__ void __launch_bounds__(256) tc_scan_pieces_kernel(float* __restrict__
         count = owner_of_work((long long)bh * T + T - 1, total, G) - owner_of_work((long long)bh * T, total, G) + 1;
     }
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (e >= n_per) return;
-    float* p = part + (size_t)bh * S * n_per + e;
-    float run = carry ? state[(size_t)bh * n_per + e] : 0.f;
+    const bool mine = e < n_per;
+    float* p = part + (size_t)bh * S * n_per + (mine ? e : 0);
+    float run = carry && mine ? state[(size_t)bh * n_per + e] : 0.f;
+    if (!mine) count = 0;
     for (int s0 = 0; s0 < count; s0 += 8) {      // eight independent loads in flight, then the scan in piece order
         float t[8];
 #pragma unroll
@@ -171,7 +172,8 @@ __global__ void __launch_bounds__(256) tc_scan_pieces_kernel(float* __restrict__
                 run += t[k];
             }
     }
-    state[(size_t)bh * n_per + e] = run;
+    if (mine) state[(size_t)bh * n_per + e] = run;
+    grid_end(beside);
 }
 
 // MODE 0: the forward sweep described above.
@@ -213,7 +215,6 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     const int w0 = cw.w0, nwork = cw.w1 - cw.w0;
     auto work_of = [&](int it) { return MODE == 0 ? w0 + it : w0 + nwork - 1 - it; };                 // (head, tile) of the CTA's it-th item
     auto starts = [&](int it) { return it == 0 || (MODE == 0 && (w0 + it) % T == 0); };          // a piece begins with this item
-    grid_launch_dependents();
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    grid_begin(false);
     bool ok = true;
 
     if (warp == 0) {
@@ -578,7 +579,7 @@ inline hla_status launch_causal_sweep(const Dims& D, int BH, const float* qf, co
     if (!set_smem(tc_causal_forward_kernel<DV, 0>, CaCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_scan_pieces");
-    launch_pdl(tc_scan_pieces_kernel<3>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, state, S, D.ld, G, T, carry ? 1 : 0);
+    launch_pdl(tc_scan_pieces_kernel<3>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, state, S, D.ld, G, T, carry ? 1 : 0, false);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_causal_forward");
     launch_pdl(tc_causal_forward_kernel<DV, 0>, G > 0 ? dim3(G) : dim3(S, BH), dim3(kCaThreads), CaCfg<DV>::kSmem, rec.st, mapV, mapO, qf, kf,
@@ -602,7 +603,7 @@ inline hla_status launch_causal_state_build(const Dims& D, int BH, const float* 
     if (!set_smem(tc_state_build_kernel<DV, 3>, SbCfg<3>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_state_build");
     launch_pdl(tc_state_build_kernel<DV, 3>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapV, kf, reinterpret_cast<float*>(ws + off_part), D.N, D.S,
-               D.ld, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, (const float*)nullptr, 0.f, 1);
+               D.ld, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, (const float*)nullptr, 0.f, 1, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
@@ -620,8 +621,7 @@ template <int DV>
 __global__ void __launch_bounds__(256) tc_delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO, float* __restrict__ delta,
                                                        long long rows) {
     constexpr int LPR = DV / 8;                 // lanes per row
-    grid_launch_dependents();
-    grid_dependency_wait();
+    grid_begin(false);
     const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
     const long long row = t / LPR;
     const int part = (int)(t % LPR);
@@ -650,11 +650,12 @@ inline hla_status launch_causal_delta(const Dims& D, int BH, const void* O, cons
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
-// Backward of the causal operator at the feature level, value side: the gradient state of every piece, its suffix scan,
-// and the sweep that gives dV (delta must have been computed).
-template <int DV>
+// Backward of the causal operator at the feature level, value side: the gradient state of every piece (beside the kernel before, which
+// must itself have waited for delta), its suffix scan, and the sweep that gives dV.  `between` (run_between: there is such a step) is
+// launched before the scan, which then runs beside it.
+template <int DV, typename Between>
 inline hla_status launch_causal_backward_values(const Dims& D, int BH, const float* qf, const float* kf, const void* dO, void* dV, char* ws,
-                                                const hla_ws_layout& L, size_t off_gpart, size_t off_delta, LaunchRec& rec) {
+                                                const hla_ws_layout& L, size_t off_gpart, size_t off_delta, LaunchRec& rec, bool run_between, Between&& between) {
     CUtensorMap mapdO, mapdV;
     if (!make_map_bhnd(&mapdO, dO, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapdV, dV, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
     int* status = reinterpret_cast<int*>(ws + L.status);
@@ -666,10 +667,14 @@ inline hla_status launch_causal_backward_values(const Dims& D, int BH, const flo
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_dstate_build");
     launch_pdl(tc_state_build_kernel<DV, 3, true>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapdO, qf, part, D.N, D.S, D.ld, status,
-               (const float*)eta, (const float*)delta, D.eps, 0);
+               (const float*)eta, (const float*)delta, D.eps, 0, true);
     if (!rec.end()) return HLA_ERR_CUDA;
+    if (run_between) {
+        const hla_status e = between();
+        if (e != HLA_OK) return e;
+    }
     rec.begin("tc_scan_pieces");
-    launch_pdl(tc_scan_pieces_kernel<3, true>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, dstate, D.S, D.ld, 0, T, 0);
+    launch_pdl(tc_scan_pieces_kernel<3, true>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, dstate, D.S, D.ld, 0, T, 0, run_between);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dv");
     launch_pdl(tc_causal_forward_kernel<DV, 1>, dim3(D.S, BH), dim3(kCaThreads), CaCfg<DV>::kSmem, rec.st, mapdO, mapdV, qf, kf, (const float*)part,

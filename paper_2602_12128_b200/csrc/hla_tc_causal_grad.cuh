@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                                                                        const float* __restrict__ qf, const float* __restrict__ kf,
                                                                        const float* __restrict__ eta, const float* __restrict__ delta,
                                                                        const float* __restrict__ init, float* __restrict__ out, int N, int BH, int S, int ld,
-                                                                       int G, float eps, int* status) {
+                                                                       int G, float eps, int* status, bool beside) {
     using Cfg = CgCfg<DV>;
     constexpr int kStageBytes = Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
@@ -98,7 +98,6 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
         }
     };
     auto starts = [&](int it) { return it == 0 || (DIR == 0 && (w0 + it) % T == 0); };      // a piece begins with this item
-    grid_launch_dependents();
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -129,7 +128,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    grid_begin(beside);
     bool ok = true;
 
     if (warp >= kCgEpiWarp0) {
@@ -500,6 +499,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
+    grid_end(beside);
 }
 
 // The pieces the forward swept, and the prefix states of which it left in the workspace: S slots per head, G as in CaWork.
@@ -524,32 +524,35 @@ inline hla_status launch_causal_backward_features(const Dims& D, int BH, const f
         if (!set_smem(tc_causal_grad_kernel<DV, 0>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
         rec.begin("tc_causal_dq");
         launch_pdl(tc_causal_grad_kernel<DV, 0>, fwd.G > 0 ? dim3(fwd.G) : dim3(fwd.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapdO, mapV, qf, kf, eta, delta,
-                   reinterpret_cast<const float*>(ws + fwd.off), dqf, D.N, BH, fwd.S, D.ld, fwd.G, D.eps, status);
+                   reinterpret_cast<const float*>(ws + fwd.off), dqf, D.N, BH, fwd.S, D.ld, fwd.G, D.eps, status, false);
         return rec.end() ? HLA_OK : HLA_ERR_CUDA;
     }
     if (!set_smem(tc_causal_grad_kernel<DV, 1>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dk");
     launch_pdl(tc_causal_grad_kernel<DV, 1>, dim3(D.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapV, mapdO, qf, kf, eta, delta,
-               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, D.ld, 0, D.eps, status);
+               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, D.ld, 0, D.eps, status, true);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
-// dO . o, then dq on the forward states, then the gradient states (in a region of their own, so that the forward's stay), dV and dk on them.
-template <int DV>
+// dO . o, then dq on the forward states, beside it the gradient states (in a region of their own, so that the forward's stay), their scan
+// (beside `between`, the next step of the query side), dV and beside it dk.
+template <int DV, typename Between>
 inline hla_status launch_causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf,
                                          float* dkf, void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta,
-                                         LaunchRec& rec) {
+                                         LaunchRec& rec, bool run_between, Between&& between) {
     hla_status s = launch_causal_delta<DV>(D, BH, O, dO, ws, off_delta, rec);
     if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, false, rec);
-    if (s == HLA_OK) s = launch_causal_backward_values<DV>(D, BH, qf, kf, dO, dV, ws, L, off_gpart, off_delta, rec);
+    if (s == HLA_OK) s = launch_causal_backward_values<DV>(D, BH, qf, kf, dO, dV, ws, L, off_gpart, off_delta, rec, run_between, between);
     if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, true, rec);
     return s;
 }
+template <typename Between>
 inline hla_status causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf, float* dkf,
-                                  void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta, LaunchRec& rec) {
+                                  void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta, LaunchRec& rec,
+                                  bool run_between, Between&& between) {
     if (D.F != 3) return HLA_ERR_UNSUPPORTED;
-    if (D.d == 128) return launch_causal_backward<128>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec);
-    return launch_causal_backward<64>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec);
+    if (D.d == 128) return launch_causal_backward<128>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec, run_between, between);
+    return launch_causal_backward<64>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec, run_between, between);
 }
 
 }  // namespace tc

@@ -146,7 +146,6 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
     constexpr int HC = DV / 4;
     constexpr int XST = Cfg::kXStages;
     extern __shared__ uint8_t smem_raw[];
-    grid_launch_dependents();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
     uint64_t* x_full = bars;           // [2]
@@ -215,7 +214,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;     // h[b] at columns 128*b, dg at 256, dX at 384
-    grid_dependency_wait();
+    grid_begin(false);
     bool ok = true;
 
     if (warp == 0) {
@@ -452,51 +451,40 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-template <int DV, int F>
-inline hla_status launch_phi_backward(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K, void* dQ,
-                                      void* dK, char* ws, const hla_ws_layout& L, int sm_count, LaunchRec& rec) {
-    constexpr int NM = MT<F>::kMaps, DP = MT<F>::kDphi;
+// One side of the phi backward: dQ from the query features' gradients, or dK from those of the key maps.
+template <int DV, int F, bool KSIDE>
+inline hla_status launch_phi_backward(const Dims& D, int BH, const hla_mlp* phi, const void* X, void* dX, char* ws, const hla_ws_layout& L, int sm_count,
+                                      LaunchRec& rec) {
+    constexpr int NM = KSIDE ? MT<F>::kMaps : 1, DP = MT<F>::kDphi;
     const long long rows = (long long)BH * D.N;
-    CUtensorMap mapQ, mapK, mapdQ, mapdK;
-    PhiMaps mq, mk;
-    PhiBwdPtrs pq{}, pk{};
-    if (!make_map_2d(&mapQ, Q, (size_t)rows, DV, kTileTokens) || !make_map_2d(&mapK, K, (size_t)rows, DV, kTileTokens)) return HLA_ERR_CUDA;
-    if (!make_map_2d(&mapdQ, dQ, (size_t)rows, DV, kTileTokens) || !make_map_2d(&mapdK, dK, (size_t)rows, DV, kTileTokens)) return HLA_ERR_CUDA;
-    if (!make_map_2d(&mq.w1[0], phi_q->W1, DV, DV, DV)) return HLA_ERR_CUDA;
-    mq.w1[1] = mq.w1[0];
-    mq.w1[2] = mq.w1[0];
-    pq.b1[0] = static_cast<const __nv_bfloat16*>(phi_q->b1);
-    pq.W2[0] = static_cast<const __nv_bfloat16*>(phi_q->W2);
+    CUtensorMap mapX, mapdX;
+    PhiMaps maps;
+    PhiBwdPtrs ptrs{};
+    if (!make_map_2d(&mapX, X, (size_t)rows, DV, kTileTokens) || !make_map_2d(&mapdX, dX, (size_t)rows, DV, kTileTokens)) return HLA_ERR_CUDA;
     for (int f = 0; f < NM; ++f) {
-        if (!make_map_2d(&mk.w1[f], phi_k[f].W1, DV, DV, DV)) return HLA_ERR_CUDA;
-        pk.b1[f] = static_cast<const __nv_bfloat16*>(phi_k[f].b1);
-        pk.W2[f] = static_cast<const __nv_bfloat16*>(phi_k[f].W2);
+        if (!make_map_2d(&maps.w1[f], phi[f].W1, DV, DV, DV)) return HLA_ERR_CUDA;
+        ptrs.b1[f] = static_cast<const __nv_bfloat16*>(phi[f].b1);
+        ptrs.W2[f] = static_cast<const __nv_bfloat16*>(phi[f].W2);
     }
-    for (int f = NM; f < 3; ++f) mk.w1[f] = mk.w1[0];
-    int* status = reinterpret_cast<int*>(ws + L.status);
-    if (!set_smem(tc_phi_backward_kernel<DV, 1, false, DP>, PbCfg<DV, 1, DP>::kSmem) || !set_smem(tc_phi_backward_kernel<DV, NM, true, DP>, PbCfg<DV, NM, DP>::kSmem))
-        return HLA_ERR_CUDA;
+    for (int f = NM; f < 3; ++f) maps.w1[f] = maps.w1[0];
+    if (!set_smem(tc_phi_backward_kernel<DV, NM, KSIDE, DP>, PbCfg<DV, NM, DP>::kSmem)) return HLA_ERR_CUDA;
     const long long tiles = (rows + kTileTokens - 1) / kTileTokens;
     const int grid = (int)(tiles < sm_count ? tiles : sm_count);
-    cudaStream_t st = rec.st;
-    rec.begin("tc_phi_backward_q");
-    launch_pdl(tc_phi_backward_kernel<DV, 1, false, DP>, grid, dim3(kPbThreads), PbCfg<DV, 1, DP>::kSmem, st,
-        mapQ, mq, mapdQ, pq, reinterpret_cast<const float*>(ws + L.qf), reinterpret_cast<const float*>(ws + L.dqf), static_cast<__nv_bfloat16*>(dQ), rows, D.N, status);
-    if (!rec.end()) return HLA_ERR_CUDA;
-    rec.begin("tc_phi_backward_k");
-    launch_pdl(tc_phi_backward_kernel<DV, NM, true, DP>, grid, dim3(kPbThreads), PbCfg<DV, NM, DP>::kSmem, st,
-        mapK, mk, mapdK, pk, reinterpret_cast<const float*>(ws + L.kf), reinterpret_cast<const float*>(ws + L.dkf), static_cast<__nv_bfloat16*>(dK), rows, D.N, status);
+    rec.begin(KSIDE ? "tc_phi_backward_k" : "tc_phi_backward_q");
+    launch_pdl(tc_phi_backward_kernel<DV, NM, KSIDE, DP>, grid, dim3(kPbThreads), PbCfg<DV, NM, DP>::kSmem, rec.st, mapX, maps, mapdX, ptrs,
+               reinterpret_cast<const float*>(ws + (KSIDE ? L.kf : L.qf)), reinterpret_cast<const float*>(ws + (KSIDE ? L.dkf : L.dqf)),
+               static_cast<__nv_bfloat16*>(dX), rows, D.N, reinterpret_cast<int*>(ws + L.status));
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
-inline hla_status phi_backward(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K, void* dQ, void* dK,
-                               char* ws, const hla_ws_layout& L, int sm_count, LaunchRec& rec) {
+template <bool KSIDE>
+inline hla_status phi_backward(const Dims& D, int BH, const hla_mlp* phi, const void* X, void* dX, char* ws, const hla_ws_layout& L, int sm_count, LaunchRec& rec) {
     if (D.F == 3) {
-        if (D.d == 128) return launch_phi_backward<128, 3>(D, BH, phi_q, phi_k, Q, K, dQ, dK, ws, L, sm_count, rec);
-        return launch_phi_backward<64, 3>(D, BH, phi_q, phi_k, Q, K, dQ, dK, ws, L, sm_count, rec);
+        if (D.d == 128) return launch_phi_backward<128, 3, KSIDE>(D, BH, phi, X, dX, ws, L, sm_count, rec);
+        return launch_phi_backward<64, 3, KSIDE>(D, BH, phi, X, dX, ws, L, sm_count, rec);
     }
-    if (D.d == 128) return launch_phi_backward<128, 2>(D, BH, phi_q, phi_k, Q, K, dQ, dK, ws, L, sm_count, rec);
-    return launch_phi_backward<64, 2>(D, BH, phi_q, phi_k, Q, K, dQ, dK, ws, L, sm_count, rec);
+    if (D.d == 128) return launch_phi_backward<128, 2, KSIDE>(D, BH, phi, X, dX, ws, L, sm_count, rec);
+    return launch_phi_backward<64, 2, KSIDE>(D, BH, phi, X, dX, ws, L, sm_count, rec);
 }
 
 }  // namespace tc

@@ -42,6 +42,16 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 __device__ __forceinline__ void grid_start_beside() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // Lets the next kernel's blocks be scheduled as soon as every block of this one has started.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The two ends of a kernel that can run either way.  The next kernel is let go only here, after the wait: if it is one that runs beside
+// this one, it relies on everything before this one being complete.
+__device__ __forceinline__ void grid_begin(bool beside) {
+    if (beside) grid_start_beside();
+    else grid_dependency_wait();
+    grid_launch_dependents();
+}
+__device__ __forceinline__ void grid_end(bool beside) {
+    if (beside) grid_dependency_wait();
+}
 
 // ---- mbarrier -------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

@@ -35,8 +35,7 @@ __global__ void __launch_bounds__(32 * kFoldGroups) vmod_fold_kernel(VmlpPtrs a,
                                                                      int* __restrict__ clear) {
     constexpr int d = D;
     __shared__ float sc[kFoldGroups][32], ss[kFoldGroups][32];
-    grid_launch_dependents();
-    grid_dependency_wait();
+    grid_begin(false);
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 16) clear[threadIdx.x] = 0;
     const VmlpPtrs p = blockIdx.x == 0 ? a : b;
     __nv_bfloat16* wf = w1f + (size_t)blockIdx.x * d * d;
@@ -167,12 +166,11 @@ template <int DV, bool COMBINE>
 __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW1,
                                                                         const __grid_constant__ CUtensorMap mapW2, const __grid_constant__ CUtensorMap mapAux,
                                                                         const __grid_constant__ CUtensorMap mapY2, const __grid_constant__ CUtensorMap mapOut,
-                                                                        long long rows, int* status) {
+                                                                        long long rows, int* status, bool beside) {
     using Cfg = VfCfg<DV, COMBINE>;
     constexpr int HC = DV / 4;
     constexpr int XST = Cfg::kXStages;
     extern __shared__ uint8_t smem_raw[];
-    grid_launch_dependents();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float* stat = reinterpret_cast<float*>(smem + Cfg::kOffStat);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
@@ -233,7 +231,7 @@ __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_dependency_wait();
+    grid_begin(beside);
     bool ok = true;
 
     if (warp == 0) {
@@ -413,6 +411,7 @@ __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
+    grid_end(beside);
 }
 
 // ---- backward of one map (input gradient) ---------------------------------------------------------------------------
@@ -457,11 +456,10 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
                                                                          const __grid_constant__ CUtensorMap mapW2, const __grid_constant__ CUtensorMap mapAux,
                                                                          const __grid_constant__ CUtensorMap mapdO, const __grid_constant__ CUtensorMap mapY,
                                                                          const __grid_constant__ CUtensorMap mapdX, const __nv_bfloat16* __restrict__ aux,
-                                                                         int accumulate, long long rows, int* status) {
+                                                                         int accumulate, long long rows, int* status, bool beside) {
     using Cfg = VbCfg<DV>;
     constexpr int HC = DV / 4;
     extern __shared__ uint8_t smem_raw[];
-    grid_launch_dependents();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float2* stat = reinterpret_cast<float2*>(smem + Cfg::kOffStat);
     float2* lnp = reinterpret_cast<float2*>(smem + Cfg::kOffLnp);
@@ -528,7 +526,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    grid_begin(beside);
     // c and b1' (fp32, from the two bf16 halves the folding kernel wrote) for the row means of the LayerNorm backward
     for (int j = tid; j < DV; j += kVbThreads) {
         cb[j] = __bfloat162float(aux[j]) + __bfloat162float(aux[DV + j]);
@@ -795,6 +793,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
+    grid_end(beside);
 }
 
 // ---- host side ---------------------------------------------------------------------------------------------------------
@@ -845,17 +844,17 @@ inline hla_status launch_vmod(const VmodPlan& P, long long rows, const hla_vmlp*
     const int grid = (int)(tiles < sm_count ? tiles : sm_count);
     // Y2 = phi_v2(V)
     rec.begin("tc_vmlp_forward");
-    launch_pdl(tc_vmlp_forward_kernel<DV, false>, grid, dim3(kVfThreads), VfCfg<DV, false>::kSmem, st, mapV, mapW1[1], mapW2[1], mapAux[1], mapY2, mapY2, rows, status);
+    launch_pdl(tc_vmlp_forward_kernel<DV, false>, grid, dim3(kVfThreads), VfCfg<DV, false>::kSmem, st, mapV, mapW1[1], mapW2[1], mapAux[1], mapY2, mapY2, rows, status, false);
     if (!rec.end()) return HLA_ERR_CUDA;
     if (!backward) {      // Out = T + phi_v1(T) (.) Y2
         CUtensorMap mapOut;
         if (!make_map_2d(&mapOut, Out, (size_t)rows, DV, kTileTokens)) return HLA_ERR_CUDA;
         rec.begin("tc_vmlp_forward_combine");
-        launch_pdl(tc_vmlp_forward_kernel<DV, true>, grid, dim3(kVfThreads), VfCfg<DV, true>::kSmem, st, mapT, mapW1[0], mapW2[0], mapAux[0], mapY2, mapOut, rows, status);
+        launch_pdl(tc_vmlp_forward_kernel<DV, true>, grid, dim3(kVfThreads), VfCfg<DV, true>::kSmem, st, mapT, mapW1[0], mapW2[0], mapAux[0], mapY2, mapOut, rows, status, false);
         return rec.end() ? HLA_OK : HLA_ERR_CUDA;
     }
-    rec.begin("tc_vmlp_forward");      // Y1 = phi_v1(T)
-    launch_pdl(tc_vmlp_forward_kernel<DV, false>, grid, dim3(kVfThreads), VfCfg<DV, false>::kSmem, st, mapT, mapW1[0], mapW2[0], mapAux[0], mapY1, mapY1, rows, status);
+    rec.begin("tc_vmlp_forward");      // Y1 = phi_v1(T), beside Y2
+    launch_pdl(tc_vmlp_forward_kernel<DV, false>, grid, dim3(kVfThreads), VfCfg<DV, false>::kSmem, st, mapT, mapW1[0], mapW2[0], mapAux[0], mapY1, mapY1, rows, status, true);
     if (!rec.end()) return HLA_ERR_CUDA;
     CUtensorMap mapdO, mapdT, mapdV;
     if (!make_map_2d(&mapdO, dOut, (size_t)rows, DV, kTileTokens) || !make_map_2d(&mapdT, dT, (size_t)rows, DV, kTileTokens) ||
@@ -863,11 +862,11 @@ inline hla_status launch_vmod(const VmodPlan& P, long long rows, const hla_vmlp*
         return HLA_ERR_CUDA;
     rec.begin("tc_vmlp_backward_t");   // dT = dOut + J1^T (dOut (.) Y2)
     launch_pdl(tc_vmlp_backward_kernel<DV, true>, grid, dim3(kVbThreads), VbCfg<DV>::kSmem, st, mapT, mapW1[0], mapW2[0], mapAux[0], mapdO, mapY2, mapdT,
-               (const bf*)aux, 0, rows, status);
+               (const bf*)aux, 0, rows, status, false);
     if (!rec.end()) return HLA_ERR_CUDA;
-    rec.begin("tc_vmlp_backward_v");   // dV (+)= J2^T (dOut (.) Y1)
+    rec.begin("tc_vmlp_backward_v");   // dV (+)= J2^T (dOut (.) Y1), beside dT
     launch_pdl(tc_vmlp_backward_kernel<DV, false>, grid, dim3(kVbThreads), VbCfg<DV>::kSmem, st, mapV, mapW1[1], mapW2[1], mapAux[1], mapdO, mapY1, mapdV,
-               (const bf*)(aux + (size_t)16 * DV), accumulate_dV, rows, status);
+               (const bf*)(aux + (size_t)16 * DV), accumulate_dV, rows, status, true);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 

@@ -62,11 +62,10 @@ struct WgMaps {
 template <int DV, int DP>
 __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __grid_constant__ WgMaps maps, const float* __restrict__ feat,
                                                                      const float* __restrict__ dfeat, float* __restrict__ wpart, long long rows, int N,
-                                                                     int* status) {
+                                                                     int* status, bool beside) {
     using Cfg = WgCfg<DV, DP>;
     constexpr int HC = DV / 4;
     extern __shared__ uint8_t smem_raw[];
-    grid_launch_dependents();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
     uint64_t* x_full = bars;           // [2] TMA
@@ -136,7 +135,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    grid_begin(beside);
     bool ok = true;
 
     if (warp == 0) {
@@ -390,6 +389,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
+    grid_end(beside);
 }
 
 struct WgradOut {
@@ -403,12 +403,11 @@ struct WgradOut {
 // maps).  A block owns 32 consecutive outputs, warp w adds the partials w, w + 8, ... of the map (coalesced 128-byte reads, independent
 // loads), and the eight warp sums are added in warp order.
 template <int DV, int DP>
-__global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __restrict__ wpart, WgradOut out) {
+__global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __restrict__ wpart, WgradOut out, bool beside) {
     using C1 = WgCfg<DV, DP>;
     constexpr int PF = C1::kPartFloats, oW2 = C1::kPartW2, oB1 = C1::kPartB1, oB2 = C1::kPartB2, W2C = C1::kW2Cols;
     __shared__ float red[8][32];
-    grid_launch_dependents();
-    grid_dependency_wait();
+    grid_begin(beside);
     const int m = blockIdx.y;
     const int nctas = out.first[m + 1] - out.first[m];
     const int total = DV * DV + DV * DP + DV + DP;   // outputs of one map
@@ -452,6 +451,7 @@ __global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __res
         }
         __syncthreads();
     }
+    grid_end(beside);
 }
 
 // CTAs of the query map, and of each of n key maps: an even share of the SMs, and no more partials in all than three per tile (or four
@@ -468,8 +468,8 @@ inline size_t wgrad_part_bytes(int d, int n, long long rows, int sm_count) {
 }
 
 // dphi_q / dphi_k: fp32 device outputs with the shapes of the weights (dphi_k points to one entry per key map); either may be null.
-// Both passes come first, then both reductions: the partials of the sides have regions of their own, so the key pass is set up while the
-// query pass drains.
+// Both passes come first, the second beside the first (the partials of the sides have regions of their own), then both reductions, the
+// second beside the first.
 template <int DV, int F>
 inline hla_status launch_phi_wgrad(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K,
                                    const hla_mlp_grad* dphi_q, const hla_mlp_grad* dphi_k, char* ws, const hla_ws_layout& L, size_t off_wpart,
@@ -506,15 +506,17 @@ inline hla_status launch_phi_wgrad(const Dims& D, int BH, const hla_mlp* phi_q, 
         const int per_head = key ? D.N : 0;
         rec.begin(key ? "tc_phi_wgrad_k" : "tc_phi_wgrad_q");
         // the first pass stages caller-provided weights before its dependency wait: no overlap with what precedes it
-        if (first) launch_serial(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status);
-        else launch_pdl(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status);
+        if (first) launch_serial(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status, false);
+        else launch_pdl(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status, true);
         first = false;
         if (!rec.end()) return HLA_ERR_CUDA;
     }
+    bool second = false;
     for (int key = 0; key < 2; ++key) {
         if (nmaps[key] == 0) continue;
         rec.begin("tc_wgrad_reduce");
-        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((DV * DV + DV * DP + DV + DP + 31) / 32, nmaps[key]), dim3(256), 0, rec.st, (const float*)wpart[key], out[key]);
+        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((DV * DV + DV * DP + DV + DP + 31) / 32, nmaps[key]), dim3(256), 0, rec.st, (const float*)wpart[key], out[key], second);
+        second = true;
         if (!rec.end()) return HLA_ERR_CUDA;
     }
     return HLA_OK;
