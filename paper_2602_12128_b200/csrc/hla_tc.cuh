@@ -593,7 +593,7 @@ template <int DV, int F>
 __global__ void __launch_bounds__(256) tc_reduce_emit_kernel(const float* __restrict__ part, float* __restrict__ state,
                                                              __nv_bfloat16* __restrict__ b3, __nv_bfloat16* __restrict__ bq, int S, int ld, int G, int T, bool beside) {
     constexpr int kN = MT<F>::kN, kPad = MT<F>::kPad;
-    __shared__ float sm[8][kMaxD + 8];
+    __shared__ __align__(16) float sm[8][kMaxD + 8];
     const int m0 = 8 * blockIdx.x, bh = blockIdx.y, tid = threadIdx.x;      // gridDim.x = kPad / 8
     grid_begin(beside);
     const size_t n_per = (size_t)kN * ld;
@@ -602,15 +602,26 @@ __global__ void __launch_bounds__(256) tc_reduce_emit_kernel(const float* __rest
         const long long total = (long long)gridDim.y * T;
         count = owner_of_work((long long)bh * T + T - 1, total, G) - owner_of_work((long long)bh * T, total, G) + 1;
     }
-    for (int i = tid; i < 8 * ld; i += 256) {
-        const int mm = i / ld, col = i - mm * ld, m = m0 + mm;
-        float a = 0.f;
+    // Four columns per thread, eight partials in flight, added in their order (bit-reproducible).  (One column at a time and one partial
+    // after the other, a block walked 2 to 3 x S dependent round trips to L2.)
+    for (int i = tid; i < 2 * ld; i += 256) {
+        const int mm = i / (ld / 4), col = 4 * (i - mm * (ld / 4)), m = m0 + mm;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         if (m < kN) {
             const float* src = part + (size_t)bh * S * n_per + (size_t)m * ld + col;
-            for (int s = 0; s < count; ++s) a += src[(size_t)s * n_per];      // fixed order: bit-reproducible
-            state[(size_t)bh * n_per + (size_t)m * ld + col] = a;
+            for (int s0 = 0; s0 < count; s0 += 8) {
+                float4 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    v[k] = s0 + k < count ? *reinterpret_cast<const float4*>(src + (size_t)(s0 + k) * n_per) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+                }
+            }
+            *reinterpret_cast<float4*>(state + (size_t)bh * n_per + (size_t)m * ld + col) = a;
         }
-        sm[mm][col] = a;
+        *reinterpret_cast<float4*>(&sm[mm][col]) = a;
     }
     __syncthreads();
     __nv_bfloat16* o3 = b3 + (size_t)bh * (DV + 16) * kPad;
