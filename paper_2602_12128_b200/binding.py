@@ -133,8 +133,15 @@ def _ptr(t) -> int:
     return t.data_ptr()
 
 
+# The handle of PyTorch's current stream without building a Stream object for it (3 of the 4 us that this took of every call; a
+# feature-level step of 12 heads x 4999 tokens, 38 us of device time, was bound by the host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else 0
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
