@@ -311,8 +311,9 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
     if (S == 0) {
         if (x->tc) {
             // One CTA per SM: S * heads CTAs run in ceil(S * heads / SMs) waves.  Take the split count that fills its
-            // waves best (each extra wave is charged 2 % for its start-up and drain), with at least 8 tiles per CTA.
-            const int smax = tiles / 8 > 1 ? (tiles / 8 < 64 ? tiles / 8 : 64) : 1;
+            // waves best (each extra wave is charged 2 % for its start-up and drain), with at least 4 tiles per CTA (8 left 60 CTAs of
+            // a step of 12 heads x 4999 tokens: 36.2 us against 34.7).
+            const int smax = tiles / 4 > 1 ? (tiles / 4 < 64 ? tiles / 4 : 64) : 1;
             double best = -1.0;
             for (int cand = 1; cand <= smax; ++cand) {
                 const long long ctas = (long long)cand * x->BH;
