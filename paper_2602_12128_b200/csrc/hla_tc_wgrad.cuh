@@ -400,56 +400,55 @@ struct WgradOut {
     int first[4];      // map i: the partials first[i] .. first[i + 1] - 1
 };
 // Adds a map's partials in a fixed order (bit-reproducible) and writes its gradients (fp32, the shapes of the weights); grid = (blocks,
-// maps).  A block owns 32 consecutive outputs, warp w adds the partials w, w + 8, ... of the map (coalesced 128-byte reads, independent
-// loads), and the eight warp sums are added in warp order.
+// maps).  A block owns 128 consecutive partial entries, a thread four of them: warp w adds the partials w, w + 8, ... of the map (512-byte
+// reads, eight in flight), and the eight warp sums are added in warp order.  The entries of dW2 (its two halves) and db2 (its four token
+// quarters) that make up one output lie in one block.  (With one entry per thread the two launches of a call took 16 us each for 11 MB.)
 template <int DV, int DP>
 __global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __restrict__ wpart, WgradOut out, bool beside) {
     using C1 = WgCfg<DV, DP>;
     constexpr int PF = C1::kPartFloats, oW2 = C1::kPartW2, oB1 = C1::kPartB1, oB2 = C1::kPartB2, W2C = C1::kW2Cols;
-    __shared__ float red[8][32];
+    static_assert(oW2 % 128 == 0 && 128 % W2C == 0 && PF % 4 == 0 && (oB2 % 128) + 64 <= 128, "entries of one output in one block");
+    __shared__ __align__(16) float red[8][128];
     grid_begin(beside);
-    const int m = blockIdx.y;
+    const int m = blockIdx.y, base = blockIdx.x * 128;
     const int nctas = out.first[m + 1] - out.first[m];
-    const int total = DV * DV + DV * DP + DV + DP;   // outputs of one map
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float* src = wpart + (size_t)out.first[m] * PF;
-    constexpr size_t stride = PF;
-    for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
-        const int i = base + lane;
-        // an output is the sum over the CTAs of `nterm` partial entries `step` floats apart, starting at `off`
-        int off = 0, nterm = 0, step = 0;
-        float scale = 1.f;
-        if (i < DV * DV) {
-            off = i; nterm = 1;
-        } else if (i < DV * DV + DV * DP) {
-            const int j = (i - DV * DV) / DP, o = (i - DV * DV) % DP;
-            off = oW2 + j * W2C + o; nterm = 2; step = DP; scale = 0.5f;      // the G tile held 2 GELU(h)
-        } else if (i < DV * DV + DV * DP + DV) {
-            off = oB1 + (i - DV * DV - DV * DP); nterm = 1;
-        } else if (i < total) {
-            off = oB2 + (i - DV * DV - DV * DP - DV); nterm = 4; step = 16;
-        }
-        float a = 0.f;
-        if (nterm == 1) {
-#pragma unroll 8
-            for (int c = warp; c < nctas; c += 8) a += src[c * stride + off];
-        } else {
-            for (int c = warp; c < nctas; c += 8)
-                for (int q = 0; q < nterm; ++q) a += src[c * stride + off + q * step];
-        }
-        red[warp][lane] = a;
-        __syncthreads();
-        if (warp == 0 && i < total) {
-            float t = red[0][lane];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, at = base + 4 * lane;
+    const float* src = wpart + (size_t)out.first[m] * PF + at;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (at < PF) {
+        for (int c0 = warp; c0 < nctas; c0 += 64) {
+            float4 v[8];
 #pragma unroll
-            for (int w = 1; w < 8; ++w) t += red[w][lane];
-            t *= scale;
-            if (i < DV * DV) out.dW1[m][i] = t;
-            else if (i < DV * DV + DV * DP) out.dW2[m][i - DV * DV] = t;
-            else if (i < DV * DV + DV * DP + DV) out.db1[m][i - DV * DV - DV * DP] = t;
-            else out.db2[m][i - DV * DV - DV * DP - DV] = t;
+            for (int k = 0; k < 8; ++k)
+                v[k] = c0 + 8 * k < nctas ? *reinterpret_cast<const float4*>(src + (size_t)(c0 + 8 * k) * PF) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
+            }
         }
-        __syncthreads();
+    }
+    *reinterpret_cast<float4*>(&red[warp][4 * lane]) = a;
+    __syncthreads();
+    const int i = threadIdx.x;
+    if (i < 128) {
+        float t = red[0][i];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) t += red[w][i];
+        red[0][i] = t;
+    }
+    __syncthreads();
+    const int e = base + i;
+    if (i < 128 && e < PF) {
+        if (e < oW2) {
+            out.dW1[m][e] = red[0][i];
+        } else if (e < oB1) {
+            const int j = (e - oW2) / W2C, o = (e - oW2) % W2C;
+            if (o < DP) out.dW2[m][j * DP + o] = 0.5f * (red[0][i] + red[0][i + DP]);      // the G tile held 2 GELU(h); dp in two halves
+        } else if (e < oB2) {
+            out.db1[m][e - oB1] = red[0][i];
+        } else if (e - oB2 < DP) {
+            out.db2[m][e - oB2] = ((red[0][i] + red[0][i + 16]) + red[0][i + 32]) + red[0][i + 48];
+        }
     }
     grid_end(beside);
 }
@@ -515,7 +514,7 @@ inline hla_status launch_phi_wgrad(const Dims& D, int BH, const hla_mlp* phi_q, 
     for (int key = 0; key < 2; ++key) {
         if (nmaps[key] == 0) continue;
         rec.begin("tc_wgrad_reduce");
-        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((DV * DV + DV * DP + DV + DP + 31) / 32, nmaps[key]), dim3(256), 0, rec.st, (const float*)wpart[key], out[key], second);
+        launch_pdl(tc_wgrad_reduce_kernel<DV, DP>, dim3((WgCfg<DV, DP>::kPartFloats + 127) / 128, nmaps[key]), dim3(256), 0, rec.st, (const float*)wpart[key], out[key], second);
         second = true;
         if (!rec.end()) return HLA_ERR_CUDA;
     }
