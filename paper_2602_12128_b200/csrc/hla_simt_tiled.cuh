@@ -11,10 +11,10 @@
 // permutations of an index, and so is G = X S^T of the key side.  Only the state itself is formed in full, because it is the layout
 // the workspace promises (P rows); the folded rows are summed when a block stages the state.
 //
-// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2547 -> 332 us (two
-// state builds 1236 -> 98, two feature gradients 557 -> 56, two readouts 277 -> 37, feature networks backward 387 -> 105, forward 104 ->
-// 72); forward with B*H = 2, N = 256, d = 16: 95 -> 25 us.  Of these, independent neighbours side by side, more splits of the gradient
-// state and the small tiles: 431 -> 332 and 37 -> 25 us.
+// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2547 -> 296 us (two
+// state builds 1236 -> 95, two feature gradients 557 -> 46, two readouts 277 -> 35, feature networks backward 387 -> 95, forward 104 ->
+// 64); forward with B*H = 2, N = 256, d = 16: 95 -> 22.6 us.  Of these, independent neighbours side by side, more splits of the gradient
+// state and the small tiles: 431 -> 332 and 37 -> 25 us; loads without index divisions and without branches between them: the rest.
 #pragma once
 #include "hla_simt.cuh"
 #include "hla_tc.cuh"
@@ -68,11 +68,14 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
     *reinterpret_cast<uint2*>(p) = make_uint2(tc::pack_bf16(v.x, v.y), tc::pack_bf16(v.z, v.w));
 }
 
-// rows [row0, row0 + n) of a matrix [.][d] into a tile with row stride ld; rows from `limit` on are zero.  All threads.
-template <typename T> __device__ __forceinline__ void stage_rows(float* tile, int ld, const T* __restrict__ src, size_t row0, int n, size_t limit, int d) {
-    const int q = d >> 2;
-    for (int i = threadIdx.x; i < n * q; i += blockDim.x) {
-        const int r = i / q, c = 4 * (i - r * q);
+// rows [row0, row0 + n) of a matrix [.][d] into a tile with row stride ld; rows from `limit` on are zero.  All threads of the block; a
+// thread takes the columns 4 cg .. 4 cg + 3 of the rows tg, tg + 8, ...
+template <int CG, typename T>
+__device__ __forceinline__ void stage_rows(float* tile, int ld, const T* __restrict__ src, size_t row0, int n, size_t limit, int d) {
+    const int c = 4 * (threadIdx.x % CG);
+    if (c >= d) return;
+#pragma unroll 8
+    for (int r = threadIdx.x / CG; r < n; r += 8) {
         const float4 v = row0 + r < limit ? load4(src + (row0 + r) * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         *reinterpret_cast<float4*>(tile + r * ld + c) = v;
     }
@@ -115,18 +118,18 @@ template <int CG, int JN, int R> __device__ __forceinline__ void tile_nt(float (
     }
 }
 
-// The value-side tile: X = V, xz = 1 (forward), or X = r dO, xz = -r (dO . O), r = 1 / (eta + eps) (backward; a warp per row).
-template <typename T, bool BWD>
+// The value-side tile: X = V, xz = 1 (forward), or X = r dO, xz = -r (dO . O), r = 1 / (eta + eps) (backward; CG lanes per row).
+template <int CG, typename T, bool BWD>
 __device__ __forceinline__ void stage_values(float* Xs, int ld, float* xz, const T* __restrict__ X, const T* __restrict__ O, const float* __restrict__ eta,
                                              const Dims& D, int bh, int tok0, int n, int limit) {
     if (!BWD) {
-        stage_rows(Xs, ld, X + (size_t)bh * D.N * D.d, (size_t)tok0, n, (size_t)limit, D.d);
+        stage_rows<CG>(Xs, ld, X + (size_t)bh * D.N * D.d, (size_t)tok0, n, (size_t)limit, D.d);
         for (int t = threadIdx.x; t < n; t += blockDim.x) xz[t] = tok0 + t < limit ? 1.f : 0.f;
         return;
     }
-    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5, c = 4 * lane;
+    const int cg = threadIdx.x % CG, c = 4 * cg;
 #pragma unroll 4
-    for (int t = threadIdx.x >> 5; t < n; t += nwarp) {
+    for (int t = threadIdx.x / CG; t < n; t += 8) {      // (n is a multiple of 8: all lanes of a warp take part in the sums)
         const int tok = tok0 + t;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         float s = 0.f, r = 0.f;
@@ -139,9 +142,10 @@ __device__ __forceinline__ void stage_values(float* Xs, int ld, float* xz, const
                 s = fmaf(x.x, o.x, fmaf(x.y, o.y, fmaf(x.z, o.z, x.w * o.w)));
             }
         }
-        s = warp_sum(s);
+#pragma unroll
+        for (int o = CG / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (c < D.d) *reinterpret_cast<float4*>(Xs + t * ld + c) = make_float4(r * x.x, r * x.y, r * x.z, r * x.w);
-        if (lane == 0) xz[t] = -r * s;
+        if (cg == 0) xz[t] = -r * s;
     }
 }
 
@@ -193,7 +197,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const
             const size_t at = BWD ? ((size_t)bh * D.N + tok0 + t) * DP + k : (((size_t)bh * F + f) * D.N + tok0 + t) * DP + k;
             fs[t * KF + f * DP + k] = tok0 + t < t1 ? __ldg(feat + at) : 0.f;
         }
-        stage_values<T, BWD>(Xs, LD, xz, X, O, eta, D, bh, tok0, kSbTok, t1);
+        stage_values<CG, T, BWD>(Xs, LD, xz, X, O, eta, D, bh, tok0, kSbTok, t1);
         __syncthreads();
         for (int t = threadIdx.x >> 6; t < kSbTok; t += NT / 64) {
             const float* f = fs + t * KF;
@@ -274,23 +278,31 @@ template <int F, bool SUM> __device__ __forceinline__ void stage_state(float* ti
         const int m = i / q, c = 4 * (i - m * q);
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         if (m < G::kN) {
+            // (all rows are loaded, those that repeat an index tuple with a zero factor: independent loads instead of a chain of branches)
             const int p = kRowTable<F>.v[m];
-            auto add = [&](int r, bool on) {
-                if (on) {
-                    const float4 v = __ldg(reinterpret_cast<const float4*>(st + (size_t)r * ld + c));
-                    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
-                }
+            auto row = [&](int r) { return __ldg(reinterpret_cast<const float4*>(st + (size_t)r * ld + c)); };
+            auto add = [&](float4 v, bool on) {
+                const float f = on ? 1.f : 0.f;
+                a.x = fmaf(f, v.x, a.x); a.y = fmaf(f, v.y, a.y); a.z = fmaf(f, v.z, a.z); a.w = fmaf(f, v.w, a.w);
             };
-            add(p, true);
-            if (SUM && F == 2) add((p % 12) * 12 + p / 12, p / 12 != p % 12);
-            if (SUM && F == 3) {
+            if (!SUM) {
+                a = row(p);
+            } else if (F == 2) {
+                const int d0 = p / 12, d1 = p % 12;
+                const float4 v0 = row(p), v1 = row(d1 * 12 + d0);
+                a = v0;
+                add(v1, d0 != d1);
+            } else {
                 const int d0 = p / 36, d1 = (p / 6) % 6, d2 = p % 6;      // d0 <= d1 <= d2
                 const bool n01 = d0 != d1, n12 = d1 != d2;
-                add(36 * d0 + 6 * d2 + d1, n12);
-                add(36 * d1 + 6 * d0 + d2, n01);
-                add(36 * d1 + 6 * d2 + d0, n01 && n12);
-                add(36 * d2 + 6 * d0 + d1, n01 && n12);
-                add(36 * d2 + 6 * d1 + d0, n01 || n12);
+                const float4 v0 = row(p), v1 = row(36 * d0 + 6 * d2 + d1), v2 = row(36 * d1 + 6 * d0 + d2), v3 = row(36 * d1 + 6 * d2 + d0),
+                             v4 = row(36 * d2 + 6 * d0 + d1), v5 = row(36 * d2 + 6 * d1 + d0);
+                a = v0;
+                add(v1, n12);
+                add(v2, n01);
+                add(v3, n01 && n12);
+                add(v4, n01 && n12);
+                add(v5, n01 || n12);
             }
         }
         *reinterpret_cast<float4*>(tile + m * ldt + c) = a;
@@ -381,7 +393,7 @@ __global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, cons
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
     tc::grid_begin(beside);
     stage_state<F, QSIDE>(Ss, LD, state + (size_t)bh * G::kP * D.ld, D.ld);
-    stage_values<T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, TM, D.N);
+    stage_values<CG, T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, TM, D.N);
     __syncthreads();
     float acc[R][JN];
 #pragma unroll
@@ -432,8 +444,8 @@ __global__ void __launch_bounds__(CG * 8) tiled_phi_forward_kernel(const T* __re
     const size_t row0 = (size_t)blockIdx.x * TM;
     const int m = blockIdx.y, cg = threadIdx.x % CG, tg = threadIdx.x / CG;
     tc::grid_begin(beside);
-    stage_rows(Xs, LD, X, row0, TM, rows, d);
-    stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
+    stage_rows<CG>(Xs, LD, X, row0, TM, rows, d);
+    stage_rows<CG>(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
     for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
     __syncthreads();
     float acc[R][4];
@@ -495,7 +507,7 @@ __global__ void __launch_bounds__(CG * 8, CG == 32 ? 1 : 64 / CG) tiled_phi_back
     const int cg = threadIdx.x % CG, tg = threadIdx.x / CG;
     const bool live = 4 * cg < d;
     tc::grid_begin(beside);
-    stage_rows(Xs, LD, X, row0, TM, rows, d);
+    stage_rows<CG>(Xs, LD, X, row0, TM, rows, d);
     for (int i = threadIdx.x; i < (4 * CG - d) * (d >> 2); i += NT)      // rows of W1 past the head width: read by tile_nt, kept finite
         *reinterpret_cast<float4*>(Ws + (d + i / (d >> 2)) * LD + 4 * (i % (d >> 2))) = make_float4(0.f, 0.f, 0.f, 0.f);
     float dx[R][4];
@@ -505,7 +517,7 @@ __global__ void __launch_bounds__(CG * 8, CG == 32 ? 1 : 64 / CG) tiled_phi_back
         for (int j = 0; j < 4; ++j) dx[i][j] = 0.f;
     for (int m = 0; m < W.nmaps; ++m) {
         if (m > 0) __syncthreads();      // the previous map's tiles have been read
-        stage_rows(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
+        stage_rows<CG>(Ws, LD, W.W1[m], 0, d, (size_t)d, d);
         for (int i = threadIdx.x; i < d * DP; i += NT) W2s[(i % DP) * LD + i / DP] = ldf(W.W2[m] + i);
         for (int i = threadIdx.x; i < TM * DP; i += NT) {
             const int t = i / DP, o = i - t * DP;
