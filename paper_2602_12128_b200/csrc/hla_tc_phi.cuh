@@ -58,15 +58,15 @@ __device__ __forceinline__ float2 times_gelu_grad2(float2 dg, float2 x) {
 // (fit_gelu_tanh.py: |GELU' error| < 5.2e-4 instead of 1.5e-4 - still an order below the bf16 rounding of dh).  V grows to
 // 27 at |x| = 6 with these constants, so the form relies on tanh.approx being accurate near saturation: measured on B200 its
 // absolute error stays below 8e-6 on [-6, 6] (its documented bound, 2^-11 relative, would allow 1.4e-2 in GELU' there).
-__device__ __forceinline__ void gelu_both2_twice(float2 x, float2& g2, float2& grad2) {
+// dh = dg GELU'(x) with dg halved, as above, and 2 GELU(x): nine packed instructions per pair.
+__device__ __forceinline__ void gelu_both2(float2 dg, float2 x, float2& g2, float2& dh) {
     const float2 t = __fmul2_rn(x, x);
     const float2 u = __fmul2_rn(x, __ffma2_rn(t, splat2(0.0352821f), splat2(0.79880136f)));
+    const float2 vn = __fmul2_rn(x, __ffma2_rn(t, splat2(-0.104597145f), splat2(-0.800572795f)));   // -V, V = x (C0 + C1 x^2) / 2
     const float2 th = make_float2(tanh_approx(u.x), tanh_approx(u.y));
     g2 = __ffma2_rn(x, th, x);
-    const float2 vn = __fmul2_rn(x, __ffma2_rn(t, splat2(-0.104597145f), splat2(-0.800572795f)));   // -V, V = x (C0 + C1 x^2) / 2
-    const float2 a1 = __ffma2_rn(vn, th, splat2(1.f));          // 1 - V th
-    const float2 b1 = __ffma2_rn(th, a1, splat2(1.f));          // 1 + th (1 - V th)
-    grad2 = __ffma2_rn(vn, splat2(-1.f), b1);                   // + V
+    const float2 q = __ffma2_rn(vn, __ffma2_rn(th, th, splat2(-1.f)), th);      // th + V (1 - th^2) = 2 GELU' - 1
+    dh = __ffma2_rn(dg, q, dg);
 }
 
 struct PhiPtrs {
