@@ -583,32 +583,36 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
 // Reduce the split partials [BH][S][56][ld] in a fixed order -> fp32 folded state [BH][56][ld]
 // (column d = folded z) and the two bf16 MMA operands of that state.
 // =======================================================================================
-// grid = (8, heads): block c of a head owns the monomials 8c .. 8c+7 (block 7 owns only the zero padding 56..63).
+// grid = (kPad / 4, heads): block c of a head owns the monomials 4c .. 4c+3 (the last ones only zero padding).
 // The partials of head bh are the slots [bh * S, bh * S + count).  With G == 0 every head has count = S slots (kernels
 // whose grid is splits x heads); with G > 0 the producer was a persistent kernel of G CTAs over heads x T work items and
 // the head's slots are its pieces, one per CTA that touched it (see owner_of_work).
-__host__ __device__ inline int owner_of_work(long long w, long long total, int G) { return (int)(((w + 1) * G - 1) / total); }
+__host__ __device__ inline int owner_of_work(long long w, long long total, int G) {
+    if (total * G < (1ll << 32)) return (int)((unsigned)((w + 1) * G - 1) / (unsigned)total);      // (a 64-bit division takes a hundred instructions)
+    return (int)(((w + 1) * G - 1) / total);
+}
 
+constexpr int kReRows = 4;
+template <int DV> constexpr int kReThreads = (kReRows * (DV + 4) / 4 + 31) / 32 * 32;      // one float4 of the state per thread: a single round of loads
 template <int DV, int F>
-__global__ void __launch_bounds__(256) tc_reduce_emit_kernel(const float* __restrict__ part, float* __restrict__ state,
-                                                             __nv_bfloat16* __restrict__ b3, __nv_bfloat16* __restrict__ bq, int S, int ld, int G, int T, bool beside) {
-    constexpr int kN = MT<F>::kN, kPad = MT<F>::kPad;
-    __shared__ __align__(16) float sm[8][kMaxD + 8];
-    const int m0 = 8 * blockIdx.x, bh = blockIdx.y, tid = threadIdx.x;      // gridDim.x = kPad / 8
-    grid_begin(beside);
-    const size_t n_per = (size_t)kN * ld;
+__global__ void __launch_bounds__(kReThreads<DV>) tc_reduce_emit_kernel(const float* __restrict__ part, float* __restrict__ state, __nv_bfloat16* __restrict__ b3,
+                                                                        __nv_bfloat16* __restrict__ bq, int S, int G, int T, bool beside) {
+    constexpr int kN = MT<F>::kN, kPad = MT<F>::kPad, LD = DV + 4, Q = LD / 4, n_per = kN * LD;
+    __shared__ __align__(16) float sm[kReRows][LD];
+    const int m0 = kReRows * blockIdx.x, bh = blockIdx.y, tid = threadIdx.x;      // gridDim.x = kPad / kReRows
     int count = S;
     if (G > 0) {
         const long long total = (long long)gridDim.y * T;
         count = owner_of_work((long long)bh * T + T - 1, total, G) - owner_of_work((long long)bh * T, total, G) + 1;
     }
+    grid_begin(beside);
     // Four columns per thread, eight partials in flight, added in their order (bit-reproducible).  (One column at a time and one partial
     // after the other, a block walked 2 to 3 x S dependent round trips to L2.)
-    for (int i = tid; i < 2 * ld; i += 256) {
-        const int mm = i / (ld / 4), col = 4 * (i - mm * (ld / 4)), m = m0 + mm;
+    if (tid < kReRows * Q) {
+        const int mm = tid / Q, col = 4 * (tid - mm * Q), m = m0 + mm;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         if (m < kN) {
-            const float* src = part + (size_t)bh * S * n_per + (size_t)m * ld + col;
+            const float* src = part + (size_t)bh * S * n_per + (size_t)m * LD + col;
             for (int s0 = 0; s0 < count; s0 += 8) {
                 float4 v[8];
 #pragma unroll
@@ -619,23 +623,16 @@ __global__ void __launch_bounds__(256) tc_reduce_emit_kernel(const float* __rest
                     a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
                 }
             }
-            *reinterpret_cast<float4*>(state + (size_t)bh * n_per + (size_t)m * ld + col) = a;
+            *reinterpret_cast<float4*>(state + (size_t)bh * n_per + (size_t)m * LD + col) = a;
         }
         *reinterpret_cast<float4*>(&sm[mm][col]) = a;
+        if (col < DV) *reinterpret_cast<uint2*>(bq + (size_t)bh * kPad * DV + (size_t)m * DV + col) = make_uint2(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w));
     }
     __syncthreads();
     __nv_bfloat16* o3 = b3 + (size_t)bh * (DV + 16) * kPad;
-    for (int row = tid; row < DV + 16; row += 256) {       // row <= DV: column `row` of the state (row == DV is z); rest zero
-        uint32_t w[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) w[e] = row <= DV ? pack_bf16(sm[2 * e][row], sm[2 * e + 1][row]) : 0u;
-        *reinterpret_cast<uint4*>(o3 + (size_t)row * kPad + m0) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-    __nv_bfloat16* oq = bq + (size_t)bh * kPad * DV;
-    for (int i = tid; i < 8 * DV; i += 256) {
-        const int mm = i / DV, g = i - mm * DV;
-        oq[(size_t)(m0 + mm) * DV + g] = __float2bfloat16_rn(sm[mm][g]);
-    }
+    for (int row = tid; row < DV + 16; row += kReThreads<DV>)       // row <= DV: column `row` of the state (row == DV is z); rest zero
+        *reinterpret_cast<uint2*>(o3 + (size_t)row * kPad + m0) =
+            row <= DV ? make_uint2(pack_bf16(sm[0][row], sm[1][row]), pack_bf16(sm[2][row], sm[3][row])) : make_uint2(0u, 0u);
     grid_end(beside);
 }
 
@@ -707,7 +704,9 @@ __global__ void __launch_bounds__(kRoThreads, 1) tc_readout_kernel(const __grid_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    // Only the state operand is the work of the kernel before this one (the reduction, which lets this kernel start once everything
+    // before itself is complete): the thread that loads it waits, the generators and the rest start at once.
+    grid_start_beside();
     bool ok = true;
 
     if (warp == kRoMmaWarp) {
@@ -715,6 +714,7 @@ __global__ void __launch_bounds__(kRoThreads, 1) tc_readout_kernel(const __grid_
             const uint32_t idesc = idesc_bf16(128, Cfg::kNmma, false, false);
             const uint32_t b3a = smem_u32(smem + Cfg::kOffB3);
             int cur_bh = -1, nload = 0;
+            grid_dependency_wait();
             for (int it = 0; it < nwork; ++it) {
                 const int work = w0 + it, bh = work / tiles_per_head;
                 const int ab = it & 1, u = it >> 1;
@@ -1222,7 +1222,9 @@ __global__ void __launch_bounds__(kBkThreads, 1) tc_bwd_key_kernel(const __grid_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;     // D3[grp] at columns 128*grp, D4[grp] at columns 256 + kD4Stride*grp
-    grid_dependency_wait();
+    // Only the gradient state is the work of the kernel before this one (the reduction): the thread that loads its operand images and the
+    // threads that read dzsym wait for it, the V tiles and the folded key tiles are on their way meanwhile.
+    grid_start_beside();
     bool ok = true;
 
     if (warp == 0) {
@@ -1242,6 +1244,7 @@ __global__ void __launch_bounds__(kBkThreads, 1) tc_bwd_key_kernel(const __grid_
             const uint32_t idesc3 = idesc_bf16(128, DV, false, false);         // dV = Tsym_k (K-major over m) * dCsym^T (K-major over m)
             const uint32_t b3a = smem_u32(smem + Cfg::kOffB3), bqa = smem_u32(smem + Cfg::kOffBq);
             int cur_bh = -1, nload = 0;
+            grid_dependency_wait();
             for (int it = 0; it < nwork; ++it) {
                 const int work = w0 + it, bh = work / tiles_per_head;
                 const int st = it & 1, u = it >> 1, grp = it & 1;
@@ -1293,12 +1296,6 @@ __global__ void __launch_bounds__(kBkThreads, 1) tc_bwd_key_kernel(const __grid_
             const int work = w0 + it, bh = work / tiles_per_head, tile = work % tiles_per_head;
             const int u = it >> 1;
             const int tok = tile * kTileTokens + row;
-            if (bh != cur_bh) {      // dzsym of the head, once per head and group instead of 56 global loads per thread and tile
-                named_barrier(1 + grp, 128);
-                if (row < M::kN) dzs[row] = __ldg(dstate + (size_t)bh * M::kN * ld + DV + (size_t)row * ld);
-                named_barrier(1 + grp, 128);
-                cur_bh = bh;
-            }
             float k[M::kKf];
 #pragma unroll
             for (int i = 0; i < M::kKf; ++i) k[i] = tok < N ? kn[i] : 0.f;
@@ -1310,6 +1307,13 @@ __global__ void __launch_bounds__(kBkThreads, 1) tc_bwd_key_kernel(const __grid_
                 store_mono_row_t<F>(smem_u32(smem + Cfg::kOffA + grp * Cfg::kABytes), row, ts, 1.f);
                 fence_proxy_async();
                 mbar_arrive(&a_full[grp]);
+            }
+            if (bh != cur_bh) {      // dzsym of the head, once per head and group instead of 56 global loads per thread and tile
+                if (cur_bh < 0) grid_dependency_wait();
+                named_barrier(1 + grp, 128);
+                if (row < M::kN) dzs[row] = *(dstate + (size_t)bh * M::kN * ld + DV + (size_t)row * ld);
+                named_barrier(1 + grp, 128);
+                cur_bh = bh;
             }
             // ---- G -> dk
             if (ok && !mbar_wait(&d4_full[grp], u & 1)) { ok = false; report_timeout(status, 406); }
@@ -1440,7 +1444,7 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
     launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (const float*)nullptr, 0.f, 1, false);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_reduce_emit");
-    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, state, b3, bq, D.S, D.ld, 0, 0, false);
+    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, state, b3, bq, D.S, 0, 0, false);
     if (!rec.end()) return HLA_ERR_CUDA;
     if (!readout) return HLA_OK;
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
@@ -1460,8 +1464,8 @@ inline hla_status reduce_pieces_f(const Plan& P, const Dims& D, int BH, char* ws
     float* state = reinterpret_cast<float*>(ws + L.state);
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_reduce_emit");
-    if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T, false);
-    else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, part, state, b3, bq, smax, D.ld, G, T, false);
+    if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<128>), 0, rec.st, part, state, b3, bq, smax, G, T, false);
+    else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<64>), 0, rec.st, part, state, b3, bq, smax, G, T, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 inline hla_status reduce_pieces(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec) {
@@ -1477,7 +1481,7 @@ inline hla_status launch_emit_from_state(const Plan& P, const Dims& D, int BH, c
     __nv_bfloat16* b3 = reinterpret_cast<__nv_bfloat16*>(ws + (gradient ? P.bd3 : P.b3));
     __nv_bfloat16* bq = reinterpret_cast<__nv_bfloat16*>(ws + (gradient ? P.bdq : P.bq));
     rec.begin("tc_reduce_emit");
-    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(MT<F>::kPad / 8, BH), dim3(256), 0, rec.st, (const float*)st, st, b3, bq, 1, D.ld, 0, 0, false);
+    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<DV>), 0, rec.st, (const float*)st, st, b3, bq, 1, 0, 0, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 inline hla_status emit_from_state(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, bool gradient, LaunchRec& rec) {
@@ -1550,7 +1554,7 @@ inline hla_status launch_core_backward(const Plan& P, const Dims& D, int BH, con
             if (e != HLA_OK) return e;
         }
         rec.begin("tc_reduce_emit");
-        launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / 8, BH), dim3(256), 0, st, part, dstate, bd3, bdq, D.S, D.ld, 0, 0, run_between);
+        launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, dstate, bd3, bdq, D.S, 0, 0, run_between);
         if (!rec.end()) return HLA_ERR_CUDA;
         if (phase == 1) return HLA_OK;
     } else {

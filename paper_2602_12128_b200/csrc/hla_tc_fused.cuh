@@ -140,8 +140,7 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;     // D1[b] at columns 128*b, D2[b] at 256 + 32*b, readout accumulator at 320
-    if (READOUT) grid_dependency_wait();
-    else grid_start_beside();
+    grid_start_beside();      // READOUT: only the state operand is the work of the kernel before this one; its loader waits for it
     bool ok = true;
 
     if (warp == 0) {
@@ -207,6 +206,7 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
             static_assert(Cfg::kB3Block % 16 == 0, "descriptor advance");
             int cur_bh = -1, nload = 0;
             bool good = true;
+            grid_dependency_wait();      // the reduction has left the state operands
             for (int it = 0; it < nwork && good; ++it) {
                 const int bh = (w0 + it) / tiles_per_head;
                 if (bh != cur_bh) {

@@ -219,13 +219,18 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
         // form 2 GELU); row kFkB1Row of the same tile holds b1: read as an MN-major operand [16 K rows][DV] it is the B
         // operand of the bias step of the first layer.  (After the dependency wait: a kernel of the caller may have just written
         // the weights.  Warp 0 has started the loads of the tiles meanwhile.)
-        for (int i = tid - 32; i < NM * DV * (DP + 1); i += kFkThreads - 32) {
-            const int m = i / (DV * (DP + 1)), j = (i / (DP + 1)) % DV, o = i % (DP + 1);
-            uint8_t* base = smem + Cfg::kOffW2 + m * Cfg::kW2Bytes + (j >> 6) * 2048;
-            const int r = o < DP ? o : kFkB1Row;
-            *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(r, (j & 63) >> 3) + (j & 7) * 2) = o < DP ? half_bf16(P.W2[m][j * DP + o]) : P.b1[m][j];
+        for (int i = tid - 32; i < NM * DV; i += kFkThreads - 32) {
+            const int m = i / DV, j = i % DV;
+            __nv_bfloat16 w[DP];
+            const __nv_bfloat16 b = P.b1[m][j];
+            load_w2_row<DP>(P.W2[m], j, w);
+            uint8_t* base = smem + Cfg::kOffW2 + m * Cfg::kW2Bytes + (j >> 6) * 2048 + (j & 7) * 2;
+#pragma unroll
+            for (int o = 0; o < DP; ++o) *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(o, (j & 63) >> 3)) = half_bf16(w[o]);
+            *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(kFkB1Row, (j & 63) >> 3)) = b;
         }
-        for (int i = tid - 32; i < NM * 16; i += kFkThreads - 32) b2s[i] = (i & 15) < DP ? __bfloat162float(P.b2[i >> 4][i & 15]) : 0.f;
+        // (the last threads, which have no row of W2 to stage)
+        for (int i = kFkThreads - 1 - tid; i < NM * 16; i += kFkThreads - 32) b2s[i] = (i & 15) < DP ? __bfloat162float(P.b2[i >> 4][i & 15]) : 0.f;
         fence_proxy_async();
         tc_fence_before();
         named_barrier(1, kFkThreads - 32);

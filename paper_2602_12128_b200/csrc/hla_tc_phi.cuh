@@ -69,6 +69,33 @@ __device__ __forceinline__ void gelu_both2(float2 dg, float2 x, float2& g2, floa
     dh = __ffma2_rn(dg, q, dg);
 }
 
+// Row j of a second-layer weight [d][DP] (hidden unit j), as the kernels stage it: one thread per (map, hidden unit), all of its loads in
+// flight at once.  (One element per thread and step, written to shared memory before the next was loaded, took the key side's 2688 elements
+// 4.6 us at the start of every call and the 6144 of its backward seven round trips to L2.)
+template <int DP> __device__ __forceinline__ void load_w2_row(const __nv_bfloat16* W2, int j, __nv_bfloat16 (&w)[DP]) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(W2 + (size_t)j * DP);      // W2 is 16-byte aligned, DP even
+    uint32_t r[DP / 2];
+#pragma unroll
+    for (int i = 0; i < DP / 2; ++i) r[i] = src[i];
+#pragma unroll
+    for (int i = 0; i < DP / 2; ++i) {
+        w[2 * i] = __ushort_as_bfloat16((unsigned short)(r[i] & 0xffffu));
+        w[2 * i + 1] = __ushort_as_bfloat16((unsigned short)(r[i] >> 16));
+    }
+}
+// Column j of a map's staged [W2^T; W2^T] tile of ROWS K rows (rows 0..DP-1 meet dp_hi, rows DP..2DP-1 meet dp_lo; row B1ROW holds b1 for
+// the bias step; the rest is zero): an MN-major operand in blocks of 64 hidden units, BLOCK bytes apart.
+template <int DP, int ROWS, int B1ROW, int BLOCK>
+__device__ __forceinline__ void stage_w2t_column(uint8_t* tile, const __nv_bfloat16* W2, const __nv_bfloat16* b1, int j) {
+    __nv_bfloat16 w[DP];
+    const __nv_bfloat16 b = b1[j];
+    load_w2_row<DP>(W2, j, w);
+    uint8_t* base = tile + (j >> 6) * BLOCK + (j & 7) * 2;
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k)
+        *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(k, (j & 63) >> 3)) = k < 2 * DP ? half_bf16(w[k % DP]) : (k == B1ROW ? b : __float2bfloat16_rn(0.f));
+}
+
 struct PhiPtrs {
     const __nv_bfloat16* b1[3];
     const __nv_bfloat16* W2[3];
@@ -170,13 +197,10 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
     const int ntiles = (int)(t1 - t0);
     const int nunits = ntiles * NMAPS;
 
-    // W2^T stacked twice (rows 0..DP-1 meet dp_hi, rows DP..2DP-1 meet dp_lo, the rest is zero but for b1), as an MN-major operand
     constexpr int kRows = 16 * Cfg::kDgSteps, kB1Abs = kRows - 16 + Cfg::kB1Row;
-    for (int i = tid; i < NMAPS * kRows * DV; i += kPbThreads) {
-        const int m = i / (kRows * DV), k = (i / DV) % kRows, j = i % DV;
-        uint8_t* base = smem + Cfg::kOffW2t + m * Cfg::kW2tBytes + (j >> 6) * Cfg::kW2tBlock;
-        *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(k, (j & 63) >> 3) + (j & 7) * 2) =
-            k < 2 * DP ? half_bf16(P.W2[m][j * DP + (k % DP)]) : (k == kB1Abs ? P.b1[m][j] : __float2bfloat16_rn(0.f));
+    for (int i = tid; i < NMAPS * DV; i += kPbThreads) {
+        const int m = i / DV;
+        stage_w2t_column<DP, kRows, kB1Abs, Cfg::kW2tBlock>(smem + Cfg::kOffW2t + m * Cfg::kW2tBytes, P.W2[m], P.b1[m], i % DV);
     }
     for (int i = tid; i < Cfg::kDpBlocks * kBlk / 16; i += kPbThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffDp)[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();

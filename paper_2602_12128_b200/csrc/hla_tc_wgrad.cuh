@@ -94,12 +94,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     float* out_cta = wpart + (size_t)blockIdx.x * Cfg::kPartFloats;
 
     constexpr int kRows = 16 * Cfg::kDgSteps, kB1Abs = kRows - 16 + Cfg::kB1Row;
-    for (int i = tid; i < kRows * DV; i += kWgThreads) {
-        const int k = i / DV, j = i % DV;
-        uint8_t* base = smem + Cfg::kOffW2t + (j >> 6) * Cfg::kW2tBlock;
-        *reinterpret_cast<__nv_bfloat16*>(base + sw128_off(k, (j & 63) >> 3) + (j & 7) * 2) =
-            k < 2 * DP ? half_bf16(W2g[j * DP + (k % DP)]) : (k == kB1Abs ? b1g[j] : __float2bfloat16_rn(0.f));
-    }
+    if (tid < DV) stage_w2t_column<DP, kRows, kB1Abs, Cfg::kW2tBlock>(smem + Cfg::kOffW2t, W2g, b1g, tid);
     for (int i = tid; i < 3 * kBlk / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffDp)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < 2 * Cfg::kXBytes / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffX)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < 4 * kBlk / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffG)[i] = make_uint4(0, 0, 0, 0);
