@@ -431,26 +431,29 @@ hla_status forward_impl(hla_ctx* ctx, const void* Q, const void* K, const void* 
     if (ctx->tc) {
         const float *qf, *kf;
         if (ctx->cfg.phi == HLA_PHI_MLP) {
+            if (ctx->cfg.causal) {
+                // the feature map of the queries and the key side leave the features of both sides in the workspace; the pieces of the
+                // key side become the pieces of the sweep
+                float* carry_copy = reinterpret_cast<float*>(ws + ctx->off_gpart);      // (scratch of the backward, which a carried call does not have)
+                s = tc::causal_maps(ctx->D, ctx->BH, &ctx->phi_q, ctx->phi_k, Q, K, V, ws, ctx->L, ctx->off_part, ctx->k_pieces, ctx->carry, carry_copy,
+                                    ctx->sm_count, ctx->rec);
+                if (s != HLA_OK) return s;
+                return tc::causal_sweep(ctx->D, ctx->BH, reinterpret_cast<const float*>(ws + ctx->L.qf), reinterpret_cast<const float*>(ws + ctx->L.kf), V, O,
+                                        ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count), ctx->carry, carry_copy, ctx->rec);
+            }
             // one kernel for the key maps and the state build -> reduction of its pieces -> one kernel for phi_q, readout
             // and normaliser
             if (phase != 2) {
                 s = tc::phik_state(ctx->D, ctx->BH, ctx->phi_k, K, V, ws, ctx->L, ctx->off_part, ctx->k_pieces, ctx->sm_count, ctx->rec);
                 if (s != HLA_OK) return s;
-                // (the causal sweep reads the pieces themselves)
-                if (!ctx->cfg.causal)
-                    s = tc::reduce_pieces(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count),
-                                          ctx->rec);
+                s = tc::reduce_pieces(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count),
+                                      ctx->rec);
                 if (s != HLA_OK || phase == 1) return s;
             } else {
                 s = tc::emit_from_state(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, false, ctx->rec);
                 if (s != HLA_OK) return s;
             }
-            // causal: only the feature map of the query side runs (no readout), which leaves the features of both sides in the
-            // workspace; the pieces of the key-side kernel become the pieces of the sweep
-            s = tc::phiq_readout(ctx->tcp, ctx->D, ctx->BH, &ctx->phi_q, Q, O, ws, ctx->L, ctx->sm_count, ctx->rec, !ctx->cfg.causal);
-            if (s != HLA_OK || !ctx->cfg.causal) return s;
-            return tc::causal_sweep(ctx->D, ctx->BH, reinterpret_cast<const float*>(ws + ctx->L.qf), reinterpret_cast<const float*>(ws + ctx->L.kf), V, O,
-                                    ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count), ctx->carry, ctx->rec);
+            return tc::phiq_readout(ctx->tcp, ctx->D, ctx->BH, &ctx->phi_q, Q, O, ws, ctx->L, ctx->sm_count, ctx->rec);
         } else {
             qf = static_cast<const float*>(Q);
             kf = static_cast<const float*>(K);

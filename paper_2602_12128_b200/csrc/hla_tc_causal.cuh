@@ -30,6 +30,7 @@
 // (selects only where the mask cuts a 32 x 32 block, conversions 32 columns at a time, out-of-line waits, rolled loops).
 #pragma once
 #include "hla_tc.cuh"
+#include "hla_tc_fused.cuh"
 #include "hla_tc_fused_k.cuh"
 
 namespace hla {
@@ -140,6 +141,53 @@ __device__ __forceinline__ void tmem_st_state(uint32_t taddr, const float (&v)[8
              __float_as_uint(v[6]), __float_as_uint(v[7]));
 }
 
+// Where a sweep finds the state before its first piece.  Either a scan has left prefix states (self = false), or the slots hold the pieces
+// themselves and every CTA adds those before its own (after `carry`, if any), in the order of the scan and to the same bits.  The sum is
+// formed in shared memory at the start of a sweep: with the scan before it and one warp per 16 rows loading what it needed, the
+// two and the release between them took 10 of the 22 us of a call of 12 heads x 500 tokens.  A CTA reads all the pieces before its own
+// from L2, so this is done for few pieces per head only.
+constexpr int kSelfPrefixPieces = 16;
+inline bool self_prefix(int S) { return S <= kSelfPrefixPieces; }
+// THREADS threads, numbered t: [56][ld] floats of the state before piece `slot` (the head's first slot is `base`, `carry` its carried
+// state or null) into `dst`
+// and, where image is not null, its bf16 operand image.  Eight loads in flight per thread.
+template <int DV, int THREADS>
+__device__ __forceinline__ void stage_initial_state(float* dst, uint8_t* image, int t, const float* __restrict__ slots, int base, int slot, bool self,
+                                                    const float* __restrict__ carry) {
+    constexpr int ld = DV + 4, kQuads = kMono * ld / 4, kItems = (kQuads + THREADS - 1) / THREADS;
+    static_assert(kItems <= 4, "loads in flight");
+    const float4* src = reinterpret_cast<const float4*>(slots) + (size_t)(self ? base : slot) * kQuads;
+    const float4* first = reinterpret_cast<const float4*>(carry);
+    const int lo = self && carry ? -1 : 0, hi = self ? slot - base : 1;      // source -1 is the carried state
+    float4 a[kItems];
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int p = lo; p < hi; p += 2) {
+        float4 v[2][kItems];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float4* from = p + j < 0 ? first : src + (size_t)(p + j) * kQuads;
+#pragma unroll
+            for (int k = 0; k < kItems; ++k) v[j][k] = p + j < hi && t + k * THREADS < kQuads ? from[t + k * THREADS] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int k = 0; k < kItems; ++k) {
+                a[k].x += v[j][k].x; a[k].y += v[j][k].y; a[k].z += v[j][k].z; a[k].w += v[j][k].w;
+            }
+    }
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        const int i = t + k * THREADS;
+        if (i >= kQuads) break;
+        reinterpret_cast<float4*>(dst)[i] = a[k];
+        const int m = i / (ld / 4), c = 4 * (i - m * (ld / 4));
+        if (image) *reinterpret_cast<uint2*>(image + (c >> 6) * (64 * 128) + sw128_off(m + kCaRowPad, (c & 63) >> 3) + (c & 7) * 2) = make_uint2(pack_bf16(a[k].x, a[k].y), pack_bf16(a[k].z, a[k].w));
+    }
+}
+
 // In-place exclusive scan of the piece states of every head, in piece order (bit-reproducible); the sum of all pieces,
 // i.e. the state after the last token, goes to `state`.  REVERSE: the scan runs from the last piece to the first (every
 // piece gets the sum of the pieces after it).  carry != 0: the scan starts from what `state` holds (the state an earlier
@@ -187,7 +235,9 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
                                                                           const float* __restrict__ qf, const float* __restrict__ kf,
                                                                           const float* __restrict__ init, float* __restrict__ eta_out,
                                                                           const float* __restrict__ eta_in, const float* __restrict__ delta, int N, int BH,
-                                                                          int S, int ld, int G, float eps, int* status) {
+                                                                          int S, int G, float eps, int* status, const float* __restrict__ carry, bool self_sum,
+                                                                          float* __restrict__ state_out) {
+    constexpr int ld = DV + 4;
     using Cfg = CaCfg<DV>;
     constexpr int kStageBytes = Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
@@ -197,10 +247,11 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     uint64_t* stage_free = bars + 2;      // [2] 2 MMA commits (one per issuing thread): every product that reads the stage has finished
     uint64_t* p_full = bars + 4;          // MMA commit
     uint64_t* pm_ready = bars + 5;        // 256 arrivals: masked bf16 block is in tensor memory
-    uint64_t* b3_ready = bars + 15;       // [2] 128 arrivals, barrier it & 1: state image of tile it (at the start of a piece also the
-                                          // state) is in place; two barriers because the image of tile it + 1 can be ready before
+    uint64_t* b3_ready = bars + 15;       // [2] 128 arrivals, barrier it & 1: state image of tile it is in place; two barriers because the image of tile it + 1 can be ready before
                                           // the readout of tile it has waited
     uint64_t* acc_free = bars + 12;       // 128 arrivals: the accumulator has been drained
+    uint64_t* state_init = bars + 18;     // 128 arrivals: the initial state of a piece is in tensor memory
+    uint64_t* staging_read = bars + 17;   // 128 arrivals, once: the first piece's has been read from the staging tile of O
     uint64_t* rd_done = bars + 13;        // [2] MMA commit after the readout of tile it, on barrier it & 1 (a waiter may lag two
                                           // tiles behind the issuing thread, which one barrier's phase parity cannot tell apart)
     uint64_t* state_full = bars + 7;      // MMA commit
@@ -226,6 +277,8 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
         mbar_init(&b3_ready[0], 128);
         mbar_init(&b3_ready[1], 128);
         mbar_init(acc_free, 128);
+        mbar_init(state_init, 128);
+        mbar_init(staging_read, 128);
         mbar_init(&rd_done[0], 1);
         mbar_init(&rd_done[1], 1);
         mbar_init(state_full, 1);
@@ -247,8 +300,25 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_begin(false);
+    grid_dependency_wait();
     bool ok = true;
+    if (warp >= kCaMaskWarp0 && warp < kCaStateMmaWarp) {
+        // the state before the first piece: image, and in fp32 the staging tile of O (first used when the first tile is done)
+        constexpr int kThreads = (kCaStateMmaWarp - kCaMaskWarp0) * 32;
+        static_assert(kMono * ld * 4 <= Cfg::kVB * kBlk, "staging tile");
+        const int t = tid - kCaMaskWarp0 * 32;
+        if (nwork > 0) {
+            const int bh = work_of(0) / T;
+            stage_initial_state<DV, kThreads>(reinterpret_cast<float*>(smem + Cfg::kOffO), smem + Cfg::kOffB3, t, init, bh * S, causal_slot(bh, T, BH, S, G), self_sum,
+                                              carry ? carry + (size_t)bh * kMono * ld : nullptr);
+            fence_proxy_async();
+        }
+        named_barrier(2, kThreads);
+        // Self-summing without state_out: the scan that runs beside this kernel overwrites the pieces and the carried state.  It starts when
+        // every CTA has got here, or, where a CTA begins another head later and reads that head's carried state then, has ended.
+        const bool reads_later = self_sum && carry && !state_out && nwork > 0 && (w0 + nwork - 1) / T != w0 / T;
+        if (t == 0 && !reads_later) grid_launch_dependents();
+    }
 
     if (warp == 0) {
         if (lane == 0) {
@@ -300,13 +370,14 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
         // chain state -> image -> readout of consecutive tiles is the long one.
         if (lane == 0) {
             const uint32_t id_s = idesc_bf16(64, Cfg::kNState, true, true);
+            int begun = 0;
             for (int it = 0; it < nwork; ++it) {
                 const int st = it & 1, u = it >> 1;
                 const uint32_t sa = smem_u32(smem + st * kStageBytes), ta = sa + Cfg::kOffT;
                 // the state after the previous tile must have been read out of tensor memory; the first tile of a piece
                 // waits for the initial state
                 if (it > 0 && !mbar_wait_c(state_read, (it - 1) & 1)) { report_timeout(status, 911); break; }
-                if (starts(it) && !mbar_wait_c(&b3_ready[it & 1], (it >> 1) & 1)) { report_timeout(status, 912); break; }
+                if (starts(it) && !mbar_wait_c(state_init, begun++ & 1)) { report_timeout(status, 912); break; }
                 if (!mbar_wait_c(&stage_ready[st], u & 1)) { report_timeout(status, 904); break; }
                 tc_fence_after();
                 {      // state += Tsym^T * [V | 1]
@@ -452,22 +523,39 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
                 if (it >= 2 && ok && !mbar_wait_c(&rd_done[it & 1], ((it - 2) >> 1) & 1)) { ok = false; report_timeout(status, 914); }
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                const float* src = init + ((size_t)causal_slot(bh, T, BH, S, G) * kMono + (mine ? m : 0)) * ld;
+                if (it == 0) {      // (the image is written: the readout need not wait for the copy in tensor memory)
+                    mbar_arrive(&b3_ready[0]);
+                    const float* src = reinterpret_cast<const float*>(smem + Cfg::kOffO) + (mine ? m : 0) * ld;
+#pragma unroll 4
+                    for (int c = 0; c < Cfg::kNState / 8; ++c) {
+                        const float4 x = *reinterpret_cast<const float4*>(src + 8 * c);
+                        const float4 y = 8 * c + 4 < ld ? *reinterpret_cast<const float4*>(src + 8 * c + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float v[8] = {mine ? x.x : 0.f, mine ? x.y : 0.f, mine ? x.z : 0.f, mine ? x.w : 0.f, mine ? y.x : 0.f, mine ? y.y : 0.f, mine ? y.z : 0.f, mine ? y.w : 0.f};
+                        tmem_st_state(sa + 8 * c, v);
+                    }
+                } else {
+                    // a later piece: with self_sum it is the first of its head, and what precedes it is the carried state or nothing
+                    const float* src = (self_sum ? carry + (size_t)bh * kMono * ld : init + (size_t)causal_slot(bh, T, BH, S, G) * kMono * ld) + (mine ? m : 0) * ld;
 #pragma unroll 1
-                for (int c0 = 0; c0 < kChunks; c0 += kStateBatch) {
-                    float v[kStateBatch][8];
-                    load_state_chunks(v, src, c0, ld, mine);
+                    for (int c0 = 0; c0 < kChunks; c0 += kStateBatch) {
+                        float v[kStateBatch][8];
+                        load_state_chunks(v, src, c0, ld, mine && (!self_sum || carry));
 #pragma unroll
-                    for (int k = 0; k < kStateBatch; ++k) {
-                        const int c = c0 + k;
-                        if (8 * c < Cfg::kNState) tmem_st_state(sa + 8 * c, v[k]);
-                        if (c < kChunks) store_chunk(it, c, v[k]);
+                        for (int k = 0; k < kStateBatch; ++k) {
+                            const int c = c0 + k;
+                            if (8 * c < Cfg::kNState) tmem_st_state(sa + 8 * c, v[k]);
+                            if (c < kChunks) store_chunk(it, c, v[k]);
+                        }
                     }
                 }
                 tmem_st_wait();
                 tc_fence_before();
-                fence_proxy_async();
-                mbar_arrive(&b3_ready[it & 1]);
+                if (it > 0) {
+                    fence_proxy_async();
+                    mbar_arrive(&b3_ready[it & 1]);
+                }
+                else mbar_arrive(staging_read);
+                mbar_arrive(state_init);
             }
             if (ok && !mbar_wait_c(state_full, it & 1)) { ok = false; report_timeout(status, 908); }
             ok = __all_sync(0xffffffffu, ok);
@@ -509,7 +597,23 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
                 fence_proxy_async();
                 mbar_arrive(&b3_ready[(it + 1) & 1]);
             } else {
-                mbar_arrive(state_read);      // nothing is read: the next tile (if any) starts a piece with a state of its own
+                // the next tile (if any) starts a piece with a state of its own; the state after a head's last token is what the head leaves
+                if (MODE == 0 && state_out && work % T == T - 1) {
+                    tc_fence_after();
+                    float* dst = state_out + ((size_t)bh * kMono + (mine ? m : 0)) * ld;
+#pragma unroll 1
+                    for (int c = 0; c < Cfg::kNState / 8; ++c) {
+                        uint32_t r[8];
+                        tmem_ld8(sa + 8 * c, r);
+                        tmem_ld_wait();
+                        if (!mine) continue;
+                        const bool z = 8 * c >= DV;      // column d, then padding
+                        *reinterpret_cast<uint4*>(dst + 8 * c) = z ? make_uint4(r[0], 0u, 0u, 0u) : make_uint4(r[0], r[1], r[2], r[3]);
+                        if (!z) *reinterpret_cast<uint4*>(dst + 8 * c + 4) = make_uint4(r[4], r[5], r[6], r[7]);
+                    }
+                    tc_fence_before();
+                }
+                mbar_arrive(state_read);
             }
         }
     } else {
@@ -519,7 +623,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
         const uint32_t os = smem_u32(smem + Cfg::kOffO);
         for (int it = 0; it < nwork; ++it) {
             const int work = work_of(it), bh = work / T, tile = work % T;
-            if (!mbar_wait_c(acc_full, it & 1)) {
+            if (!mbar_wait_c(acc_full, it & 1) || (it == 0 && !mbar_wait_c(staging_read, 0))) {
                 report_timeout(status, 909);
                 *abort_flag = 1;
             }
@@ -565,11 +669,56 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// Exclusive scan of the piece states, then the causal sweep.  The pieces are those of the kernel that built them:
-// G == 0: S pieces per head from a (S, heads) grid; G > 0: the pieces of a persistent kernel of G CTAs (at most S per head).
+// The feature maps of a causal forward in one launch: CTAs 0 .. key_grid - 1 are the key side (features, states of the pieces), the others the
+// map of the queries.  Short calls are chains of launches, and as two kernels side by side the two cost a launch and a release more (2 of
+// 22 us at 12 heads x 500 tokens); long ones run the query CTAs as the key CTAs leave their SMs.
+struct PhiqArgs {
+    CUtensorMap Q, W1;
+    const __nv_bfloat16 *b1, *W2, *b2;
+};
+template <int DV>
+__global__ void __launch_bounds__(kFkThreads, 1) tc_causal_maps_kernel(const __grid_constant__ PhikArgs k, const __grid_constant__ PhiqArgs q, float* __restrict__ kf_out,
+                                                                       float* __restrict__ qf_out, float* __restrict__ part, int N, int BH, int smax, int* status,
+                                                                       const float* __restrict__ carry, float* __restrict__ carry_copy, int key_grid) {
+    if ((int)blockIdx.x < key_grid)
+        phik_state_cta<DV, 3>(k.K, k.maps, k.V, k.ptrs, kf_out, part, N, BH, smax, status, carry, carry_copy, blockIdx.x, key_grid);
+    else
+        phiq_cta<DV, 3, false>(q.Q, q.W1, q.Q, q.Q, q.b1, q.W2, q.b2, qf_out, nullptr, N, BH, 0.f, status, blockIdx.x - key_grid, gridDim.x - key_grid);
+}
+template <int DV>
+inline hla_status launch_causal_maps(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K, const void* V, char* ws,
+                                     const hla_ws_layout& L, size_t off_part, int smax, bool carry, float* carry_copy, int sm_count, LaunchRec& rec) {
+    static_assert(kFkThreads == kFqThreads, "one block size");
+    constexpr int kSmem = FkCfg<DV, 3>::kSmem > FqCfg<DV, 3>::kSmem ? FkCfg<DV, 3>::kSmem : FqCfg<DV, 3>::kSmem;
+    PhikArgs k;
+    PhiqArgs q;
+    if (!phik_args<DV, 3>(k, D, BH, phi_k, K, V) || !make_map_bhnd(&q.Q, Q, BH, D.N, DV, kTileTokens) || !make_map_2d(&q.W1, phi_q->W1, DV, DV, DV) ||
+        !set_smem(tc_causal_maps_kernel<DV>, kSmem))
+        return HLA_ERR_CUDA;
+    q.b1 = static_cast<const __nv_bfloat16*>(phi_q->b1);
+    q.W2 = static_cast<const __nv_bfloat16*>(phi_q->W2);
+    q.b2 = static_cast<const __nv_bfloat16*>(phi_q->b2);
+    const int grid = fused_key_grid(BH, D.N, sm_count);      // of each side
+    rec.begin("tc_causal_maps");
+    launch_pdl(tc_causal_maps_kernel<DV>, 2 * grid, dim3(kFkThreads), kSmem, rec.st, k, q, reinterpret_cast<float*>(ws + L.kf), reinterpret_cast<float*>(ws + L.qf),
+               reinterpret_cast<float*>(ws + off_part), D.N, BH, smax, reinterpret_cast<int*>(ws + L.status),
+               carry ? reinterpret_cast<const float*>(ws + L.state) : (const float*)nullptr, carry_copy, grid);
+    return rec.end() ? HLA_OK : HLA_ERR_CUDA;
+}
+inline hla_status causal_maps(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K, const void* V, char* ws,
+                              const hla_ws_layout& L, size_t off_part, int smax, bool carry, float* carry_copy, int sm_count, LaunchRec& rec) {
+    if (D.d == 128) return launch_causal_maps<128>(D, BH, phi_q, phi_k, Q, K, V, ws, L, off_part, smax, carry, carry_copy, sm_count, rec);
+    return launch_causal_maps<64>(D, BH, phi_q, phi_k, Q, K, V, ws, L, off_part, smax, carry, carry_copy, sm_count, rec);
+}
+
+// The causal sweep.  The pieces are those of the kernel that built them: G == 0: S pieces per head from a (S, heads) grid; G > 0: the pieces
+// of a persistent kernel of G CTAs (at most S per head), which has also copied the carried state, if any, to carry_copy.
+//   few pieces, G > 0: the sweep alone (it writes the state after the last token; the slots keep the pieces);
+//   few pieces, G == 0: the sweep, beside it the scan, which leaves prefix states and the state after the last token;
+//   else: the scan, then the sweep.
 template <int DV>
 inline hla_status launch_causal_sweep(const Dims& D, int BH, const float* qf, const float* kf, const void* V, void* O, char* ws, const hla_ws_layout& L,
-                                      size_t off_part, int S, int G, bool carry, LaunchRec& rec) {
+                                      size_t off_part, int S, int G, bool carry, float* carry_copy, LaunchRec& rec) {
     CUtensorMap mapV, mapO;
     if (!make_map_bhnd(&mapV, V, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapO, O, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
     int* status = reinterpret_cast<int*>(ws + L.status);
@@ -578,20 +727,26 @@ inline hla_status launch_causal_sweep(const Dims& D, int BH, const float* qf, co
     float* eta = reinterpret_cast<float*>(ws + L.eta);
     if (!set_smem(tc_causal_forward_kernel<DV, 0>, CaCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
-    rec.begin("tc_scan_pieces");
-    launch_pdl(tc_scan_pieces_kernel<3>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, state, S, D.ld, G, T, carry ? 1 : 0, false);
-    if (!rec.end()) return HLA_ERR_CUDA;
+    const bool self_sum = self_prefix(S), alone = self_sum && G > 0;
+    auto scan = [&]() {
+        rec.begin("tc_scan_pieces");
+        launch_pdl(tc_scan_pieces_kernel<3>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, state, S, D.ld, G, T, carry ? 1 : 0, self_sum);
+        return rec.end();
+    };
+    if (!self_sum && !scan()) return HLA_ERR_CUDA;
     rec.begin("tc_causal_forward");
     launch_pdl(tc_causal_forward_kernel<DV, 0>, G > 0 ? dim3(G) : dim3(S, BH), dim3(kCaThreads), CaCfg<DV>::kSmem, rec.st, mapV, mapO, qf, kf,
-               (const float*)part, eta, (const float*)nullptr, (const float*)nullptr, D.N, BH, S, D.ld, G, D.eps, status);
-    return rec.end() ? HLA_OK : HLA_ERR_CUDA;
+               (const float*)part, eta, (const float*)nullptr, (const float*)nullptr, D.N, BH, S, G, D.eps, status,
+               (const float*)(!carry ? nullptr : alone ? carry_copy : state), self_sum, alone ? state : (float*)nullptr);
+    if (!rec.end()) return HLA_ERR_CUDA;
+    return alone || !self_sum || scan() ? HLA_OK : HLA_ERR_CUDA;
 }
 
 inline hla_status causal_sweep(const Dims& D, int BH, const float* qf, const float* kf, const void* V, void* O, char* ws, const hla_ws_layout& L,
-                               size_t off_part, int S, int G, bool carry, LaunchRec& rec) {
+                               size_t off_part, int S, int G, bool carry, float* carry_copy, LaunchRec& rec) {
     if (D.F != 3) return HLA_ERR_UNSUPPORTED;
-    if (D.d == 128) return launch_causal_sweep<128>(D, BH, qf, kf, V, O, ws, L, off_part, S, G, carry, rec);
-    return launch_causal_sweep<64>(D, BH, qf, kf, V, O, ws, L, off_part, S, G, carry, rec);
+    if (D.d == 128) return launch_causal_sweep<128>(D, BH, qf, kf, V, O, ws, L, off_part, S, G, carry, carry_copy, rec);
+    return launch_causal_sweep<64>(D, BH, qf, kf, V, O, ws, L, off_part, S, G, carry, carry_copy, rec);
 }
 
 // Feature-level causal forward: state of every piece (the non-causal state build, one piece per split) -> scan -> sweep.
@@ -613,7 +768,7 @@ inline hla_status causal_forward(const Dims& D, int BH, const float* qf, const f
     const hla_status s = D.d == 128 ? launch_causal_state_build<128>(D, BH, kf, V, ws, L, off_part, rec)
                                     : launch_causal_state_build<64>(D, BH, kf, V, ws, L, off_part, rec);
     if (s != HLA_OK) return s;
-    return causal_sweep(D, BH, qf, kf, V, O, ws, L, off_part, D.S, 0, carry, rec);
+    return causal_sweep(D, BH, qf, kf, V, O, ws, L, off_part, D.S, 0, carry, nullptr, rec);
 }
 
 // delta_i = dO_i . o_i for every token row (bf16 rows of d values, fp32 sum): d / 8 lanes per row, 16 bytes per lane.
@@ -678,7 +833,7 @@ inline hla_status launch_causal_backward_values(const Dims& D, int BH, const flo
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dv");
     launch_pdl(tc_causal_forward_kernel<DV, 1>, dim3(D.S, BH), dim3(kCaThreads), CaCfg<DV>::kSmem, rec.st, mapdO, mapdV, qf, kf, (const float*)part,
-               (float*)nullptr, (const float*)eta, (const float*)delta, D.N, BH, D.S, D.ld, 0, D.eps, status);
+               (float*)nullptr, (const float*)eta, (const float*)delta, D.N, BH, D.S, 0, D.eps, status, (const float*)nullptr, false, (float*)nullptr);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 

@@ -61,8 +61,9 @@ template <int DV, int DIR>
 __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
                                                                        const float* __restrict__ qf, const float* __restrict__ kf,
                                                                        const float* __restrict__ eta, const float* __restrict__ delta,
-                                                                       const float* __restrict__ init, float* __restrict__ out, int N, int BH, int S, int ld,
-                                                                       int G, float eps, int* status, bool beside) {
+                                                                       const float* __restrict__ init, float* __restrict__ out, int N, int BH, int S,
+                                                                       int G, float eps, int* status, bool beside, bool self_sum) {
+    constexpr int ld = DV + 4;
     using Cfg = CgCfg<DV>;
     constexpr int kStageBytes = Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
@@ -130,6 +131,15 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
     const uint32_t tmem = *tmem_slot;
     grid_begin(beside);
     bool ok = true;
+    // the state before the first piece: image, and in fp32 the X tile of the second stage (TMA loads it once the first image is in place)
+    float* init0 = reinterpret_cast<float*>(smem + kStageBytes + Cfg::kOffX);
+    static_assert(kMono * ld * 4 <= Cfg::kVB * kBlk, "staging tile");
+    if (nwork > 0) {
+        const int bh = work_of(0) / T;
+        stage_initial_state<DV, kCgThreads>(init0, nullptr, tid, init, bh * S, causal_slot(bh, T, BH, S, G), self_sum, nullptr);
+        fence_proxy_async();
+    }
+    __syncthreads();
 
     if (warp >= kCgEpiWarp0) {
         reg_inc<kCgEpiRegs>();
@@ -206,6 +216,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                 for (int it = 0; it < nwork; ++it, step(p, 1)) {
                     const int st = it & 1, u = it >> 1, tile = p.tile, bh = p.bh;
                     if (!mbar_wait(&stage_free[st], (u & 1) ^ 1)) { report_timeout(status, 921); break; }
+                    if (it == 1 && !mbar_wait(&b3_ready[0], 0)) { report_timeout(status, 938); break; }
                     mbar_arrive_expect_tx(&stage_ready[st], 2 * DV * kTileTokens * 2);
                     for (int b = 0; b < Cfg::kVB; ++b) {
                         tma_load_3d(smem + st * kStageBytes + b * kBlk, &mapY, &stage_ready[st], b * 64, tile * kTileTokens, bh);
@@ -432,12 +443,13 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
-                    const float* src = init + ((size_t)causal_slot(pos_of(it).bh, T, BH, S, G) * kMono + (mine ? m : 0)) * ld;
+                    // (with self_sum a later piece is the first of its head: nothing precedes it)
+                    const float* src = (it == 0 ? init0 : init + (self_sum ? 0 : (size_t)causal_slot(pos_of(it).bh, T, BH, S, G) * kMono * ld)) + (mine ? m : 0) * ld;
                     const uint32_t b3img = b3base + (it & 1) * Cfg::kB3Bytes;
 #pragma unroll 1
                     for (int c0 = 0; c0 < (DV + 8) / 8; c0 += kStateBatch) {
                         float v[kStateBatch][8];
-                        load_state_chunks(v, src, c0, ld, mine);
+                        load_state_chunks(v, src, c0, ld, mine && (it == 0 || !self_sum));
 #pragma unroll
                         for (int k = 0; k < kStateBatch; ++k) {
                             const int c = c0 + k;
@@ -502,13 +514,14 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
     grid_end(beside);
 }
 
-// The pieces the forward swept, and the prefix states of which it left in the workspace: S slots per head, G as in CaWork.
+// The pieces the forward swept and what it left in their slots (S per head, G as in CaWork): the pieces themselves or their prefix states.
 struct CausalPieces {
     size_t off;
     int S, G;
+    bool self() const { return G > 0 && self_prefix(S); }
 };
 
-// Feature gradients of the causal operator: the forward sweep for dq on the prefix states that the forward left in the workspace (they were
+// Feature gradients of the causal operator: the forward sweep for dq on the piece or prefix states that the forward left in the workspace (they were
 // rebuilt here at first: a pass over the keys and V and a scan, 59 us of a training step with 24 heads x 32760 tokens); then, on the
 // gradient states the value-gradient pass left (suffix sums), the backward sweep for dk.
 template <int DV>
@@ -524,13 +537,13 @@ inline hla_status launch_causal_backward_features(const Dims& D, int BH, const f
         if (!set_smem(tc_causal_grad_kernel<DV, 0>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
         rec.begin("tc_causal_dq");
         launch_pdl(tc_causal_grad_kernel<DV, 0>, fwd.G > 0 ? dim3(fwd.G) : dim3(fwd.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapdO, mapV, qf, kf, eta, delta,
-                   reinterpret_cast<const float*>(ws + fwd.off), dqf, D.N, BH, fwd.S, D.ld, fwd.G, D.eps, status, false);
+                   reinterpret_cast<const float*>(ws + fwd.off), dqf, D.N, BH, fwd.S, fwd.G, D.eps, status, false, fwd.self());
         return rec.end() ? HLA_OK : HLA_ERR_CUDA;
     }
     if (!set_smem(tc_causal_grad_kernel<DV, 1>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dk");
     launch_pdl(tc_causal_grad_kernel<DV, 1>, dim3(D.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapV, mapdO, qf, kf, eta, delta,
-               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, D.ld, 0, D.eps, status, true);
+               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, 0, D.eps, status, true, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 

@@ -46,24 +46,20 @@ template <int DV, int F> struct FqCfg {
     static constexpr int kSmem = kSmemUsed > 120 * 1024 ? kSmemUsed : 120 * 1024;   // one CTA per SM (512 TMEM columns)
 };
 
-// Q [BH][N][DV] bf16 (3-D map, rows past N read as zero), O the same (stores are clipped at N).  READOUT = false: the feature
-// map only (the causal operator reads its states tile by tile in a sweep of its own and needs just the query features):
-// the readout product, its epilogue and the monomial tile are left out, O and eta are not written.  It then needs nothing of the kernel
-// before it (the key side of the same call, which lets it start only once everything before the call is complete): it waits for that
-// kernel at its end instead of its start, so that the two run side by side where they do not fill the SMs (12 heads x 500 tokens: a
-// quarter of a call).
-template <int DV, int F, bool READOUT = true>
-__global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapW1,
-                                                                        const __grid_constant__ CUtensorMap mapB3, const __grid_constant__ CUtensorMap mapO,
-                                                                        const __nv_bfloat16* __restrict__ b1g, const __nv_bfloat16* __restrict__ W2g,
-                                                                        const __nv_bfloat16* __restrict__ b2g, float* __restrict__ qf_out,
-                                                                        float* __restrict__ eta_out, int N, int BH, float eps, int* status) {
+// Q [BH][N][DV] bf16 (3-D map, rows past N read as zero), O the same (stores are clipped at N).  CTA `bid` of `G`.  READOUT = false: the
+// feature map only (the causal operator reads its states tile by tile in a sweep of its own and needs just the query features):
+// the readout product, its epilogue and the monomial tile are left out, O and eta are not written.
+template <int DV, int F, bool READOUT>
+__device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensorMap& mapW1, const CUtensorMap& mapB3, const CUtensorMap& mapO,
+                                         const __nv_bfloat16* __restrict__ b1g, const __nv_bfloat16* __restrict__ W2g, const __nv_bfloat16* __restrict__ b2g,
+                                         float* __restrict__ qf_out, float* __restrict__ eta_out, int N, int BH, float eps, int* status, int bid, int G) {
     using Cfg = FqCfg<DV, F>;
     using M = MT<F>;
     constexpr int DP = M::kDphi;
     constexpr int HC = DV / 4;          // hidden units per GELU thread
     extern __shared__ uint8_t smem_raw[];
-    grid_launch_dependents();
+    if (READOUT) grid_launch_dependents();
+    else grid_begin(false);      // first of its call: a kernel of the caller may have just written the weights that are staged now
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float* bias = reinterpret_cast<float*>(smem + Cfg::kOffBias);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
@@ -88,7 +84,7 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tiles_per_head = (N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles_per_head;
-    const int w0 = (int)(total * blockIdx.x / gridDim.x), w1 = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    const int w0 = (int)(total * bid / G), w1 = (int)(total * (bid + 1) / G);
     const int nwork = w1 - w0;
 
     // second-layer weights as a K-major MMA operand [16 rows (outputs, 6 used)][DV], and the biases
@@ -140,7 +136,7 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;     // D1[b] at columns 128*b, D2[b] at 256 + 32*b, readout accumulator at 320
-    grid_start_beside();      // READOUT: only the state operand is the work of the kernel before this one; its loader waits for it
+    if (READOUT) grid_start_beside();      // only the state operand is the work of the kernel before this one; its loader waits for it
     bool ok = true;
 
     if (warp == 0) {
@@ -345,10 +341,18 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
-    if (!READOUT) grid_dependency_wait();      // what follows this kernel may rely on the key side too
 }
 
-template <int DV, int F, bool READOUT>
+template <int DV, int F>
+__global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapW1,
+                                                                        const __grid_constant__ CUtensorMap mapB3, const __grid_constant__ CUtensorMap mapO,
+                                                                        const __nv_bfloat16* __restrict__ b1g, const __nv_bfloat16* __restrict__ W2g,
+                                                                        const __nv_bfloat16* __restrict__ b2g, float* __restrict__ qf_out,
+                                                                        float* __restrict__ eta_out, int N, int BH, float eps, int* status) {
+    phiq_cta<DV, F, true>(mapQ, mapW1, mapB3, mapO, b1g, W2g, b2g, qf_out, eta_out, N, BH, eps, status, blockIdx.x, gridDim.x);
+}
+
+template <int DV, int F>
 inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, const hla_mlp* phi_q, const void* Q, void* O, char* ws,
                                       const hla_ws_layout& L, int sm_count, LaunchRec& rec) {
     CUtensorMap mapQ, mapW1, mapB3, mapO;
@@ -356,12 +360,12 @@ inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, cons
     if (!make_map_bhnd(&mapQ, Q, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapO, O, BH, D.N, DV, kTileTokens) ||
         !make_map_2d(&mapW1, phi_q->W1, DV, DV, DV) || !make_map_2d(&mapB3, b3, (size_t)BH * (DV + 16), MT<F>::kPad, DV + 16))
         return HLA_ERR_CUDA;
-    if (!set_smem(tc_phiq_readout_kernel<DV, F, READOUT>, FqCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
+    if (!set_smem(tc_phiq_readout_kernel<DV, F>, FqCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles;
     const int grid = (int)(total < sm_count ? total : sm_count);
-    rec.begin(READOUT ? "tc_phiq_readout" : "tc_phiq");
-    launch_pdl(tc_phiq_readout_kernel<DV, F, READOUT>, grid, dim3(kFqThreads), FqCfg<DV, F>::kSmem, rec.st,
+    rec.begin("tc_phiq_readout");
+    launch_pdl(tc_phiq_readout_kernel<DV, F>, grid, dim3(kFqThreads), FqCfg<DV, F>::kSmem, rec.st,
         mapQ, mapW1, mapB3, mapO, static_cast<const __nv_bfloat16*>(phi_q->b1), static_cast<const __nv_bfloat16*>(phi_q->W2),
         static_cast<const __nv_bfloat16*>(phi_q->b2), reinterpret_cast<float*>(ws + L.qf), reinterpret_cast<float*>(ws + L.eta), D.N, BH, D.eps,
         reinterpret_cast<int*>(ws + L.status));
@@ -369,18 +373,13 @@ inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, cons
 }
 
 inline hla_status phiq_readout(const Plan& P, const Dims& D, int BH, const hla_mlp* phi_q, const void* Q, void* O, char* ws, const hla_ws_layout& L,
-                               int sm_count, LaunchRec& rec, bool readout = true) {
+                               int sm_count, LaunchRec& rec) {
     if (D.F == 3) {
-        if (!readout) {
-            if (D.d == 128) return launch_phiq_readout<128, 3, false>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
-            return launch_phiq_readout<64, 3, false>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
-        }
-        if (D.d == 128) return launch_phiq_readout<128, 3, true>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
-        return launch_phiq_readout<64, 3, true>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
+        if (D.d == 128) return launch_phiq_readout<128, 3>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
+        return launch_phiq_readout<64, 3>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
     }
-    if (!readout) return HLA_ERR_UNSUPPORTED;
-    if (D.d == 128) return launch_phiq_readout<128, 2, true>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
-    return launch_phiq_readout<64, 2, true>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
+    if (D.d == 128) return launch_phiq_readout<128, 2>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
+    return launch_phiq_readout<64, 2>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
 }
 
 }  // namespace tc

@@ -123,10 +123,12 @@ __device__ __forceinline__ void folded_row_store2(uint32_t tile, uint32_t row, c
     (folded_chunk_store2<C>(tile, row, k1, k2, std::make_integer_sequence<int, 8>{}), ...);
 }
 
+// CTA `bid` of `G`.  carry, carry_copy: the state a causal call starts from, and where it is copied (or null).
 template <int DV, int F>
-__global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ PhiMaps maps,
-                                                                      const __grid_constant__ CUtensorMap mapV, PhiPtrs P, float* __restrict__ kf_out,
-                                                                      float* __restrict__ part, int N, int BH, int ld, int smax, int* status) {
+__device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const PhiMaps& maps, const CUtensorMap& mapV, const PhiPtrs& P, float* __restrict__ kf_out,
+                                               float* __restrict__ part, int N, int BH, int smax, int* status, const float* __restrict__ carry,
+                                               float* __restrict__ carry_copy, int bid, int G) {
+    constexpr int ld = DV + 4;
     using Cfg = FkCfg<DV, F>;
     using M = MT<F>;
     using Col = FkCols<F>;
@@ -158,8 +160,7 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int T = (N + kTileTokens - 1) / kTileTokens;      // tiles per head
     const long long total = (long long)BH * T;
-    const int G = gridDim.x;
-    const int w0 = (int)(total * blockIdx.x / G), w1 = (int)(total * (blockIdx.x + 1) / G);
+    const int w0 = (int)(total * bid / G), w1 = (int)(total * (bid + 1) / G);
     const int nwork = w1 - w0;
     auto head_of = [&](int it) { return (w0 + it) / T; };
     auto piece_ends = [&](int it) { return it == nwork - 1 || head_of(it + 1) != head_of(it); };
@@ -210,9 +211,9 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
         tmem_st_wait();
     }
     grid_dependency_wait();
-    if (blockIdx.x == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
-    // Only now may the next kernel start: the kernels of a call that stage weights before their own wait (or, the causal query map, do
-    // not wait at all until their end) rely on everything before the call being complete.
+    if (bid == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
+    // Only now may the next kernel start: the kernels of a call that stage weights before their own wait rely on everything before the
+    // call being complete.
     grid_launch_dependents();
     if (warp > 0) {
         // second-layer weights as a K-major MMA operand [16 rows (outputs, 6 used)][DV] per map, halved (the GELU warps
@@ -231,6 +232,10 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
         }
         // (the last threads, which have no row of W2 to stage)
         for (int i = kFkThreads - 1 - tid; i < NM * 16; i += kFkThreads - 32) b2s[i] = (i & 15) < DP ? __bfloat162float(P.b2[i >> 4][i & 15]) : 0.f;
+        // the carried state of a causal call, which its sweep reads while it writes the new one
+        if (carry)
+            for (long long i = (long long)bid * (kFkThreads - 32) + tid - 32; i < (long long)BH * M::kN * ld / 4; i += (long long)G * (kFkThreads - 32))
+                reinterpret_cast<float4*>(carry_copy)[i] = reinterpret_cast<const float4*>(carry)[i];
         fence_proxy_async();
         tc_fence_before();
         named_barrier(1, kFkThreads - 32);
@@ -366,22 +371,25 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
             if (lane == 0) mbar_arrive(f_empty);
             if (piece_ends(it)) {
                 const int bh = head_of(it);
-                const int piece = blockIdx.x - owner_of_work((long long)bh * T, total, G);
+                const int piece = bid - owner_of_work((long long)bh * T, total, G);
                 float* out = part + ((size_t)bh * smax + piece) * M::kN * ld;
                 auto put = [&](int m, float v) {
-                    if (m < M::kN) {
-                        out[(size_t)m * ld + DV] = v;
-                        for (int c = DV + 1; c < ld; ++c) out[(size_t)m * ld + c] = 0.f;
-                    }
+                    if (m < M::kN) *reinterpret_cast<float4*>(out + (size_t)m * ld + DV) = make_float4(v, 0.f, 0.f, 0.f);
                 };
+                // The 8 sums of a chunk over the 16 lanes that share it (lane bits 1..4): each of three steps halves the values a lane
+                // still holds, then one more adds the two halves of the rows: 8 shuffles instead of 32.  Value 4 b4 + 2 b3 + b2 (bits of the
+                // lane number) ends up in the lane.
+                float v4[4], v2[2], v1;
+                const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    float v = z0[e];
+                for (int e = 0; e < 4; ++e) v4[e] = (b4 ? z0[4 + e] : z0[e]) + __shfl_xor_sync(0xffffffffu, b4 ? z0[e] : z0[4 + e], 16);
 #pragma unroll
-                    for (int o = 2; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (lane < 2) put(8 * (2 * zw + lane) + e, v);
-                    z0[e] = 0.f;
-                }
+                for (int e = 0; e < 2; ++e) v2[e] = (b3 ? v4[2 + e] : v4[e]) + __shfl_xor_sync(0xffffffffu, b3 ? v4[e] : v4[2 + e], 8);
+                v1 = (b2 ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? v2[0] : v2[1], 4);
+                v1 += __shfl_xor_sync(0xffffffffu, v1, 2);
+                if (!(lane & 2)) put(8 * (2 * zw + (lane & 1)) + (lane >> 2), v1);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) z0[e] = 0.f;
                 if (M::kBlocks == 2) {      // (every warp runs the shuffles; warps 2 and 3 hold zeros)
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
@@ -447,18 +455,22 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                const int piece = blockIdx.x - owner_of_work((long long)bh * T, total, G);
+                const int piece = bid - owner_of_work((long long)bh * T, total, G);
                 float* out = part + ((size_t)bh * smax + piece) * M::kN * ld;
                 const int g = quarter * 32 + lane;       // TMEM lane = value channel
                 if (quarter * 32 < DV) {
 #pragma unroll
-                    for (int c = 0; c < (M::kN + 7) / 8; ++c) {
-                        uint32_t rr[8];
-                        tmem_ld8(tmem + Col::kC + lane_base + 8 * c, rr);
+                    for (int c = 0; c < M::kN; c += 32) {      // (32 columns per wait)
+                        uint32_t rr[4][8];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (c + 8 * k < M::kN) tmem_ld8(tmem + Col::kC + lane_base + c + 8 * k, rr[k]);
                         tmem_ld_wait();
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (8 * c + e < M::kN) out[(size_t)(8 * c + e) * ld + g] = __uint_as_float(rr[e]);
+                        for (int k = 0; k < 4; ++k)
+#pragma unroll
+                            for (int e = 0; e < 8; ++e)
+                                if (c + 8 * k + e < M::kN) out[(size_t)(c + 8 * k + e) * ld + g] = __uint_as_float(rr[k][e]);
                     }
                 }
                 tc_fence_before();
@@ -503,6 +515,13 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __gr
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
+template <int DV, int F>
+__global__ void __launch_bounds__(kFkThreads, 1) tc_phik_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ PhiMaps maps,
+                                                                      const __grid_constant__ CUtensorMap mapV, const __grid_constant__ PhiPtrs P,
+                                                                      float* __restrict__ kf_out, float* __restrict__ part, int N, int BH, int smax, int* status) {
+    phik_state_cta<DV, F>(mapK, maps, mapV, P, kf_out, part, N, BH, smax, status, nullptr, nullptr, blockIdx.x, gridDim.x);
+}
+
 // Largest number of pieces any head has when BH * T work items are dealt to G CTAs.
 inline int fused_key_max_pieces(int BH, int T, int G) {
     const long long total = (long long)BH * T;
@@ -518,25 +537,34 @@ inline int fused_key_grid(int BH, int N, int sm_count) {
     return (int)(total < sm_count ? total : sm_count);
 }
 
+// Tensor maps and pointers of the key side.
+struct PhikArgs {
+    CUtensorMap K, V;
+    PhiMaps maps;
+    PhiPtrs ptrs;
+};
+template <int DV, int F> inline bool phik_args(PhikArgs& a, const Dims& D, int BH, const hla_mlp* phi_k, const void* K, const void* V) {
+    a.ptrs = PhiPtrs{};
+    if (!make_map_bhnd(&a.K, K, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&a.V, V, BH, D.N, DV, kTileTokens)) return false;
+    for (int f = 0; f < MT<F>::kMaps; ++f) {
+        if (!make_map_2d(&a.maps.w1[f], phi_k[f].W1, DV, DV, DV)) return false;
+        a.ptrs.b1[f] = static_cast<const __nv_bfloat16*>(phi_k[f].b1);
+        a.ptrs.W2[f] = static_cast<const __nv_bfloat16*>(phi_k[f].W2);
+        a.ptrs.b2[f] = static_cast<const __nv_bfloat16*>(phi_k[f].b2);
+    }
+    for (int f = MT<F>::kMaps; f < 3; ++f) a.maps.w1[f] = a.maps.w1[0];
+    return true;
+}
+
 template <int DV, int F>
 inline hla_status launch_phik_state(const Dims& D, int BH, const hla_mlp* phi_k, const void* K, const void* V, char* ws, const hla_ws_layout& L,
                                     size_t off_part, int smax, int sm_count, LaunchRec& rec) {
-    CUtensorMap mapK, mapV;
-    PhiMaps mk;
-    PhiPtrs pk{};
-    if (!make_map_bhnd(&mapK, K, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapV, V, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
-    for (int f = 0; f < MT<F>::kMaps; ++f) {
-        if (!make_map_2d(&mk.w1[f], phi_k[f].W1, DV, DV, DV)) return HLA_ERR_CUDA;
-        pk.b1[f] = static_cast<const __nv_bfloat16*>(phi_k[f].b1);
-        pk.W2[f] = static_cast<const __nv_bfloat16*>(phi_k[f].W2);
-        pk.b2[f] = static_cast<const __nv_bfloat16*>(phi_k[f].b2);
-    }
-    for (int f = MT<F>::kMaps; f < 3; ++f) mk.w1[f] = mk.w1[0];
-    if (!set_smem(tc_phik_state_kernel<DV, F>, FkCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
+    PhikArgs a;
+    if (!phik_args<DV, F>(a, D, BH, phi_k, K, V) || !set_smem(tc_phik_state_kernel<DV, F>, FkCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
     const int grid = fused_key_grid(BH, D.N, sm_count);
     rec.begin("tc_phik_state");
-    launch_pdl(tc_phik_state_kernel<DV, F>, grid, dim3(kFkThreads), FkCfg<DV, F>::kSmem, rec.st, mapK, mk, mapV, pk, reinterpret_cast<float*>(ws + L.kf),
-                  reinterpret_cast<float*>(ws + off_part), D.N, BH, D.ld, smax, reinterpret_cast<int*>(ws + L.status));
+    launch_pdl(tc_phik_state_kernel<DV, F>, grid, dim3(kFkThreads), FkCfg<DV, F>::kSmem, rec.st, a.K, a.maps, a.V, a.ptrs, reinterpret_cast<float*>(ws + L.kf),
+                  reinterpret_cast<float*>(ws + off_part), D.N, BH, smax, reinterpret_cast<int*>(ws + L.status));
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
