@@ -388,9 +388,10 @@ template <int F> __device__ __forceinline__ void key_folded_grad_t(const float (
 // State build
 // =======================================================================================
 constexpr int kSbThreads = 320;            // warp 0: TMA, warp 1: MMA, warps 2..9: two generator groups of 128 threads
-template <int F> struct SbCfg {
-    static constexpr int kStages = F == 3 ? 4 : 3;
-    static constexpr int kStageBytes = 2 * kBlk + MT<F>::kBlocks * kBlk;   // V (two 64-column blocks) + folded key tile
+template <int F, bool GRAD = false> struct SbCfg {
+    static constexpr int kStages = GRAD ? 2 : (F == 3 ? 4 : 3);
+    static constexpr int kOffO = (2 + MT<F>::kBlocks) * kBlk;              // GRAD: the O tile, behind V (two 64-column blocks) and the folded key tile
+    static constexpr int kStageBytes = kOffO + (GRAD ? 2 * kBlk : 0);
     static constexpr int kOffZ = kStages * kStageBytes;                    // zred [8 warps][kPad] floats
     static constexpr int kOffBars = kOffZ + 8 * MT<F>::kPad * 4;
     static constexpr int kSmem = 1024 + kOffBars + 256;
@@ -400,14 +401,15 @@ template <int F> struct SbCfg {
 // GRAD = false: the state of Theorem 4.2, rows = folded key features of `kf`, values = V.
 // GRAD = true (3 factors only): the gradient of that state when every token sees only the tokens up to itself,
 // [dCsym | dzsym] = sum_i r_i mono_i (x) [dO_i | -delta_i]: `kf` points to the query features, the value map to dO,
-// r_i = 1 / (eta_i + eps) and delta_i = dO_i . o_i come from `eta` and `delta`.
+// r_i = 1 / (eta_i + eps) from `eta`.  delta_i = dO_i . o_i is formed here, from the dO tile that the product reads anyway and the O tile
+// (mapO), and left in `delta` for the sweeps that follow: as a kernel of its own it read dO once more (24 heads x 32760 tokens: 72 us,
+// bound by those reads, of a causal step of 1.12 ms; this pass takes as long as that kernel did, and the 45 us it took without O are saved).
 template <int DV, int F, bool GRAD = false>
-__global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __grid_constant__ CUtensorMap mapV, const float* __restrict__ kf,
-                                                                       float* __restrict__ part, int N, int S, int ld, int* status,
-                                                                       const float* __restrict__ eta = nullptr, const float* __restrict__ delta = nullptr,
-                                                                       float eps = 0.f, int clear = 0, bool beside = false) {
+__global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
+                                                                       const float* __restrict__ kf, float* __restrict__ part, int N, int S, int ld, int* status,
+                                                                       const float* __restrict__ eta, float* __restrict__ delta, float eps, int clear) {
     using M = MT<F>;
-    using Cfg = SbCfg<F>;
+    using Cfg = SbCfg<F, GRAD>;
     constexpr int kStages = Cfg::kStages, kStageBytes = Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -428,9 +430,8 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     float* out = part + ((size_t)bh * S + s) * M::kN * ld;
 
     if (ntiles == 0) {   // an empty split contributes zeros (never split 0)
-        grid_begin(beside);
+        grid_begin(false);
         for (int i = tid; i < M::kN * ld; i += kSbThreads) out[i] = 0.f;
-        grid_end(beside);
         return;
     }
     if (DV == 64) {      // rows 64..127 of the MMA's M dimension read a second V block: keep it zero
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_begin(beside);
+    grid_begin(false);
     if (clear && s == 0 && bh == 0 && tid < 16) status[tid] = 0;      // first kernel of a forward: a new record of device-side time-outs
     bool ok = true;
 
@@ -468,8 +469,11 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
                 const int st = it % kStages, u = it / kStages;
                 if (!mbar_wait(&empty[st], (u & 1) ^ 1)) { report_timeout(status, 101); break; }
                 uint8_t* vs = smem + st * kStageBytes;
-                mbar_arrive_expect_tx(&full_v[st], DV * kTileTokens * 2);
-                for (int b = 0; b < DV / 64; ++b) tma_load_3d(vs + b * kBlk, &mapV, &full_v[st], b * 64, (tile0 + it) * kTileTokens, bh);
+                mbar_arrive_expect_tx(&full_v[st], (GRAD ? 2 : 1) * DV * kTileTokens * 2);
+                for (int b = 0; b < DV / 64; ++b) {
+                    tma_load_3d(vs + b * kBlk, &mapV, &full_v[st], b * 64, (tile0 + it) * kTileTokens, bh);
+                    if (GRAD) tma_load_3d(vs + Cfg::kOffO + b * kBlk, &mapO, &full_v[st], b * 64, (tile0 + it) * kTileTokens, bh);
+                }
             }
         }
     } else if (warp == 1) {
@@ -496,13 +500,12 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
         for (int i = 0; i < M::kN; ++i) zacc[i] = 0.f;
         // The key features of the group's next tile are loaded while the current one is processed (row index clamped:
         // the loads are unconditional, out-of-range rows are zeroed when used).
-        float k[M::kKf], kn[M::kKf], en = 0.f, dn = 0.f;
+        float k[M::kKf], kn[M::kKf], en = 0.f;
         auto prefetch = [&](int it) {
             const int tok = min((tile0 + it) * kTileTokens + row, N - 1);
             if constexpr (GRAD) {
                 load_feat<M::kDphi>(kn, kf + ((size_t)bh * N + tok) * M::kDphi);
                 en = __ldg(eta + (size_t)bh * N + tok);
-                dn = __ldg(delta + (size_t)bh * N + tok);
             } else {
 #pragma unroll
                 for (int f = 0; f < F; ++f) load_feat<M::kDphi>(kn + M::kDphi * f, kf + (((size_t)bh * F + f) * N + tok) * M::kDphi);
@@ -514,7 +517,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
             const int tok = (tile0 + it) * kTileTokens + row;
 #pragma unroll
             for (int i = 0; i < (GRAD ? M::kDphi : M::kKf); ++i) k[i] = tok < N ? kn[i] : 0.f;
-            const float rr = GRAD && tok < N ? 1.f / (en + eps) : 0.f, nd = -dn;
+            const float rr = GRAD && tok < N ? 1.f / (en + eps) : 0.f;
             if (it + 2 < ntiles) prefetch(it + 2);
             float ts[M::kN];
             if constexpr (GRAD) {
@@ -523,10 +526,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
                 for (int i = 0; i < M::kDphi; ++i) q[i] = k[i];
                 query_monomials_t<F>(q, ts);
 #pragma unroll
-                for (int i = 0; i < M::kN; ++i) {
-                    ts[i] *= rr;
-                    zacc[i] = fmaf(nd, ts[i], zacc[i]);
-                }
+                for (int i = 0; i < M::kN; ++i) ts[i] *= rr;
             } else {
                 key_folded_t<F>(k, ts);
 #pragma unroll
@@ -535,6 +535,26 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
             if (ok && !mbar_wait(&empty[st], (u & 1) ^ 1)) { ok = false; report_timeout(status, 103); }
             if (ok) {
                 store_mono_row_t<F>(smem_u32(smem + st * kStageBytes + 2 * kBlk), row, ts, 1.f);
+                if constexpr (GRAD) {
+                    if (!mbar_wait(&full_v[st], u & 1)) { ok = false; report_timeout(status, 105); continue; }
+                    const uint8_t *dO = smem + st * kStageBytes, *o = dO + Cfg::kOffO;
+                    float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+                    for (int c = 0; c < DV / 8; ++c) {
+                        const uint32_t at = (c >> 3) * kBlk + sw128_off(row, c & 7);
+                        const uint4 x = *reinterpret_cast<const uint4*>(dO + at), y = *reinterpret_cast<const uint4*>(o + at);
+                        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            d[e] = fmaf(__uint_as_float(xs[e] << 16), __uint_as_float(ys[e] << 16), d[e]);
+                            d[e] = fmaf(__uint_as_float(xs[e] & 0xffff0000u), __uint_as_float(ys[e] & 0xffff0000u), d[e]);
+                        }
+                    }
+                    const float dl = (d[0] + d[1]) + (d[2] + d[3]);
+                    if (tok < N) delta[(size_t)bh * N + tok] = dl;
+#pragma unroll
+                    for (int i = 0; i < M::kN; ++i) zacc[i] = fmaf(-dl, ts[i], zacc[i]);
+                }
                 fence_proxy_async();
                 mbar_arrive(&full_t[st]);
             }
@@ -576,7 +596,6 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, Cfg::kTmemCols);
-    grid_end(beside);
 }
 
 // =======================================================================================
@@ -1441,7 +1460,7 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
     if (!set_smem(tc_state_build_kernel<DV, F>, SbCfg<F>::kSmem) || !set_smem(tc_readout_kernel<DV, F>, RoCfg<DV, F>::kSmem)) return HLA_ERR_CUDA;
     cudaStream_t st = rec.st;
     rec.begin("tc_state_build");
-    launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (const float*)nullptr, 0.f, 1, false);
+    launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (float*)nullptr, 0.f, 1);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_reduce_emit");
     launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, state, b3, bq, D.S, 0, 0, false);

@@ -757,8 +757,8 @@ inline hla_status launch_causal_state_build(const Dims& D, int BH, const float* 
     if (!make_map_bhnd(&mapV, V, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
     if (!set_smem(tc_state_build_kernel<DV, 3>, SbCfg<3>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_state_build");
-    launch_pdl(tc_state_build_kernel<DV, 3>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapV, kf, reinterpret_cast<float*>(ws + off_part), D.N, D.S,
-               D.ld, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, (const float*)nullptr, 0.f, 1, false);
+    launch_pdl(tc_state_build_kernel<DV, 3>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapV, mapV, kf, reinterpret_cast<float*>(ws + off_part), D.N,
+               D.S, D.ld, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, (float*)nullptr, 0.f, 1);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
@@ -771,69 +771,38 @@ inline hla_status causal_forward(const Dims& D, int BH, const float* qf, const f
     return causal_sweep(D, BH, qf, kf, V, O, ws, L, off_part, D.S, 0, carry, nullptr, rec);
 }
 
-// delta_i = dO_i . o_i for every token row (bf16 rows of d values, fp32 sum): d / 8 lanes per row, 16 bytes per lane.
+// Backward of the causal operator at the feature level, value side.  First the gradient state of every piece and delta_i = dO_i . o_i;
+// then, beside the kernel before it, the suffix scan of those states; then the sweep that gives dV.
 template <int DV>
-__global__ void __launch_bounds__(256) tc_delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO, float* __restrict__ delta,
-                                                       long long rows) {
-    constexpr int LPR = DV / 8;                 // lanes per row
-    grid_begin(false);
-    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
-    const long long row = t / LPR;
-    const int part = (int)(t % LPR);
-    float a = 0.f;
-    if (row < rows) {
-        const uint4 x = *reinterpret_cast<const uint4*>(O + row * DV + 8 * part);
-        const uint4 y = *reinterpret_cast<const uint4*>(dO + row * DV + 8 * part);
-        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            a = fmaf(__uint_as_float(xs[e] << 16), __uint_as_float(ys[e] << 16), a);
-            a = fmaf(__uint_as_float(xs[e] & 0xffff0000u), __uint_as_float(ys[e] & 0xffff0000u), a);
-        }
-    }
-#pragma unroll
-    for (int o = LPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (row < rows && part == 0) delta[row] = a;
-}
-
-template <int DV>
-inline hla_status launch_causal_delta(const Dims& D, int BH, const void* O, const void* dO, char* ws, size_t off_delta, LaunchRec& rec) {
-    const long long rows = (long long)BH * D.N;
-    rec.begin("tc_delta");
-    launch_pdl(tc_delta_kernel<DV>, dim3((unsigned)((rows * (DV / 8) + 255) / 256)), dim3(256), 0, rec.st, static_cast<const __nv_bfloat16*>(O),
-               static_cast<const __nv_bfloat16*>(dO), reinterpret_cast<float*>(ws + off_delta), rows);
+inline hla_status launch_causal_gradient_states(const Dims& D, int BH, const float* qf, const void* O, const void* dO, char* ws, const hla_ws_layout& L,
+                                                size_t off_gpart, size_t off_delta, LaunchRec& rec) {
+    CUtensorMap mapdO, mapO;
+    if (!make_map_bhnd(&mapdO, dO, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapO, O, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
+    if (!set_smem(tc_state_build_kernel<DV, 3, true>, SbCfg<3, true>::kSmem)) return HLA_ERR_CUDA;
+    rec.begin("tc_dstate_build");
+    launch_pdl(tc_state_build_kernel<DV, 3, true>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3, true>::kSmem, rec.st, mapdO, mapO, qf,
+               reinterpret_cast<float*>(ws + off_gpart), D.N, D.S, D.ld, reinterpret_cast<int*>(ws + L.status), reinterpret_cast<const float*>(ws + L.eta),
+               reinterpret_cast<float*>(ws + off_delta), D.eps, 0);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
-
-// Backward of the causal operator at the feature level, value side: the gradient state of every piece (beside the kernel before, which
-// must itself have waited for delta), its suffix scan, and the sweep that gives dV.  `between` (run_between: there is such a step) is
-// launched before the scan, which then runs beside it.
-template <int DV, typename Between>
+inline hla_status launch_causal_gradient_scan(const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_gpart, LaunchRec& rec) {
+    const int T = (D.N + kTileTokens - 1) / kTileTokens;
+    rec.begin("tc_scan_pieces");
+    launch_pdl(tc_scan_pieces_kernel<3, true>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, reinterpret_cast<float*>(ws + off_gpart),
+               reinterpret_cast<float*>(ws + L.dstate), D.S, D.ld, 0, T, 0, true);
+    return rec.end() ? HLA_OK : HLA_ERR_CUDA;
+}
+template <int DV>
 inline hla_status launch_causal_backward_values(const Dims& D, int BH, const float* qf, const float* kf, const void* dO, void* dV, char* ws,
-                                                const hla_ws_layout& L, size_t off_gpart, size_t off_delta, LaunchRec& rec, bool run_between, Between&& between) {
+                                                const hla_ws_layout& L, size_t off_gpart, size_t off_delta, LaunchRec& rec) {
     CUtensorMap mapdO, mapdV;
     if (!make_map_bhnd(&mapdO, dO, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapdV, dV, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
-    int* status = reinterpret_cast<int*>(ws + L.status);
-    float* part = reinterpret_cast<float*>(ws + off_gpart);
-    float* dstate = reinterpret_cast<float*>(ws + L.dstate);
-    float* eta = reinterpret_cast<float*>(ws + L.eta);
-    float* delta = reinterpret_cast<float*>(ws + off_delta);
-    if (!set_smem(tc_state_build_kernel<DV, 3, true>, SbCfg<3>::kSmem) || !set_smem(tc_causal_forward_kernel<DV, 1>, CaCfg<DV>::kSmem)) return HLA_ERR_CUDA;
-    const int T = (D.N + kTileTokens - 1) / kTileTokens;
-    rec.begin("tc_dstate_build");
-    launch_pdl(tc_state_build_kernel<DV, 3, true>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<3>::kSmem, rec.st, mapdO, qf, part, D.N, D.S, D.ld, status,
-               (const float*)eta, (const float*)delta, D.eps, 0, true);
-    if (!rec.end()) return HLA_ERR_CUDA;
-    if (run_between) {
-        const hla_status e = between();
-        if (e != HLA_OK) return e;
-    }
-    rec.begin("tc_scan_pieces");
-    launch_pdl(tc_scan_pieces_kernel<3, true>, dim3((kMono * D.ld + 255) / 256, BH), dim3(256), 0, rec.st, part, dstate, D.S, D.ld, 0, T, 0, run_between);
-    if (!rec.end()) return HLA_ERR_CUDA;
+    if (!set_smem(tc_causal_forward_kernel<DV, 1>, CaCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dv");
-    launch_pdl(tc_causal_forward_kernel<DV, 1>, dim3(D.S, BH), dim3(kCaThreads), CaCfg<DV>::kSmem, rec.st, mapdO, mapdV, qf, kf, (const float*)part,
-               (float*)nullptr, (const float*)eta, (const float*)delta, D.N, BH, D.S, 0, D.eps, status, (const float*)nullptr, false, (float*)nullptr);
+    launch_pdl(tc_causal_forward_kernel<DV, 1>, dim3(D.S, BH), dim3(kCaThreads), CaCfg<DV>::kSmem, rec.st, mapdO, mapdV, qf, kf,
+               reinterpret_cast<const float*>(ws + off_gpart), (float*)nullptr, reinterpret_cast<const float*>(ws + L.eta),
+               reinterpret_cast<const float*>(ws + off_delta), D.N, BH, D.S, 0, D.eps, reinterpret_cast<int*>(ws + L.status), (const float*)nullptr, false,
+               (float*)nullptr);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 

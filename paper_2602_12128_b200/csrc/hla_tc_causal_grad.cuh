@@ -547,15 +547,17 @@ inline hla_status launch_causal_backward_features(const Dims& D, int BH, const f
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
-// dO . o, then dq on the forward states, beside it the gradient states (in a region of their own, so that the forward's stay), their scan
-// (beside `between`, the next step of the query side), dV and beside it dk.
+// Gradient states (in a region of their own, so that the forward's stay) and dO . o, then dq on the forward states, beside it the scan of the
+// gradient states, `between` (the next step of the query side, if any), dV and beside it dk.
 template <int DV, typename Between>
 inline hla_status launch_causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf,
                                          float* dkf, void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta,
                                          LaunchRec& rec, bool run_between, Between&& between) {
-    hla_status s = launch_causal_delta<DV>(D, BH, O, dO, ws, off_delta, rec);
+    hla_status s = launch_causal_gradient_states<DV>(D, BH, qf, O, dO, ws, L, off_gpart, off_delta, rec);
     if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, false, rec);
-    if (s == HLA_OK) s = launch_causal_backward_values<DV>(D, BH, qf, kf, dO, dV, ws, L, off_gpart, off_delta, rec, run_between, between);
+    if (s == HLA_OK) s = launch_causal_gradient_scan(D, BH, ws, L, off_gpart, rec);
+    if (s == HLA_OK && run_between) s = between();
+    if (s == HLA_OK) s = launch_causal_backward_values<DV>(D, BH, qf, kf, dO, dV, ws, L, off_gpart, off_delta, rec);
     if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, true, rec);
     return s;
 }
