@@ -322,7 +322,7 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
                 if (score > best + 1e-9) { best = score; S = cand; }
             }
         } else {
-            S = simt::tiled(D) ? simt::tiled_splits(x->BH, c.N, P, x->sm_count) : (2 * x->sm_count + x->BH - 1) / x->BH;
+            S = simt::tiled(D) ? simt::tiled_splits(x->BH, c.N, P, c.d, x->sm_count) : (2 * x->sm_count + x->BH - 1) / x->BH;
         }
     }
     if (S > tiles) S = tiles;

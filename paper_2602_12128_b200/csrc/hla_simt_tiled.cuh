@@ -25,7 +25,9 @@ namespace simt {
 // The per-token kernels work on tiles of TM = 8 R tokens, a thread holds the tokens tg + 8 i, i < R: R = 8 where that gives every SM a
 // block, else R = 2 (512 rows: 32 blocks instead of 8, and a quarter of the serial work in each).
 constexpr int kSbTok = 32;        // tokens per step of the state build
-constexpr int kSbRows = 64;       // state rows per block of the state build
+// State rows per block of the state build, in groups of 8 (a thread's rows): 72 of the 216 or 144 rows of the forward, all 56 or 78 of the
+// gradient state.  (Blocks of 64 rows did a seventh of their work on padding.)
+template <int F, bool BWD> constexpr int kSbGroups = !BWD ? 9 : (F == 3 ? 7 : 10);
 
 template <int F> struct Geo {
     using M = tc::MT<F>;
@@ -151,85 +153,133 @@ __device__ __forceinline__ void stage_values(float* Xs, int ld, float* xz, const
 
 // ---- state build -------------------------------------------------------------------------------
 // Forward: rows = the P products T_k[p], X = V.  Backward: rows = the M monomials of q (the gradient is the same for every permutation
-// of a row's indices), X = r dO.  Block = (split, 64 rows, head), thread = 8 rows x 4 columns; the T tile of a step is formed by threads
-// that own one row each, so that a row's digits are decoded once per block.
+// of a row's indices), X = r dO, xz = -r (dO . O).  Block = (split, 8 RG rows, head), thread = 8 rows x 4 columns; the T tile of a step and
+// its part of z are formed by threads that own one row each (CG / 8 threads per row, alternate tokens), so that a row's digits are decoded
+// once per block.  The next step's inputs are on their way (in registers) while a step is computed: with the loads between two barriers of
+// the same step, 18 % of the FMA rate; at B*H = 12, N = 3000, d = 64 that kernel took 62 us, of which 22 were a second wave of 24 blocks.
 template <typename T, int F, int CG, bool BWD>
-__global__ void __launch_bounds__(CG * 8) tiled_state_build_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X, const T* __restrict__ O,
-                                                                   const float* __restrict__ eta, float* __restrict__ part, int S, bool beside, int* __restrict__ clear) {
+__global__ void __launch_bounds__(CG * kSbGroups<F, BWD>, CG == 32 ? 2 : 64 / CG) tiled_state_build_kernel(Dims D, const float* __restrict__ feat, const T* __restrict__ X,
+                                                                                                const T* __restrict__ O, const float* __restrict__ eta,
+                                                                                                float* __restrict__ part, int S, bool beside, int* __restrict__ clear) {
     using G = Geo<F>;
-    constexpr int NT = CG * 8, DP = G::kDphi, LD = 4 * CG + 4, LT = kSbRows + 4, KF = BWD ? DP : G::kKf, ROWS = BWD ? G::kN : G::kP;
+    constexpr int RG = kSbGroups<F, BWD>, NR = 8 * RG, NT = CG * RG, DP = G::kDphi, LD = 4 * CG + 4, LT = NR + 4, NF = BWD ? 1 : F, ROWS = BWD ? G::kN : G::kP;
+    constexpr int PER = CG / 8;                            // threads per row of T
+    constexpr int XI = (kSbTok + RG - 1) / RG;             // rows of X per thread and step
+    constexpr int FQ = NF * kSbTok * DP / 2, FI = (FQ + NT - 1) / NT;      // float2 of features per step, and per thread
     __shared__ __align__(16) float Ts[kSbTok * LT];
     __shared__ __align__(16) float Xs[kSbTok * LD];
-    __shared__ float fs[kSbTok * KF];
+    __shared__ __align__(16) float fs[NF * kSbTok * DP];     // [map][token][feature]: each map's part is one run of the input
     __shared__ float xz[kSbTok];
-    const int s = blockIdx.x, row0 = blockIdx.y * kSbRows, bh = blockIdx.z;
+    __shared__ float zs[PER * NR];
+    const int s = blockIdx.x, row0 = blockIdx.y * NR, bh = blockIdx.z;
     const int cg = threadIdx.x % CG, rg = threadIdx.x / CG;      // columns 4 cg .., rows 8 rg ..
-    const int per = ((D.N + S - 1) / S + kSbTok - 1) / kSbTok * kSbTok;
-    const int t0 = s * per, t1 = min(D.N, t0 + per);
-    // the row this thread forms: feature indices of its factors
-    const int row = row0 + (threadIdx.x & 63);
+    const int steps = (D.N + kSbTok - 1) / kSbTok;
+    const int t0 = (int)((long long)steps * s / S) * kSbTok, t1 = min(D.N, (int)((long long)steps * (s + 1) / S) * kSbTok);
+    // the row this thread forms: offsets of its factors in fs
+    const int trow = threadIdx.x % NR, row = row0 + trow, tpar = threadIdx.x / NR;
     int dig[F];
     {
-        int rem = BWD ? kRowTable<F>.v[row < ROWS ? row : 0] : row;
+        int rem = row < ROWS ? (BWD ? kRowTable<F>.v[row < ROWS ? row : 0] : row) : 0;
 #pragma unroll
         for (int f = F - 1; f >= 0; --f) {
-            dig[f] = rem % DP + (BWD ? 0 : f * DP);
+            dig[f] = rem % DP + (BWD ? 0 : f * (kSbTok * DP));
             rem /= DP;
         }
-        if (row >= ROWS)
-            for (int f = 0; f < F; ++f) dig[f] = 0;
     }
+    const float live = row < ROWS ? 1.f : 0.f;
     tc::grid_begin(beside);
     if (clear && s == 0 && blockIdx.y == 0 && bh == 0 && threadIdx.x < 16) clear[threadIdx.x] = 0;
-    float acc[8][4];
+    float2 acc[8][2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
     float zacc = 0.f;
     if (4 * cg >= D.d) {      // columns past the head width: never staged, kept finite
-        for (int t = rg; t < kSbTok; t += 8) *reinterpret_cast<float4*>(Xs + t * LD + 4 * cg) = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t = rg; t < kSbTok; t += RG) *reinterpret_cast<float4*>(Xs + t * LD + 4 * cg) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    float4 xn[XI], on[BWD ? XI : 1];
+    float en[BWD ? XI : 1];
+    float2 fn[FI];
+    auto load_step = [&](int tok0) {
+#pragma unroll
+        for (int i = 0; i < XI; ++i) {
+            const int t = rg + RG * i, tok = tok0 + t;
+            const bool in = t < kSbTok && tok < t1;
+            const size_t at = (size_t)bh * D.N + (in ? tok : t0);
+            xn[i] = in && 4 * cg < D.d ? load4(X + at * D.d + 4 * cg) : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (BWD) {
+                on[i] = in && 4 * cg < D.d ? load4(O + at * D.d + 4 * cg) : make_float4(0.f, 0.f, 0.f, 0.f);
+                en[i] = in ? 1.f / (__ldg(eta + at) + D.eps) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < FI; ++i) {
+            const int e = threadIdx.x + NT * i, f = e / (kSbTok * DP / 2), j = e - f * (kSbTok * DP / 2);      // token j / (DP / 2)
+            const bool in = e < FQ && 2 * j < (t1 - tok0) * DP;
+            const size_t at = BWD ? ((size_t)bh * D.N + tok0) * DP : (((size_t)bh * F + (in ? f : 0)) * D.N + tok0) * DP;
+            fn[i] = in ? __ldg(reinterpret_cast<const float2*>(feat + at) + j) : make_float2(0.f, 0.f);
+        }
+    };
+    if (t0 < t1) load_step(t0);
     for (int tok0 = t0; tok0 < t1; tok0 += kSbTok) {
         __syncthreads();
-        for (int i = threadIdx.x; i < kSbTok * KF; i += NT) {
-            const int f = i / (kSbTok * DP), j = i - f * (kSbTok * DP), t = j / DP, k = j - t * DP;      // (BWD: f = 0)
-            const size_t at = BWD ? ((size_t)bh * D.N + tok0 + t) * DP + k : (((size_t)bh * F + f) * D.N + tok0 + t) * DP + k;
-            fs[t * KF + f * DP + k] = tok0 + t < t1 ? __ldg(feat + at) : 0.f;
+#pragma unroll
+        for (int i = 0; i < XI; ++i) {
+            const int t = rg + RG * i;
+            float4 x = xn[i];
+            if (BWD) {
+                const float r = en[i];
+                float v = fmaf(x.x, on[i].x, fmaf(x.y, on[i].y, fmaf(x.z, on[i].z, x.w * on[i].w)));
+                const unsigned lanes = CG == 32 ? 0xffffffffu : ((1u << (CG & 31)) - 1u) << (threadIdx.x & 31 & ~(CG - 1));      // the row's CG lanes
+#pragma unroll
+                for (int o = CG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(lanes, v, o);
+                if (cg == 0 && t < kSbTok) xz[t] = -r * v;
+                x = make_float4(r * x.x, r * x.y, r * x.z, r * x.w);
+            } else if (cg == 0 && t < kSbTok) {
+                xz[t] = tok0 + t < t1 ? 1.f : 0.f;
+            }
+            if (t < kSbTok && 4 * cg < D.d) *reinterpret_cast<float4*>(Xs + t * LD + 4 * cg) = x;
         }
-        stage_values<CG, T, BWD>(Xs, LD, xz, X, O, eta, D, bh, tok0, kSbTok, t1);
+#pragma unroll
+        for (int i = 0; i < FI; ++i)
+            if (threadIdx.x + NT * i < FQ) reinterpret_cast<float2*>(fs)[threadIdx.x + NT * i] = fn[i];
         __syncthreads();
-        for (int t = threadIdx.x >> 6; t < kSbTok; t += NT / 64) {
-            const float* f = fs + t * KF;
-            float v = f[dig[0]] * f[dig[1]];
+        if (tok0 + kSbTok < t1) load_step(tok0 + kSbTok);
+#pragma unroll 8
+        for (int t = tpar; t < kSbTok; t += PER) {
+            const float* f = fs + t * DP;
+            float v = live * f[dig[0]] * f[dig[1]];
             if (F == 3) v *= f[dig[F - 1]];
-            Ts[t * LT + (threadIdx.x & 63)] = row < ROWS ? v : 0.f;
+            Ts[t * LT + trow] = v;
+            zacc = fmaf(v, xz[t], zacc);
         }
         __syncthreads();
 #pragma unroll 4
         for (int t = 0; t < kSbTok; ++t) {
             const float4 a0 = ld4(Ts + t * LT + 8 * rg), a1 = ld4(Ts + t * LT + 8 * rg + 4), x = ld4(Xs + t * LD + 4 * cg);
             const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                acc[i][0] = fmaf(av[i], x.x, acc[i][0]);
-                acc[i][1] = fmaf(av[i], x.y, acc[i][1]);
-                acc[i][2] = fmaf(av[i], x.z, acc[i][2]);
-                acc[i][3] = fmaf(av[i], x.w, acc[i][3]);
+                const float2 a = make_float2(av[i], av[i]);
+                acc[i][0] = __ffma2_rn(a, x0, acc[i][0]);
+                acc[i][1] = __ffma2_rn(a, x1, acc[i][1]);
             }
-        }
-        if (threadIdx.x < kSbRows) {
-#pragma unroll 4
-            for (int t = 0; t < kSbTok; ++t) zacc = fmaf(Ts[t * LT + threadIdx.x], xz[t], zacc);
         }
     }
     float* out = part + ((size_t)bh * S + s) * ROWS * D.ld;
     if (4 * cg < D.d) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            if (row0 + 8 * rg + i < ROWS) store4(out + (size_t)(row0 + 8 * rg + i) * D.ld + 4 * cg, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+            if (row0 + 8 * rg + i < ROWS) store4(out + (size_t)(row0 + 8 * rg + i) * D.ld + 4 * cg, make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y));
     }
-    if (threadIdx.x < kSbRows && row < ROWS) store4(out + (size_t)row * D.ld + D.d, make_float4(zacc, 0.f, 0.f, 0.f));
+    zs[threadIdx.x] = zacc;      // [PER][NR]
+    __syncthreads();
+    if (threadIdx.x < NR && row < ROWS) {
+        float z = zs[threadIdx.x];
+#pragma unroll
+        for (int k = 1; k < PER; ++k) z += zs[k * NR + threadIdx.x];
+        store4(out + (size_t)row * D.ld + D.d, make_float4(z, 0.f, 0.f, 0.f));
+    }
     tc::grid_end(beside);
 }
 
@@ -586,16 +636,21 @@ __global__ void __launch_bounds__(CG * 8, CG == 32 ? 1 : 64 / CG) tiled_phi_back
 
 // ---- host --------------------------------------------------------------------------------------
 inline bool tiled(const Dims& D) { return (D.F == 3 && D.dphi == 6) || (D.F == 2 && D.dphi == 12); }
-// Token splits of a state build: six blocks per SM over all row blocks and heads (a step is loads, two barriers and 1024 FMAs per thread,
-// so it takes that many blocks side by side to cover them; three per SM: 85 us a build against 49 at B*H = 12, N = 3000, d = 64).
-inline int tiled_splits(int BH, int N, int P, int sm_count) {
-    const int blocks = BH * ((P + kSbRows - 1) / kSbRows), S = (6 * sm_count + blocks - 1) / blocks, most = (N + kSbTok - 1) / kSbTok;
-    return S < most ? S : most;
+// Token splits of a state build: as many blocks as the SMs hold at once (at least 64 / CG of CG x 9 threads; a wave that is nearly empty
+// costs as much as a full one), but at least two steps of 32 tokens per block where that leaves every SM one.
+inline int tiled_split_count(int blocks_per_split, int N, int d, int sm_count) {
+    const int held = (d <= 32 ? 8 : (d <= 64 ? 4 : 2)) * sm_count, steps = (N + kSbTok - 1) / kSbTok;
+    int S = held / blocks_per_split;
+    if (S > steps) S = steps;
+    if (S < 1) S = 1;
+    const int per = (steps + S - 1) / S;      // the same longest run of steps with the fewest splits
+    return (steps + per - 1) / per;
 }
-// The gradient state has M instead of P rows: as many more splits for the same bytes of partials.
-template <int F> inline int tiled_gradient_splits(const Dims& D) {
-    const int S = (int)((long long)D.S * Geo<F>::kP / Geo<F>::kN), most = (D.N + kSbTok - 1) / kSbTok;
-    return S < most ? S : (most > D.S ? most : D.S);
+inline int tiled_splits(int BH, int N, int P, int d, int sm_count) { return tiled_split_count(BH * (P / 72), N, d, sm_count); }
+// The gradient state has M instead of P rows: more splits, within the same bytes of partials.
+template <int F> inline int tiled_gradient_splits(const Dims& D, int BH, int sm_count) {
+    const int room = (int)((long long)D.S * Geo<F>::kP / Geo<F>::kN), S = tiled_split_count(BH, D.N, D.d, sm_count);
+    return S < room ? S : room;
 }
 template <int F, int CG, int R> struct TiledSmem {
     using G = Geo<F>;
@@ -649,7 +704,7 @@ template <typename T, int F, int CG, int R> struct Tiled {
     static const T* in(const void* p) { return static_cast<const T*>(p); }
     static T* out(void* p) { return static_cast<T*>(p); }
 
-    static bool forward(const TiledArgs& a, LaunchRec& rec) {
+    static bool forward(const TiledArgs& a, int, LaunchRec& rec) {
         const Dims& D = a.D;
         const size_t rows = (size_t)a.BH * D.N;
         const unsigned rb = (unsigned)((rows + TM - 1) / TM), tb = (unsigned)((D.N + TM - 1) / TM);
@@ -662,21 +717,21 @@ template <typename T, int F, int CG, int R> struct Tiled {
                         rows, D.N, D.d, true))
                 return false;
         }
-        return launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, false>, dim3(D.S, (G::kP + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.kf, in(a.V),
+        return launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, false>, dim3(D.S, G::kP / 72, a.BH), CG * kSbGroups<F, false>, 0, D, a.kf, in(a.V),
                       in(nullptr), a.eta, a.part, D.S, false, a.clear) &&
                launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, false>, reduce_grid(a, G::kP), 256, 0, a.state, a.part, a.BH, D.S, D.ld) &&
                launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, R, true>, dim3(tb, a.BH), NT, S::readout, D, a.qf, a.state, out(a.Oout), a.eta, false);
     }
-    static bool backward(const TiledArgs& a, LaunchRec& rec) {
+    static bool backward(const TiledArgs& a, int sm_count, LaunchRec& rec) {
         const Dims& D = a.D;
         const size_t rows = (size_t)a.BH * D.N;
         const unsigned rb = (unsigned)((rows + TM - 1) / TM), tb = (unsigned)((D.N + TM - 1) / TM);
-        const int Sg = tiled_gradient_splits<F>(D);
+        const int Sg = tiled_gradient_splits<F>(D, a.BH, sm_count);
         // dq, and beside it the partials of dC, dz;  their sum;  dk^f, and beside it dV;  the feature networks of Q (dq is long complete) beside
         // that, then those of K
         if (!(launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state, a.dqf,
                      false) &&
-              launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(Sg, (G::kN + kSbRows - 1) / kSbRows, a.BH), NT, 0, D, a.qf, in(a.dO), in(a.O),
+              launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(Sg, 1, a.BH), CG * kSbGroups<F, true>, 0, D, a.qf, in(a.dO), in(a.O),
                      a.eta, a.part, Sg, true, nullptr) &&
               launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, Sg, D.ld) &&
               launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::grad, D, a.kf, in(a.V), in(nullptr), a.eta, a.dstate,
@@ -692,15 +747,15 @@ template <typename T, int F, int CG, int R> struct Tiled {
 };
 
 // The column groups of a block: the smallest of 8, 16, 32 (x 4 columns) that covers the head width.
-template <typename T, int F, int R> inline bool run_tiled_r(const TiledArgs& a, bool fwd, LaunchRec& rec) {
-    if (a.D.d <= 32) return fwd ? Tiled<T, F, 8, R>::forward(a, rec) : Tiled<T, F, 8, R>::backward(a, rec);
-    if (a.D.d <= 64) return fwd ? Tiled<T, F, 16, R>::forward(a, rec) : Tiled<T, F, 16, R>::backward(a, rec);
-    return fwd ? Tiled<T, F, 32, R>::forward(a, rec) : Tiled<T, F, 32, R>::backward(a, rec);
+template <typename T, int F, int R> inline bool run_tiled_r(const TiledArgs& a, bool fwd, int sm_count, LaunchRec& rec) {
+    if (a.D.d <= 32) return fwd ? Tiled<T, F, 8, R>::forward(a, sm_count, rec) : Tiled<T, F, 8, R>::backward(a, sm_count, rec);
+    if (a.D.d <= 64) return fwd ? Tiled<T, F, 16, R>::forward(a, sm_count, rec) : Tiled<T, F, 16, R>::backward(a, sm_count, rec);
+    return fwd ? Tiled<T, F, 32, R>::forward(a, sm_count, rec) : Tiled<T, F, 32, R>::backward(a, sm_count, rec);
 }
 template <typename T> inline bool run_tiled(const TiledArgs& a, bool fwd, int sm_count, LaunchRec& rec) {
     const bool few = (long long)a.BH * ((a.D.N + 63) / 64) < sm_count;
-    if (a.D.F == 3) return few ? run_tiled_r<T, 3, 2>(a, fwd, rec) : run_tiled_r<T, 3, 8>(a, fwd, rec);
-    return few ? run_tiled_r<T, 2, 2>(a, fwd, rec) : run_tiled_r<T, 2, 8>(a, fwd, rec);
+    if (a.D.F == 3) return few ? run_tiled_r<T, 3, 2>(a, fwd, sm_count, rec) : run_tiled_r<T, 3, 8>(a, fwd, sm_count, rec);
+    return few ? run_tiled_r<T, 2, 2>(a, fwd, sm_count, rec) : run_tiled_r<T, 2, 8>(a, fwd, sm_count, rec);
 }
 
 }  // namespace simt
