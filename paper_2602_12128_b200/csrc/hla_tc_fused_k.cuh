@@ -347,9 +347,11 @@ __device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const Ph
         float z0[8], z1[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) z0[e] = z1[e] = 0.f;
-        auto add_chunk = [](float (&z)[8], uint32_t addr) {
-            uint32_t w[4];
+        // A tile is read into registers and released before the sums are formed: the feature warps wait for it to write the next one.
+        auto load_chunk = [](uint32_t (&w)[4], uint32_t addr) {
             asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr) : "memory");
+        };
+        auto add_chunk = [](float (&z)[8], const uint32_t (&w)[4]) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 z[2 * e] += __uint_as_float(w[e] << 16);
@@ -361,14 +363,21 @@ __device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const Ph
             if (ok && !mbar_wait(f_full, it & 1)) { ok = false; report_timeout(status, 805); }
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
+            uint32_t w[kTileTokens / 16][4], v[M::kBlocks == 2 ? kTileTokens / 32 : 1][4];
 #pragma unroll
-            for (int j = 0; j < kTileTokens / 16; ++j) add_chunk(z0, fa + sw128_off((lane >> 1) + 16 * j, 2 * zw + (lane & 1)));
+            for (int j = 0; j < kTileTokens / 16; ++j) load_chunk(w[j], fa + sw128_off((lane >> 1) + 16 * j, 2 * zw + (lane & 1)));
             if (second) {
 #pragma unroll
-                for (int j = 0; j < kTileTokens / 32; ++j) add_chunk(z1, fa + kBlk + sw128_off(lane + 32 * j, zw));
+                for (int j = 0; j < kTileTokens / 32; ++j) load_chunk(v[M::kBlocks == 2 ? j : 0], fa + kBlk + sw128_off(lane + 32 * j, zw));
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(f_empty);
+#pragma unroll
+            for (int j = 0; j < kTileTokens / 16; ++j) add_chunk(z0, w[j]);
+            if (second) {
+#pragma unroll
+                for (int j = 0; j < kTileTokens / 32; ++j) add_chunk(z1, v[M::kBlocks == 2 ? j : 0]);
+            }
             if (piece_ends(it)) {
                 const int bh = head_of(it);
                 const int piece = bid - owner_of_work((long long)bh * T, total, G);
