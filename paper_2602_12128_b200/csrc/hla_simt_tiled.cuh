@@ -295,11 +295,7 @@ __global__ void __launch_bounds__(256) tiled_reduce_kernel(float* __restrict__ o
         const int c = i % q, row = (i / q) % ROWS, bh = i / (q * ROWS);
         const float4* src = reinterpret_cast<const float4*>(part) + ((size_t)bh * S * ROWS + row) * q + c;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-        for (int s = 0; s < S; ++s) {
-            const float4 v = __ldg(src + (size_t)s * ROWS * q);
-            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
-        }
+        tc::add_partials<8>(a, reinterpret_cast<const float*>(src), (size_t)ROWS * ld, 0, 1, S);
         float4* o = reinterpret_cast<float4*>(out) + (size_t)bh * G::kP * q + c;
         if (!FOLDED) {
             o[(size_t)row * q] = a;

@@ -170,18 +170,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
-// The same without the attribute, for a kernel that reads caller-provided memory (the phi weights) before its wait and
-// may directly follow a kernel of the caller that wrote it: it starts only after everything before it has completed.
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_serial(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 // ---- small device helpers ----------------------------------------------------------------
 __device__ __forceinline__ void report_timeout(int* status, int where) {
     atomicExch(status + kStatusTimeout, 1);
@@ -611,6 +599,20 @@ __host__ __device__ inline int owner_of_work(long long w, long long total, int G
     return (int)(((w + 1) * G - 1) / total);
 }
 
+// a += the float4 at src + c stride for c = first, first + step, ... < count, in this order, K loads in flight.  (A load past the end repeats
+// the last one: as conditional loads they were issued one after the other.)
+template <int K> __device__ __forceinline__ void add_partials(float4& a, const float* __restrict__ src, size_t stride, int first, int step, int count) {
+    for (int c0 = first; c0 < count; c0 += K * step) {
+        float4 v[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] = *reinterpret_cast<const float4*>(src + (size_t)min(c0 + k * step, count - 1) * stride);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const bool on = c0 + k * step < count;
+            a.x += on ? v[k].x : 0.f; a.y += on ? v[k].y : 0.f; a.z += on ? v[k].z : 0.f; a.w += on ? v[k].w : 0.f;
+        }
+    }
+}
 constexpr int kReRows = 4;
 template <int DV> constexpr int kReThreads = (kReRows * (DV + 4) / 4 + 31) / 32 * 32;      // one float4 of the state per thread: a single round of loads
 template <int DV, int F>
@@ -625,23 +627,15 @@ __global__ void __launch_bounds__(kReThreads<DV>) tc_reduce_emit_kernel(const fl
         count = owner_of_work((long long)bh * T + T - 1, total, G) - owner_of_work((long long)bh * T, total, G) + 1;
     }
     grid_begin(beside);
-    // Four columns per thread, eight partials in flight, added in their order (bit-reproducible).  (One column at a time and one partial
-    // after the other, a block walked 2 to 3 x S dependent round trips to L2.)
+    // Four columns per thread, sixteen partials in flight, added in their order (bit-reproducible): a head of the feature-level calls has ten
+    // splits, one of 12 heads 13 or 14 pieces.
     if (tid < kReRows * Q) {
         const int mm = tid / Q, col = 4 * (tid - mm * Q), m = m0 + mm;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         if (m < kN) {
             const float* src = part + (size_t)bh * S * n_per + (size_t)m * LD + col;
-            for (int s0 = 0; s0 < count; s0 += 8) {
-                float4 v[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    v[k] = s0 + k < count ? *reinterpret_cast<const float4*>(src + (size_t)(s0 + k) * n_per) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
-                }
-            }
+            if (count <= 8) add_partials<8>(a, src, n_per, 0, 1, count);
+            else add_partials<16>(a, src, n_per, 0, 1, count);
             *reinterpret_cast<float4*>(state + (size_t)bh * n_per + (size_t)m * LD + col) = a;
         }
         *reinterpret_cast<float4*>(&sm[mm][col]) = a;

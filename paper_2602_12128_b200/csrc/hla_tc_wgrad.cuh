@@ -94,7 +94,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     float* out_cta = wpart + (size_t)blockIdx.x * Cfg::kPartFloats;
 
     constexpr int kRows = 16 * Cfg::kDgSteps, kB1Abs = kRows - 16 + Cfg::kB1Row;
-    if (tid < DV) stage_w2t_column<DP, kRows, kB1Abs, Cfg::kW2tBlock>(smem + Cfg::kOffW2t, W2g, b1g, tid);
     for (int i = tid; i < 3 * kBlk / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffDp)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < 2 * Cfg::kXBytes / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffX)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < 4 * kBlk / 16; i += kWgThreads) reinterpret_cast<uint4*>(smem + Cfg::kOffG)[i] = make_uint4(0, 0, 0, 0);
@@ -131,6 +130,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) tc_phi_wgrad_kernel(const __gri
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     grid_begin(beside);
+    // (after the dependency wait: a kernel of the caller may have just written the weights)
+    if (tid < DV) stage_w2t_column<DP, kRows, kB1Abs, Cfg::kW2tBlock>(smem + Cfg::kOffW2t, W2g, b1g, tid);
+    fence_proxy_async();
+    __syncthreads();
     bool ok = true;
 
     if (warp == 0) {
@@ -409,18 +412,7 @@ __global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __res
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, at = base + 4 * lane;
     const float* src = wpart + (size_t)out.first[m] * PF + at;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (at < PF) {
-        for (int c0 = warp; c0 < nctas; c0 += 64) {
-            float4 v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                v[k] = c0 + 8 * k < nctas ? *reinterpret_cast<const float4*>(src + (size_t)(c0 + 8 * k) * PF) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
-            }
-        }
-    }
+    if (at < PF) add_partials<8>(a, src, PF, warp, 8, nctas);
     *reinterpret_cast<float4*>(&red[warp][4 * lane]) = a;
     __syncthreads();
     const int i = threadIdx.x;
@@ -498,9 +490,7 @@ inline hla_status launch_phi_wgrad(const Dims& D, int BH, const hla_mlp* phi_q, 
         const float* dfeat = reinterpret_cast<const float*>(ws + (key ? L.dkf : L.dqf));
         const int per_head = key ? D.N : 0;
         rec.begin(key ? "tc_phi_wgrad_k" : "tc_phi_wgrad_q");
-        // the first pass stages caller-provided weights before its dependency wait: no overlap with what precedes it
-        if (first) launch_serial(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status, false);
-        else launch_pdl(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status, true);
+        launch_pdl(tc_phi_wgrad_kernel<DV, DP>, maps.first[n], dim3(kWgThreads), WgCfg<DV, DP>::kSmem, rec.st, maps, feat, dfeat, wpart[key], rows, per_head, status, !first);
         first = false;
         if (!rec.end()) return HLA_ERR_CUDA;
     }
