@@ -447,7 +447,7 @@ hla_status forward_impl(hla_ctx* ctx, const void* Q, const void* K, const void* 
                 s = tc::phik_state(ctx->D, ctx->BH, ctx->phi_k, K, V, ws, ctx->L, ctx->off_part, ctx->k_pieces, ctx->sm_count, ctx->rec);
                 if (s != HLA_OK) return s;
                 s = tc::reduce_pieces(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count),
-                                      ctx->rec);
+                                      phase == 0 && tc::query_starts_early(ctx->BH, ctx->D.N, ctx->sm_count) ? tc::Start::kLetGo : tc::Start::kWait, ctx->rec);
                 if (s != HLA_OK || phase == 1) return s;
             } else {
                 s = tc::emit_from_state(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, false, ctx->rec);

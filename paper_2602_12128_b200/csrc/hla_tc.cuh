@@ -613,11 +613,16 @@ template <int K> __device__ __forceinline__ void add_partials(float4& a, const f
         }
     }
 }
+// How it starts.  kWait: after its predecessor, and only then is the next kernel let go.  kBeside: beside its predecessor (see
+// grid_begin).  kLetGo: after its predecessor, but the next kernel (the fused query side, which waits for this one where it needs its
+// result) may start on every SM that the predecessor leaves: it relies on what precedes the predecessor only, and that is complete,
+// because the predecessor (the fused key side) lets this kernel go after its own wait.
+enum class Start { kWait, kBeside, kLetGo };
 constexpr int kReRows = 4;
 template <int DV> constexpr int kReThreads = (kReRows * (DV + 4) / 4 + 31) / 32 * 32;      // one float4 of the state per thread: a single round of loads
 template <int DV, int F>
 __global__ void __launch_bounds__(kReThreads<DV>) tc_reduce_emit_kernel(const float* __restrict__ part, float* __restrict__ state, __nv_bfloat16* __restrict__ b3,
-                                                                        __nv_bfloat16* __restrict__ bq, int S, int G, int T, bool beside) {
+                                                                        __nv_bfloat16* __restrict__ bq, int S, int G, int T, Start how) {
     constexpr int kN = MT<F>::kN, kPad = MT<F>::kPad, LD = DV + 4, Q = LD / 4, n_per = kN * LD;
     __shared__ __align__(16) float sm[kReRows][LD];
     const int m0 = kReRows * blockIdx.x, bh = blockIdx.y, tid = threadIdx.x;      // gridDim.x = kPad / kReRows
@@ -626,7 +631,12 @@ __global__ void __launch_bounds__(kReThreads<DV>) tc_reduce_emit_kernel(const fl
         const long long total = (long long)gridDim.y * T;
         count = owner_of_work((long long)bh * T + T - 1, total, G) - owner_of_work((long long)bh * T, total, G) + 1;
     }
-    grid_begin(beside);
+    if (how == Start::kLetGo) {
+        grid_launch_dependents();
+        grid_dependency_wait();
+    } else {
+        grid_begin(how == Start::kBeside);
+    }
     // Four columns per thread, sixteen partials in flight, added in their order (bit-reproducible): a head of the feature-level calls has ten
     // splits, one of 12 heads 13 or 14 pieces.
     if (tid < kReRows * Q) {
@@ -646,7 +656,7 @@ __global__ void __launch_bounds__(kReThreads<DV>) tc_reduce_emit_kernel(const fl
     for (int row = tid; row < DV + 16; row += kReThreads<DV>)       // row <= DV: column `row` of the state (row == DV is z); rest zero
         *reinterpret_cast<uint2*>(o3 + (size_t)row * kPad + m0) =
             row <= DV ? make_uint2(pack_bf16(sm[0][row], sm[1][row]), pack_bf16(sm[2][row], sm[3][row])) : make_uint2(0u, 0u);
-    grid_end(beside);
+    grid_end(how == Start::kBeside);
 }
 
 // =======================================================================================
@@ -1457,7 +1467,7 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
     launch_pdl(tc_state_build_kernel<DV, F>, dim3(D.S, BH), dim3(kSbThreads), SbCfg<F>::kSmem, st, mapV, mapV, kf, part, D.N, D.S, D.ld, status, (const float*)nullptr, (float*)nullptr, 0.f, 1);
     if (!rec.end()) return HLA_ERR_CUDA;
     rec.begin("tc_reduce_emit");
-    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, state, b3, bq, D.S, 0, 0, false);
+    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, state, b3, bq, D.S, 0, 0, Start::kWait);
     if (!rec.end()) return HLA_ERR_CUDA;
     if (!readout) return HLA_OK;
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
@@ -1470,19 +1480,19 @@ inline hla_status launch_core_forward(const Plan& P, const Dims& D, int BH, cons
 
 // Reduction of the pieces the fused key-side kernel (G CTAs over heads x T tiles, at most `smax` pieces per head) left.
 template <int F>
-inline hla_status reduce_pieces_f(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec) {
+inline hla_status reduce_pieces_f(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, Start how, LaunchRec& rec) {
     __nv_bfloat16* b3 = reinterpret_cast<__nv_bfloat16*>(ws + P.b3);
     __nv_bfloat16* bq = reinterpret_cast<__nv_bfloat16*>(ws + P.bq);
     float* part = reinterpret_cast<float*>(ws + off_part);
     float* state = reinterpret_cast<float*>(ws + L.state);
     const int T = (D.N + kTileTokens - 1) / kTileTokens;
     rec.begin("tc_reduce_emit");
-    if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<128>), 0, rec.st, part, state, b3, bq, smax, G, T, false);
-    else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<64>), 0, rec.st, part, state, b3, bq, smax, G, T, false);
+    if (D.d == 128) launch_pdl(tc_reduce_emit_kernel<128, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<128>), 0, rec.st, part, state, b3, bq, smax, G, T, how);
+    else launch_pdl(tc_reduce_emit_kernel<64, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<64>), 0, rec.st, part, state, b3, bq, smax, G, T, how);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
-inline hla_status reduce_pieces(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, LaunchRec& rec) {
-    return D.F == 3 ? reduce_pieces_f<3>(P, D, BH, ws, L, off_part, smax, G, rec) : reduce_pieces_f<2>(P, D, BH, ws, L, off_part, smax, G, rec);
+inline hla_status reduce_pieces(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, size_t off_part, int smax, int G, Start how, LaunchRec& rec) {
+    return D.F == 3 ? reduce_pieces_f<3>(P, D, BH, ws, L, off_part, smax, G, how, rec) : reduce_pieces_f<2>(P, D, BH, ws, L, off_part, smax, G, how, rec);
 }
 
 // The two bf16 operand images of a state that already sits, summed, in the workspace (the state region, or with
@@ -1494,7 +1504,7 @@ inline hla_status launch_emit_from_state(const Plan& P, const Dims& D, int BH, c
     __nv_bfloat16* b3 = reinterpret_cast<__nv_bfloat16*>(ws + (gradient ? P.bd3 : P.b3));
     __nv_bfloat16* bq = reinterpret_cast<__nv_bfloat16*>(ws + (gradient ? P.bdq : P.bq));
     rec.begin("tc_reduce_emit");
-    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<DV>), 0, rec.st, (const float*)st, st, b3, bq, 1, 0, 0, false);
+    launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(MT<F>::kPad / kReRows, BH), dim3(kReThreads<DV>), 0, rec.st, (const float*)st, st, b3, bq, 1, 0, 0, Start::kWait);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 inline hla_status emit_from_state(const Plan& P, const Dims& D, int BH, char* ws, const hla_ws_layout& L, bool gradient, LaunchRec& rec) {
@@ -1567,7 +1577,7 @@ inline hla_status launch_core_backward(const Plan& P, const Dims& D, int BH, con
             if (e != HLA_OK) return e;
         }
         rec.begin("tc_reduce_emit");
-        launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, dstate, bd3, bdq, D.S, 0, 0, run_between);
+        launch_pdl(tc_reduce_emit_kernel<DV, F>, dim3(kPad / kReRows, BH), dim3(kReThreads<DV>), 0, st, part, dstate, bd3, bdq, D.S, 0, 0, run_between ? Start::kBeside : Start::kWait);
         if (!rec.end()) return HLA_ERR_CUDA;
         if (phase == 1) return HLA_OK;
     } else {

@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(kFkThreads, 1) tc_causal_maps_kernel(const __g
     if ((int)blockIdx.x < key_grid)
         phik_state_cta<DV, 3>(k.K, k.maps, k.V, k.ptrs, kf_out, part, N, BH, smax, status, carry, carry_copy, blockIdx.x, key_grid);
     else
-        phiq_cta<DV, 3, false>(q.Q, q.W1, q.Q, q.Q, q.b1, q.W2, q.b2, qf_out, nullptr, N, BH, 0.f, status, blockIdx.x - key_grid, gridDim.x - key_grid);
+        phiq_cta<DV, 3, false>(q.Q, q.W1, q.Q, q.Q, q.b1, q.W2, q.b2, qf_out, nullptr, N, BH, 0.f, status, blockIdx.x - key_grid, gridDim.x - key_grid, 0, 0);
 }
 template <int DV>
 inline hla_status launch_causal_maps(const Dims& D, int BH, const hla_mlp* phi_q, const hla_mlp* phi_k, const void* Q, const void* K, const void* V, char* ws,

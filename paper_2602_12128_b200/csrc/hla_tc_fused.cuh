@@ -46,13 +46,21 @@ template <int DV, int F> struct FqCfg {
     static constexpr int kSmem = kSmemUsed > 120 * 1024 ? kSmemUsed : 120 * 1024;   // one CTA per SM (512 TMEM columns)
 };
 
+// Whether the CTAs of the query side may start while the reduction before them is still waiting for the key side: with few tiles per CTA the
+// set-up and the first tiles it hides count (24 heads x 4096 tokens, 5 tiles per CTA: 32.2 -> 30.2 us; 12 heads x 12600, 8 tiles:
+// 266 -> 264 us); in long calls they take bandwidth from the key side's last CTAs (24 heads x 32760, 41 tiles: 239.7 -> 241 us).
+inline bool query_starts_early(int BH, int N, int sm_count) { return (long long)BH * ((N + kTileTokens - 1) / kTileTokens) <= 16ll * sm_count; }
+// First work item of CTA c: even shares, but `fewer` items less for the last `late` CTAs.
+__host__ __device__ inline int query_share(long long total, int c, int G, int late, int fewer) {
+    return (int)((total + (long long)late * fewer) * c / G) - (c > G - late ? fewer * (c - (G - late)) : 0);
+}
 // Q [BH][N][DV] bf16 (3-D map, rows past N read as zero), O the same (stores are clipped at N).  CTA `bid` of `G`.  READOUT = false: the
 // feature map only (the causal operator reads its states tile by tile in a sweep of its own and needs just the query features):
 // the readout product, its epilogue and the monomial tile are left out, O and eta are not written.
 template <int DV, int F, bool READOUT>
 __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensorMap& mapW1, const CUtensorMap& mapB3, const CUtensorMap& mapO,
                                          const __nv_bfloat16* __restrict__ b1g, const __nv_bfloat16* __restrict__ W2g, const __nv_bfloat16* __restrict__ b2g,
-                                         float* __restrict__ qf_out, float* __restrict__ eta_out, int N, int BH, float eps, int* status, int bid, int G) {
+                                         float* __restrict__ qf_out, float* __restrict__ eta_out, int N, int BH, float eps, int* status, int bid, int G, int late, int fewer) {
     using Cfg = FqCfg<DV, F>;
     using M = MT<F>;
     constexpr int DP = M::kDphi;
@@ -84,7 +92,7 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tiles_per_head = (N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles_per_head;
-    const int w0 = (int)(total * bid / G), w1 = (int)(total * (bid + 1) / G);
+    const int w0 = query_share(total, bid, G, late, fewer), w1 = query_share(total, bid + 1, G, late, fewer);
     const int nwork = w1 - w0;
 
     // second-layer weights as a K-major MMA operand [16 rows (outputs, 6 used)][DV], and the biases
@@ -348,8 +356,8 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
                                                                         const __grid_constant__ CUtensorMap mapB3, const __grid_constant__ CUtensorMap mapO,
                                                                         const __nv_bfloat16* __restrict__ b1g, const __nv_bfloat16* __restrict__ W2g,
                                                                         const __nv_bfloat16* __restrict__ b2g, float* __restrict__ qf_out,
-                                                                        float* __restrict__ eta_out, int N, int BH, float eps, int* status) {
-    phiq_cta<DV, F, true>(mapQ, mapW1, mapB3, mapO, b1g, W2g, b2g, qf_out, eta_out, N, BH, eps, status, blockIdx.x, gridDim.x);
+                                                                        float* __restrict__ eta_out, int N, int BH, float eps, int* status, int late, int fewer) {
+    phiq_cta<DV, F, true>(mapQ, mapW1, mapB3, mapO, b1g, W2g, b2g, qf_out, eta_out, N, BH, eps, status, blockIdx.x, gridDim.x, late, fewer);
 }
 
 template <int DV, int F>
@@ -364,11 +372,16 @@ inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, cons
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles;
     const int grid = (int)(total < sm_count ? total : sm_count);
+    // (see query_starts_early) the blocks of the reduction, twelve to an SM, sit on the SMs that the last CTAs are waiting for: those start 4 to
+    // 10 us late and would end as late.  They get up to four tiles less (a tile takes 0.8 to 1.4 us), at most half of their share.
+    const bool early = query_starts_early(BH, D.N, sm_count);
+    int late = early ? (MT<F>::kPad / kReRows * BH + 11) / 12 : 0, fewer = (int)(total / grid / 2 < 4 ? total / grid / 2 : 4);
+    if (late > grid / 2) late = 0;
     rec.begin("tc_phiq_readout");
     launch_pdl(tc_phiq_readout_kernel<DV, F>, grid, dim3(kFqThreads), FqCfg<DV, F>::kSmem, rec.st,
         mapQ, mapW1, mapB3, mapO, static_cast<const __nv_bfloat16*>(phi_q->b1), static_cast<const __nv_bfloat16*>(phi_q->W2),
         static_cast<const __nv_bfloat16*>(phi_q->b2), reinterpret_cast<float*>(ws + L.qf), reinterpret_cast<float*>(ws + L.eta), D.N, BH, D.eps,
-        reinterpret_cast<int*>(ws + L.status));
+        reinterpret_cast<int*>(ws + L.status), late, fewer);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
