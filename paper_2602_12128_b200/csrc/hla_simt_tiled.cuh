@@ -11,10 +11,11 @@
 // permutations of an index, and so is G = X S^T of the key side.  Only the state itself is formed in full, because it is the layout
 // the workspace promises (P rows); the folded rows are summed when a block stages the state.
 //
-// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2547 -> 296 us (two
-// state builds 1236 -> 95, two feature gradients 557 -> 46, two readouts 277 -> 35, feature networks backward 387 -> 95, forward 104 ->
-// 64); forward with B*H = 2, N = 256, d = 16: 95 -> 22.6 us.  Of these, independent neighbours side by side, more splits of the gradient
-// state and the small tiles: 431 -> 332 and 37 -> 25 us; loads without index divisions and without branches between them: the rest.
+// Measured on B200, fp32, F = 3, against the kernels of hla_simt.cuh: training step with B*H = 12, N = 3000, d = 64: 2602 -> 265 us (two
+// state builds 1236 -> 63, two feature gradients 557 -> 46, two readouts 277 -> 35, feature networks backward 387 -> 94, forward 104 ->
+// 63); forward with B*H = 2, N = 256, d = 16: 94 -> 19.8 us.  Of these, independent neighbours side by side, more splits of the gradient
+// state and the small tiles: 431 -> 332 and 37 -> 25 us; loads without index divisions and without branches between them: 296 and 22.6;
+// the state build as it is now: the rest.
 #pragma once
 #include "hla_simt.cuh"
 #include "hla_tc.cuh"

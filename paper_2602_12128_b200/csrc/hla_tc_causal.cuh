@@ -6,8 +6,8 @@
 //     [num | eta]_i = mono_i . [Csym | zsym](tokens before the tile)  +  sum_{j in tile, j <= i} (mono_i . Tsym_j) [v_j | 1]
 // The first term is the readout of the non-causal path against the state *before* the tile; the second is a 128 x 128
 // block of the masked attention matrix times the value tile.  The sequence of a head is cut into pieces (one per CTA that
-// touches the head); a first pass builds the state of every piece, a fixed-order exclusive scan over the pieces of a head
-// gives each piece its initial state, and the kernel below sweeps a piece tile by tile:
+// touches the head); a first pass builds the state of every piece, a fixed-order exclusive prefix sum over the pieces of
+// a head gives each piece its initial state, and the kernel below sweeps a piece tile by tile:
 //
 //     P      = mono tile * Tsym tile^T                    (MMA, K = 64)      P[i][j] = prod_f (q_i . k^f_j)
 //     acc    = mono tile * [Csym | zsym]                  (MMA, K = 64)      state before the tile, bf16 image in shared memory
