@@ -36,21 +36,22 @@ __device__ __forceinline__ float2 gelu2_twice(float2 x) {
 __device__ __forceinline__ __nv_bfloat16 half_bf16(__nv_bfloat16 w) { return __float2bfloat16_rn(0.5f * __bfloat162float(w)); }
 // dg GELU'(x) of a pair of elements, with dg already halved (the 1/2 sits in the staged W2^T, exact in bf16), through one tanh.approx
 // per element:
-//   th = tanh(x (a + b x^2)),   2 GELU'(x) ~ (1 + th) (1 + C0 x (1 - th)) = 1 + th + C0 x (1 - th^2)
-// (the derivative of a tanh-form GELU with a linear inner derivative); a, b, C0 are fitted against the exact derivative
-// (fit_gelu_tanh.py: |error| < 1.33e-4 before the 2^-11 relative error of tanh.approx).  Seven packed instructions per pair; the form
-// with a cubic inner derivative (1.23e-4) needed nine, and a packed fp32 instruction holds the FMA pipe for two cycles: sixteen
-// warps with 32 elements per thread took 1445 cycles, with this form 1265 (the special-function pipe alone needs 1024).  Phi backward of
-// the training shape (B = 2, H = 24, N = 32760, d = 128): key side 424 -> 398 us, query side 189 -> 184 us (at the power cap, where fewer
-// instructions count and more overlap does not: h single- and dg double-buffered, with a fifth fewer cycles, took 404 and 190 us).
-constexpr float kGradA = 0.70650562f, kGradB = 0.03061539f, kGradC0 = 0.88953152f;
+//   th = tanh(x (a + b x^2)),   2 GELU'(x) ~ (1 + th) (1 + V (1 - th)) = 1 + V + th (1 - V th),   V = x (C0 + C1 x^2)
+// (the derivative of a tanh-form GELU whose inner derivative is a free polynomial); a, b, C0, C1 are fitted against the
+// exact derivative (fit_gelu_tanh.py, which prints twice C0 and C1: |error| < 1.5e-4, 3.8e-5 in the mean square over N(0,1), before the 2^-11 relative error of
+// tanh.approx; < 1.3e-3 with it).  Evaluated with -V so that every step is one packed multiply or fma: nine packed and two
+// special-function instructions per pair of elements.  (A linear inner derivative, C1 = 0, takes seven, but its mean-square error is
+// 8.6e-5: errors of gradients against 64 bits grew by up to 0.6 %, for 1 % of a training step (B = 2, H = 24, N = 32760, d = 128:
+// 1286 against 1299 us).)
+constexpr float kGradA = 0.69631102f, kGradB = 0.02936904f, kGradC0 = 0.89902785f, kGradC1 = -0.010848315f;
 __device__ __forceinline__ float2 times_gelu_grad2(float2 dg, float2 x) {
     const float2 t = __fmul2_rn(x, x);
     const float2 u = __fmul2_rn(x, __ffma2_rn(t, splat2(kGradB), splat2(kGradA)));
-    const float2 v = __fmul2_rn(x, splat2(-kGradC0));
     const float2 th = make_float2(tanh_approx(u.x), tanh_approx(u.y));
-    const float2 q = __ffma2_rn(v, __ffma2_rn(th, th, splat2(-1.f)), th);
-    return __ffma2_rn(dg, q, dg);
+    const float2 vn = __fmul2_rn(x, __ffma2_rn(t, splat2(-kGradC1), splat2(-kGradC0)));      // -V
+    const float2 a1 = __ffma2_rn(vn, th, splat2(1.f));          // 1 - V th
+    const float2 b1 = __ffma2_rn(th, a1, splat2(1.f));          // 1 + th (1 - V th)
+    return __fmul2_rn(dg, __ffma2_rn(vn, splat2(-1.f), b1));    // + V
 }
 
 // 2 GELU(x) and 2 GELU'(x) of the same elements through ONE tanh.approx each (the weight gradients need both): the tanh
