@@ -150,16 +150,21 @@ constexpr int kSelfPrefixPieces = 16;
 inline bool self_prefix(int S) { return S <= kSelfPrefixPieces; }
 // THREADS threads, numbered t: [56][ld] floats of the state before piece `slot` (the head's first slot is `base`, `carry` its carried
 // state or null) into `dst`
-// and, where image is not null, its bf16 operand image.  Eight loads in flight per thread.
+// and, where image is not null, its bf16 operand image.  Eight loads in flight per thread.  Returns the thread's part.
+template <int DV, int THREADS> struct StatePart {
+    static constexpr int kQuads = kMono * (DV + 4) / 4, kItems = (kQuads + THREADS - 1) / THREADS;
+    float4 q[kItems];      // quads t, t + THREADS, ..
+};
 template <int DV, int THREADS>
-__device__ __forceinline__ void stage_initial_state(float* dst, uint8_t* image, int t, const float* __restrict__ slots, int base, int slot, bool self,
-                                                    const float* __restrict__ carry) {
-    constexpr int ld = DV + 4, kQuads = kMono * ld / 4, kItems = (kQuads + THREADS - 1) / THREADS;
+__device__ __forceinline__ StatePart<DV, THREADS> stage_initial_state(float* dst, uint8_t* image, int t, const float* __restrict__ slots, int base, int slot, bool self,
+                                                                      const float* __restrict__ carry) {
+    constexpr int ld = DV + 4, kQuads = StatePart<DV, THREADS>::kQuads, kItems = StatePart<DV, THREADS>::kItems;
     static_assert(kItems <= 4, "loads in flight");
     const float4* src = reinterpret_cast<const float4*>(slots) + (size_t)(self ? base : slot) * kQuads;
     const float4* first = reinterpret_cast<const float4*>(carry);
     const int lo = self && carry ? -1 : 0, hi = self ? slot - base : 1;      // source -1 is the carried state
-    float4 a[kItems];
+    StatePart<DV, THREADS> part;
+    float4(&a)[kItems] = part.q;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
@@ -186,6 +191,20 @@ __device__ __forceinline__ void stage_initial_state(float* dst, uint8_t* image, 
         const int m = i / (ld / 4), c = 4 * (i - m * (ld / 4));
         if (image) *reinterpret_cast<uint2*>(image + (c >> 6) * (64 * 128) + sw128_off(m + kCaRowPad, (c & 63) >> 3) + (c & 7) * 2) = make_uint2(pack_bf16(a[k].x, a[k].y), pack_bf16(a[k].z, a[k].w));
     }
+    return part;
+}
+// `out` = the state before a piece + the piece, the last step of the same sum: what a head leaves when the piece is its last.
+template <int DV, int THREADS>
+__device__ __forceinline__ void store_state_after(float* __restrict__ out, const StatePart<DV, THREADS>& before, int t, const float* __restrict__ piece) {
+    using P = StatePart<DV, THREADS>;
+    float4 v[P::kItems];
+#pragma unroll
+    for (int k = 0; k < P::kItems; ++k)
+        if (t + k * THREADS < P::kQuads) v[k] = reinterpret_cast<const float4*>(piece)[t + k * THREADS];
+#pragma unroll
+    for (int k = 0; k < P::kItems; ++k)
+        if (t + k * THREADS < P::kQuads)
+            reinterpret_cast<float4*>(out)[t + k * THREADS] = make_float4(before.q[k].x + v[k].x, before.q[k].y + v[k].y, before.q[k].z + v[k].z, before.q[k].w + v[k].w);
 }
 
 // In-place exclusive scan of the piece states of every head, in piece order (bit-reproducible); the sum of all pieces,
@@ -266,6 +285,10 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     const int w0 = cw.w0, nwork = cw.w1 - cw.w0;
     auto work_of = [&](int it) { return MODE == 0 ? w0 + it : w0 + nwork - 1 - it; };                 // (head, tile) of the CTA's it-th item
     auto starts = [&](int it) { return it == 0 || (MODE == 0 && (w0 + it) % T == 0); };          // a piece begins with this item
+    // The state after a head's last token is what the head leaves.  Its last CTA adds it up in fp32 from the states of the pieces.  (The
+    // accumulator of the sweep holds it too, but every tile's products were added onto the full sum there, and not rounded to nearest:
+    // after 400 carried calls that state was off by more than 400 roundings of fp32.)
+    auto ends_here = [&](int bh) { return MODE == 0 && state_out && (bh + 1) * T <= cw.w1; };
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -307,10 +330,11 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
         constexpr int kThreads = (kCaStateMmaWarp - kCaMaskWarp0) * 32;
         static_assert(kMono * ld * 4 <= Cfg::kVB * kBlk, "staging tile");
         const int t = tid - kCaMaskWarp0 * 32;
+        const int bh = work_of(0) / T, slot = causal_slot(bh, T, BH, S, G);
+        StatePart<DV, kThreads> before;
         if (nwork > 0) {
-            const int bh = work_of(0) / T;
-            stage_initial_state<DV, kThreads>(reinterpret_cast<float*>(smem + Cfg::kOffO), smem + Cfg::kOffB3, t, init, bh * S, causal_slot(bh, T, BH, S, G), self_sum,
-                                              carry ? carry + (size_t)bh * kMono * ld : nullptr);
+            before = stage_initial_state<DV, kThreads>(reinterpret_cast<float*>(smem + Cfg::kOffO), smem + Cfg::kOffB3, t, init, bh * S, slot, self_sum,
+                                                       carry ? carry + (size_t)bh * kMono * ld : nullptr);
             fence_proxy_async();
         }
         named_barrier(2, kThreads);
@@ -318,6 +342,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
         // every CTA has got here, or, where a CTA begins another head later and reads that head's carried state then, has ended.
         const bool reads_later = self_sum && carry && !state_out && nwork > 0 && (w0 + nwork - 1) / T != w0 / T;
         if (t == 0 && !reads_later) grid_launch_dependents();
+        if (nwork > 0 && ends_here(bh)) store_state_after<DV, kThreads>(state_out + (size_t)bh * kMono * ld, before, t, init + (size_t)slot * kMono * ld);
     }
 
     if (warp == 0) {
@@ -597,23 +622,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
                 fence_proxy_async();
                 mbar_arrive(&b3_ready[(it + 1) & 1]);
             } else {
-                // the next tile (if any) starts a piece with a state of its own; the state after a head's last token is what the head leaves
-                if (MODE == 0 && state_out && work % T == T - 1) {
-                    tc_fence_after();
-                    float* dst = state_out + ((size_t)bh * kMono + (mine ? m : 0)) * ld;
-#pragma unroll 1
-                    for (int c = 0; c < Cfg::kNState / 8; ++c) {
-                        uint32_t r[8];
-                        tmem_ld8(sa + 8 * c, r);
-                        tmem_ld_wait();
-                        if (!mine) continue;
-                        const bool z = 8 * c >= DV;      // column d, then padding
-                        *reinterpret_cast<uint4*>(dst + 8 * c) = z ? make_uint4(r[0], 0u, 0u, 0u) : make_uint4(r[0], r[1], r[2], r[3]);
-                        if (!z) *reinterpret_cast<uint4*>(dst + 8 * c + 4) = make_uint4(r[4], r[5], r[6], r[7]);
-                    }
-                    tc_fence_before();
-                }
-                mbar_arrive(state_read);
+                mbar_arrive(state_read);      // nothing is read: the next tile (if any) starts a piece with a state of its own
             }
         }
     } else {
@@ -663,6 +672,20 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
             if (MODE == 0 && tok < N) eta_out[(size_t)bh * N + tok] = eta;
         }
         if (etid == 0) tma_store_wait_all0();
+    }
+    if (MODE == 0 && state_out) {      // heads that begin and end in this CTA behind its first piece: the carried state, if any, and their only piece
+        constexpr int kQuads = kMono * ld / 4;
+        const int h0 = cw.w0 / T + 1, n = (cw.w1 / T - h0) * kQuads;
+#pragma unroll 2
+        for (int i = tid; i < n; i += kCaThreads) {
+            const int h = h0 + i / kQuads, q = i % kQuads;
+            float4 x = reinterpret_cast<const float4*>(init + (size_t)h * S * kMono * ld)[q];
+            if (carry) {
+                const float4 c = reinterpret_cast<const float4*>(carry + (size_t)h * kMono * ld)[q];
+                x = make_float4(c.x + x.x, c.y + x.y, c.z + x.z, c.w + x.w);
+            }
+            reinterpret_cast<float4*>(state_out + (size_t)h * kMono * ld)[q] = x;
+        }
     }
     tc_fence_before();
     __syncthreads();
