@@ -261,7 +261,9 @@ hla_status hla_value_mod_backward(hla_ctx *ctx, const void *T, const void *V, co
  * workspace, and calls no memory-allocating routine.
  *
  *   - Contexts whose hla_workspace_bytes() exceeds HLA_STATIC_WS_BYTES are
- *     refused with HLA_ERR_WORKSPACE before anything is enqueued.
+ *     refused with HLA_ERR_WORKSPACE before anything is enqueued.  (The split
+ *     count that n_splits = 0 stands for is lowered where the workspace would
+ *     be too large for speed only.)
  *   - The first call on a device looks up the array's device address (with
  *     that device current) and remembers it; make that first call outside any
  *     stream capture.  Later calls on the same device only enqueue work.

@@ -85,6 +85,21 @@ simt::PhiWeights<T> pack_weights(const hla_mlp* m, int n) {
     return w;
 }
 
+// One CTA per SM: S * heads CTAs run in ceil(S * heads / SMs) waves.  The split count that fills its waves best (each extra wave is charged
+// 2 % for its start-up and drain), with at least `least` tiles per CTA.
+int wave_splits(int BH, int tiles, int least, int sm_count) {
+    const int smax = tiles / least > 1 ? (tiles / least < 64 ? tiles / least : 64) : 1;
+    int S = 1;
+    double best = -1.0;
+    for (int cand = 1; cand <= smax; ++cand) {
+        const long long ctas = (long long)cand * BH;
+        const long long waves = (ctas + sm_count - 1) / sm_count;
+        const double score = (double)ctas / (double)(waves * sm_count) - 0.02 * (double)(waves - 1);
+        if (score > best + 1e-9) { best = score; S = cand; }
+    }
+    return S;
+}
+
 int reduce_blocks(size_t total) {
     size_t b = (total + 255) / 256;
     return (int)(b > 4096 ? 4096 : (b < 1 ? 1 : b));
@@ -307,63 +322,62 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
     }
     const int tile = x->tc ? tc::kTileTokens : simt::kTok;
     const int tiles = (c.N + tile - 1) / tile;
-    int S = c.n_splits;
+    // Splits of the rule, and the fewest that a workspace in the library's own array may be had with (see below).
+    int S = c.n_splits, fewest = c.n_splits;
     if (S == 0) {
         if (x->tc) {
-            // One CTA per SM: S * heads CTAs run in ceil(S * heads / SMs) waves.  Take the split count that fills its
-            // waves best (each extra wave is charged 2 % for its start-up and drain), with at least 4 tiles per CTA (8 left 60 CTAs of
-            // a step of 12 heads x 4999 tokens: 36.2 us against 34.7).
-            const int smax = tiles / 4 > 1 ? (tiles / 4 < 64 ? tiles / 4 : 64) : 1;
-            double best = -1.0;
-            for (int cand = 1; cand <= smax; ++cand) {
-                const long long ctas = (long long)cand * x->BH;
-                const long long waves = (ctas + x->sm_count - 1) / x->sm_count;
-                const double score = (double)ctas / (double)(waves * x->sm_count) - 0.02 * (double)(waves - 1);
-                if (score > best + 1e-9) { best = score; S = cand; }
-            }
+            // At least 4 tiles per CTA (8 left 60 CTAs of a step of 12 heads x 4999 tokens: 36.2 us against 34.7).
+            S = wave_splits(x->BH, tiles, 4, x->sm_count);
+            fewest = wave_splits(x->BH, tiles, 8, x->sm_count);
         } else {
-            S = simt::tiled(D) ? simt::tiled_splits(x->BH, c.N, P, c.d, x->sm_count) : (2 * x->sm_count + x->BH - 1) / x->BH;
+            fewest = (2 * x->sm_count + x->BH - 1) / x->BH;
+            S = simt::tiled(D) ? simt::tiled_splits(x->BH, c.N, P, c.d, x->sm_count) : fewest;
         }
     }
     if (S > tiles) S = tiles;
     if (S < 1) S = 1;
-    D.S = S;
 
     const bool mlp = c.phi == HLA_PHI_MLP;
     const size_t tok = (size_t)x->BH * c.N;
-    Carver cv;
     hla_ws_layout& L = x->L;
-    L.status = cv.take(64);
-    L.qf = mlp ? cv.take(tok * c.d_phi * 4) : kNone;
-    L.kf = mlp ? cv.take(tok * c.F * c.d_phi * 4) : kNone;
     const int state_rows = x->tc ? tc::n_mono(c.F) : P;
-    L.state = cv.take((size_t)x->BH * state_rows * D.ld * 4);
-    L.eta = cv.take(tok * 4);
-    L.dstate = cv.take((size_t)x->BH * state_rows * D.ld * 4);
-    L.dqf = mlp ? cv.take(tok * c.d_phi * 4) : kNone;
-    L.dkf = mlp ? cv.take(tok * c.F * c.d_phi * 4) : kNone;
     L.state_ld = D.ld;
     L.state_rows = state_rows;
-    L.n_splits = S;
     L.tensor_core = x->tc ? 1 : 0;
-    // partial states: S per head from the split kernels, or the pieces of the fused key-side kernel (folded rows)
-    x->k_pieces = 0;
-    size_t part_bytes = (size_t)x->BH * S * state_rows * D.ld * 4;
-    if (x->tc && mlp) {
-        x->k_pieces = tc::fused_key_max_pieces(x->BH, tiles, tc::fused_key_grid(x->BH, c.N, x->sm_count));
-        const size_t need = (size_t)x->BH * x->k_pieces * tc::n_mono(c.F) * D.ld * 4;
-        if (need > part_bytes) part_bytes = need;
-    }
-    x->off_part = cv.take(part_bytes);
-    x->off_wpart = (x->tc && mlp) ? cv.take(tc::wgrad_part_bytes(c.d, c.F, (long long)x->BH * c.N, x->sm_count)) : kNone;
-    if (x->tc) cv.off = tc::plan(x->tcp, D, x->BH, cv.off);
-    x->off_delta = c.causal ? cv.take(tok * 4) : kNone;      // dO . o per token (causal backward)
-    x->off_gpart = c.causal ? cv.take((size_t)x->BH * S * state_rows * D.ld * 4) : kNone;
+    x->k_pieces = x->tc && mlp ? tc::fused_key_max_pieces(x->BH, tiles, tc::fused_key_grid(x->BH, c.N, x->sm_count)) : 0;
     x->carry = false;
     x->vmod = c.value_mod != 0;
     x->phi_v_set = false;
-    if (x->vmod) cv.off = tc::vmod_plan(x->vmp, c.d, (long long)x->BH * c.N, cv.off);
-    x->ws_bytes = cv.off;
+    auto lay_out = [&](int splits) {
+        Carver cv;
+        D.S = L.n_splits = splits;
+        L.status = cv.take(64);
+        L.qf = mlp ? cv.take(tok * c.d_phi * 4) : kNone;
+        L.kf = mlp ? cv.take(tok * c.F * c.d_phi * 4) : kNone;
+        L.state = cv.take((size_t)x->BH * state_rows * D.ld * 4);
+        L.eta = cv.take(tok * 4);
+        L.dstate = cv.take((size_t)x->BH * state_rows * D.ld * 4);
+        L.dqf = mlp ? cv.take(tok * c.d_phi * 4) : kNone;
+        L.dkf = mlp ? cv.take(tok * c.F * c.d_phi * 4) : kNone;
+        // partial states: one per split and head from the split kernels, or the pieces of the fused key-side kernel (folded rows)
+        const int parts = splits > x->k_pieces ? splits : x->k_pieces;
+        x->off_part = cv.take((size_t)x->BH * parts * state_rows * D.ld * 4);
+        x->off_wpart = (x->tc && mlp) ? cv.take(tc::wgrad_part_bytes(c.d, c.F, (long long)x->BH * c.N, x->sm_count)) : kNone;
+        if (x->tc) cv.off = tc::plan(x->tcp, D, x->BH, cv.off);
+        x->off_delta = c.causal ? cv.take(tok * 4) : kNone;      // dO . o per token (causal backward)
+        x->off_gpart = c.causal ? cv.take((size_t)x->BH * splits * state_rows * D.ld * 4) : kNone;
+        if (x->vmod) cv.off = tc::vmod_plan(x->vmp, c.d, (long long)x->BH * c.N, cv.off);
+        return cv.off;
+    };
+    x->ws_bytes = lay_out(S);
+    // hla_forward_static takes what fits in the library's own array.  More splits than `fewest` are there for speed only: they may not
+    // cost a configuration that call, so a workspace that fits with fewer of them gets as many as fit.
+    if (x->ws_bytes > HLA_STATIC_WS_BYTES && fewest < S) {
+        int fit = S;
+        if (lay_out(fewest) <= HLA_STATIC_WS_BYTES)
+            do --fit; while (lay_out(fit) > HLA_STATIC_WS_BYTES);
+        x->ws_bytes = lay_out(fit);
+    }
     *out = x;
     return HLA_OK;
 }

@@ -53,6 +53,19 @@ def test_create_defaults_and_layout():
     binding.hla_destroy(ctx)
 
 
+@pytest.mark.parametrize("kw", [dict(H=17, N=1400, d=32, dtype=binding.HLA_F32), dict(B=2, H=7, N=3534, d=16), dict(B=4, H=5, N=2349, d=8, F=2, dtype=binding.HLA_F32),
+                                dict(H=25, N=11045, F=2, phi=binding.HLA_PHI_NONE), dict(H=33, N=8458, d=64, phi=binding.HLA_PHI_NONE, causal=1)])
+def test_splits_for_speed_do_not_push_a_workspace_out_of_the_static_array(kw):
+    st, ctx = create(**kw)
+    assert st == binding.HLA_OK
+    S = binding.hla_workspace_layout(ctx).n_splits
+    assert binding.hla_workspace_bytes(ctx) <= binding.HLA_STATIC_WS_BYTES
+    binding.hla_destroy(ctx)
+    st, ctx = create(n_splits=S + 1, **kw)      # as many as fit
+    assert st == binding.HLA_OK and binding.hla_workspace_bytes(ctx) > binding.HLA_STATIC_WS_BYTES
+    binding.hla_destroy(ctx)
+
+
 def test_feature_level_entry_has_no_feature_regions():
     st, ctx = create(phi=binding.HLA_PHI_NONE, dtype=binding.HLA_F32, d=16, F=2)
     assert st == binding.HLA_OK
