@@ -315,6 +315,8 @@ __global__ void __launch_bounds__(256) tiled_reduce_kernel(float* __restrict__ o
     }
 }
 
+__device__ float4 g_no_row;      // zeros, read in place of a row that is left out; never written
+
 // Folded rows of a head's state into a tile [kNp][ldt] (columns 0 .. d: d values, then z; the padding rows are zero).
 //   SUM = true: sum over the distinct permutations of the row's indices (what the readout of q (x) .. (x) q sees);
 //   SUM = false: the row itself (a gradient state, the same for all permutations).
@@ -325,31 +327,32 @@ template <int F, bool SUM> __device__ __forceinline__ void stage_state(float* ti
         const int m = i / q, c = 4 * (i - m * q);
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         if (m < G::kN) {
-            // (all rows are loaded, those that repeat an index tuple with a zero factor: independent loads instead of a chain of branches)
+            // Every row is a load, those that repeat an index tuple one of zeros: independent loads instead of a chain of branches.  (A zero
+            // factor made NaN of an infinite row; choosing or masking the loaded values took 21.5 us for a forward of 2 heads x 256 tokens
+            // instead of 20.0.)
             const int p = kRowTable<F>.v[m];
-            auto row = [&](int r) { return __ldg(reinterpret_cast<const float4*>(st + (size_t)r * ld + c)); };
-            auto add = [&](float4 v, bool on) {
-                const float f = on ? 1.f : 0.f;
-                a.x = fmaf(f, v.x, a.x); a.y = fmaf(f, v.y, a.y); a.z = fmaf(f, v.z, a.z); a.w = fmaf(f, v.w, a.w);
+            auto row = [&](int r, bool on = true) { return __ldg(on ? reinterpret_cast<const float4*>(st + (size_t)r * ld + c) : &g_no_row); };
+            auto add = [&](float4 v) {
+                a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
             };
             if (!SUM) {
                 a = row(p);
             } else if (F == 2) {
                 const int d0 = p / 12, d1 = p % 12;
-                const float4 v0 = row(p), v1 = row(d1 * 12 + d0);
+                const float4 v0 = row(p), v1 = row(d1 * 12 + d0, d0 != d1);
                 a = v0;
-                add(v1, d0 != d1);
+                add(v1);
             } else {
                 const int d0 = p / 36, d1 = (p / 6) % 6, d2 = p % 6;      // d0 <= d1 <= d2
                 const bool n01 = d0 != d1, n12 = d1 != d2;
-                const float4 v0 = row(p), v1 = row(36 * d0 + 6 * d2 + d1), v2 = row(36 * d1 + 6 * d0 + d2), v3 = row(36 * d1 + 6 * d2 + d0),
-                             v4 = row(36 * d2 + 6 * d0 + d1), v5 = row(36 * d2 + 6 * d1 + d0);
+                const float4 v0 = row(p), v1 = row(36 * d0 + 6 * d2 + d1, n12), v2 = row(36 * d1 + 6 * d0 + d2, n01), v3 = row(36 * d1 + 6 * d2 + d0, n01 && n12),
+                             v4 = row(36 * d2 + 6 * d0 + d1, n01 && n12), v5 = row(36 * d2 + 6 * d1 + d0, n01 || n12);
                 a = v0;
-                add(v1, n12);
-                add(v2, n01);
-                add(v3, n01 && n12);
-                add(v4, n01 && n12);
-                add(v5, n01 || n12);
+                add(v1);
+                add(v2);
+                add(v3);
+                add(v4);
+                add(v5);
             }
         }
         *reinterpret_cast<float4*>(tile + m * ldt + c) = a;
