@@ -182,6 +182,10 @@ hla_status hla_set_carry(hla_ctx *ctx, int carry);
  * (their rows leave the kernel as 32-byte stores); anything else is refused with
  * HLA_ERR_INVALID_ARG before a launch.
  * Gradients with respect to the phi weights are not computed by this call.
+ * In HLA_PHI_MLP mode dQ may be the buffer of Q, V, O or dO and dK that of K; with
+ * features given, dK may be that of K and, without the mask, dQ that of Q.  (Such a call runs
+ * its kernels one after the other where they would otherwise run side by side, and
+ * hla_backward_weights needs the Q and K that it overwrites.)
  * With causal = 1, O must be the output of that forward (the call reads it for
  * dO_i . o_i; without the mask it is not read) and V, O, dO, dV must be 16-byte
  * aligned like every tensor.
@@ -236,7 +240,7 @@ hla_status hla_backward_weights(hla_ctx *ctx, const void *Q, const void *K, cons
  *     dT = dOut + J1^T (dOut (.) phi_v2(V)),     dV = J2^T (dOut (.) phi_v1(T))      (J: Jacobian of a map w.r.t. its input)
  * the gradients of sum(dOut * Out) with respect to T and V (weights fixed).  With accumulate_dV != 0 the V-side
  * gradient is added to what dV already holds (the dV that hla_backward wrote for the same step), else dV is overwritten.
- * Out, dT, dV must be 32-byte aligned.  Out may not alias T or V.  hla_value_mod_forward clears the device status words
+ * Out, dT, dV must be 32-byte aligned.  Out may not alias T or V; dT may be the buffer of T, and dV that of V, T or dOut.  hla_value_mod_forward clears the device status words
  * like hla_forward does (read hla_last_device_status before it if the record of hla_forward matters); the backward
  * keeps them.  A whole step is then
  *     hla_forward -> hla_value_mod_forward;   hla_value_mod_backward -> hla_backward(dO = dT) with accumulate_dV = 0 and

@@ -63,6 +63,12 @@ struct Carver {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Whether n bytes at a and m bytes at b share memory.
+bool overlap(const void* a, size_t n, const void* b, size_t m) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + m && y < x + n;
+}
+
 int ipow(int b, int e) {
     long long r = 1;
     for (int i = 0; i < e; ++i) {
@@ -239,6 +245,9 @@ hla_status backward_simt(hla_ctx* c, const void* Q, const void* K, const void* V
         a.dQ = dQ; a.dK = dK; a.dV = dV;
         a.dqf = mlp ? reinterpret_cast<float*>(ws + c->L.dqf) : static_cast<float*>(dQ);
         a.dkf = mlp ? reinterpret_cast<float*>(ws + c->L.dkf) : static_cast<float*>(dK);
+        // gradients over inputs that a kernel beside or after theirs still reads
+        const size_t tok = (size_t)c->BH * c->D.N, val = tok * c->D.d * sizeof(T), qn = tok * c->D.dphi * 4, kn = qn * c->D.F;
+        a.in_order = mlp ? overlap(dQ, val, V, val) : overlap(dQ, qn, Q, qn) || overlap(dQ, qn, O, val) || overlap(dQ, qn, dO, val) || overlap(dK, kn, K, kn);
         return simt::run_tiled<T>(a, false, c->sm_count, c->rec) ? HLA_OK : HLA_ERR_CUDA;
     }
     const float* qf = mlp ? reinterpret_cast<const float*>(ws + c->L.qf) : static_cast<const float*>(Q);
@@ -521,14 +530,17 @@ hla_status backward_impl(hla_ctx* ctx, const void* Q, const void* K, const void*
         const float* kf = mlp ? reinterpret_cast<const float*>(ws + ctx->L.kf) : static_cast<const float*>(K);
         float* dqf = mlp ? reinterpret_cast<float*>(ws + ctx->L.dqf) : static_cast<float*>(dQ);
         float* dkf = mlp ? reinterpret_cast<float*>(ws + ctx->L.dkf) : static_cast<float*>(dK);
-        // the feature network of the queries needs only the query side's result: its backward is launched in the middle of the core's
-        const bool inside = mlp && phase == 0;
+        // the feature network of the queries needs only the query side's result: its backward is launched in the middle of the core's, unless
+        // dQ lies over an input that the rest of the core reads; likewise dk beside dV
+        const size_t tok = (size_t)ctx->BH * ctx->D.N, val = tok * ctx->D.d * 2, qn = tok * ctx->D.dphi * 4, kn = qn * ctx->D.F;
+        const bool inside = mlp && phase == 0 && !overlap(dQ, val, V, val) && !(ctx->cfg.causal && overlap(dQ, val, dO, val));
+        const bool dk_beside = mlp || !(overlap(dK, kn, K, kn) || overlap(dK, kn, Q, qn) || overlap(dK, kn, dO, val));
         auto query_map = [&]() { return tc::phi_backward<false>(ctx->D, ctx->BH, &ctx->phi_q, Q, dQ, ws, ctx->L, ctx->sm_count, ctx->rec); };
         if (ctx->cfg.causal) {
             if (ctx->carry) return HLA_ERR_UNSUPPORTED;      // a chunk that started from a carried state has no backward here
             const tc::CausalPieces fwd = mlp ? tc::CausalPieces{ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count)}
                                              : tc::CausalPieces{ctx->off_part, ctx->D.S, 0};
-            s = tc::causal_backward(ctx->D, ctx->BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, ctx->L, fwd, ctx->off_gpart, ctx->off_delta, ctx->rec, inside, query_map);
+            s = tc::causal_backward(ctx->D, ctx->BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, ctx->L, fwd, ctx->off_gpart, ctx->off_delta, ctx->rec, dk_beside, inside, query_map);
         } else {
             s = tc::core_backward(ctx->tcp, ctx->D, ctx->BH, qf, kf, V, dO, dqf, dkf, dV, ws, ctx->L, ctx->off_part, ctx->sm_count, ctx->rec, phase, inside, query_map);
         }
@@ -623,9 +635,11 @@ hla_status value_mod_call(hla_ctx* ctx, const void* T, const void* V, const void
     tc::HostCacheScope scope(&ctx->hc);
     const long long rows = (long long)ctx->BH * ctx->D.N;
     int* status = reinterpret_cast<int*>(ws + ctx->L.status);
+    const size_t val = (size_t)rows * ctx->D.d * 2;
+    const bool dV_beside = !(overlap(dV, val, dOut, val) || overlap(dV, val, T, val));      // (the pass for dT reads T and dOut)
     if (ctx->D.d == 128)
-        return tc::launch_vmod<128>(ctx->vmp, rows, ctx->phi_v, T, V, dOut, Out, dT, dV, accumulate, backward, ws, status, ctx->sm_count, ctx->rec);
-    return tc::launch_vmod<64>(ctx->vmp, rows, ctx->phi_v, T, V, dOut, Out, dT, dV, accumulate, backward, ws, status, ctx->sm_count, ctx->rec);
+        return tc::launch_vmod<128>(ctx->vmp, rows, ctx->phi_v, T, V, dOut, Out, dT, dV, accumulate, backward, dV_beside, ws, status, ctx->sm_count, ctx->rec);
+    return tc::launch_vmod<64>(ctx->vmp, rows, ctx->phi_v, T, V, dOut, Out, dT, dV, accumulate, backward, dV_beside, ws, status, ctx->sm_count, ctx->rec);
 }
 }  // namespace
 

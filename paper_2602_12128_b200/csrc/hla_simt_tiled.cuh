@@ -670,6 +670,7 @@ struct TiledArgs {
     const float *qf, *kf;      // features: given, or in the workspace
     float *qf_out, *kf_out, *dqf, *dkf, *part, *state, *dstate, *eta;
     const hla_mlp *phi_q, *phi_k;      // null: features are given
+    bool in_order;             // backward: gradients lie over inputs, no kernel may run beside another (see Tiled::backward)
     int* clear;                // status words, cleared by a kernel of the forward (none of these kernels waits, so none reports)
 };
 
@@ -727,20 +728,30 @@ template <typename T, int F, int CG, int R> struct Tiled {
         const size_t rows = (size_t)a.BH * D.N;
         const unsigned rb = (unsigned)((rows + TM - 1) / TM), tb = (unsigned)((D.N + TM - 1) / TM);
         const int Sg = tiled_gradient_splits<F>(D, a.BH, sm_count);
+        auto dq = [&]() {
+            return launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state,
+                          a.dqf, false);
+        };
+        auto partials = [&](bool beside) {
+            return launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(Sg, 1, a.BH), CG * kSbGroups<F, true>, 0, D, a.qf, in(a.dO), in(a.O),
+                          a.eta, a.part, Sg, beside, nullptr);
+        };
+        auto sum = [&]() { return launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, Sg, D.ld); };
+        auto dk = [&]() {
+            return launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::grad, D, a.kf, in(a.V), in(nullptr), a.eta, a.dstate,
+                          a.dkf, false);
+        };
+        auto dv = [&](bool beside) {
+            return launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::readout, D, a.kf, a.dstate, out(a.dV), a.eta, beside);
+        };
         // dq, and beside it the partials of dC, dz;  their sum;  dk^f, and beside it dV;  the feature networks of Q (dq is long complete) beside
-        // that, then those of K
-        if (!(launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, true>, dim3(tb, a.BH), NT, S::grad, D, a.qf, in(a.dO), in(a.O), a.eta, a.state, a.dqf,
-                     false) &&
-              launch(rec, "simt_state_build", tiled_state_build_kernel<T, F, CG, true>, dim3(Sg, 1, a.BH), CG * kSbGroups<F, true>, 0, D, a.qf, in(a.dO), in(a.O),
-                     a.eta, a.part, Sg, true, nullptr) &&
-              launch(rec, "simt_reduce_partials", tiled_reduce_kernel<F, true>, reduce_grid(a, G::kN), 256, 0, a.dstate, a.part, a.BH, Sg, D.ld) &&
-              launch(rec, "simt_feature_grad", tiled_feature_grad_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::grad, D, a.kf, in(a.V), in(nullptr), a.eta, a.dstate,
-                     a.dkf, false) &&
-              launch(rec, "simt_readout", tiled_readout_kernel<T, F, CG, R, false>, dim3(tb, a.BH), NT, S::readout, D, a.kf, a.dstate, out(a.dV), a.eta, true)))
-            return false;
+        // that, then those of K.  One after the other, each input is read for the last time before a gradient of its own shape is written
+        // over it (dQ over Q, dK over K, dQ over V with the feature networks).
+        const bool beside = !a.in_order;
+        if (!(beside ? dq() && partials(true) && sum() && dk() && dv(true) : partials(false) && sum() && dq() && dv(false) && dk())) return false;
         if (!a.phi_q) return true;
         return launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, R, false>, dim3(rb), NT, S::phi_bwd, in(a.Q), weights(a.phi_q, 1), a.qf, a.dqf,
-                      out(a.dQ), rows, D.N, D.d, true) &&
+                      out(a.dQ), rows, D.N, D.d, beside) &&
                launch(rec, "simt_phi_backward", tiled_phi_backward_kernel<T, G::kDphi, CG, R, true>, dim3(rb), NT, S::phi_bwd, in(a.K), weights(a.phi_k, F), a.kf, a.dkf,
                       out(a.dK), rows, D.N, D.d, false);
     }

@@ -527,7 +527,7 @@ struct CausalPieces {
 template <int DV>
 inline hla_status launch_causal_backward_features(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* dO, float* dqf, float* dkf,
                                                   char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta, bool second,
-                                                  LaunchRec& rec) {
+                                                  bool beside, LaunchRec& rec) {
     CUtensorMap mapV, mapdO;
     if (!make_map_bhnd(&mapV, V, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapdO, dO, BH, D.N, DV, kTileTokens)) return HLA_ERR_CUDA;
     int* status = reinterpret_cast<int*>(ws + L.status);
@@ -543,31 +543,31 @@ inline hla_status launch_causal_backward_features(const Dims& D, int BH, const f
     if (!set_smem(tc_causal_grad_kernel<DV, 1>, CgCfg<DV>::kSmem)) return HLA_ERR_CUDA;
     rec.begin("tc_causal_dk");
     launch_pdl(tc_causal_grad_kernel<DV, 1>, dim3(D.S, BH), dim3(kCgThreads), CgCfg<DV>::kSmem, rec.st, mapV, mapdO, qf, kf, eta, delta,
-               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, 0, D.eps, status, true, false);
+               reinterpret_cast<const float*>(ws + off_gpart), dkf, D.N, BH, D.S, 0, D.eps, status, beside, false);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
 // Gradient states (in a region of their own, so that the forward's stay) and dO . o, then dq on the forward states, beside it the scan of the
-// gradient states, `between` (the next step of the query side, if any), dV and beside it dk.
+// gradient states, `between` (the next step of the query side, if any), dV and beside it (dk_beside) dk.
 template <int DV, typename Between>
 inline hla_status launch_causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf,
                                          float* dkf, void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta,
-                                         LaunchRec& rec, bool run_between, Between&& between) {
+                                         LaunchRec& rec, bool dk_beside, bool run_between, Between&& between) {
     hla_status s = launch_causal_gradient_states<DV>(D, BH, qf, O, dO, ws, L, off_gpart, off_delta, rec);
-    if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, false, rec);
+    if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, false, false, rec);
     if (s == HLA_OK) s = launch_causal_gradient_scan(D, BH, ws, L, off_gpart, rec);
     if (s == HLA_OK && run_between) s = between();
     if (s == HLA_OK) s = launch_causal_backward_values<DV>(D, BH, qf, kf, dO, dV, ws, L, off_gpart, off_delta, rec);
-    if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, true, rec);
+    if (s == HLA_OK) s = launch_causal_backward_features<DV>(D, BH, qf, kf, V, dO, dqf, dkf, ws, L, fwd, off_gpart, off_delta, true, dk_beside, rec);
     return s;
 }
 template <typename Between>
 inline hla_status causal_backward(const Dims& D, int BH, const float* qf, const float* kf, const void* V, const void* O, const void* dO, float* dqf, float* dkf,
                                   void* dV, char* ws, const hla_ws_layout& L, const CausalPieces& fwd, size_t off_gpart, size_t off_delta, LaunchRec& rec,
-                                  bool run_between, Between&& between) {
+                                  bool dk_beside, bool run_between, Between&& between) {
     if (D.F != 3) return HLA_ERR_UNSUPPORTED;
-    if (D.d == 128) return launch_causal_backward<128>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec, run_between, between);
-    return launch_causal_backward<64>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec, run_between, between);
+    if (D.d == 128) return launch_causal_backward<128>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec, dk_beside, run_between, between);
+    return launch_causal_backward<64>(D, BH, qf, kf, V, O, dO, dqf, dkf, dV, ws, L, fwd, off_gpart, off_delta, rec, dk_beside, run_between, between);
 }
 
 }  // namespace tc

@@ -814,7 +814,7 @@ inline size_t vmod_plan(VmodPlan& p, int d, long long rows, size_t off) {
 
 template <int DV>
 inline hla_status launch_vmod(const VmodPlan& P, long long rows, const hla_vmlp* v, const void* T, const void* V, const void* dOut, void* Out, void* dT,
-                              void* dV, int accumulate_dV, bool backward, char* ws, int* status, int sm_count, LaunchRec& rec) {
+                              void* dV, int accumulate_dV, bool backward, bool dV_beside, char* ws, int* status, int sm_count, LaunchRec& rec) {
     using bf = __nv_bfloat16;
     bf* w1f = reinterpret_cast<bf*>(ws + P.w1f);
     bf* aux = reinterpret_cast<bf*>(ws + P.aux);
@@ -864,9 +864,9 @@ inline hla_status launch_vmod(const VmodPlan& P, long long rows, const hla_vmlp*
     launch_pdl(tc_vmlp_backward_kernel<DV, true>, grid, dim3(kVbThreads), VbCfg<DV>::kSmem, st, mapT, mapW1[0], mapW2[0], mapAux[0], mapdO, mapY2, mapdT,
                (const bf*)aux, 0, rows, status, false);
     if (!rec.end()) return HLA_ERR_CUDA;
-    rec.begin("tc_vmlp_backward_v");   // dV (+)= J2^T (dOut (.) Y1), beside dT
+    rec.begin("tc_vmlp_backward_v");   // dV (+)= J2^T (dOut (.) Y1), beside dT unless dV lies over an input of that pass
     launch_pdl(tc_vmlp_backward_kernel<DV, false>, grid, dim3(kVbThreads), VbCfg<DV>::kSmem, st, mapV, mapW1[1], mapW2[1], mapAux[1], mapdO, mapY1, mapdV,
-               (const bf*)(aux + (size_t)16 * DV), accumulate_dV, rows, status, true);
+               (const bf*)(aux + (size_t)16 * DV), accumulate_dV, rows, status, dV_beside);
     return rec.end() ? HLA_OK : HLA_ERR_CUDA;
 }
 
