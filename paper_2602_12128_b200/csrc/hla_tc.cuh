@@ -905,9 +905,8 @@ __global__ void __launch_bounds__(kBqThreads, 1) tc_bwd_query_kernel(const __gri
     const int tile0 = s * tiles_per;
     const int ntiles = max(0, min(tiles, tile0 + tiles_per) - tile0);
     float* out = part + ((size_t)bh * S + s) * M::kN * ld;
-    grid_launch_dependents();
     if (ntiles == 0) {
-        grid_dependency_wait();
+        grid_begin(false);
         for (int i = tid; i < M::kN * ld; i += kBqThreads) out[i] = 0.f;
         return;
     }
@@ -943,7 +942,7 @@ __global__ void __launch_bounds__(kBqThreads, 1) tc_bwd_query_kernel(const __gri
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_dependency_wait();
+    grid_begin(false);      // first kernel of a backward: the next one stages weights before its own wait, which a kernel of the caller may have just written
     // (zsym is read by the generator warps only; the named barrier keeps the other warps out of it)
     if (warp >= 4) {
         if (tid - 128 < M::kPad) zsym[tid - 128] = tid - 128 < M::kN ? state[((size_t)bh * M::kN + tid - 128) * ld + DV] : 0.f;
