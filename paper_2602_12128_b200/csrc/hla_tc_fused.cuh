@@ -66,8 +66,12 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
     constexpr int DP = M::kDphi;
     constexpr int HC = DV / 4;          // hidden units per GELU thread
     extern __shared__ uint8_t smem_raw[];
-    if (READOUT) grid_launch_dependents();
-    else grid_begin(false);      // first of its call: a kernel of the caller may have just written the weights that are staged now
+    if (READOUT) {
+        grid_launch_dependents();
+        grid_start_beside();      // only the state operand is the work of the kernel before this one; its loader waits for it
+    } else {
+        grid_begin(false);      // first of its call: a kernel of the caller may have just written the weights that are staged now
+    }
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float* bias = reinterpret_cast<float*>(smem + Cfg::kOffBias);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBars);
@@ -144,7 +148,6 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;     // D1[b] at columns 128*b, D2[b] at 256 + 32*b, readout accumulator at 320
-    if (READOUT) grid_start_beside();      // only the state operand is the work of the kernel before this one; its loader waits for it
     bool ok = true;
 
     if (warp == 0) {

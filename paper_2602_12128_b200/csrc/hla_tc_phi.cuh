@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
     const int ntiles = (int)(t1 - t0);
     const int nunits = ntiles * NMAPS;
 
+    grid_start_beside();      // the weights are older than the kernel before this one, which released this one after its own wait or behind one that waited
     constexpr int kRows = 16 * Cfg::kDgSteps, kB1Abs = kRows - 16 + Cfg::kB1Row;
     for (int i = tid; i < NMAPS * DV; i += kPbThreads) {
         const int m = i / DV;

@@ -38,8 +38,8 @@ template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setma
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The start of a kernel that needs nothing of its predecessor, only of the kernels before that one: the predecessor lets it be scheduled
 // after its own dependency wait (so those kernels are complete), and it calls grid_dependency_wait at its end, so that what follows may
-// rely on both.  The fence orders its reads after that; nothing is waited for.
-__device__ __forceinline__ void grid_start_beside() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// rely on both.  The fences order its reads, and those of the TMA unit, after that; nothing is waited for.
+__device__ __forceinline__ void grid_start_beside() { asm volatile("fence.acq_rel.gpu;\n\tfence.proxy.async.global;" ::: "memory"); }
 // Lets the next kernel's blocks be scheduled as soon as every block of this one has started.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // The two ends of a kernel that can run either way.  The next kernel is let go only here, after the wait: if it is one that runs beside
