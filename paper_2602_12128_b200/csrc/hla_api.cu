@@ -466,17 +466,18 @@ hla_status forward_impl(hla_ctx* ctx, const void* Q, const void* K, const void* 
             }
             // one kernel for the key maps and the state build -> reduction of its pieces -> one kernel for phi_q, readout
             // and normaliser
+            const bool early = phase == 0 && tc::query_starts_early(ctx->BH, ctx->D.N, ctx->sm_count);
             if (phase != 2) {
                 s = tc::phik_state(ctx->D, ctx->BH, ctx->phi_k, K, V, ws, ctx->L, ctx->off_part, ctx->k_pieces, ctx->sm_count, ctx->rec);
                 if (s != HLA_OK) return s;
                 s = tc::reduce_pieces(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, ctx->off_part, ctx->k_pieces, tc::fused_key_grid(ctx->BH, ctx->D.N, ctx->sm_count),
-                                      phase == 0 && tc::query_starts_early(ctx->BH, ctx->D.N, ctx->sm_count) ? tc::Start::kLetGo : tc::Start::kWait, ctx->rec);
+                                      early ? tc::Start::kLetGo : tc::Start::kWait, ctx->rec);
                 if (s != HLA_OK || phase == 1) return s;
             } else {
                 s = tc::emit_from_state(ctx->tcp, ctx->D, ctx->BH, ws, ctx->L, false, ctx->rec);
                 if (s != HLA_OK) return s;
             }
-            return tc::phiq_readout(ctx->tcp, ctx->D, ctx->BH, &ctx->phi_q, Q, O, ws, ctx->L, ctx->sm_count, ctx->rec);
+            return tc::phiq_readout(ctx->tcp, ctx->D, ctx->BH, &ctx->phi_q, Q, O, ws, ctx->L, early, ctx->sm_count, ctx->rec);
         } else {
             qf = static_cast<const float*>(Q);
             kf = static_cast<const float*>(K);

@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kFqThreads, 1) tc_phiq_readout_kernel(const __
 
 template <int DV, int F>
 inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, const hla_mlp* phi_q, const void* Q, void* O, char* ws,
-                                      const hla_ws_layout& L, int sm_count, LaunchRec& rec) {
+                                      const hla_ws_layout& L, bool early, int sm_count, LaunchRec& rec) {
     CUtensorMap mapQ, mapW1, mapB3, mapO;
     __nv_bfloat16* b3 = reinterpret_cast<__nv_bfloat16*>(ws + P.b3);
     if (!make_map_bhnd(&mapQ, Q, BH, D.N, DV, kTileTokens) || !make_map_bhnd(&mapO, O, BH, D.N, DV, kTileTokens) ||
@@ -375,9 +375,9 @@ inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, cons
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles;
     const int grid = (int)(total < sm_count ? total : sm_count);
-    // (see query_starts_early) the blocks of the reduction, twelve to an SM, sit on the SMs that the last CTAs are waiting for: those start 4 to
-    // 10 us late and would end as late.  They get up to four tiles less (a tile takes 0.8 to 1.4 us), at most half of their share.
-    const bool early = query_starts_early(BH, D.N, sm_count);
+    // early: the reduction lets this kernel go before its own wait (see query_starts_early).  Its blocks, twelve to an SM, sit on the SMs
+    // that the last CTAs are waiting for: those start 4 to 10 us late and would end as late.  They get up to four tiles less (a tile takes
+    // 0.8 to 1.4 us), at most half of their share.
     int late = early ? (MT<F>::kPad / kReRows * BH + 11) / 12 : 0, fewer = (int)(total / grid / 2 < 4 ? total / grid / 2 : 4);
     if (late > grid / 2) late = 0;
     rec.begin("tc_phiq_readout");
@@ -389,13 +389,13 @@ inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, cons
 }
 
 inline hla_status phiq_readout(const Plan& P, const Dims& D, int BH, const hla_mlp* phi_q, const void* Q, void* O, char* ws, const hla_ws_layout& L,
-                               int sm_count, LaunchRec& rec) {
+                               bool early, int sm_count, LaunchRec& rec) {
     if (D.F == 3) {
-        if (D.d == 128) return launch_phiq_readout<128, 3>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
-        return launch_phiq_readout<64, 3>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
+        if (D.d == 128) return launch_phiq_readout<128, 3>(P, D, BH, phi_q, Q, O, ws, L, early, sm_count, rec);
+        return launch_phiq_readout<64, 3>(P, D, BH, phi_q, Q, O, ws, L, early, sm_count, rec);
     }
-    if (D.d == 128) return launch_phiq_readout<128, 2>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
-    return launch_phiq_readout<64, 2>(P, D, BH, phi_q, Q, O, ws, L, sm_count, rec);
+    if (D.d == 128) return launch_phiq_readout<128, 2>(P, D, BH, phi_q, Q, O, ws, L, early, sm_count, rec);
+    return launch_phiq_readout<64, 2>(P, D, BH, phi_q, Q, O, ws, L, early, sm_count, rec);
 }
 
 }  // namespace tc
