@@ -338,11 +338,10 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
             fence_proxy_async();
         }
         named_barrier(2, kThreads);
-        // Self-summing without state_out: the scan that runs beside this kernel overwrites the pieces and the carried state.  It starts when
-        // every CTA has got here, or, where a CTA begins another head later and reads that head's carried state then, has ended.
-        const bool reads_later = self_sum && carry && !state_out && nwork > 0 && (w0 + nwork - 1) / T != w0 / T;
-        if (t == 0 && !reads_later) grid_launch_dependents();
         if (nwork > 0 && ends_here(bh)) store_state_after<DV, kThreads>(state_out + (size_t)bh * kMono * ld, before, t, init + (size_t)slot * kMono * ld);
+        // Self-summing without state_out (one head per CTA): the scan that runs beside this kernel overwrites the pieces and the carried state.
+        // It starts when every CTA has got here.
+        if (t == 0) grid_launch_dependents();
     }
 
     if (warp == 0) {
