@@ -335,7 +335,8 @@ hla_status hla_create(const hla_config* cfg, hla_ctx** out) {
     int S = c.n_splits, fewest = c.n_splits;
     if (S == 0) {
         if (x->tc) {
-            // At least 4 tiles per CTA (8 left 60 CTAs of a step of 12 heads x 4999 tokens: 36.2 us against 34.7).
+            // At least 4 tiles per CTA.  Feature-level steps with at least 2, 4 and 8, us: 12 heads x 4999 tokens, d = 64, 41.2, 32.2 and 35.1;
+            // 24 x 2500, d = 128, 40.8, 39.2 and 42.3; 4 x 4000, d = 128, 28.9, 28.5 and 31.2; 12 x 2000, d = 64, 28.9, 28.9 and 30.1.
             S = wave_splits(x->BH, tiles, 4, x->sm_count);
             fewest = wave_splits(x->BH, tiles, 8, x->sm_count);
         } else {
@@ -466,7 +467,7 @@ hla_status forward_impl(hla_ctx* ctx, const void* Q, const void* K, const void* 
             }
             // one kernel for the key maps and the state build -> reduction of its pieces -> one kernel for phi_q, readout
             // and normaliser
-            const bool early = phase == 0 && tc::query_starts_early(ctx->BH, ctx->D.N, ctx->sm_count);
+            const bool early = phase == 0 && tc::query_starts_early(ctx->D.F, ctx->BH, ctx->D.N, ctx->sm_count);
             if (phase != 2) {
                 s = tc::phik_state(ctx->D, ctx->BH, ctx->phi_k, K, V, ws, ctx->L, ctx->off_part, ctx->k_pieces, ctx->sm_count, ctx->rec);
                 if (s != HLA_OK) return s;

@@ -153,9 +153,8 @@ inline bool make_map_2d(CUtensorMap* m, const void* ptr, size_t rows, int cols, 
     return true;
 }
 
-// Launch with programmatic stream serialization (see grid_dependency_wait): the kernel's blocks may start while the
-// previous kernel of the stream drains; every kernel launched this way waits for its predecessor before it touches
-// global memory that the library's kernels write or read.
+// Launch with programmatic stream serialization (see grid_dependency_wait for the rules): the kernel's blocks may start while the previous
+// kernel of the stream drains.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -145,7 +145,9 @@ __device__ __forceinline__ void tmem_st_state(uint32_t taddr, const float (&v)[8
 // themselves and every CTA adds those before its own (after `carry`, if any), in the order of the scan and to the same bits.  The sum is
 // formed in shared memory at the start of a sweep: with the scan before it and one warp per 16 rows loading what it needed, the
 // two and the release between them took 10 of the 22 us of a call of 12 heads x 500 tokens.  A CTA reads all the pieces before its own
-// from L2, so this is done for few pieces per head only.
+// from L2, so this is done for few pieces per head only.  Forward with the phi maps, d = 128, in the sweep against by a scan, us: 24 heads x 4000
+// tokens (7 pieces) 53.9 and 58.3; 12 x 12600 (13) 87.0 and 85.3; 10 x 12600 (16) 73.0 and 74.7; 8 x 12600 (19) 59.6 and 61.1; 4 x 4000 (32)
+// 31.5 and 27.3; 2 x 8000 (63) 42.1 and 29.1.
 constexpr int kSelfPrefixPieces = 16;
 inline bool self_prefix(int S) { return S <= kSelfPrefixPieces; }
 // THREADS threads, numbered t: [56][ld] floats of the state before piece `slot` (the head's first slot is `base`, `carry` its carried

@@ -46,10 +46,16 @@ template <int DV, int F> struct FqCfg {
     static constexpr int kSmem = kSmemUsed > 120 * 1024 ? kSmemUsed : 120 * 1024;   // one CTA per SM (512 TMEM columns)
 };
 
+// CTAs of the query side that wait for the SMs on which the blocks of the reduction sit, twelve to an SM.
+inline int query_late_ctas(int F, int BH) { return (mono_pad(F) / kReRows * BH + 11) / 12; }
 // Whether the CTAs of the query side may start while the reduction before them is still waiting for the key side: with few tiles per CTA the
-// set-up and the first tiles it hides count (24 heads x 4096 tokens, 5 tiles per CTA: 32.2 -> 30.2 us; 12 heads x 12600, 8 tiles:
-// 266 -> 264 us); in long calls they take bandwidth from the key side's last CTAs (24 heads x 32760, 41 tiles: 239.7 -> 241 us).
-inline bool query_starts_early(int BH, int N, int sm_count) { return (long long)BH * ((N + kTileTokens - 1) / kTileTokens) <= 16ll * sm_count; }
+// set-up and the first tiles that it hides count (d = 128, early against not, us: 24 heads x 4096 tokens, 5 tiles per SM, 41.3 and 43.7;
+// 12 x 12600, 8 tiles, 53.4 and 57.0; 24 x 11000, 14 tiles, 73.7 and 75.7; 48 x 2000 42.2 and 43.8).  In long calls the early CTAs take bandwidth
+// from the key side's last ones (24 x 32760, 41 tiles, 241 and 239.7), and with so many heads that the late CTAs are more than half of
+// all, their smaller shares cannot be made up for (64 heads: x 1000 d = 64 26.3 and 25.8, x 3600 72.2 and 71.8; 96 x 2000 64.4 and 64.0).
+inline bool query_starts_early(int F, int BH, int N, int sm_count) {
+    return (long long)BH * ((N + kTileTokens - 1) / kTileTokens) <= 16ll * sm_count && query_late_ctas(F, BH) <= sm_count / 2;
+}
 // First work item of CTA c: even shares, but `fewer` items less for the last `late` CTAs.
 __host__ __device__ inline int query_share(long long total, int c, int G, int late, int fewer) {
     return (int)((total + (long long)late * fewer) * c / G) - (c > G - late ? fewer * (c - (G - late)) : 0);
@@ -375,10 +381,10 @@ inline hla_status launch_phiq_readout(const Plan& P, const Dims& D, int BH, cons
     const int tiles = (D.N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles;
     const int grid = (int)(total < sm_count ? total : sm_count);
-    // early: the reduction lets this kernel go before its own wait (see query_starts_early).  Its blocks, twelve to an SM, sit on the SMs
-    // that the last CTAs are waiting for: those start 4 to 10 us late and would end as late.  They get up to four tiles less (a tile takes
+    // early: the reduction lets this kernel go before its own wait (see query_starts_early).  Its blocks sit on the SMs that the last CTAs
+    // are waiting for: those start 4 to 10 us late and would end as late.  They get up to four tiles less (a tile takes
     // 0.8 to 1.4 us), at most half of their share.
-    int late = early ? (MT<F>::kPad / kReRows * BH + 11) / 12 : 0, fewer = (int)(total / grid / 2 < 4 ? total / grid / 2 : 4);
+    int late = early ? query_late_ctas(F, BH) : 0, fewer = (int)(total / grid / 2 < 4 ? total / grid / 2 : 4);
     if (late > grid / 2) late = 0;
     rec.begin("tc_phiq_readout");
     launch_pdl(tc_phiq_readout_kernel<DV, F>, grid, dim3(kFqThreads), FqCfg<DV, F>::kSmem, rec.st,

@@ -31,10 +31,14 @@ template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setma
 template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // ---- programmatic dependent launch --------------------------------------------------
-// Every tensor-core kernel is launched with the programmatic-stream-serialization attribute: its blocks may be
-// scheduled while the previous kernel of the stream is still draining, run their set-up (barriers, TMEM, weight
-// staging) and then wait here until the previous kernel has completed and its writes are visible.  No global memory
-// that another kernel of the library writes or reads is touched before this wait.
+// The kernels are launched with the programmatic-stream-serialization attribute: their blocks may be scheduled as soon as every block of the
+// previous kernel of the stream has called grid_launch_dependents (or has ended), run their set-up (barriers, TMEM, tables) and wait
+// here until the previous kernel has completed and its writes are visible.  Two rules keep this sound:
+//   - What a kernel reads or overwrites before its own wait (or without one at its start, see below) belongs to kernels older than its
+//     predecessor: inputs, weights, features.  A kernel in front of such a one therefore lets it go only after its own wait, or always runs
+//     behind a kernel that has done so (the readout, the key pass and the fused query side behind a reduction; the reduction of a short
+//     forward, Start::kLetGo, behind the fused key side).  The first kernel of every call waits before it lets the next one go.
+//   - Every kernel waits for its predecessor before it ends, so that a completed kernel stands for all before it.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The start of a kernel that needs nothing of its predecessor, only of the kernels before that one: the predecessor lets it be scheduled
 // after its own dependency wait (so those kernels are complete), and it calls grid_dependency_wait at its end, so that what follows may

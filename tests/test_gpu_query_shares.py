@@ -1,5 +1,5 @@
 """Fused query side with uneven shares (its last CTAs start late and get fewer tiles): one and two tiles per CTA, shares that do not divide,
-the longest calls that do it and the first that does not.  Every row of O and eta is written, and right in the first, a middle and the last head."""
+the longest calls and the most heads that do it and the first that does not.  Every row of O and eta is written, and right in the first, a middle and the last head."""
 import numpy as np
 import pytest
 import torch
@@ -11,7 +11,8 @@ from hla_testlib import TOL, dev_weights, relerr, to_dev, to_np
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,H,N", [(128, 37, 512), (64, 37, 1025), (128, 5, 128 * 59 + 1), (64, 16, 128 * 148), (64, 16, 128 * 148 + 1)])
+@pytest.mark.parametrize("d,H,N", [(128, 37, 512), (64, 37, 1025), (128, 5, 128 * 59 + 1), (64, 16, 128 * 148), (64, 16, 128 * 148 + 1),
+                                     (128, 44, 300), (128, 45, 300), (64, 55, 300), (64, 56, 300)])
 @pytest.mark.parametrize("F,dphi", [(3, 6), (2, 12)])
 def test_every_tile_has_an_owner(d, H, N, F, dphi):
     s = synth.HlaShape("t", 1, H, N, d, "bf16", "rms_qk", F=F, d_phi=dphi)
