@@ -92,13 +92,14 @@ simt::PhiWeights<T> pack_weights(const hla_mlp* m, int n) {
 }
 
 // One CTA per SM: S * heads CTAs run in ceil(S * heads / SMs) waves.  The split count that fills its waves best (each extra wave is charged
-// 2 % for its start-up and drain), with at least `least` tiles per CTA.
+// 2 % for its start-up and drain), with at least 8 tiles per CTA, or `least` as long as one wave holds all CTAs.
 int wave_splits(int BH, int tiles, int least, int sm_count) {
-    const int smax = tiles / least > 1 ? (tiles / least < 64 ? tiles / least : 64) : 1;
+    const int smax = tiles / least < 64 ? tiles / least : 64;
     int S = 1;
     double best = -1.0;
-    for (int cand = 1; cand <= smax; ++cand) {
+    for (int cand = 1; cand <= smax || cand == 1; ++cand) {
         const long long ctas = (long long)cand * BH;
+        if (cand > 1 && cand > tiles / 8 && ctas > sm_count) break;
         const long long waves = (ctas + sm_count - 1) / sm_count;
         const double score = (double)ctas / (double)(waves * sm_count) - 0.02 * (double)(waves - 1);
         if (score > best + 1e-9) { best = score; S = cand; }

@@ -53,16 +53,29 @@ def test_create_defaults_and_layout():
     binding.hla_destroy(ctx)
 
 
-@pytest.mark.parametrize("kw", [dict(H=17, N=1400, d=32, dtype=binding.HLA_F32), dict(B=2, H=7, N=3534, d=16), dict(B=4, H=5, N=2349, d=8, F=2, dtype=binding.HLA_F32),
-                                dict(H=25, N=11045, F=2, phi=binding.HLA_PHI_NONE), dict(H=33, N=8458, d=64, phi=binding.HLA_PHI_NONE, causal=1)])
+@pytest.mark.parametrize("kw", [dict(H=25, N=11045, F=2, phi=binding.HLA_PHI_NONE), dict(H=33, N=8458, d=64, phi=binding.HLA_PHI_NONE, causal=1),
+                                dict(H=17, N=1400, d=32, dtype=binding.HLA_F32), dict(B=2, H=7, N=3534, d=16), dict(B=4, H=5, N=2349, d=8, F=2, dtype=binding.HLA_F32),
+                                dict(H=4, N=7642, d=64, causal=1)])
 def test_splits_for_speed_do_not_push_a_workspace_out_of_the_static_array(kw):
     st, ctx = create(**kw)
     assert st == binding.HLA_OK
     S = binding.hla_workspace_layout(ctx).n_splits
     assert binding.hla_workspace_bytes(ctx) <= binding.HLA_STATIC_WS_BYTES
     binding.hla_destroy(ctx)
+    if kw.get("phi") == binding.HLA_PHI_NONE:      # (fits with the count that one wave of CTAs takes)
+        return
     st, ctx = create(n_splits=S + 1, **kw)      # as many as fit
     assert st == binding.HLA_OK and binding.hla_workspace_bytes(ctx) > binding.HLA_STATIC_WS_BYTES
+    binding.hla_destroy(ctx)
+
+
+@pytest.mark.parametrize("H,N,least", [(8, 20000, 8), (20, 15000, 8), (12, 4999, 4), (4, 4000, 4), (1, 700, 4), (300, 300, 1)])
+def test_several_waves_of_splits_have_eight_tiles_each(H, N, least):
+    st, ctx = create(H=H, N=N, d=64, phi=binding.HLA_PHI_NONE, causal=1)
+    assert st == binding.HLA_OK
+    S, tiles = binding.hla_workspace_layout(ctx).n_splits, (N + 127) // 128
+    assert S == 1 or tiles // S >= least
+    assert S == 1 or S * H <= 148 or tiles // S >= 8
     binding.hla_destroy(ctx)
 
 
