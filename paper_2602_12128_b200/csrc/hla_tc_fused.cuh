@@ -52,9 +52,11 @@ inline int query_late_ctas(int F, int BH) { return (mono_pad(F) / kReRows * BH +
 // set-up and the first tiles that it hides count (d = 128, early against not, us: 24 heads x 4096 tokens, 5 tiles per SM, 41.3 and 43.7;
 // 12 x 12600, 8 tiles, 53.4 and 57.0; 24 x 11000, 14 tiles, 73.7 and 75.7; 48 x 2000 42.2 and 43.8).  In long calls the early CTAs take bandwidth
 // from the key side's last ones (24 x 32760, 41 tiles, 241 and 239.7), and with so many heads that the late CTAs are more than half of
-// all, their smaller shares cannot be made up for (64 heads: x 1000 d = 64 26.3 and 25.8, x 3600 72.2 and 71.8; 96 x 2000 64.4 and 64.0).
+// all, their smaller shares cannot be made up for (64 heads: x 1000 d = 64 26.3 and 25.8, x 3600 72.2 and 71.8; 96 x 2000 64.4 and 64.0) unless
+// the tiles leave SMs free (d = 64: 60 heads x 128 tokens 12.9 and 14.5; 100 x 128 16.9 and 17.0; 60 x 256 17.1 and 17.3).
 inline bool query_starts_early(int F, int BH, int N, int sm_count) {
-    return (long long)BH * ((N + kTileTokens - 1) / kTileTokens) <= 16ll * sm_count && query_late_ctas(F, BH) <= sm_count / 2;
+    const long long total = (long long)BH * ((N + kTileTokens - 1) / kTileTokens);
+    return total <= sm_count || (total <= 16ll * sm_count && query_late_ctas(F, BH) <= sm_count / 2);
 }
 // First work item of CTA c: even shares, but `fewer` items less for the last `late` CTAs.
 __host__ __device__ inline int query_share(long long total, int c, int G, int late, int fewer) {

@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d,H,N", [(128, 37, 512), (64, 37, 1025), (128, 5, 128 * 59 + 1), (64, 16, 128 * 148), (64, 16, 128 * 148 + 1),
-                                     (128, 44, 300), (128, 45, 300), (64, 55, 300), (64, 56, 300)])
+                                     (128, 44, 300), (128, 45, 300), (64, 55, 300), (64, 56, 300),
+                                     (64, 148, 100), (64, 149, 100)])
 @pytest.mark.parametrize("F,dphi", [(3, 6), (2, 12)])
 def test_every_tile_has_an_owner(d, H, N, F, dphi):
     s = synth.HlaShape("t", 1, H, N, d, "bf16", "rms_qk", F=F, d_phi=dphi)
