@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             for (int it = 0; it < ntiles; ++it) {
                 const int st = it % kStages, u = it / kStages;
                 if (!mbar_wait(&empty[st], (u & 1) ^ 1)) { report_timeout(status, 101); break; }
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) tc_state_build_kernel(const __g
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16(128, M::kPad, true, true);
             for (int it = 0; it < ntiles; ++it) {
                 const int st = it % kStages, u = it / kStages;
@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(kRoThreads, 1) tc_readout_kernel(const __grid_
     bool ok = true;
 
     if (warp == kRoMmaWarp) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16(128, Cfg::kNmma, false, false);
             const uint32_t b3a = smem_u32(smem + Cfg::kOffB3);
             int cur_bh = -1, nload = 0;
@@ -1249,7 +1249,7 @@ __global__ void __launch_bounds__(kBkThreads, 1) tc_bwd_key_kernel(const __grid_
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             for (int it = 0; it < nwork; ++it) {
                 const int work = w0 + it, bh = work / tiles_per_head, tile = work % tiles_per_head;
                 const int st = it & 1, u = it >> 1;
@@ -1260,7 +1260,7 @@ __global__ void __launch_bounds__(kBkThreads, 1) tc_bwd_key_kernel(const __grid_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc4 = idesc_bf16(128, M::kPad, false, false);    // G  = V (K-major over g) * dCsym (K-major over g)
             const uint32_t idesc3 = idesc_bf16(128, DV, false, false);         // dV = Tsym_k (K-major over m) * dCsym^T (K-major over m)
             const uint32_t b3a = smem_u32(smem + Cfg::kOffB3), bqa = smem_u32(smem + Cfg::kOffBq);

@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     }
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             for (int it = 0; it < nwork; ++it) {
                 const int st = it & 1, u = it >> 1, work = work_of(it);
                 if (!mbar_wait_c(&stage_free[st], (u & 1) ^ 1)) { report_timeout(status, 901); break; }
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t id_p = idesc_bf16(128, 128, false, false);
             const uint32_t id_r = idesc_bf16(128, Cfg::kNAcc, false, true);
             const uint32_t b3base = smem_u32(smem + Cfg::kOffB3);
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kCaThreads, 1) tc_causal_forward_kernel(const 
     } else if (warp == kCaStateMmaWarp) {
         // The state products are issued by a thread of their own: they depend on nothing the other products make, and the
         // chain state -> image -> readout of consecutive tiles is the long one.
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t id_s = idesc_bf16(64, Cfg::kNState, true, true);
             int begun = 0;
             for (int it = 0; it < nwork; ++it) {

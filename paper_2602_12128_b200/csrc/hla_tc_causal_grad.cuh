@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
     } else if (warp < kCgRowWarp0) {
         reg_dec<kCgIssueRegs>();
         if (warp == 0) {
-            if (lane == 0) {
+            if (elect_one()) {
                 Pos p = pos_of(0);
                 for (int it = 0; it < nwork; ++it, step(p, 1)) {
                     const int st = it & 1, u = it >> 1, tile = p.tile, bh = p.bh;
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                 }
             }
         } else if (warp == 1) {
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t id_r = idesc_bf16(128, 64, false, false);
                 const uint32_t id_w = idesc_bf16(128, 64, false, true);
                 const uint32_t b3base = smem_u32(smem + Cfg::kOffB3);
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                 }
             }
         } else if (warp == kCgScMmaWarp) {
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t id_s = idesc_bf16(128, 128, false, false);
                 for (int it = 0; it < nwork; ++it) {
                     const int st = it & 1, u = it >> 1;
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) tc_causal_grad_kernel(const __g
                 }
             }
         } else {
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t id_st = idesc_bf16(64, Cfg::kNState, true, true);
                 for (int it = 0; it < nwork; ++it) {
                     const int st = it & 1, u = it >> 1;

@@ -159,7 +159,7 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0 && nwork > 0) {
+        if (elect_one() && nwork > 0) {
             mbar_arrive_expect_tx(w_full, Cfg::kW1Bytes);
             for (int b = 0; b < DV / 64; ++b) tma_load_2d(smem + Cfg::kOffW1 + b * (DV * 128), &mapW1, w_full, b * 64, 0);
             for (int it = 0; it < nwork; ++it) {
@@ -172,7 +172,7 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && nwork > 0) {      // D1[b] = Q tile * W1
+        if (elect_one() && nwork > 0) {      // D1[b] = Q tile * W1
             const uint32_t idesc1 = idesc_bf16(128, DV, false, true);   // Q K-major, W1 [in][hidden] MN-major
             const uint64_t xd = smem_desc_sw128(smem_u32(smem + Cfg::kOffX), 16, 1024);
             const uint64_t wd = smem_desc_sw128(smem_u32(smem + Cfg::kOffW1), DV * 128, 1024);
@@ -196,7 +196,7 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
             if (!good) report_timeout(status, 702);
         }
     } else if (warp == 1) {
-        if (lane == 0 && nwork > 0) {      // D2[b] = G[b] * W2
+        if (elect_one() && nwork > 0) {      // D2[b] = G[b] * W2
             const uint32_t idesc2 = idesc_bf16(128, 16, false, false);           // G from TMEM, W2 operand K-major
             const uint64_t vd = smem_desc_sw128(smem_u32(smem + Cfg::kOffW2), 16, 1024);
             bool good = true;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void phiq_cta(const CUtensorMap& mapQ, const CUtensor
             if (!good) report_timeout(status, 703);
         }
     } else if (warp == kFqReadoutMmaWarp) {
-        if (READOUT && lane == 0 && nwork > 0) {      // [num | eta] = monomial tile * state operand of the tile's head
+        if (READOUT && elect_one() && nwork > 0) {      // [num | eta] = monomial tile * state operand of the tile's head
             const uint32_t idesc3 = idesc_bf16(128, Cfg::kNmma, false, false);   // monomial tile K-major, state operand K-major over the monomials
             const uint64_t ad = smem_desc_sw128(smem_u32(smem + Cfg::kOffA), 16, 1024);
             const uint64_t bd = smem_desc_sw128(smem_u32(smem + Cfg::kOffB3), 16, 1024);

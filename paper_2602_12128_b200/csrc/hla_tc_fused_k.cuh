@@ -244,7 +244,7 @@ __device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const Ph
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_arrive_expect_tx(w_full, NM * Cfg::kW1Bytes);
             for (int m = 0; m < NM; ++m)
                 for (int b = 0; b < DV / 64; ++b)
@@ -259,7 +259,7 @@ __device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const Ph
             }
         }
     } else if (warp == 2) {
-        if (lane == 0) {      // D1[b] = K tile * W1[m] + 1 * b1[m]
+        if (elect_one()) {      // D1[b] = K tile * W1[m] + 1 * b1[m]
             const uint32_t idesc1 = idesc_bf16(128, DV, false, true);   // K tile K-major, W1 [in][hidden] MN-major
             const uint64_t xd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffX), 16, 1024);
             const uint64_t wd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffW1), DV * 128, 1024);
@@ -281,7 +281,7 @@ __device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const Ph
             if (!good) report_timeout(status, 802);
         }
     } else if (warp == 1) {
-        if (lane == 0) {      // D2[b] = G[b] * W2[m]
+        if (elect_one()) {      // D2[b] = G[b] * W2[m]
             const uint32_t idesc2 = idesc_bf16(128, 16, false, false);  // G from TMEM, W2 operand K-major
             const uint64_t vd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffW2), 16, 1024);
             bool good = true;
@@ -300,7 +300,7 @@ __device__ __forceinline__ void phik_state_cta(const CUtensorMap& mapK, const Ph
             if (!good) report_timeout(status, 803);
         }
     } else if (warp == kFkStateWarp) {
-        if (lane == 0) {      // Csym^T += V tile^T (MN-major, M = value channels) * folded key tile (MN-major, N = 64), K = 128 tokens
+        if (elect_one()) {      // Csym^T += V tile^T (MN-major, M = value channels) * folded key tile (MN-major, N = 64), K = 128 tokens
             const uint32_t idesc = idesc_bf16(128, M::kPad, true, true);
             const uint32_t va = smem_u32(smem + Cfg::kOffV), fa = smem_u32(smem + Cfg::kOffF);
             auto load_v = [&](int it) {

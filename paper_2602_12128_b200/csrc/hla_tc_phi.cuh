@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0 && ntiles > 0) {
+        if (elect_one() && ntiles > 0) {
             mbar_arrive_expect_tx(w_full, NMAPS * Cfg::kW1Bytes);
             for (int m = 0; m < NMAPS; ++m)
                 for (int b = 0; b < DV / 64; ++b)
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && ntiles > 0) {      // h[b] = X * W1[m]
+        if (elect_one() && ntiles > 0) {      // h[b] = X * W1[m]
             const uint32_t idesc1 = idesc_bf16(128, DV, false, true);    // X K-major, W1 [in][hidden] MN-major
             const uint64_t xd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffX), 16, 1024);
             const uint64_t wd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffW1), DV * 128, 1024);
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
             if (!good) report_timeout(status, 602);
         }
     } else if (warp == 1) {
-        if (lane == 0 && ntiles > 0) {
+        if (elect_one() && ntiles > 0) {
             const uint32_t idesc_dg = idesc_bf16(128, DV, false, true);  // dg = dp (K-major) * W2^T (MN-major)
             const uint32_t idesc2 = idesc_bf16(128, DV, false, false);   // dX = dh (TMEM) * W1 as [in][hidden] (K-major)
             const uint64_t pd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffDp), 16, 1024);

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0 && ntiles > 0) {
+        if (elect_one() && ntiles > 0) {
             mbar_arrive_expect_tx(w_full, 2 * Cfg::kWBytes + Cfg::kAuxBytes);
             for (int b = 0; b < DV / 64; ++b) {
                 tma_load_2d(smem + Cfg::kOffW1 + b * (DV * 128), &mapW1, w_full, b * 64, 0);
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && ntiles > 0) {      // D1[b] = X W1' + [-mu, sigma] [c; b1']
+        if (elect_one() && ntiles > 0) {      // D1[b] = X W1' + [-mu, sigma] [c; b1']
             const uint32_t idesc1 = idesc_bf16(128, DV, false, true);   // X K-major, W1' [in][hidden] MN-major
             const uint64_t xd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffX), 16, 1024);
             const uint64_t wd = smem_desc_sw128(smem_u32(smem + Cfg::kOffW1), DV * 128, 1024);
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __
             if (!good) report_timeout(status, 1102);
         }
     } else if (warp == 1) {
-        if (lane == 0 && ntiles > 0) {      // D2 = G W2 + 1 b2
+        if (elect_one() && ntiles > 0) {      // D2 = G W2 + 1 b2
             const uint32_t idesc2 = idesc_bf16(128, DV, false, true);   // G from TMEM, W2 [hidden][out] MN-major
             const uint64_t wd = smem_desc_sw128(smem_u32(smem + Cfg::kOffW2), DV * 128, 1024);
             const uint64_t ad = smem_desc_sw128(smem_u32(smem + Cfg::kOffAux), 2048, 1024);
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
     bool ok = true;
 
     if (warp == 0) {
-        if (lane == 0 && ntiles > 0) {
+        if (elect_one() && ntiles > 0) {
             mbar_arrive_expect_tx(w_full, 2 * Cfg::kWBytes + Cfg::kAuxBytes);
             for (int b = 0; b < DV / 64; ++b) {
                 tma_load_2d(smem + Cfg::kOffW1 + b * (DV * 128), &mapW1, w_full, b * 64, 0);
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && ntiles > 0) {      // h = X W1' + [-mu, sigma] [c; b1']
+        if (elect_one() && ntiles > 0) {      // h = X W1' + [-mu, sigma] [c; b1']
             const uint32_t idesc1 = idesc_bf16(128, DV, false, true);
             const uint64_t xd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffX), 16, 1024);
             const uint64_t wd = smem_desc_sw128(smem_u32(smem + Cfg::kOffW1), DV * 128, 1024);
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
             if (!good) report_timeout(status, 1202);
         }
     } else if (warp == 1) {
-        if (lane == 0 && ntiles > 0) {
+        if (elect_one() && ntiles > 0) {
             const uint32_t idesc_k = idesc_bf16(128, DV, false, false);
             const uint64_t yd = smem_desc_sw128(smem_u32(smem + Cfg::kOffDy), 16, 1024);       // dy tile, K-major over the output channels
             const uint64_t w2d = smem_desc_sw128(smem_u32(smem + Cfg::kOffW2), 16, 1024);      // W2 [hidden][out] read K-major: N = hidden, K = out
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
         }
     } else if (warp == kVbStoreWarp) {
         // the result tile leaves through TMA; its X stage is free for the next load once the store has read it
-        if (lane == 0) {
+        if (elect_one()) {
             for (int it = 0; it < ntiles; ++it) {
                 const int st = it & 1;
                 if (!mbar_wait(&o_full[st], (it >> 1) & 1)) { report_timeout(status, 1210); break; }
