@@ -36,22 +36,22 @@ __device__ __forceinline__ float2 gelu2_twice(float2 x) {
 __device__ __forceinline__ __nv_bfloat16 half_bf16(__nv_bfloat16 w) { return __float2bfloat16_rn(0.5f * __bfloat162float(w)); }
 // dg GELU'(x) of a pair of elements, with dg already halved (the 1/2 sits in the staged W2^T, exact in bf16), through one tanh.approx
 // per element:
-//   th = tanh(x (a + b x^2)),   2 GELU'(x) ~ (1 + th) (1 + V (1 - th)) = 1 + V + th (1 - V th),   V = x (C0 + C1 x^2)
+//   th = tanh(x (a + b x^2)),   2 GELU'(x) ~ (1 + th) (1 + V (1 - th)) = 1 + th + V (1 - th^2),   V = x (C0 + C1 x^2)
 // (the derivative of a tanh-form GELU whose inner derivative is a free polynomial); a, b, C0, C1 are fitted against the
 // exact derivative (fit_gelu_tanh.py, which prints twice C0 and C1: |error| < 1.5e-4, 3.8e-5 in the mean square over N(0,1), before the 2^-11 relative error of
-// tanh.approx; < 1.3e-3 with it).  Evaluated with -V so that every step is one packed multiply or fma: nine packed and two
-// special-function instructions per pair of elements.  (A linear inner derivative, C1 = 0, takes seven, but its mean-square error is
-// 8.6e-5: errors of gradients against 64 bits grew by up to 0.6 %, for 1 % of a training step (B = 2, H = 24, N = 32760, d = 128:
-// 1286 against 1299 us).)
+// tanh.approx; < 1.3e-3 with it).  Evaluated as dg + dg (th + V (1 - th^2)) with -V so that every step is one packed multiply or fma: eight
+// packed and two special-function instructions per pair of elements.  Sixteen warps alone on an SM take 1280 cycles for a 128 x 128 tile,
+// bound by the FMA pipe; as 1 + V + th (1 - V th) it was nine instructions and 1376 cycles, and V cancelled against itself for large |x|.  (A
+// linear inner derivative, C1 = 0, saves one or two more, but its mean-square error is 8.6e-5: errors of gradients against 64 bits grew by
+// up to 0.6 %.)
 constexpr float kGradA = 0.69631102f, kGradB = 0.02936904f, kGradC0 = 0.89902785f, kGradC1 = -0.010848315f;
 __device__ __forceinline__ float2 times_gelu_grad2(float2 dg, float2 x) {
     const float2 t = __fmul2_rn(x, x);
     const float2 u = __fmul2_rn(x, __ffma2_rn(t, splat2(kGradB), splat2(kGradA)));
     const float2 th = make_float2(tanh_approx(u.x), tanh_approx(u.y));
     const float2 vn = __fmul2_rn(x, __ffma2_rn(t, splat2(-kGradC1), splat2(-kGradC0)));      // -V
-    const float2 a1 = __ffma2_rn(vn, th, splat2(1.f));          // 1 - V th
-    const float2 b1 = __ffma2_rn(th, a1, splat2(1.f));          // 1 + th (1 - V th)
-    return __fmul2_rn(dg, __ffma2_rn(vn, splat2(-1.f), b1));    // + V
+    const float2 q = __ffma2_rn(vn, __ffma2_rn(th, th, splat2(-1.f)), th);      // th + V (1 - th^2) = 2 GELU' - 1
+    return __ffma2_rn(dg, q, dg);
 }
 
 // 2 GELU(x) and 2 GELU'(x) of the same elements through ONE tanh.approx each (the weight gradients need both): the tanh
@@ -387,28 +387,50 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
         // dp = dfeat (.) 1[feat > 0] of one token row as the A operand [dp_hi | dp_lo] of the dg product: the two bf16 halves
         // of every value, so that dg is exact to ~2^-17.  DP = 6: the two slots share one block (K columns 16 slot ..);
         // DP = 12: one block per slot.  The producer runs up to two units ahead of the dg products.
+        // A row's loads are issued kAhead units before their use, and the row two units behind those is asked for in L2: with one round trip
+        // to DRAM per unit the last of the four warps set the kernel's pace (its tile came 1200 to 2300 cycles into a unit of 2500; two maps,
+        // 12 x 32760 tokens, 85 -> 78 us).  More units in registers would spill (72 per thread).
         const int row = tid - kPbDpWarp0 * 32;
         const uint32_t dpblk = smem_u32(smem + Cfg::kOffDp);
-        for (int unit = 0; unit < nunits; ++unit) {
-            const int it = unit / NMAPS, m = unit % NMAPS, slot = unit & 1;
+        constexpr int kAhead = DP == 6 ? 2 : 1;
+        float2 fr[kAhead][DP / 2], gr[kAhead][DP / 2];
+        auto offset = [&](int unit) {
+            const int it = unit / NMAPS, m = unit % NMAPS;
             long long grow = (t0 + it) * kTileTokens + row;
-            const bool live = grow < rows;
-            grow = live ? grow : rows - 1;
-            size_t off;
-            if (KSIDE) {
-                const uint32_t bh = (uint32_t)grow / (uint32_t)N, n = (uint32_t)grow - bh * (uint32_t)N;   // rows < 2^31 (checked on the host)
-                off = (((size_t)bh * NMAPS + m) * N + n) * DP;
-            } else {
-                off = (size_t)grow * DP;
+            grow = grow < rows ? grow : rows - 1;
+            if (!KSIDE) return (size_t)grow * DP;
+            const uint32_t bh = (uint32_t)grow / (uint32_t)N, n = (uint32_t)grow - bh * (uint32_t)N;   // rows < 2^31 (checked on the host)
+            return (((size_t)bh * NMAPS + m) * N + n) * DP;
+        };
+        auto fetch = [&](int unit, float2 (&f)[DP / 2], float2 (&g)[DP / 2]) {
+            const size_t off = offset(unit);
+#pragma unroll
+            for (int i = 0; i < DP / 2; ++i) {
+                f[i] = ld_early(feat + off + 2 * i);
+                g[i] = ld_early(dfeat + off + 2 * i);
             }
+            if (unit + 2 < nunits) {
+                const size_t next = offset(unit + 2);
+                prefetch_l2(feat + next);
+                prefetch_l2(dfeat + next);
+            }
+        };
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k)
+            if (k < nunits) fetch(k, fr[k], gr[k]);
+        for (int u0 = 0; u0 < nunits && ok; u0 += kAhead)
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            const int unit = u0 + k, slot = unit & 1;
+            if (unit >= nunits || !ok) break;
+            const bool live = (t0 + unit / NMAPS) * kTileTokens + row < rows;
             float d[DP];
 #pragma unroll
             for (int i = 0; i < DP / 2; ++i) {
-                const float2 f = __ldg(reinterpret_cast<const float2*>(feat + off) + i);
-                const float2 g = __ldg(reinterpret_cast<const float2*>(dfeat + off) + i);
-                d[2 * i] = (live && f.x > 0.f) ? g.x : 0.f;
-                d[2 * i + 1] = (live && f.y > 0.f) ? g.y : 0.f;
+                d[2 * i] = (live && fr[k][i].x > 0.f) ? gr[k][i].x : 0.f;
+                d[2 * i + 1] = (live && fr[k][i].y > 0.f) ? gr[k][i].y : 0.f;
             }
+            if (unit + kAhead < nunits) fetch(unit + kAhead, fr[k], gr[k]);
             uint32_t w[DP];      // [hi pairs | lo pairs]
 #pragma unroll
             for (int i = 0; i < DP / 2; ++i) {
@@ -416,8 +438,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
                 w[i] = pack_bf16(d[2 * i], d[2 * i + 1]);
                 w[DP / 2 + i] = pack_bf16(l0, l1);
             }
-            if (ok && !mbar_wait(&dp_free[slot], ((unit >> 1) & 1) ^ 1)) { ok = false; report_timeout(status, 611); }
-            if (!ok) break;
+            if (!mbar_wait(&dp_free[slot], ((unit >> 1) & 1) ^ 1)) { ok = false; report_timeout(status, 611); break; }
             if constexpr (DP == 6) {
                 st_shared_v4(dpblk + sw128_off(row, 2 * slot), w[0], w[1], w[2], w[3]);
                 st_shared_v4(dpblk + sw128_off(row, 2 * slot + 1), w[4], w[5], 0u, 0u);
