@@ -25,6 +25,13 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
     return pred != 0;
 }
+// The same for a warp with a second loop for one other thread: which lane is elected is not specified, so the other one is found from
+// `leader`, the elected lane's index (in every lane), and not from a lane number.
+__device__ __forceinline__ bool elect_one(int& leader) {
+    uint32_t pred;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync %1|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred), "=r"(leader));
+    return pred != 0;
+}
 
 // ---- registers per thread ------------------------------------------------------------
 // Registers per thread of the calling group of four warps (all four execute it; a multiple of 8): a group that needs few

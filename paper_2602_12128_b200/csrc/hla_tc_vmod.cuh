@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(kVfThreads, 1) tc_vmlp_forward_kernel(const __
 }
 
 // ---- backward of one map (input gradient) ---------------------------------------------------------------------------
-// warp 0: TMA (lane 0: weights and X tiles, lane 1: dOut and Yother tiles), warp 1: dg and dxhat MMAs, warp 2: h MMAs, warps
+// warp 0: TMA (the elected lane: weights and X tiles, its neighbour: dOut and Yother tiles), warp 1: dg and dxhat MMAs, warp 2: h MMAs, warps
 // 3..18: GELU' (thread = token row x quarter of the hidden units), warps 19..22: dy = dOut (.) Yother, row statistics and the residual, warps 23..26: LayerNorm backward,
 // warp 27: TMA stores.
 // Shared-memory tiles: X (two stages, kept until the tile's output is formed: the LayerNorm backward needs xhat; the result
@@ -536,7 +536,9 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
     bool ok = true;
 
     if (warp == 0) {
-        if (elect_one() && ntiles > 0) {
+        int leader;
+        const bool first = elect_one(leader);
+        if (first && ntiles > 0) {
             mbar_arrive_expect_tx(w_full, 2 * Cfg::kWBytes + Cfg::kAuxBytes);
             for (int b = 0; b < DV / 64; ++b) {
                 tma_load_2d(smem + Cfg::kOffW1 + b * (DV * 128), &mapW1, w_full, b * 64, 0);
@@ -550,7 +552,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) tc_vmlp_backward_kernel(const _
                 for (int b = 0; b < DV / 64; ++b)
                     tma_load_2d(smem + Cfg::kOffX + st * Cfg::kXBytes + b * kBlk, &mapX, &x_full[st], b * 64, (int)((t0 + it) * kTileTokens));
             }
-        } else if (lane == 1) {
+        } else if (lane == (leader ^ 1)) {
             // dOut and Yother tiles: free once the dg product of the previous tile has read dy and the dy warps are done with dOut
             for (int it = 0; it < ntiles; ++it) {
                 if (it > 0 && !(mbar_wait(dy_empty, (it - 1) & 1) && mbar_wait(do_free, (it - 1) & 1))) { report_timeout(status, 1205); break; }
