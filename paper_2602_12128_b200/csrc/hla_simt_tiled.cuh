@@ -139,8 +139,11 @@ template <int R> __device__ __forceinline__ void tile_nn_packed(float (&acc)[R][
     }
 }
 // The contraction of tile_nt below into a tile that starts at zero, even and odd k summed apart in packed instructions: half the issue
-// slots, which the loads need, at the price of twice the accumulators.  Feature gradients of a step of 12 heads x 3000 tokens, d = 64: the step 263
-// -> 259 us; in the networks' backward, which keeps a dX tile besides, 94 -> 100 us.
+// slots, which the loads need, at the price of twice the accumulators.  Feature gradients of both sides, 12 heads x 3000 tokens, tile_nt -> this:
+// d = 64 45 -> 43.5 us (F = 3), 66 -> 60 (F = 2), d = 128 78 -> 74, 95 -> 89; 12 x 2000, d = 96, 63.5 -> 57.5, 70.5 -> 64.  Not up to d = 32, where the
+// registers of the two warps of a block decide how many blocks an SM holds (96 -> 158 with F = 3, 167 -> 219 with F = 2; 7 -> 6 and 5 -> 4 blocks): 40
+// heads x 3000, d = 32, 76.6 -> 84.4 and 107 -> 119 us, the steps 423 -> 427.5 and 481 -> 492.5; 12 heads, d = 16, F = 2, the step 174.4 -> 182.4.
+// Not in the networks' backward either, which keeps a dX tile besides: 94 -> 100 us.
 template <int CG, int JN, int R> __device__ __forceinline__ void tile_nt_packed(float (&acc)[R][JN], const float* A, int lda, const float* B, int ldb, int K) {
     float2 p[R][JN];
 #pragma unroll
@@ -506,7 +509,15 @@ __global__ void __launch_bounds__(CG * 8) tiled_feature_grad_kernel(Dims D, cons
     stage_values<CG, T, QSIDE>(Xs, LD, xz, X, O, eta, D, bh, tok0, TM, D.N);
     __syncthreads();
     float acc[R][JN];
-    tile_nt_packed<CG, JN, R>(acc, Xs + tg * LD, LD, Ss + cg * LD, LD, D.d);
+    if constexpr (CG == 8) {      // d <= 32
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < JN; ++j) acc[i][j] = 0.f;
+        tile_nt<CG, JN, R>(acc, Xs + tg * LD, LD, Ss + cg * LD, LD, D.d);
+    } else {
+        tile_nt_packed<CG, JN, R>(acc, Xs + tg * LD, LD, Ss + cg * LD, LD, D.d);
+    }
 #pragma unroll
     for (int j = 0; j < JN; ++j) {
         const int m = cg + CG * j;
