@@ -387,13 +387,13 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
         // dp = dfeat (.) 1[feat > 0] of one token row as the A operand [dp_hi | dp_lo] of the dg product: the two bf16 halves
         // of every value, so that dg is exact to ~2^-17.  DP = 6: the two slots share one block (K columns 16 slot ..);
         // DP = 12: one block per slot.  The producer runs up to two units ahead of the dg products.
-        // A row's loads are issued kAhead units before their use, and the row two units behind those is asked for in L2: with one round trip
-        // to DRAM per unit the last of the four warps set the kernel's pace (its tile came 1200 to 2300 cycles into a unit of 2500; two maps,
-        // 12 x 32760 tokens, 85 -> 78 us).  More units in registers would spill (72 per thread).
+        // A row's loads are issued a unit before their use.  The wider rows of the two-factor key side come from DRAM too late even so, and the row
+        // three units on is asked for in L2 then (the first sector of its 48 bytes; two maps, 12 x 32760 tokens: loads at their use 85.6 us,
+        // a unit ahead 82, with the prefetch 81.6, at 1.93 GHz 75.6 and 71.9).  Elsewhere the prefetch and a second row in registers cost more than they
+        // hide: 48 x 32760 tokens, d = 128, three maps 412 us at the use, 409 a unit ahead, 417 with both, one map 201, 197 and 204.
         const int row = tid - kPbDpWarp0 * 32;
         const uint32_t dpblk = smem_u32(smem + Cfg::kOffDp);
-        constexpr int kAhead = DP == 6 ? 2 : 1;
-        float2 fr[kAhead][DP / 2], gr[kAhead][DP / 2];
+        float2 fr[DP / 2], gr[DP / 2];
         auto offset = [&](int unit) {
             const int it = unit / NMAPS, m = unit % NMAPS;
             long long grow = (t0 + it) * kTileTokens + row;
@@ -402,35 +402,30 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
             const uint32_t bh = (uint32_t)grow / (uint32_t)N, n = (uint32_t)grow - bh * (uint32_t)N;   // rows < 2^31 (checked on the host)
             return (((size_t)bh * NMAPS + m) * N + n) * DP;
         };
-        auto fetch = [&](int unit, float2 (&f)[DP / 2], float2 (&g)[DP / 2]) {
+        auto fetch = [&](int unit) {
             const size_t off = offset(unit);
 #pragma unroll
             for (int i = 0; i < DP / 2; ++i) {
-                f[i] = ld_early(feat + off + 2 * i);
-                g[i] = ld_early(dfeat + off + 2 * i);
+                fr[i] = ld_early(feat + off + 2 * i);
+                gr[i] = ld_early(dfeat + off + 2 * i);
             }
-            if (unit + 2 < nunits) {
+            if (KSIDE && DP == 12 && unit + 2 < nunits) {
                 const size_t next = offset(unit + 2);
                 prefetch_l2(feat + next);
                 prefetch_l2(dfeat + next);
             }
         };
-#pragma unroll
-        for (int k = 0; k < kAhead; ++k)
-            if (k < nunits) fetch(k, fr[k], gr[k]);
-        for (int u0 = 0; u0 < nunits && ok; u0 += kAhead)
-#pragma unroll
-        for (int k = 0; k < kAhead; ++k) {
-            const int unit = u0 + k, slot = unit & 1;
-            if (unit >= nunits || !ok) break;
+        if (nunits > 0) fetch(0);
+        for (int unit = 0; unit < nunits; ++unit) {
+            const int slot = unit & 1;
             const bool live = (t0 + unit / NMAPS) * kTileTokens + row < rows;
             float d[DP];
 #pragma unroll
             for (int i = 0; i < DP / 2; ++i) {
-                d[2 * i] = (live && fr[k][i].x > 0.f) ? gr[k][i].x : 0.f;
-                d[2 * i + 1] = (live && fr[k][i].y > 0.f) ? gr[k][i].y : 0.f;
+                d[2 * i] = (live && fr[i].x > 0.f) ? gr[i].x : 0.f;
+                d[2 * i + 1] = (live && fr[i].y > 0.f) ? gr[i].y : 0.f;
             }
-            if (unit + kAhead < nunits) fetch(unit + kAhead, fr[k], gr[k]);
+            if (unit + 1 < nunits) fetch(unit + 1);
             uint32_t w[DP];      // [hi pairs | lo pairs]
 #pragma unroll
             for (int i = 0; i < DP / 2; ++i) {
