@@ -289,7 +289,12 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
             if (!good) report_timeout(status, 602);
         }
     } else if (warp == 1) {
-        if (elect_one() && ntiles > 0) {
+        // One map, d = 128: a thread found by its lane number, whose products go out 240 cycles apart.  From an elected thread, 64 apart, this side
+        // takes 6 % longer (48 x 32760 tokens 186 -> 198 us, 24 x 32760 97.4 -> 102.5, two factors 12 x 32760 53.9 -> 55.3; causal step 1062 -> 1071 us);
+        // the reason is not known: without the wait for dg above, or with dg issued behind dX, it takes 229 and 227 us.  At d = 64 the elected thread is
+        // the better one (step of 24 heads x 4096 tokens 80.0 against 82.2 us), and with several maps per tile everywhere.
+        const bool one = NMAPS == 1 && DV == 128 ? lane == 0 : elect_one();
+        if (one && ntiles > 0) {
             const uint32_t idesc_dg = idesc_bf16(128, DV, false, true);  // dg = dp (K-major) * W2^T (MN-major)
             const uint32_t idesc2 = idesc_bf16(128, DV, false, false);   // dX = dh (TMEM) * W1 as [in][hidden] (K-major)
             const uint64_t pd0 = smem_desc_sw128(smem_u32(smem + Cfg::kOffDp), 16, 1024);
