@@ -392,10 +392,11 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
         // dp = dfeat (.) 1[feat > 0] of one token row as the A operand [dp_hi | dp_lo] of the dg product: the two bf16 halves
         // of every value, so that dg is exact to ~2^-17.  DP = 6: the two slots share one block (K columns 16 slot ..);
         // DP = 12: one block per slot.  The producer runs up to two units ahead of the dg products.
-        // A row's loads are issued a unit before their use.  The wider rows of the two-factor key side come from DRAM too late even so, and the row
-        // three units on is asked for in L2 then (the first sector of its 48 bytes; two maps, 12 x 32760 tokens: loads at their use 85.6 us,
-        // a unit ahead 82, with the prefetch 81.6, at 1.93 GHz 75.6 and 71.9).  Elsewhere the prefetch and a second row in registers cost more than they
-        // hide: 48 x 32760 tokens, d = 128, three maps 412 us at the use, 409 a unit ahead, 417 with both, one map 201, 197 and 204.
+        // A row's loads are issued a unit before their use.  Where that is too late, on the key side with two maps (48-byte rows) or d = 64 (short
+        // units), the row three units on is also asked for in L2 (the first sector of its 24 or 48 bytes): two maps, 12 x 32760 tokens, d = 128, loads at
+        // their use 85.6 us, a unit ahead 82.2, with the prefetch 81.5 (at 1.93 GHz 75.6 and 71.9); three maps, 48 x 32760, d = 64, 271 and 228.
+        // Elsewhere the prefetch and a second row in registers cost more than they hide: 48 x 32760 tokens, d = 128, three maps 412 us at
+        // the use, 409 a unit ahead, 417 with both, one map 201, 197 and 204.
         const int row = tid - kPbDpWarp0 * 32;
         const uint32_t dpblk = smem_u32(smem + Cfg::kOffDp);
         float2 fr[DP / 2], gr[DP / 2];
@@ -414,7 +415,7 @@ __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __
                 fr[i] = ld_early(feat + off + 2 * i);
                 gr[i] = ld_early(dfeat + off + 2 * i);
             }
-            if (KSIDE && DP == 12 && unit + 2 < nunits) {
+            if (KSIDE && (DP == 12 || DV == 64) && unit + 2 < nunits) {
                 const size_t next = offset(unit + 2);
                 prefetch_l2(feat + next);
                 prefetch_l2(dfeat + next);
