@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(kRoThreads, 1) tc_readout_kernel(const __grid_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 10);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 11);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int tiles_per_head = (N + kTileTokens - 1) / kTileTokens;
     const long long total = (long long)BH * tiles_per_head;
     const int w0 = (int)(total * blockIdx.x / gridDim.x), w1 = (int)(total * (blockIdx.x + 1) / gridDim.x);
@@ -851,8 +851,8 @@ __global__ void __launch_bounds__(kRoThreads, 1) tc_readout_kernel(const __grid_
 // (column d = deta/r, the rest zero).  Accumulator row 8+m then holds dCsym[m][0..d-1], dzsym[m], 0, 0, 0: one row of
 // the partial state, and dz costs no product of its own.  Rows 0..7 of the accumulator are not used.
 //
-// The tensor pipe needs ~100 cycles per MMA of this size (set by the operand bytes it reads from shared memory, not by
-// the arithmetic), so the MMAs per tile are kept at 16 and are issued by two threads (D2: warp 1, dC: warp 2).
+// The MMAs of a tile followed one another every ~100 cycles in this kernel when one thread issued 24 of them; they are 16 now, issued by two
+// threads (D2: warp 1, dC: warp 2).  (Alone and back to back, products of 128 x 64 take 48 cycles and of 128 x 128 64.)
 // =======================================================================================
 constexpr int kBqGroups = 3;                            // generator groups of 128 threads; tile `it` belongs to group it % 3
 constexpr int kBqThreads = 128 + 128 * kBqGroups;       // warp 0: TMA, warp 1: D2 MMAs, warp 2: dC MMAs, warp 3 idle, warps 4..: generators

@@ -20,10 +20,10 @@
 // the two MMA-issuing threads and the barrier protocol are those of the forward sweep.
 //
 // Warp roles: 0 TMA (X and Y tiles), 2 MMA issue (Sc), 1 MMA issue (readout, Sm * W), 3 MMA issue (state), 4..7 operand
-// rows W, 8..15 mask, 16..19 state image, 20..23 and 24..27 epilogue (two groups, alternate tiles).  A lone thread needs
-// well over a hundred cycles per product it issues, more than the product takes, so the 32 products of a tile are spread
-// over three threads; Sc has two buffers in tensor memory (by tile parity), which lets the Sc product and the mask of the
-// next tile run while the readout of this one is still being issued.
+// rows W, 8..15 mask, 16..19 state image, 20..23 and 24..27 epilogue (two groups, alternate tiles).  The 32 products of a tile
+// are spread over three threads; Sc has two buffers in tensor memory (by tile parity), which lets the Sc product and the mask of the
+// next tile run while the readout of this one is still being issued.  (The split was made when a thread issued a product every 240
+// cycles; from an elected thread, 64 apart, it has not been measured against fewer threads.)
 #pragma once
 #include "hla_tc_causal.cuh"
 

@@ -41,8 +41,9 @@ __device__ __forceinline__ __nv_bfloat16 half_bf16(__nv_bfloat16 w) { return __f
 // exact derivative (fit_gelu_tanh.py, which prints twice C0 and C1: |error| < 1.5e-4, 3.8e-5 in the mean square over N(0,1), before the 2^-11 relative error of
 // tanh.approx; < 1.3e-3 with it).  Evaluated as dg + dg (th + V (1 - th^2)) with -V so that every step is one packed multiply or fma: eight
 // packed and two special-function instructions per pair of elements.  Sixteen warps alone on an SM take 1280 cycles for a 128 x 128 tile,
-// bound by the FMA pipe; as 1 + V + th (1 - V th) it was nine instructions and 1376 cycles, and V cancelled against itself for large |x|.  (A
-// linear inner derivative, C1 = 0, saves one or two more, but its mean-square error is 8.6e-5: errors of gradients against 64 bits grew by
+// bound by the FMA pipe; as 1 + V + th (1 - V th) it was nine instructions and 1376 cycles, and V cancelled against itself for large |x|; the
+// kernels with it take 1 % less (three maps, 48 x 32760 tokens, 626 -> 619 thousand cycles, backward of the value maps 178 -> 175).  (A
+// linear inner derivative, C1 = 0, saves one more, but its mean-square error is 8.6e-5: errors of gradients against 64 bits grew by
 // up to 0.6 %.)
 constexpr float kGradA = 0.69631102f, kGradB = 0.02936904f, kGradC0 = 0.89902785f, kGradC1 = -0.010848315f;
 __device__ __forceinline__ float2 times_gelu_grad2(float2 dg, float2 x) {
@@ -109,11 +110,11 @@ struct PhiMaps {
 // =======================================================================================
 // Backward of the feature networks with respect to their input (weights fixed):
 //   dp  = dfeat (.) 1[feat > 0]                 ReLU mask from the features the forward kept
-//   dg  = dp * W2^T                             6 FMAs per hidden unit on the ALUs
+//   dg  = dp * W2^T                             tensor cores, dp split into two bf16 halves
 //   dh  = dg (.) GELU'(h),  h = X W1 + b1       h recomputed on the tensor cores
 //   dX  = sum over the maps of dh * W1^T        tensor cores, accumulated over the maps in TMEM
 // Per 128-token tile: X is TMA-loaded once, every map's h goes through TMEM, the dh tile is
-// written as the second MMA's A operand, and the W1 image in shared memory serves both MMAs
+// written over h in TMEM as the second MMA's A operand, and the W1 image in shared memory serves both MMAs
 // (MN-major B for X W1, K-major B for dh W1^T).
 // =======================================================================================
 struct PhiBwdPtrs {
@@ -163,8 +164,8 @@ template <int DV, int NMAPS, int DP> struct PbCfg {
 //   dg = [dp_hi | dp_lo] * [W2^T; W2^T]  [128 x DV], K = 16: dp = dfeat (.) 1[feat > 0] split into two bf16 halves, so dg is exact to ~2^-17
 //   dX += dh * W1^T                     [128 x DV], K = DV,  dh = dg (.) GELU'(h + b1) formed by the 16 epilogue warps
 // h and the dh tile are double-buffered; dg is taken into registers at the start of a unit so that the next unit's dg
-// product overlaps this unit's arithmetic; the dX accumulator of a tile is drained one unit late, straight from
-// registers to global memory.  The epilogue threads also write the dp tiles (one feature pair each, one unit ahead).
+// product overlaps this unit's arithmetic; the dX accumulator of a tile is drained by warps of its own through a staging tile and a
+// TMA store, and warps of their own write the dp tiles ahead of the dg products (the list of the warps is above).
 template <int DV, int NMAPS, bool KSIDE, int DP>
 __global__ void __launch_bounds__(kPbThreads, 1) tc_phi_backward_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ PhiMaps maps,
                                                                         const __grid_constant__ CUtensorMap mapdX, PhiBwdPtrs P,

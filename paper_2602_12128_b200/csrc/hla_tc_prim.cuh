@@ -17,9 +17,9 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // a wait gives up 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 // True in exactly one lane of a converged warp.  Code that a single thread runs (TMA and MMA issue loops) is entered through this
-// instead of `lane == 0`: the compiler then knows the region has one active thread.  Without that every tcgen05.mma is wrapped in a loop
-// over the active lanes that makes its descriptors uniform: 240 to 270 cycles from one product to the next for a lone thread, against
-// 64 (128 x 128 x 16, operands in shared memory) or 9 (128 x 16 x 16, A in TMEM), which is the products' own time.
+// instead of `lane == 0`: the compiler then knows the region has one active thread.  Without that a lone thread takes 240 to 270 cycles
+// from one tcgen05.mma to the next (presumably for making its operands uniform lane by lane), against 64 (128 x 128 x 16, operands in
+// shared memory) or 9 (128 x 16 x 16, A in TMEM), which is the products' own time.
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
