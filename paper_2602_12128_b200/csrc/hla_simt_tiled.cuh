@@ -106,8 +106,9 @@ template <int R> __device__ __forceinline__ void tile_nn(float (&acc)[R][4], con
     }
 }
 // The same (bit for bit) in packed instructions on pairs of columns: a multiplier is copied into both halves of a register pair, which leaves three
-// issue slots where four single fmas were (the loads need them).  Two feature networks forward, 12 heads x 3000 tokens, d = 64: 64.7 -> 62.6 us; in
-// their backward, which is short of registers, 94.3 -> 95.7, and the readout is the same either way.
+// issue slots where four single fmas were (the loads need them).  Feature networks forward, 12 heads x 3000 tokens, d = 64: 64.7 -> 62.6 us; in
+// their backward, which is short of registers, 94.3 -> 95.7, and the readout is the same either way.  The forward call, 12 x 3000: d = 64 110.2 ->
+// 107.1 us, 32 72.7 -> 70.0, 16 64.3 -> 62.0; up to d = 32 its two launches, which overlap, can also fit together worse: 12 x 4096, d = 32, 87.0 -> 89.6.
 template <int R> __device__ __forceinline__ void tile_nn_packed(float (&acc)[R][4], const float* A, int lda, const float* B, int ldb, int K) {
     float2 p[R][2];
 #pragma unroll
